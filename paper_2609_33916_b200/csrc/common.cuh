@@ -220,10 +220,16 @@ cudaError_t mat_bwd(const Problem &p, const void *Q, const void *K, const void *
 
 // ---- SIMT fp32 path (simt_kernels.cu) -------------------------------------------------
 // dtype: MOA_BF16 or MOA_F32 storage; arithmetic is fp32 FMA throughout.
+// What the forward of a fused call prepares for its backward (all null for a plain forward): D = rowsum(dO o O) [B*H, n]
+// from the fp32 O it holds, and the cleared dQ accumulator [B*H, n, d] (null: not wanted).
+struct SimtPrep {
+    const void *dO = nullptr;
+    float *Dv = nullptr, *dQzero = nullptr;
+};
 cudaError_t simt_fwd(const Problem &p, int dtype, const void *Q, const void *K, const void *V,
-                     void *O, float *L, cudaStream_t st);
-// D_i = sum_k dO_ik O_ik
-cudaError_t row_dot(const Problem &p, int dtype, const void *dO, const void *O, float *Dv, cudaStream_t st);
+                     void *O, float *L, const SimtPrep &pr, cudaStream_t st);
+// D_i = sum_k dO_ik O_ik; dQzero (may be null): fp32 [B*H, n, d] to clear
+cudaError_t row_dot(const Problem &p, int dtype, const void *dO, const void *O, float *Dv, float *dQzero, cudaStream_t st);
 // dK, dV always; dQ contributions are atomically added into dQacc (fp32 [B,H,n,d], pre-zeroed)
 // when dQacc != nullptr.
 cudaError_t simt_bwd_kv(const Problem &p, int dtype, const void *Q, const void *K, const void *V,

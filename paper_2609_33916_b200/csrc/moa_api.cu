@@ -274,11 +274,11 @@ moa_status run_materialized(const moa_attn_desc *d, const void *Q, const void *K
 }
 
 moa_status run_fwd(const moa_attn_desc *d, const void *Q, const void *K, const void *V, void *O, float *L,
-                   const FwdForBwd &fb, cudaStream_t st)
+                   const FwdForBwd &fb, const SimtPrep &sp, cudaStream_t st)
 {
-    // fb: what the tensor-core forward of a fused call prepares for its backward (empty otherwise)
+    // fb, sp: what the forward of a fused call prepares for its backward (empty otherwise)
     const cudaError_t e = use_tc_fwd(d) ? tc_fwd(to_problem(d), Q, K, V, O, L, fb, st)
-                             : simt_fwd(to_problem(d), d->dtype, Q, K, V, O, L, st);
+                             : simt_fwd(to_problem(d), d->dtype, Q, K, V, O, L, sp, st);
     return e == cudaSuccess ? MOA_OK : MOA_ERR_CUDA;
 }
 
@@ -309,13 +309,13 @@ moa_status run_bwd(const moa_attn_desc *d, const void *Q, const void *K, const v
         else MOA_TRY(convert_f32_to_bf16(dQacc, dQ, elems, p.scale, st));
         return MOA_OK;
     }
-    MOA_TRY(row_dot(p, d->dtype, dO, O, Dv, st));
-    if (mode == MOA_DQ_SEPARATE_PASS) {
+    const bool separate = mode == MOA_DQ_SEPARATE_PASS;
+    float *acc = separate ? nullptr : d->dtype == MOA_F32 ? (float *)dQ : dQacc;   // fp32 output accumulates in place
+    if (!prepared) MOA_TRY(row_dot(p, d->dtype, dO, O, Dv, acc, st));
+    if (separate) {
         MOA_TRY(simt_bwd_kv(p, d->dtype, Q, K, V, dO, L, Dv, dK, dV, nullptr, st));
         MOA_TRY(simt_bwd_dq(p, d->dtype, Q, K, V, dO, L, Dv, dQ, st));
     } else {
-        float *acc = d->dtype == MOA_F32 ? (float *)dQ : dQacc;   // fp32 output accumulates in place
-        MOA_TRY(cudaMemsetAsync(acc, 0, elems * sizeof(float), st));
         MOA_TRY(simt_bwd_kv(p, d->dtype, Q, K, V, dO, L, Dv, dK, dV, acc, st));
         if (d->dtype == MOA_BF16) MOA_TRY(convert_f32_to_bf16(dQacc, dQ, elems, 1.f, st));
     }
@@ -388,7 +388,7 @@ moa_status moa_attn_fwd(const moa_attn_desc *desc, const void *Q, const void *K,
     if ((s = check_arch()) != MOA_OK) return s;
     if (desc->materialize)
         return run_materialized(desc, Q, K, V, nullptr, O, L, nullptr, nullptr, nullptr, ws, false, (cudaStream_t)stream);
-    return run_fwd(desc, Q, K, V, O, L, FwdForBwd{}, (cudaStream_t)stream);
+    return run_fwd(desc, Q, K, V, O, L, FwdForBwd{}, SimtPrep{}, (cudaStream_t)stream);
 }
 
 moa_status moa_attn_bwd(const moa_attn_desc *desc, const void *Q, const void *K, const void *V,
@@ -456,8 +456,18 @@ moa_status moa_attn_fused_fwd_bwd(const moa_attn_desc *desc, const void *Q, cons
         fb.dO = dO;
         if (w.dqacc_bytes) fb.zero_acc = (float *)((char *)ws + w.d_bytes + w.lp_bytes);
     }
-    if ((s = run_fwd(desc, Q, K, V, O, L, fb, (cudaStream_t)stream)) != MOA_OK) return s;
-    return run_bwd(desc, Q, K, V, O, L, dO, dQ, dK, dV, ws, both_tc, (cudaStream_t)stream);
+    // CUDA-core path: D and the cleared accumulator come out of the forward as well
+    SimtPrep sp;
+    const bool both_simt = !use_tc_fwd(desc) && !use_tc_bwd(desc);
+    if (both_simt) {
+        const BwdWorkspace w = bwd_workspace(desc);
+        sp.dO = dO;
+        sp.Dv = (float *)ws;
+        if (resolved_dq_mode(desc) != MOA_DQ_SEPARATE_PASS)
+            sp.dQzero = desc->dtype == MOA_F32 ? (float *)dQ : (float *)((char *)ws + w.d_bytes + w.lp_bytes);
+    }
+    if ((s = run_fwd(desc, Q, K, V, O, L, fb, sp, (cudaStream_t)stream)) != MOA_OK) return s;
+    return run_bwd(desc, Q, K, V, O, L, dO, dQ, dK, dV, ws, both_tc || both_simt, (cudaStream_t)stream);
 }
 
 moa_status moa_attn_fused_rowparallel(const moa_attn_desc *desc, const void *Q, const void *K, const void *V,

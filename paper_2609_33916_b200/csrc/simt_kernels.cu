@@ -1,11 +1,14 @@
 // fp32 SIMT kernels: the MOA_F32 path, and a generic path for any dtype/shape.
 //
-// Tiles of 64 query rows x 64 keys, 256 threads as a 16 x 16 grid; thread (ty,tx)
-// owns score rows ty*4..ty*4+3 and score columns tx, tx+16, tx+32, tx+48, and the
-// output columns tx+16c.  Online softmax in the forward; the backward recomputes P
-// from the stored logsumexp, one CTA per key tile (each dK/dV element has exactly
-// one writer), dQ either by fp32 atomics or by a separate query-parallel kernel.
+// Online softmax in the forward; the backward recomputes P from the stored logsumexp,
+// one CTA or cluster per key tile (each dK/dV element has exactly one writer), dQ either
+// by fp32 atomics or by a separate query-parallel kernel.  The forward and the key-parallel
+// backward are register-tiled (below); the two comparison variants (the query-parallel dQ
+// pass and the row-parallel single kernel) keep plain tiles of 64 query rows x 64 keys,
+// 256 threads as a 16 x 16 grid; thread (ty,tx) owns score rows ty*4..ty*4+3 and score
+// columns tx, tx+16, tx+32, tx+48, and the output columns tx+16c.
 #include "common.cuh"
+#include "ptx.cuh"
 #include <math.h>
 
 namespace moa {
@@ -40,122 +43,381 @@ __device__ __forceinline__ float group16_sum(float v)
     return v;
 }
 
-// ------------------------------------------------------------------------- forward
-template <typename T, int D>
-__global__ void __launch_bounds__(NTHREADS)
-simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
-                T *__restrict__ O, float *__restrict__ L, int n, int causal, float scale, int nqt)
-{
-    constexpr int LD = D + 1;
-    constexpr int NC = D / 16;
-    extern __shared__ float smem[];
-    float *Qs = smem, *Ks = Qs + BM * LD, *Vs = Ks + BN * LD, *Ss = Vs + BN * LD;
+// ---------------------------------------------------------- register-tiled kernels: shared pieces
+// What bounds the two kernels below is the FMA pipe (fp32 in, fp32 accumulate: no tensor-core form keeps 24 bits), so
+// everything is arranged to feed it from as few instructions as possible:
+//   * the products run on packed pairs (fma.rn.f32x2: one instruction for two multiply-adds), operands come from shared
+//     memory 16 bytes at a time, a thread computes R x 4 or more outputs: 3 loads per 16 packed multiply-adds at R = 8;
+//   * a contraction over d reads both operands along their rows and keeps even and odd partial sums in the two halves of
+//     a pair; a contraction over keys or queries packs two neighbouring rows of the output, so one operand is a pair as it
+//     lies in memory and the other a duplicated scalar;
+//   * rows are padded by 16 bytes: the 16 lanes that read 16 rows at one column fall on different banks;
+//   * P (and dS) go through shared memory only between the lanes of one warp, and the loads of the next tile are
+//     asynchronous and run under the product that does not need their buffer;
+//   * a CTA cluster shares one output tile when there are fewer tiles than the chip has room for: the ranks take the tiles
+//     of the other axis in turn, and their partial results are added through distributed shared memory, in rank order.
+constexpr int SNT = 128;         // threads per CTA: lane tx = tid % 16 along columns, ty = tid / 16 along rows
+constexpr int STY = SNT / 16;
 
-    int qt = blockIdx.x % nqt;
-    const int bh = blockIdx.x / nqt;
+__device__ __forceinline__ void cp_async16(float *dst, const float *src, bool live)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    const int bytes = live ? 16 : 0;      // 0: zero-filled
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// ROWS x D tile of src (row row0 first, rows past n zero) into padded rows of D + 4 floats.  fp32: asynchronous copies, to
+// be committed by the caller; bf16: widened on the way.
+template <typename T, int ROWS, int D>
+__device__ __forceinline__ void tile_in(float *dst, const T *src, int row0, int n)
+{
+    constexpr int V = 16 / (int)sizeof(T), PER_ROW = D / V;
+#pragma unroll
+    for (int it = 0; it < ROWS * PER_ROW / SNT; ++it) {
+        const int idx = it * SNT + threadIdx.x, r = idx / PER_ROW, c = (idx % PER_ROW) * V;
+        const bool live = row0 + r < n;
+        const T *from = src + (size_t)(live ? row0 + r : 0) * D + c;
+        float *to = dst + r * (D + 4) + c;
+        if (sizeof(T) == 4) {
+            cp_async16(to, reinterpret_cast<const float *>(from), live);
+        } else {
+            uint4 u = make_uint4(0, 0, 0, 0);
+            if (live) u = *reinterpret_cast<const uint4 *>(from);
+            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+            float f[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {      // bf16 -> fp32 is a shift
+                f[2 * i] = __uint_as_float(w[i] << 16);
+                f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+            }
+            *reinterpret_cast<float4 *>(to) = make_float4(f[0], f[1], f[2], f[3]);
+            *reinterpret_cast<float4 *>(to + 4) = make_float4(f[4], f[5], f[6], f[7]);
+        }
+    }
+}
+
+// four consecutive outputs of a row
+__device__ __forceinline__ void store4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
+__device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v)
+{
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+}
+__device__ __forceinline__ float4 load4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16 *p)
+{
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
+}
+
+// out[i][b] = A[a_row0 + i][:] . B[tx + 16 b][:], contraction over D; rows of D + 4 floats
+template <int R, int NB, int D>
+__device__ __forceinline__ void dot_rows(float (&out)[R][NB], const float *A, const float *B, int a_row0, int tx)
+{
+    constexpr int LD = D + 4;
+    uint64_t acc[R][NB];
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) acc[i][b] = 0ull;
+    const float *ap = A + a_row0 * LD, *bp = B + tx * LD;
+#pragma unroll 2
+    for (int k = 0; k < D; k += 4) {
+        ulonglong2 av[R], bv[NB];
+#pragma unroll
+        for (int i = 0; i < R; ++i) av[i] = *reinterpret_cast<const ulonglong2 *>(ap + i * LD + k);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) bv[b] = *reinterpret_cast<const ulonglong2 *>(bp + 16 * b * LD + k);
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                acc[i][b] = ptx::fma_f32x2(av[i].x, bv[b].x, acc[i][b]);
+                acc[i][b] = ptx::fma_f32x2(av[i].y, bv[b].y, acc[i][b]);
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            float lo, hi;
+            ptx::unpack_f32x2(acc[i][b], lo, hi);
+            out[i][b] = lo + hi;
+        }
+}
+
+// acc[i2][c] (rows 2 i2 and 2 i2 + 1 of the thread's R rows, packed) += sum_{j < K} W[j][R rows] X[j][4 tx + 64 v + 0..3];
+// W: rows of LW floats, the thread's R rows consecutive at w0; X: rows of D + 4 floats
+template <int R, int K, int D>
+__device__ __forceinline__ void add_rows(uint64_t (&acc)[R / 2][D / 16], const float *W, int LW, int w0, const float *X, int tx)
+{
+    static_assert(R == 2 || R % 4 == 0, "a thread's rows are read 8 or 16 bytes at a time");
+    constexpr int LD = D + 4;
+    const float *wp = W + w0, *xp = X + 4 * tx;
+#pragma unroll 4
+    for (int j = 0; j < K; ++j) {
+        uint64_t wv[R / 2], xv[D / 16];
+        if (R == 2) {
+            wv[0] = *reinterpret_cast<const uint64_t *>(wp + j * LW);
+        } else {
+#pragma unroll
+            for (int i = 0; i < R / 4; ++i) {
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(wp + j * LW + 4 * i);
+                wv[2 * i] = u.x;
+                wv[2 * i + 1] = u.y;
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < D / 64; ++v) {
+            const float4 f = *reinterpret_cast<const float4 *>(xp + j * LD + 64 * v);
+            xv[4 * v] = ptx::pack_f32x2(f.x, f.x);
+            xv[4 * v + 1] = ptx::pack_f32x2(f.y, f.y);
+            xv[4 * v + 2] = ptx::pack_f32x2(f.z, f.z);
+            xv[4 * v + 3] = ptx::pack_f32x2(f.w, f.w);
+        }
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+            for (int c = 0; c < D / 16; ++c) acc[i][c] = ptx::fma_f32x2(wv[i], xv[c], acc[i][c]);
+    }
+}
+
+// rows 2 i2, 2 i2 + 1 of a packed accumulator -> two float4 of column group v
+template <int C>
+__device__ __forceinline__ void unpack_rows(const uint64_t (&acc)[C], int v, float4 &even, float4 &odd)
+{
+    ptx::unpack_f32x2(acc[4 * v], even.x, odd.x);
+    ptx::unpack_f32x2(acc[4 * v + 1], even.y, odd.y);
+    ptx::unpack_f32x2(acc[4 * v + 2], even.z, odd.z);
+    ptx::unpack_f32x2(acc[4 * v + 3], even.w, odd.w);
+}
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// address of `p` (this CTA's shared memory) in the CTA of rank r, and loads from there
+__device__ __forceinline__ uint32_t remote(const void *p, uint32_t r)
+{
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(r));
+    return d;
+}
+__device__ __forceinline__ float4 remote_f4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ float remote_f1(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// ------------------------------------------------------------------------- forward
+// CTA: BM = 8 R query rows; a warp has 2 R rows to itself, a thread R rows x 4 keys of the score tile and R rows x D / 16
+// columns of O.  The `split` ranks of a cluster take the key tiles of their rows in turn (rank r: tiles r, r + split, ...), each
+// with its own online softmax; at the end rank r merges rows r BM / split ... of all ranks' partial results.
+// In a fused call (dO != nullptr) the merge also gives D = rowsum(dO o O), from the fp32 O, and clears its rows of dQ.
+template <int R, int D>
+struct SimtFwd {
+    static constexpr int BM = STY * R, LD = D + 4, LP = 2 * R + 4;
+    static constexpr int kFloats = (BM + 2 * BN) * LD + 4 * BN * LP;      // Q, K, V, P^T of the four warps
+    static constexpr size_t kSmem = kFloats * sizeof(float);
+};
+
+template <typename T, int R, int D>
+__global__ void __launch_bounds__(SNT, R == 8 ? 3 : D == 128 ? 2 : 4)
+simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, T *__restrict__ O,
+                float *__restrict__ L, const T *__restrict__ dO, float *__restrict__ Dv, float *__restrict__ dQzero, int n,
+                int causal, float scale, int nqt, int split)
+{
+    using S = SimtFwd<R, D>;
+    constexpr int BM = S::BM, LD = S::LD, LP = S::LP, NC = D / 16;
+    extern __shared__ float smem[];
+    float *Qs = smem, *Ks = Qs + BM * LD, *Vs = Ks + BN * LD;
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, warp = tid / 32;
+    float *Pw = Vs + BN * LD + warp * BN * LP;      // this warp's P^T: [key][2 R rows]
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const int rank = split > 1 ? (int)cluster_rank() : 0;
+    const int job = (int)blockIdx.x / split;
+    int qt = job % nqt;
+    const int bh = job / nqt;
     if (causal) qt = nqt - 1 - qt;  // longest rows first
     const int q0 = qt * BM;
     const size_t base = (size_t)bh * n * D;
     Q += base; K += base; V += base; O += base; L += (size_t)bh * n;
 
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    load_tile<T, D>(Qs, Q, q0, n);
-
-    float m[4], l[4], o[4][NC];
+    float m[R], l[R];
+    uint64_t o[R / 2][NC];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        m[a] = -INFINITY; l[a] = 0.f;
+    for (int i = 0; i < R; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
 #pragma unroll
-        for (int c = 0; c < NC; ++c) o[a][c] = 0.f;
-    }
+    for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) o[i][c] = 0ull;
     const int kend = causal ? min(n, q0 + BM) : n;
-    for (int k0 = 0; k0 < kend; k0 += BN) {
+    const int step = BN * split;
+    int k0 = rank * BN;
+    if (k0 < kend) {
+        tile_in<T, BM, D>(Qs, Q, q0, n);
+        tile_in<T, BN, D>(Ks, K, k0, n);
+        cp_commit();
+        tile_in<T, BN, D>(Vs, V, k0, n);
+        cp_commit();
+    }
+    for (; k0 < kend; k0 += step) {
+        const bool more = k0 + step < kend;
+        cp_wait<1>();                 // K (and Q) are here; V may still be on its way
         __syncthreads();
-        load_tile<T, D>(Ks, K, k0, n);
-        load_tile<T, D>(Vs, V, k0, n);
+        float s[R][4];
+        dot_rows<R, 4, D>(s, Qs, Ks, ty * R, tx);
         __syncthreads();
-        float s[4][4];
+        if (more) tile_in<T, BN, D>(Ks, K, k0 + step, n);      // runs under the softmax and the P V product
+        cp_commit();
+        const bool mask = k0 + BN > n || (causal && k0 + BN - 1 > q0);
+        uint64_t al[R / 2];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) s[a][b] = 0.f;
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) {
-            float qv[4], kv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) qv[a] = Qs[(ty * 4 + a) * LD + k];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) kv[b] = Ks[(tx + 16 * b) * LD + k];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) s[a][b] = fmaf(qv[a], kv[b], s[a][b]);
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int row = q0 + ty * 4 + a;
+        for (int i = 0; i < R; ++i) {
+            const int row = q0 + ty * R + i;
             float mx = -INFINITY;
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                const int col = k0 + tx + 16 * b;
-                float v = s[a][b] * scale;
-                if (col >= n || (causal && col > row)) v = -INFINITY;
-                s[a][b] = v;
+                float v = s[i][b] * scale;
+                if (mask) {
+                    const int col = k0 + tx + 16 * b;
+                    if (col >= n || (causal && col > row)) v = -INFINITY;
+                }
+                s[i][b] = v;
                 mx = fmaxf(mx, v);
             }
             mx = group16_max(mx);
-            float mn = fmaxf(m[a], mx);
-            if (mn == -INFINITY) mn = 0.f;  // whole row masked so far (padding rows only)
-            const float alpha = expf(m[a] - mn);
+            const float mn = fmaxf(m[i], mx);
+            const float ref = mn == -INFINITY ? 0.f : mn;      // no key visible so far
+            const float alpha = expf(m[i] - ref);
             float sum = 0.f;
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                const float pv = expf(s[a][b] - mn);
-                sum += pv;
-                Ss[(ty * 4 + a) * SLD + tx + 16 * b] = pv;
+                s[i][b] = expf(s[i][b] - ref);
+                sum += s[i][b];
             }
-            sum = group16_sum(sum);
-            l[a] = l[a] * alpha + sum;
-            m[a] = mn;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) o[a][c] *= alpha;
+            l[i] = l[i] * alpha + group16_sum(sum);
+            m[i] = mn;
+            if (i & 1) {
+                float other, none;
+                ptx::unpack_f32x2(al[i / 2], other, none);
+                al[i / 2] = ptx::pack_f32x2(other, alpha);
+            } else {
+                al[i / 2] = ptx::pack_f32x2(alpha, 0.f);
+            }
         }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            float *dst = Pw + (tx + 16 * b) * LP + (ty % 2) * R;
+            if (R == 2) {
+                *reinterpret_cast<float2 *>(dst) = make_float2(s[0][b], s[R - 1][b]);
+            } else {
+#pragma unroll
+                for (int i = 0; i + 3 < R; i += 4)
+                    *reinterpret_cast<float4 *>(dst + i) = make_float4(s[i][b], s[i + 1][b], s[i + 2][b], s[i + 3][b]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) o[i][c] = ptx::mul_f32x2(o[i][c], al[i]);
+        cp_wait<1>();                 // V is here; the next K may still be on its way
+        __syncthreads();              // (also: every lane's part of P^T is written)
+        add_rows<R, BN, D>(o, Pw, LP, (ty % 2) * R, Vs, tx);
         __syncthreads();
-#pragma unroll 4
-        for (int j = 0; j < BN; ++j) {
-            float pv[4], vv[NC];
+        if (more) tile_in<T, BN, D>(Vs, V, k0 + step, n);
+        cp_commit();
+    }
+    cp_wait<0>();
+    __syncthreads();
+    // partial results into shared memory: O [BM][LD] over Q, then m, l
+    float *Om = smem, *Mm = Ks, *Lm = Ks + BM;
 #pragma unroll
-            for (int a = 0; a < 4; ++a) pv[a] = Ss[(ty * 4 + a) * SLD + j];
+    for (int i = 0; i < R / 2; ++i)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) vv[c] = Vs[j * LD + tx + 16 * c];
+        for (int v = 0; v < D / 64; ++v) {
+            float4 e, od;
+            unpack_rows<NC>(o[i], v, e, od);
+            *reinterpret_cast<float4 *>(Om + (ty * R + 2 * i) * LD + 64 * v + 4 * tx) = e;
+            *reinterpret_cast<float4 *>(Om + (ty * R + 2 * i + 1) * LD + 64 * v + 4 * tx) = od;
+        }
+    if (tx == 0)
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+        for (int i = 0; i < R; ++i) { Mm[ty * R + i] = m[i]; Lm[ty * R + i] = l[i]; }
+    if (split > 1) cluster_barrier();
+    else __syncthreads();
+    constexpr int LPR = D / 4;         // lanes per row, 16 bytes each
+    const int per = BM / split;        // rows this rank finishes
+    for (int r = tid / LPR; r < per; r += SNT / LPR) {
+        const int rr = rank * per + r, row = q0 + rr, c = (tid % LPR) * 4;
+        float mt = -INFINITY;
+        for (int k = 0; k < split; ++k) mt = fmaxf(mt, remote_f1(remote(Mm + rr, k)));
+        const float ref = mt == -INFINITY ? 0.f : mt;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        float lt = 0.f;
+        for (int k = 0; k < split; ++k) {
+            const float w = expf(remote_f1(remote(Mm + rr, k)) - ref);
+            const float4 v = remote_f4(remote(Om + rr * LD + c, k));
+            lt = fmaf(remote_f1(remote(Lm + rr, k)), w, lt);
+            a.x = fmaf(v.x, w, a.x); a.y = fmaf(v.y, w, a.y); a.z = fmaf(v.z, w, a.z); a.w = fmaf(v.w, w, a.w);
+        }
+        const bool live = row < n;
+        const float inv = 1.f / lt;
+        a.x *= inv; a.y *= inv; a.z *= inv; a.w *= inv;
+        const size_t at = (size_t)row * D + c;
+        if (live) {
+            store4(O + at, a);
+            if (c == 0) L[row] = mt + logf(lt);
+        }
+        if (dO != nullptr) {
+            float dot = 0.f;
+            if (live) {
+                const float4 g = load4(dO + base + at);
+                dot = fmaf(g.x, a.x, fmaf(g.y, a.y, fmaf(g.z, a.z, g.w * a.w)));
+                if (dQzero) store4(dQzero + base + at, make_float4(0.f, 0.f, 0.f, 0.f));
+            }
+            // the lanes of a row, 16 (D = 64) or 32 consecutive ones, go through this loop together
+            const uint32_t who = D == 64 ? 0xFFFFu << (tid & 16) : 0xFFFFFFFFu;
 #pragma unroll
-                for (int c = 0; c < NC; ++c) o[a][c] = fmaf(pv[a], vv[c], o[a][c]);
+            for (int d = LPR / 2; d >= 1; d >>= 1) dot += __shfl_xor_sync(who, dot, d);
+            if (live && c == 0) Dv[(size_t)bh * n + row] = dot;
         }
     }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int row = q0 + ty * 4 + a;
-        if (row >= n) continue;
-        const float inv = 1.f / l[a];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) O[(size_t)row * D + tx + 16 * c] = from_float<T>(o[a][c] * inv);
-        if (tx == 0) L[row] = m[a] + logf(l[a]);
-    }
+    if (split > 1) cluster_barrier();      // nobody leaves while another rank may still read its shared memory
 }
 
-// ---------------------------------------------------- rowsum(dO o O), one warp per row
+// ---------------------------------------- rowsum(dO o O), and dQ (or its accumulator) cleared: one warp per row
 template <typename T>
 __global__ void row_dot_kernel(const T *__restrict__ dO, const T *__restrict__ O,
-                               float *__restrict__ Dv, size_t rows, int d)
+                               float *__restrict__ Dv, float *__restrict__ dQzero, size_t rows, int d)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t row = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     if (row >= rows) return;
     const int lane = threadIdx.x % 32;
     float acc = 0.f;
-    for (int c = lane; c < d; c += 32)
-        acc = fmaf(to_float<T>(dO[row * d + c]), to_float<T>(O[row * d + c]), acc);
+    for (int c = 4 * lane; c < d; c += 128) {
+        const float4 a = load4(dO + row * d + c), b = load4(O + row * d + c);
+        acc = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc))));
+        if (dQzero) store4(dQzero + row * d + c, make_float4(0.f, 0.f, 0.f, 0.f));
+    }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) Dv[row] = acc;
@@ -210,102 +472,200 @@ __device__ __forceinline__ void load_rowvec(float *dst, const float *src, int ro
     for (int r = threadIdx.x; r < BM; r += NTHREADS) dst[r] = (row0 + r) < n ? src[row0 + r] : 0.f;
 }
 
-// ----------------------------------------- backward, one CTA per key tile: dK, dV (+dQ red)
-template <typename T, int D>
-__global__ void __launch_bounds__(NTHREADS)
+// ----------------------------------------- backward, one CTA (or cluster) per key tile: dK, dV (+dQ red)
+// CTA: BN = 8 R keys against query tiles of BM rows; a warp has 2 R keys to itself, a thread R keys x BM / 16 queries of the
+// score tile, R keys x D / 16 columns of dK and dV, and BM / 8 queries x D / 16 columns of the dQ tile.  P, then dS in its
+// place, is exchanged inside a warp ([query][key], the warp's own keys); dQ needs the dS of all warps, so a transposed copy
+// ([key][query]) goes through a CTA barrier, behind which the next Q and dO tiles are requested: they arrive under the dQ
+// product.  The `split` ranks of a cluster take the query tiles of their keys in turn and add their dK, dV at the end.
+template <int R, int D>
+struct SimtBwd {
+    static constexpr int BN = STY * R, BM = D == 64 ? 64 : 32, LD = D + 4;
+    static constexpr int LPS = BN + 4, LST = BM + 4;      // rows of P / dS [query][key] and of dS^T [key][query]
+    static constexpr int kFloats = 2 * (BN + BM) * LD + BM * LPS + BN * LST + 2 * BM;
+    static constexpr size_t kSmem = kFloats * sizeof(float);
+    static_assert(BN <= BM, "the partial dK, dV are staged over Q, dO");
+};
+
+template <typename T, int R, int D>
+__global__ void __launch_bounds__(SNT, 2)
 simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
                    const T *__restrict__ dO, const float *__restrict__ L, const float *__restrict__ Dv,
                    T *__restrict__ dK, T *__restrict__ dV, float *__restrict__ dQacc,
-                   int n, int causal, float scale, int nkt)
+                   int n, int causal, float scale, int nkt, int split)
 {
-    constexpr int LD = D + 1;
-    constexpr int NC = D / 16;
+    using S = SimtBwd<R, D>;
+    constexpr int BN = S::BN, BM = S::BM, LD = S::LD, LPS = S::LPS, LST = S::LST, NC = D / 16, QB = BM / 16, RQ = BM / STY;
     extern __shared__ float smem[];
     float *Ks = smem, *Vs = Ks + BN * LD, *Qs = Vs + BN * LD, *dOs = Qs + BM * LD;
-    float *Ps = dOs + BM * LD, *dSs = Ps + BM * SLD, *Ls = dSs + BM * SLD, *Ds = Ls + BM;
+    float *Ps = dOs + BM * LD, *dSt = Ps + BM * LPS, *Ls = dSt + BN * LST, *Ds = Ls + BM;
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
 
-    const int kt = blockIdx.x % nkt;   // causal: key tile 0 has the most work and comes first
-    const int bh = blockIdx.x / nkt;
+    const int rank = split > 1 ? (int)cluster_rank() : 0;
+    const int job = (int)blockIdx.x / split;
+    const int kt = job % nkt;   // causal: key tile 0 has the most work and comes first
+    const int bh = job / nkt;
     const int k0 = kt * BN;
     const size_t base = (size_t)bh * n * D;
     Q += base; K += base; V += base; dO += base; dV += base;
     if (dK) dK += base;
     L += (size_t)bh * n; Dv += (size_t)bh * n;
     if (dQacc) dQacc += base;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 
-    load_tile<T, D>(Ks, K, k0, n);
-    load_tile<T, D>(Vs, V, k0, n);
-    float dk[4][NC], dv[4][NC];
+    uint64_t dk[R / 2][NC], dv[R / 2][NC];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int i = 0; i < R / 2; ++i)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) { dk[a][c] = 0.f; dv[a][c] = 0.f; }
+        for (int c = 0; c < NC; ++c) { dk[i][c] = 0ull; dv[i][c] = 0ull; }
 
-    const int qstart = causal ? (k0 / BM) * BM : 0;
-    for (int q0 = qstart; q0 < n; q0 += BM) {
+    const int step = BM * split;
+    int q0 = (causal ? k0 / BM * BM : 0) + rank * BM;
+    if (q0 < n) {
+        tile_in<T, BN, D>(Ks, K, k0, n);
+        tile_in<T, BN, D>(Vs, V, k0, n);
+        tile_in<T, BM, D>(Qs, Q, q0, n);
+        tile_in<T, BM, D>(dOs, dO, q0, n);
+        cp_commit();
+    }
+    // launched as a programmatic dependent of the kernel that writes L and D and clears dQ
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (; q0 < n; q0 += step) {
+        if (tid < BM) {
+            const bool live = q0 + tid < n;
+            Ls[tid] = live ? L[q0 + tid] : 0.f;
+            Ds[tid] = live ? Dv[q0 + tid] : 0.f;
+        }
+        cp_wait<0>();
         __syncthreads();
-        load_tile<T, D>(Qs, Q, q0, n);
-        load_tile<T, D>(dOs, dO, q0, n);
-        load_rowvec(Ls, L, q0, n);
-        load_rowvec(Ds, Dv, q0, n);
+        const bool mask = k0 + BN > n || q0 + BM > n || (causal && k0 + BN - 1 > q0);
+        float p[R][QB];
+        dot_rows<R, QB, D>(p, Ks, Qs, ty * R, tx);
+#pragma unroll
+        for (int b = 0; b < QB; ++b) {
+            const int q = tx + 16 * b, row = q0 + q;
+            const float Li = Ls[q];
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                p[i][b] = expf(p[i][b] * scale - Li);
+                if (mask) {
+                    const int col = k0 + ty * R + i;
+                    if (row >= n || col >= n || (causal && col > row)) p[i][b] = 0.f;
+                }
+            }
+        }
+        auto put_rows = [&](const float (&v)[R][QB]) {      // [query][key]: this thread's R keys of each of its queries
+#pragma unroll
+            for (int b = 0; b < QB; ++b) {
+                float *dst = Ps + (tx + 16 * b) * LPS + ty * R;
+                if (R == 2) {
+                    *reinterpret_cast<float2 *>(dst) = make_float2(v[0][b], v[R - 1][b]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i + 3 < R; i += 4)
+                        *reinterpret_cast<float4 *>(dst + i) = make_float4(v[i][b], v[i + 1][b], v[i + 2][b], v[i + 3][b]);
+                }
+            }
+            __syncwarp();
+        };
+        put_rows(p);
+        add_rows<R, BM, D>(dv, Ps, LPS, ty * R, dOs, tx);
+        if (dK != nullptr || dQacc != nullptr) {
+            float ds[R][QB];
+            dot_rows<R, QB, D>(ds, Vs, dOs, ty * R, tx);
+#pragma unroll
+            for (int b = 0; b < QB; ++b) {
+                const int q = tx + 16 * b;
+                const float Di = Ds[q];
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    ds[i][b] = p[i][b] * (ds[i][b] - Di) * scale;
+                    dSt[(ty * R + i) * LST + q] = ds[i][b];
+                }
+            }
+            __syncwarp();              // the warp's lanes have read P
+            put_rows(ds);
+            add_rows<R, BM, D>(dk, Ps, LPS, ty * R, Qs, tx);
+        }
         __syncthreads();
-        bwd_tile_p_ds<D>(Qs, dOs, Ks, Vs, Ls, Ds, Ps, dSs, q0, k0, n, causal, scale, tx, ty);
-        __syncthreads();
-        // dV[key][c] += sum_q P[q][key] dO[q][c] ; dK[key][c] += sum_q (scale dS)[q][key] Q[q][c]
-#pragma unroll 2
-        for (int q = 0; q < BM; ++q) {
-            float pv[4], gv[4], gq[NC], qq[NC];
+        if (q0 + step < n) {           // arrives under the dQ product
+            tile_in<T, BM, D>(Qs, Q, q0 + step, n);
+            tile_in<T, BM, D>(dOs, dO, q0 + step, n);
+            cp_commit();
+        }
+        if (dQacc != nullptr) {
+            uint64_t dq[RQ / 2][NC];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) { pv[a] = Ps[q * SLD + ty * 4 + a]; gv[a] = dSs[q * SLD + ty * 4 + a]; }
+            for (int i = 0; i < RQ / 2; ++i)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) { gq[c] = dOs[q * LD + tx + 16 * c]; qq[c] = Qs[q * LD + tx + 16 * c]; }
+                for (int c = 0; c < NC; ++c) dq[i][c] = 0ull;
+            add_rows<RQ, BN, D>(dq, dSt, LST, ty * RQ, Ks, tx);
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int i = 0; i < RQ / 2; ++i)
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    dv[a][c] = fmaf(pv[a], gq[c], dv[a][c]);
-                    dk[a][c] = fmaf(gv[a], qq[c], dk[a][c]);
+                for (int v = 0; v < D / 64; ++v) {
+                    float4 r[2];
+                    unpack_rows<NC>(dq[i], v, r[0], r[1]);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int row = q0 + ty * RQ + 2 * i + e;
+                        if (row < n)       // 16 lanes cover 256 consecutive bytes of the row
+                            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dQacc + (size_t)row * D + 64 * v + 4 * tx),
+                                         "f"(r[e].x), "f"(r[e].y), "f"(r[e].z), "f"(r[e].w) : "memory");
+                    }
                 }
         }
-        if (dQacc) {
-            // dQ[q][c] += sum_key (scale dS)[q][key] K[key][c]
-            float dq[4][NC];
+    }
+    if (split == 1) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+        for (int i = 0; i < R / 2; ++i)
 #pragma unroll
-                for (int c = 0; c < NC; ++c) dq[a][c] = 0.f;
-#pragma unroll 2
-            for (int j = 0; j < BN; ++j) {
-                float gv[4], kk[NC];
+            for (int v = 0; v < D / 64; ++v) {
+                float4 a[2], g[2];
+                unpack_rows<NC>(dk[i], v, a[0], a[1]);
+                unpack_rows<NC>(dv[i], v, g[0], g[1]);
 #pragma unroll
-                for (int a = 0; a < 4; ++a) gv[a] = dSs[(ty * 4 + a) * SLD + j];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) kk[c] = Ks[j * LD + tx + 16 * c];
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) dq[a][c] = fmaf(gv[a], kk[c], dq[a][c]);
+                for (int e = 0; e < 2; ++e) {
+                    const int row = k0 + ty * R + 2 * i + e;
+                    if (row >= n) continue;
+                    const size_t at = (size_t)row * D + 64 * v + 4 * tx;
+                    if (dK) store4(dK + at, a[e]);   // nullptr: dV only
+                    store4(dV + at, g[e]);
+                }
             }
+        return;
+    }
+    // partial dK over Q, dV over dO (all tiles are done with them: the barrier in front of the last dQ product)
+    __syncthreads();
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const int row = q0 + ty * 4 + a;
-                if (row >= n) continue;
+    for (int i = 0; i < R / 2; ++i)
 #pragma unroll
-                for (int c = 0; c < NC; ++c) atomicAdd(&dQacc[(size_t)row * D + tx + 16 * c], dq[a][c]);
+        for (int v = 0; v < D / 64; ++v) {
+            float4 a[2], g[2];
+            unpack_rows<NC>(dk[i], v, a[0], a[1]);
+            unpack_rows<NC>(dv[i], v, g[0], g[1]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int at = (ty * R + 2 * i + e) * LD + 64 * v + 4 * tx;
+                *reinterpret_cast<float4 *>(Qs + at) = a[e];
+                *reinterpret_cast<float4 *>(dOs + at) = g[e];
             }
         }
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int row = k0 + ty * 4 + a;
+    cluster_barrier();
+    constexpr int LPR = D / 4;
+    const int per = BN / split;
+    for (int r = tid / LPR; r < per; r += SNT / LPR) {
+        const int rr = rank * per + r, row = k0 + rr, c = (tid % LPR) * 4;
         if (row >= n) continue;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            if (dK) dK[(size_t)row * D + tx + 16 * c] = from_float<T>(dk[a][c]);   // nullptr: dV only
-            dV[(size_t)row * D + tx + 16 * c] = from_float<T>(dv[a][c]);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), g = a;
+        for (int k = 0; k < split; ++k) {
+            const float4 x = remote_f4(remote(Qs + rr * LD + c, k)), y = remote_f4(remote(dOs + rr * LD + c, k));
+            a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+            g.x += y.x; g.y += y.y; g.z += y.z; g.w += y.w;
         }
+        if (dK) store4(dK + (size_t)row * D + c, a);
+        store4(dV + (size_t)row * D + c, g);
     }
+    cluster_barrier();
 }
 
 // ----------------------------------------- backward, one CTA per query tile: dQ, no atomics
@@ -617,7 +977,6 @@ convert_rows_kernel(const float *__restrict__ src, int src_ld, __nv_bfloat16 *__
     }
 }
 
-constexpr size_t fwd_smem(int D) { return (size_t)(3 * BM * (D + 1) + BM * SLD) * sizeof(float); }
 constexpr size_t bwd_smem(int D) { return (size_t)(4 * BM * (D + 1) + 2 * BM * SLD + 2 * BM) * sizeof(float); }
 
 template <typename K>
@@ -626,30 +985,78 @@ cudaError_t set_smem(K kernel, size_t bytes)
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <typename T, int D>
-cudaError_t fwd_t(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, cudaStream_t st)
+// How many ranks share an output tile: doubled while all CTAs still fit on the chip at once (`slots`), every rank keeps at
+// least one tile of the other axis (`others`), and the cluster stays portable (8).
+int simt_split(long long tiles, int others, long long slots)
 {
-    const int nqt = (p.n + BM - 1) / BM;
-    cudaError_t e = set_smem(simt_fwd_kernel<T, D>, fwd_smem(D));
-    if (e != cudaSuccess) return e;
-    LaunchScope scope(MOA_KERNEL_FWD, st);
-    simt_fwd_kernel<T, D><<<(unsigned)(nqt * p.BH()), NTHREADS, fwd_smem(D), st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, (T *)O, L, p.n, p.causal, p.scale, nqt);
-    return cudaGetLastError();
+    int s = 1;
+    while (s < 8 && 2 * s <= others && tiles * 2 * s <= slots) s *= 2;
+    return s;
 }
 
+template <typename... KArgs, typename... Args>
+cudaError_t launch_simt(void (*kernel)(KArgs...), long long ctas, int split, size_t smem, bool dependent, cudaStream_t st, Args... args)
+{
+    cudaError_t e = set_smem(kernel, smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(SNT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = dependent && pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// Rows per thread: the widest tile (fewest shared-memory loads per multiply-add) whose tiles, shared by clusters as far as
+// that goes, still give most SMs a CTA; narrower tiles below that, where the time is one CTA's latency.
+template <typename T, int R, int D>
+cudaError_t fwd_r(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const SimtPrep &pr,
+                  cudaStream_t st)
+{
+    using S = SimtFwd<R, D>;
+    const int nqt = (p.n + S::BM - 1) / S::BM, nkt = (p.n + BN - 1) / BN;
+    const long long tiles = (long long)nqt * p.BH(), slots = (long long)device_info().sms * (R == 8 ? 3 : D == 128 ? 2 : 4);
+    if (R > 2 && tiles * (nkt < 8 ? nkt : 8) < device_info().sms)
+        return fwd_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, O, L, pr, st);
+    const int split = simt_split(tiles, nkt, slots);
+    LaunchScope scope(MOA_KERNEL_FWD, st);
+    return launch_simt(simt_fwd_kernel<T, R, D>, tiles * split, split, S::kSmem, false, st, (const T *)Q, (const T *)K, (const T *)V,
+                       (T *)O, L, (const T *)pr.dO, pr.Dv, pr.dQzero, p.n, p.causal, p.scale, nqt, split);
+}
+template <typename T, int D>
+cudaError_t fwd_t(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const SimtPrep &pr,
+                  cudaStream_t st)
+{
+    return fwd_r<T, D == 64 ? 8 : 4, D>(p, Q, K, V, O, L, pr, st);
+}
+
+template <typename T, int R, int D>
+cudaError_t bwd_kv_r(const Problem &p, const void *Q, const void *K, const void *V, const void *dO, const float *L,
+                     const float *Dv, void *dK, void *dV, float *dQacc, cudaStream_t st)
+{
+    using S = SimtBwd<R, D>;
+    const int nkt = (p.n + S::BN - 1) / S::BN, nqt = (p.n + S::BM - 1) / S::BM;
+    const long long tiles = (long long)nkt * p.BH(), slots = 2LL * device_info().sms;
+    if (R > 2 && tiles * (nqt < 8 ? nqt : 8) < device_info().sms)
+        return bwd_kv_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, dO, L, Dv, dK, dV, dQacc, st);
+    const int split = simt_split(tiles, nqt, slots);
+    LaunchScope scope(MOA_KERNEL_BWD_KV, st);
+    return launch_simt(simt_bwd_kv_kernel<T, R, D>, tiles * split, split, S::kSmem, true, st, (const T *)Q, (const T *)K,
+                       (const T *)V, (const T *)dO, L, Dv, (T *)dK, (T *)dV, dQacc, p.n, p.causal, p.scale, nkt, split);
+}
 template <typename T, int D>
 cudaError_t bwd_kv_t(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
                      const float *L, const float *Dv, void *dK, void *dV, float *dQacc, cudaStream_t st)
 {
-    const int nkt = (p.n + BN - 1) / BN;
-    cudaError_t e = set_smem(simt_bwd_kv_kernel<T, D>, bwd_smem(D));
-    if (e != cudaSuccess) return e;
-    LaunchScope scope(MOA_KERNEL_BWD_KV, st);
-    simt_bwd_kv_kernel<T, D><<<(unsigned)(nkt * p.BH()), NTHREADS, bwd_smem(D), st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, (const T *)dO, L, Dv, (T *)dK, (T *)dV, dQacc,
-        p.n, p.causal, p.scale, nkt);
-    return cudaGetLastError();
+    return bwd_kv_r<T, D == 64 ? 8 : 4, D>(p, Q, K, V, dO, L, Dv, dK, dV, dQacc, st);
 }
 
 template <typename T, int D>
@@ -700,9 +1107,9 @@ cudaError_t rowpar_t(const Problem &p, const void *Q, const void *K, const void 
 }  // namespace
 
 cudaError_t simt_fwd(const Problem &p, int dtype, const void *Q, const void *K, const void *V,
-                     void *O, float *L, cudaStream_t st)
+                     void *O, float *L, const SimtPrep &pr, cudaStream_t st)
 {
-    MOA_DISPATCH(fwd_t, p, Q, K, V, O, L, st);
+    MOA_DISPATCH(fwd_t, p, Q, K, V, O, L, pr, st);
 }
 
 cudaError_t simt_bwd_kv(const Problem &p, int dtype, const void *Q, const void *K, const void *V,
@@ -724,17 +1131,17 @@ cudaError_t simt_bwd_dq(const Problem &p, int dtype, const void *Q, const void *
     MOA_DISPATCH(bwd_dq_t, p, Q, K, V, dO, L, Dv, dQ, st);
 }
 
-cudaError_t row_dot(const Problem &p, int dtype, const void *dO, const void *O, float *Dv, cudaStream_t st)
+cudaError_t row_dot(const Problem &p, int dtype, const void *dO, const void *O, float *Dv, float *dQzero, cudaStream_t st)
 {
     const size_t rows = (size_t)p.BH() * p.n;
     const int wpb = 8;
     const unsigned grid = (unsigned)((rows + wpb - 1) / wpb);
     LaunchScope scope(MOA_KERNEL_PREPROCESS, st);
     if (dtype == MOA_F32)
-        row_dot_kernel<float><<<grid, wpb * 32, 0, st>>>((const float *)dO, (const float *)O, Dv, rows, p.d);
+        row_dot_kernel<float><<<grid, wpb * 32, 0, st>>>((const float *)dO, (const float *)O, Dv, dQzero, rows, p.d);
     else
         row_dot_kernel<__nv_bfloat16><<<grid, wpb * 32, 0, st>>>((const __nv_bfloat16 *)dO,
-                                                                 (const __nv_bfloat16 *)O, Dv, rows, p.d);
+                                                                 (const __nv_bfloat16 *)O, Dv, dQzero, rows, p.d);
     return cudaGetLastError();
 }
 
