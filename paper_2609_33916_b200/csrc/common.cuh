@@ -221,7 +221,7 @@ cudaError_t mat_bwd(const Problem &p, const void *Q, const void *K, const void *
 // ---- SIMT fp32 path (simt_kernels.cu) -------------------------------------------------
 // dtype: MOA_BF16 or MOA_F32 storage; arithmetic is fp32 FMA throughout.
 // What the forward of a fused call prepares for its backward (all null for a plain forward): D = rowsum(dO o O) [B*H, n]
-// from the fp32 O it holds, and the cleared dQ accumulator [B*H, n, d] (null: not wanted).
+// and the cleared dQ accumulator [B*H, n, d] (null: not wanted).
 struct SimtPrep {
     const void *dO = nullptr;
     float *Dv = nullptr, *dQzero = nullptr;

@@ -113,6 +113,12 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16 *p)
                        __uint_as_float(u.y & 0xFFFF0000u));
 }
 
+template <typename T> __device__ __forceinline__ float4 as_stored(float4 v)
+{
+    return make_float4(to_float(from_float<T>(v.x)), to_float(from_float<T>(v.y)), to_float(from_float<T>(v.z)),
+                       to_float(from_float<T>(v.w)));
+}
+
 // out[i][b] = A[a_row0 + i][:] . B[tx + 16 b][:], contraction over D; rows of D + 4 floats
 template <int R, int NB, int D>
 __device__ __forceinline__ void dot_rows(float (&out)[R][NB], const float *A, const float *B, int a_row0, int tx)
@@ -229,7 +235,7 @@ __device__ __forceinline__ float remote_f1(uint32_t a)
 // CTA: BM = 8 R query rows; a warp has 2 R rows to itself, a thread R rows x 4 keys of the score tile and R rows x D / 16
 // columns of O.  The `split` ranks of a cluster take the key tiles of their rows in turn (rank r: tiles r, r + split, ...), each
 // with its own online softmax; at the end rank r merges rows r BM / split ... of all ranks' partial results.
-// In a fused call (dO != nullptr) the merge also gives D = rowsum(dO o O), from the fp32 O, and clears its rows of dQ.
+// In a fused call (dO != nullptr) the merge also gives D = rowsum(dO o O) and clears its rows of dQ.
 template <int R, int D>
 struct SimtFwd {
     static constexpr int BM = STY * R, LD = D + 4, LP = 2 * R + 4;
@@ -389,8 +395,9 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         if (dO != nullptr) {
             float dot = 0.f;
             if (live) {
-                const float4 g = load4(dO + base + at);
-                dot = fmaf(g.x, a.x, fmaf(g.y, a.y, fmaf(g.z, a.z, g.w * a.w)));
+                // (from O as stored, like the separate backward call: the same gradients either way, bit for bit)
+                const float4 g = load4(dO + base + at), r = as_stored<T>(a);
+                dot = fmaf(g.x, r.x, fmaf(g.y, r.y, fmaf(g.z, r.z, g.w * r.w)));
                 if (dQzero) store4(dQzero + base + at, make_float4(0.f, 0.f, 0.f, 0.f));
             }
             // the lanes of a row, 16 (D = 64) or 32 consecutive ones, go through this loop together
