@@ -489,7 +489,7 @@ cudaError_t launch_ring(const RingPlan &p, const __nv_bfloat16 *x, const __nv_bf
                         const __nv_bfloat16 *dy, const __nv_bfloat16 *dx_add, __nv_bfloat16 *out, float *part, int n, int d,
                         float eps, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(rmsnorm_ring_kernel<kV, kBwd>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    cudaError_t e = allow_smem<rmsnorm_ring_kernel<kV, kBwd>>(p.smem);
     if (e != cudaSuccess) return e;
     rmsnorm_ring_kernel<kV, kBwd><<<p.grid, kRingThreads, p.smem, st>>>(x, g, r_in, r_out, dy, dx_add, out, part, n, d, eps,
                                                                         p.m, device_status_ptr());

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <atomic>
+#include <mutex>
 #include "moa_attn.h"
 
 namespace moa {
@@ -139,6 +141,26 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, si
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// Lets `Kernel` use `bytes` of dynamic shared memory (cudaFuncSetAttribute).  The driver call is made once per kernel and
+// device and again only for more than any call before asked for; it took a tenth of a small call's host time.
+template <auto Kernel>
+cudaError_t allow_smem(size_t bytes)
+{
+    constexpr int kMaxDev = 64;
+    static std::atomic<size_t> allowed[kMaxDev];
+    static std::mutex mu;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool known = dev >= 0 && dev < kMaxDev;
+    if (known && allowed[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    std::lock_guard<std::mutex> lk(mu);      // (so that two threads cannot leave the smaller of two sizes in force)
+    if (known && allowed[dev].load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && known) allowed[dev].store(bytes, std::memory_order_release);
+    return e;
 }
 
 // Device address of the status word kernels write when a bounded wait expires.

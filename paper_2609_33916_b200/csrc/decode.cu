@@ -458,16 +458,14 @@ cudaError_t launch_split(const DecodeProblem &p, const void *q, const void *K, c
     if (GC >= 4) {
         constexpr int kStages = Ring<T, D>::kStages;
         const size_t smem = (size_t)kStages * 2 * kTileRows * D * sizeof(T) + 2 * kStages * sizeof(uint64_t) + 16;
-        cudaError_t e = cudaFuncSetAttribute(decode_ring_kernel<T, D, GC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(smem > merge_smem ? smem : merge_smem));
+        cudaError_t e = allow_smem<decode_ring_kernel<T, D, GC>>(smem > merge_smem ? smem : merge_smem);
         if (e != cudaSuccess) return e;
         decode_ring_kernel<T, D, GC><<<grid, kRingThreads, smem > merge_smem ? smem : merge_smem, st>>>(
             (const T *)q, (const T *)K, (const T *)V, part_o, part_ml, (T *)out, lse, counters, p.n, p.H, p.Hkv, group, splits,
             keys_per_split, (size_t)p.B * p.H, p.scale * kLog2e, device_status_ptr());
         return cudaGetLastError();
     }
-    cudaError_t e = cudaFuncSetAttribute(decode_split_kernel<T, D, GC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)merge_smem);
+    cudaError_t e = allow_smem<decode_split_kernel<T, D, GC>>(merge_smem);
     if (e != cudaSuccess) return e;
     decode_split_kernel<T, D, GC><<<grid, kThreads, merge_smem, st>>>((const T *)q, (const T *)K, (const T *)V, part_o,
                                                                       part_ml, (T *)out, lse, counters, p.n, p.H, p.Hkv,

@@ -986,12 +986,6 @@ convert_rows_kernel(const float *__restrict__ src, int src_ld, __nv_bfloat16 *__
 
 constexpr size_t bwd_smem(int D) { return (size_t)(4 * BM * (D + 1) + 2 * BM * SLD + 2 * BM) * sizeof(float); }
 
-template <typename K>
-cudaError_t set_smem(K kernel, size_t bytes)
-{
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // How many ranks share an output tile: doubled while all CTAs still fit on the chip at once (`slots`), every rank keeps at
 // least one tile of the other axis (`others`), and the cluster stays portable (8).
 int simt_split(long long tiles, int others, long long slots)
@@ -1004,8 +998,6 @@ int simt_split(long long tiles, int others, long long slots)
 template <typename... KArgs, typename... Args>
 cudaError_t launch_simt(void (*kernel)(KArgs...), long long ctas, int split, size_t smem, bool dependent, cudaStream_t st, Args... args)
 {
-    cudaError_t e = set_smem(kernel, smem);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas);
     cfg.blockDim = dim3(SNT);
@@ -1034,6 +1026,8 @@ cudaError_t fwd_r(const Problem &p, const void *Q, const void *K, const void *V,
     if (R > 2 && tiles * (nkt < 8 ? nkt : 8) < device_info().sms)
         return fwd_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, O, L, pr, st);
     const int split = simt_split(tiles, nkt, slots);
+    const cudaError_t e = allow_smem<simt_fwd_kernel<T, R, D>>(S::kSmem);
+    if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
     return launch_simt(simt_fwd_kernel<T, R, D>, tiles * split, split, S::kSmem, false, st, (const T *)Q, (const T *)K, (const T *)V,
                        (T *)O, L, (const T *)pr.dO, pr.Dv, pr.dQzero, p.n, p.causal, p.scale, nqt, split);
@@ -1055,6 +1049,8 @@ cudaError_t bwd_kv_r(const Problem &p, const void *Q, const void *K, const void 
     if (R > 2 && tiles * (nqt < 8 ? nqt : 8) < device_info().sms)
         return bwd_kv_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, dO, L, Dv, dK, dV, dQacc, st);
     const int split = simt_split(tiles, nqt, slots);
+    const cudaError_t e = allow_smem<simt_bwd_kv_kernel<T, R, D>>(S::kSmem);
+    if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
     return launch_simt(simt_bwd_kv_kernel<T, R, D>, tiles * split, split, S::kSmem, true, st, (const T *)Q, (const T *)K,
                        (const T *)V, (const T *)dO, L, Dv, (T *)dK, (T *)dV, dQacc, p.n, p.causal, p.scale, nkt, split);
@@ -1071,7 +1067,7 @@ cudaError_t bwd_dq_t(const Problem &p, const void *Q, const void *K, const void 
                      const float *L, const float *Dv, void *dQ, cudaStream_t st)
 {
     const int nqt = (p.n + BM - 1) / BM;
-    cudaError_t e = set_smem(simt_bwd_dq_kernel<T, D>, bwd_smem(D));
+    cudaError_t e = allow_smem<simt_bwd_dq_kernel<T, D>>(bwd_smem(D));
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_BWD_DQ, st);
     simt_bwd_dq_kernel<T, D><<<(unsigned)(nqt * p.BH()), NTHREADS, bwd_smem(D), st>>>(
@@ -1084,8 +1080,8 @@ cudaError_t rowpar_t(const Problem &p, const void *Q, const void *K, const void 
                      float *Dv, void *dQ, float *dKacc, float *dVacc, int sites, cudaStream_t st)
 {
     const int nqt = (p.n + BM - 1) / BM;
-    cudaError_t e = set_smem(simt_rowpar_kernel<T, D, 1>, bwd_smem(D));
-    if (e == cudaSuccess) e = set_smem(simt_rowpar_kernel<T, D, 2>, bwd_smem(D));
+    cudaError_t e = allow_smem<simt_rowpar_kernel<T, D, 1>>(bwd_smem(D));
+    if (e == cudaSuccess) e = allow_smem<simt_rowpar_kernel<T, D, 2>>(bwd_smem(D));
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_OTHER, st);
     if (sites == 2)

@@ -698,7 +698,7 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     if (!make_tensor_map_3d(&mdq, dQacc ? (const void *)dQacc : Q, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, heads, p.n, D, 32, D == 64 ? 32 : D))
         return cudaErrorInvalidValue;
     constexpr int kSmem = BwdSmem<D, kBulk>::kTotal;
-    cudaError_t e = cudaFuncSetAttribute(tc_bwd_kernel<D, kBulk, kGrouped>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_bwd_kernel<D, kBulk, kGrouped>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);

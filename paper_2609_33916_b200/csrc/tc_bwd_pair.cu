@@ -668,7 +668,7 @@ cudaError_t launch_pair(const Problem &p, const void *Q, const void *K, const vo
         return cudaErrorInvalidValue;
     auto kernel = tc_bwd_pair_kernel<kBulk, kGrouped>;
     constexpr int kSmem = PairSmem::kTotal;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_bwd_pair_kernel<kBulk, kGrouped>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128, npt = (nkt + 1) / 2;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);

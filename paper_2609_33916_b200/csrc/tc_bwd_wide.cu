@@ -455,7 +455,7 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
         return cudaErrorInvalidValue;
     auto kernel = tc_bwd_wide_kernel<kGrouped>;
     constexpr int kSmem = WideSmem::kTotal;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_bwd_wide_kernel<kGrouped>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);

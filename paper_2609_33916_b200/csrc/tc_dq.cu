@@ -218,7 +218,7 @@ cudaError_t launch_dq(const Problem &p, const void *Q, const void *K, const void
         !make_tensor_map_4d_strided(&mdo, dO, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64))
         return cudaErrorInvalidValue;
     constexpr int kSmem = DqSmem<D>::kTotal;
-    cudaError_t e = cudaFuncSetAttribute(tc_dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_dq_kernel<D>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_DQ, st);

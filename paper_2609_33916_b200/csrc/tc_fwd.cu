@@ -501,7 +501,7 @@ cudaError_t launch_fwd(const Problem &p, const void *Q, const void *K, const voi
         !make_tensor_map_4d_strided(&mv, V, bf, 2, p.B, p.kv_heads(), p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64) ||
         !make_tensor_map_4d_strided(&mo, O, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tc_fwd_kernel<D, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_fwd_kernel<D, KC>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + BM - 1) / BM;
     LaunchScope scope(MOA_KERNEL_FWD, st);
@@ -528,7 +528,7 @@ cudaError_t launch_fwd_decode(int B, int Hkv, int G, int n, float scale, const v
         !make_tensor_map_4d(&mv, V, bf, 2, B, Hkv, n, D, false, 128, 64) ||
         !make_tensor_map_4d(&mo, O_part, bf, 2, (uint64_t)splits * B, Hkv, G, D, false, 128, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tc_fwd_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_fwd_kernel<D, 1>>(kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
     tc_fwd_kernel<D, 1><<<(unsigned)(B * Hkv * splits), kThreads, kSmem, st>>>(

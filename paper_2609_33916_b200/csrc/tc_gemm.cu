@@ -549,7 +549,7 @@ cudaError_t launch_gemm_as(const Operand &A0, const Operand &B0, const Operand *
             return cudaErrorInvalidValue;
     auto kernel = tc_gemm_kernel<kAMn, kBMn, kEpi, kPair>;
     constexpr int kSmem = gemm_smem(kPair), kTileM = kPair ? 2 * GM : GM;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    cudaError_t e = allow_smem<tc_gemm_kernel<kAMn, kBMn, kEpi, kPair>>(kSmem);
     if (e != cudaSuccess) return e;
     const int tiles = ((M + kTileM - 1) / kTileM) * ((N + (kDualN ? 128 : GN) - 1) / (kDualN ? 128 : GN)) * nbatch;
     const int nparts = (A1 && !kDualN && nbatch == 1) ? 2 : 1;

@@ -545,7 +545,7 @@ cudaError_t run_group(const Problem &p, const void *Q, const void *K, const void
     cudaError_t e;
     if (stage == 0) {
         constexpr int kSmem = 3 * 128 * D * 2 + 128;
-        if ((e = cudaFuncSetAttribute(mat_fwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return e;
+        if ((e = allow_smem<mat_fwd_kernel<D>>(kSmem)) != cudaSuccess) return e;
         LaunchScope scope(MOA_KERNEL_FWD, st);
         mat_fwd_kernel<D><<<(unsigned)(nt * p.BH()), 192, kSmem, st>>>(mq, mk, mv, (__nv_bfloat16 *)O, L, (__nv_bfloat16 *)PT,
                                                                       p.n, n_pad, p.causal, p.scale * kLog2e, nt,
@@ -557,7 +557,7 @@ cudaError_t run_group(const Problem &p, const void *Q, const void *K, const void
         return cudaErrorInvalidValue;
     {
         constexpr int kSmem = MatBwdSmem<D>::kTotal;
-        if ((e = cudaFuncSetAttribute(mat_bwd_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return e;
+        if ((e = allow_smem<mat_bwd_kernel<D>>(kSmem)) != cudaSuccess) return e;
         LaunchScope scope(MOA_KERNEL_BWD_KV, st);
         mat_bwd_kernel<D><<<(unsigned)(nt * p.BH()), 320, kSmem, st>>>(mq, mk, mv, mdo, Dp_group, (const __nv_bfloat16 *)PT,
                                                                       (__nv_bfloat16 *)GST, (__nv_bfloat16 *)dK,
@@ -567,7 +567,7 @@ cudaError_t run_group(const Problem &p, const void *Q, const void *K, const void
     }
     {
         constexpr int kSmem = 2 * 128 * 128 * 2 + 2 * 128 * D * 2 + 128;
-        if ((e = cudaFuncSetAttribute(mat_dq_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return e;
+        if ((e = allow_smem<mat_dq_kernel<D>>(kSmem)) != cudaSuccess) return e;
         LaunchScope scope(MOA_KERNEL_BWD_DQ, st);
         mat_dq_kernel<D><<<(unsigned)(nt * p.BH()), 192, kSmem, st>>>(mg, mk, (__nv_bfloat16 *)dQ, p.n, n_pad, p.causal, p.scale,
                                                                      nt, heads_per_group(p, nt), device_status_ptr());
