@@ -95,6 +95,9 @@ rmsnorm_fwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
                    __nv_bfloat16 *__restrict__ y, float *__restrict__ r_out, int n, int d, float eps, int tpr)
 {
     __shared__ float red[8 * R];
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    x = ptx::after_wait(x); g = ptx::after_wait(g);
     const int c = threadIdx.x % tpr, rl = threadIdx.x / tpr, lanes = kNormThreads / tpr;
     const int nvec = d / 8;
     float gf[kV][8];
@@ -102,7 +105,7 @@ rmsnorm_fwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
     for (int j = 0; j < kV; ++j) {
         const int v = c + j * tpr;
         uint4 gv = make_uint4(0u, 0u, 0u, 0u);
-        if (v < nvec) gv = __ldg(reinterpret_cast<const uint4 *>(g) + v);
+        if (v < nvec) gv = *(reinterpret_cast<const uint4 *>(g) + v);
         unpack8(gv, gf[j]);
     }
     const long long rows_per_iter = (long long)gridDim.x * lanes * R;
@@ -158,6 +161,9 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
 {
     __shared__ float red[8 * R];
     __shared__ float acc[kNormThreads * 8];              // [row lane][tpr*8] for one j at a time
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    x = ptx::after_wait(x); g = ptx::after_wait(g); r_in = ptx::after_wait(r_in); dy = ptx::after_wait(dy); dx_add = ptx::after_wait(dx_add);
     const int c = threadIdx.x % tpr, rl = threadIdx.x / tpr, lanes = kNormThreads / tpr;
     const int nvec = d / 8;
     float gf[kV][8], dgacc[kV][8];
@@ -165,7 +171,7 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
     for (int j = 0; j < kV; ++j) {
         const int v = c + j * tpr;
         uint4 gv = make_uint4(0u, 0u, 0u, 0u);
-        if (v < nvec) gv = __ldg(reinterpret_cast<const uint4 *>(g) + v);
+        if (v < nvec) gv = *(reinterpret_cast<const uint4 *>(g) + v);
         unpack8(gv, gf[j]);
 #pragma unroll
         for (int e = 0; e < 8; ++e) dgacc[j][e] = 0.f;
@@ -186,7 +192,7 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
         // the stored r of this iteration's rows: requested here, ahead of the reductions and their barriers
         float rr[R];
 #pragma unroll
-        for (int i = 0; i < R; ++i) rr[i] = (r_in != nullptr && row0 + i < n) ? __ldg(r_in + row0 + i) : 0.f;
+        for (int i = 0; i < R; ++i) rr[i] = (r_in != nullptr && row0 + i < n) ? r_in[row0 + i] : 0.f;
         // per row: t = sum_k x_k g_k dy_k, and sum_k x_k^2 when r is not given
         float t[R], ss[R];
 #pragma unroll
@@ -288,6 +294,9 @@ rmsnorm_ring_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__
         *abortp = 0;
         fence_mbar_init();
     }
+    grid_dependency_wait();
+    grid_launch_dependents();
+    g = after_wait(g); r_in = after_wait(r_in); dx_add = after_wait(dx_add);
     for (int i = threadIdx.x; i < d; i += kRingThreads) gs[i] = __bfloat162float(g[i]);
     __syncthreads();
     float dgacc[kV][8];          // backward only (dead otherwise)
@@ -331,7 +340,7 @@ rmsnorm_ring_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__
                 const long long row = row0 + lr;
                 if (row >= n) break;                          // warp-uniform
                 float rr = 0.f;
-                if (kBwd && r_in != nullptr) rr = __ldg(r_in + row);
+                if (kBwd && r_in != nullptr) rr = r_in[row];
                 float ss = 0.f, t = 0.f;
 #pragma unroll
                 for (int j = 0; j < kV; ++j) {
@@ -415,6 +424,9 @@ __global__ void __launch_bounds__(32 * kDgWarps)
 rmsnorm_dg_kernel(const float *__restrict__ part, __nv_bfloat16 *__restrict__ dg, int parts, int d)
 {
     __shared__ float s[kDgWarps][32];
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    part = ptx::after_wait(part);
     const int cx = threadIdx.x % 32, cy = threadIdx.x / 32;
     const int col = blockIdx.x * 32 + cx;
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
@@ -491,9 +503,8 @@ cudaError_t launch_ring(const RingPlan &p, const __nv_bfloat16 *x, const __nv_bf
 {
     cudaError_t e = allow_smem<rmsnorm_ring_kernel<kV, kBwd>>(p.smem);
     if (e != cudaSuccess) return e;
-    rmsnorm_ring_kernel<kV, kBwd><<<p.grid, kRingThreads, p.smem, st>>>(x, g, r_in, r_out, dy, dx_add, out, part, n, d, eps,
-                                                                        p.m, device_status_ptr());
-    return cudaGetLastError();
+    return launch_dependent(rmsnorm_ring_kernel<kV, kBwd>, dim3(p.grid), dim3(kRingThreads), p.smem, st, x, g, r_in, r_out, dy, dx_add, out,
+                            part, n, d, eps, p.m, device_status_ptr());
 }
 template <bool kBwd>
 cudaError_t launch_ring_kv(const RingPlan &p, const __nv_bfloat16 *x, const __nv_bfloat16 *g, const float *r_in, float *r_out,
@@ -519,10 +530,8 @@ cudaError_t rmsnorm_fwd(int n, int d, float eps, const void *x, const void *g, v
     auto *yb = (__nv_bfloat16 *)y;
     LaunchScope scope(MOA_KERNEL_OTHER, st);
     if (norm_uses_ring(d)) return launch_ring_kv<false>(ring_plan(n, d, false), xb, gb, nullptr, r, nullptr, nullptr, yb, nullptr, n, d, eps, st);
-    if (p.kV == 1) rmsnorm_fwd_kernel<1, 2><<<p.grid, kNormThreads, 0, st>>>(xb, gb, yb, r, n, d, eps, p.tpr);
-    else if (p.kV == 2) rmsnorm_fwd_kernel<2, 1><<<p.grid, kNormThreads, 0, st>>>(xb, gb, yb, r, n, d, eps, p.tpr);
-    else rmsnorm_fwd_kernel<4, 1><<<p.grid, kNormThreads, 0, st>>>(xb, gb, yb, r, n, d, eps, p.tpr);
-    return cudaGetLastError();
+    const auto kernel = p.kV == 1 ? rmsnorm_fwd_kernel<1, 2> : p.kV == 2 ? rmsnorm_fwd_kernel<2, 1> : rmsnorm_fwd_kernel<4, 1>;
+    return launch_dependent(kernel, dim3(p.grid), dim3(kNormThreads), (size_t)0, st, xb, gb, yb, r, n, d, eps, p.tpr);
 }
 
 cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, const float *r, const void *dy,
@@ -544,15 +553,13 @@ cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, c
         if (e != cudaSuccess) return e;
     } else {
         LaunchScope scope(MOA_KERNEL_OTHER, st);
-        if (p.kV == 1) rmsnorm_bwd_kernel<1, 2><<<p.grid, kNormThreads, 0, st>>>(xb, gb, r, db, ab, ob, part, n, d, eps, p.tpr);
-        else if (p.kV == 2) rmsnorm_bwd_kernel<2, 1><<<p.grid, kNormThreads, 0, st>>>(xb, gb, r, db, ab, ob, part, n, d, eps, p.tpr);
-        else rmsnorm_bwd_kernel<4, 2><<<p.grid, kNormThreads, 0, st>>>(xb, gb, r, db, ab, ob, part, n, d, eps, p.tpr);
-        const cudaError_t e = cudaGetLastError();
+        const auto kernel = p.kV == 1 ? rmsnorm_bwd_kernel<1, 2> : p.kV == 2 ? rmsnorm_bwd_kernel<2, 1> : rmsnorm_bwd_kernel<4, 2>;
+        const cudaError_t e = launch_dependent(kernel, dim3(p.grid), dim3(kNormThreads), (size_t)0, st, xb, gb, r, db, ab, ob, part, n, d, eps, p.tpr);
         if (e != cudaSuccess) return e;
     }
     LaunchScope scope(MOA_KERNEL_OTHER, st);
-    rmsnorm_dg_kernel<<<(d + 31) / 32, 32 * kDgWarps, 0, st>>>(part, (__nv_bfloat16 *)dg, parts, d);
-    return cudaGetLastError();
+    return launch_dependent(rmsnorm_dg_kernel, dim3((d + 31) / 32), dim3(32 * kDgWarps), (size_t)0, st, (const float *)part, (__nv_bfloat16 *)dg,
+                            parts, d);
 }
 
 }  // namespace moa

@@ -124,23 +124,37 @@ struct LaunchScope {
 };
 
 // Launch `kernel` so that it may start before the kernel in front of it in the stream has finished (programmatic
-// dependent launch): the kernel itself calls ptx::grid_dependency_wait() before it touches anything that kernel
-// wrote.  MOA_PDL=0 in the environment turns the attribute off (plain stream order).
+// dependent launch), in clusters of `cluster` CTAs.  Every kernel launched like this keeps to two rules, which together
+// make the early start invisible:
+//   * it calls ptx::grid_dependency_wait() before it reads or writes global memory -- except that a kernel that is never the
+//     first of a call (the attention backward kernels) may read the call's own inputs before that;
+//   * it calls ptx::grid_launch_dependents() only after that wait.  So once a kernel's successor runs at all, everything in
+//     front of the kernel itself, the caller's work included, has completed.
+// What overlaps is the set-up (barriers, TMEM allocation, tensor-map fetches) and the launch latency.
+// MOA_PDL=0 in the environment turns the attribute off (plain stream order).
 bool pdl_enabled();
 template <typename... KArgs, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+cudaError_t launch_cluster(void (*kernel)(KArgs...), unsigned cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    return launch_cluster(kernel, 1u, grid, block, smem, st, args...);
 }
 
 // Lets `Kernel` use `bytes` of dynamic shared memory (cudaFuncSetAttribute).  The driver call is made once per kernel and
@@ -208,8 +222,9 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
 
 // Lp = -L*log2(e) and Dp = -rowsum(dO o O) (negated: fma/add operands), each padded per head to a
 // multiple of 128 rows (-inf / 0 past n)
+// (and, unless zero_acc is null, clears the fp32 accumulator [B*H, n, kernel_d(d)] the backward adds dQ into)
 cudaError_t tc_bwd_preprocess(const Problem &p, const void *dO, const void *O, const float *L, float *Lp, float *Dp,
-                              cudaStream_t st);
+                              float *zero_acc, cudaStream_t st);
 // dK, dV; UNSCALED dQ contributions (dS K, without the factor scale) red-added into dQacc
 // (fp32 [B,H,n,kernel_d(d)], pre-zeroed); dQacc == nullptr skips the dQ contraction altogether
 cudaError_t tc_bwd_kv(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,

@@ -265,7 +265,7 @@ moa_status run_materialized(const moa_attn_desc *d, const void *Q, const void *K
         if (mat_fwd(p, q, k, v, o, l, PT, st) != cudaSuccess) return MOA_ERR_CUDA;
         if (!with_bwd) continue;
         const char *g_do = (const char *)dO + g0 * hs;
-        if (tc_bwd_preprocess(p, g_do, o, l, Lp, Dp, st) != cudaSuccess) return MOA_ERR_CUDA;
+        if (tc_bwd_preprocess(p, g_do, o, l, Lp, Dp, nullptr, st) != cudaSuccess) return MOA_ERR_CUDA;
         if (mat_bwd(p, q, k, v, g_do, Dp, PT, GST, (char *)dQ + g0 * hs, (char *)dK + g0 * hs, (char *)dV + g0 * hs, st) !=
             cudaSuccess)
             return MOA_ERR_CUDA;
@@ -296,14 +296,13 @@ moa_status run_bwd(const moa_attn_desc *d, const void *Q, const void *K, const v
     const int mode = resolved_dq_mode(d);
 #define MOA_TRY(x) do { if ((x) != cudaSuccess) return MOA_ERR_CUDA; } while (0)
     if (use_tc_bwd(d)) {
-        if (!prepared) MOA_TRY(tc_bwd_preprocess(p, dO, O, L, Lp, Dv, st));
+        if (!prepared) MOA_TRY(tc_bwd_preprocess(p, dO, O, L, Lp, Dv, mode == MOA_DQ_SEPARATE_PASS ? nullptr : dQacc, st));
         if (mode == MOA_DQ_SEPARATE_PASS) {
             MOA_TRY(tc_bwd_kv(p, Q, K, V, dO, Lp, Dv, dK, dV, nullptr, 0, st));
             MOA_TRY(tc_bwd_dq(p, Q, K, V, dO, Lp, Dv, dQ, st));
             return MOA_OK;
         }
         const int acc_ld = kernel_d(p.d);
-        if (!prepared) MOA_TRY(cudaMemsetAsync(dQacc, 0, (size_t)p.BH() * p.n * acc_ld * sizeof(float), st));
         MOA_TRY(tc_bwd_kv(p, Q, K, V, dO, Lp, Dv, dK, dV, dQacc, mode == MOA_DQ_BULK_REDUCE, st));
         if (!p.contiguous_bhnd() || acc_ld != p.d) MOA_TRY(convert_f32_to_bf16_rows(dQacc, acc_ld, dQ, p.B, p.H, p.n, p.d, p.sq, p.scale, st));
         else MOA_TRY(convert_f32_to_bf16(dQacc, dQ, elems, p.scale, st));

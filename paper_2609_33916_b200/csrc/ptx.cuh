@@ -40,6 +40,13 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
 // scheduler that, as far as this CTA is concerned, the next kernel's CTAs may be started (they are, once every CTA of this grid
 // has said so or exited, on whatever SM resources are free).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer whose loads must stay behind the wait: the compiler may otherwise take what a `const __restrict__` pointer shows
+// for constant over the whole kernel.
+template <typename T> __device__ __forceinline__ T *after_wait(T *p)
+{
+    asm volatile("" : "+l"(p) :: "memory");
+    return p;
+}
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)

@@ -255,7 +255,8 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     float *Qs = smem, *Ks = Qs + BM * LD, *Vs = Ks + BN * LD;
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, warp = tid / 32;
     float *Pw = Vs + BN * LD + warp * BN * LP;      // this warp's P^T: [key][2 R rows]
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    ptx::grid_dependency_wait();
+    Q = ptx::after_wait(Q); K = ptx::after_wait(K); V = ptx::after_wait(V); dO = ptx::after_wait(dO);
 
     const int rank = split > 1 ? (int)cluster_rank() : 0;
     const int job = (int)blockIdx.x / split;
@@ -353,6 +354,9 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     }
     cp_wait<0>();
     __syncthreads();
+    // (only here: the grid leaves slots free, and a successor's CTAs that sit in them from the start skew the balance of its
+    // own work -- B2 H1 n2048 d64: 252 us per fused call with the trigger on top, 219 here)
+    ptx::grid_launch_dependents();
     // partial results into shared memory: O [BM][LD] over Q, then m, l
     float *Om = smem, *Mm = Ks, *Lm = Ks + BM;
 #pragma unroll
@@ -415,7 +419,9 @@ template <typename T>
 __global__ void row_dot_kernel(const T *__restrict__ dO, const T *__restrict__ O,
                                float *__restrict__ Dv, float *__restrict__ dQzero, size_t rows, int d)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    dO = ptx::after_wait(dO); O = ptx::after_wait(O);
     const size_t row = (size_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     if (row >= rows) return;
     const int lane = threadIdx.x % 32;
@@ -534,8 +540,9 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
         tile_in<T, BM, D>(dOs, dO, q0, n);
         cp_commit();
     }
-    // launched as a programmatic dependent of the kernel that writes L and D and clears dQ
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (the tiles above are the call's inputs; L, D and the cleared dQ come from the kernel in front)
+    ptx::grid_dependency_wait();
+    L = ptx::after_wait(L); Dv = ptx::after_wait(Dv);
     for (; q0 < n; q0 += step) {
         if (tid < BM) {
             const bool live = q0 + tid < n;
@@ -622,6 +629,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
                 }
         }
     }
+    ptx::grid_launch_dependents();       // (late, as in the forward)
     if (split == 1) {
 #pragma unroll
         for (int i = 0; i < R / 2; ++i)
@@ -937,7 +945,9 @@ simt_rowpar_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
 __global__ void __launch_bounds__(256)
 convert_kernel(const float *__restrict__ src, __nv_bfloat16 *__restrict__ dst, size_t count, float mul)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");      // launched as a programmatic dependent of the kernel that fills src
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    src = ptx::after_wait(src);
     const size_t quads = count / 4;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -965,7 +975,9 @@ __global__ void __launch_bounds__(256)
 convert_rows_kernel(const float *__restrict__ src, int src_ld, __nv_bfloat16 *__restrict__ dst, size_t rows, int n, int H,
                     int d, Strides ds, float mul)
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    src = ptx::after_wait(src);
     const int quads_per_row = d / 4;
     const size_t total = rows * (size_t)quads_per_row;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -995,25 +1007,6 @@ int simt_split(long long tiles, int others, long long slots)
     return s;
 }
 
-template <typename... KArgs, typename... Args>
-cudaError_t launch_simt(void (*kernel)(KArgs...), long long ctas, int split, size_t smem, bool dependent, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(SNT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = dependent && pdl_enabled() ? 1 : 0;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)split;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
 // Rows per thread: the widest tile (fewest shared-memory loads per multiply-add) whose tiles, shared by clusters as far as
 // that goes, still give most SMs a CTA; narrower tiles below that, where the time is one CTA's latency.
 template <typename T, int R, int D>
@@ -1029,7 +1022,7 @@ cudaError_t fwd_r(const Problem &p, const void *Q, const void *K, const void *V,
     const cudaError_t e = allow_smem<simt_fwd_kernel<T, R, D>>(S::kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_simt(simt_fwd_kernel<T, R, D>, tiles * split, split, S::kSmem, false, st, (const T *)Q, (const T *)K, (const T *)V,
+    return launch_cluster(simt_fwd_kernel<T, R, D>, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K, (const T *)V,
                        (T *)O, L, (const T *)pr.dO, pr.Dv, pr.dQzero, p.n, p.causal, p.scale, nqt, split);
 }
 template <typename T, int D>
@@ -1052,7 +1045,7 @@ cudaError_t bwd_kv_r(const Problem &p, const void *Q, const void *K, const void 
     const cudaError_t e = allow_smem<simt_bwd_kv_kernel<T, R, D>>(S::kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
-    return launch_simt(simt_bwd_kv_kernel<T, R, D>, tiles * split, split, S::kSmem, true, st, (const T *)Q, (const T *)K,
+    return launch_cluster(simt_bwd_kv_kernel<T, R, D>, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K,
                        (const T *)V, (const T *)dO, L, Dv, (T *)dK, (T *)dV, dQacc, p.n, p.causal, p.scale, nkt, split);
 }
 template <typename T, int D>
@@ -1141,11 +1134,10 @@ cudaError_t row_dot(const Problem &p, int dtype, const void *dO, const void *O, 
     const unsigned grid = (unsigned)((rows + wpb - 1) / wpb);
     LaunchScope scope(MOA_KERNEL_PREPROCESS, st);
     if (dtype == MOA_F32)
-        row_dot_kernel<float><<<grid, wpb * 32, 0, st>>>((const float *)dO, (const float *)O, Dv, dQzero, rows, p.d);
-    else
-        row_dot_kernel<__nv_bfloat16><<<grid, wpb * 32, 0, st>>>((const __nv_bfloat16 *)dO,
-                                                                 (const __nv_bfloat16 *)O, Dv, dQzero, rows, p.d);
-    return cudaGetLastError();
+        return launch_dependent(row_dot_kernel<float>, dim3(grid), dim3(wpb * 32), (size_t)0, st, (const float *)dO, (const float *)O,
+                                Dv, dQzero, rows, p.d);
+    return launch_dependent(row_dot_kernel<__nv_bfloat16>, dim3(grid), dim3(wpb * 32), (size_t)0, st, (const __nv_bfloat16 *)dO,
+                            (const __nv_bfloat16 *)O, Dv, dQzero, rows, p.d);
 }
 
 cudaError_t convert_f32_to_bf16(const float *src, void *dst, size_t count, float mul, cudaStream_t st)

@@ -76,10 +76,12 @@ template <int D>
 __global__ void __launch_bounds__(256)
 bwd_preprocess_kernel(const __nv_bfloat16 *__restrict__ dO, const __nv_bfloat16 *__restrict__ O,
                       const float *__restrict__ L, float *__restrict__ Lp, float *__restrict__ Dp,
-                      int n, int n_pad, size_t padded_rows, int H, Strides so, int d)
+                      float *__restrict__ zero_acc, int n, int n_pad, size_t padded_rows, int H, Strides so, int d)
 {
     // d <= D: the head dimension in memory (lanes past it contribute zeros)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // the backward kernel behind this one may set itself up
+    grid_dependency_wait();
+    grid_launch_dependents();      // the backward kernel behind this one may set itself up
+    L = after_wait(L); dO = after_wait(dO); O = after_wait(O);
     constexpr int kLanesPerRow = D / 8;
     constexpr int kRowsPerPass = 32 / kLanesPerRow;
     constexpr int kPasses = 4;
@@ -109,6 +111,14 @@ bwd_preprocess_kernel(const __nv_bfloat16 *__restrict__ dO, const __nv_bfloat16 
             if (l == 0) lv[p] = L[row];
         }
     }
+    if (zero_acc != nullptr)      // under the loads: the rows of the dQ accumulator, 32 bytes per lane
+#pragma unroll
+        for (int p = 0; p < kPasses; ++p)
+            if (real[p]) {
+                const size_t prow = prow0 + (size_t)p * kRowsPerPass, bh = prow / (size_t)n_pad;
+                float4 *z = reinterpret_cast<float4 *>(zero_acc + (bh * (size_t)n + (prow - bh * (size_t)n_pad)) * D) + 2 * l;
+                z[0] = z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
 #pragma unroll
     for (int p = 0; p < kPasses; ++p) {
         const uint32_t x[4] = {a[p].x, a[p].y, a[p].z, a[p].w}, y[4] = {b[p].x, b[p].y, b[p].z, b[p].w};
@@ -237,7 +247,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_launch_dependents();      // the dQ conversion that follows may be set up while this grid drains
     const uint32_t tbase = *tmem_base_s;
     // a misaligned shared-memory base (swizzled tiles would be misplaced) turns every role into a no-op
     const int niter = (*abortp == 0) ? niter_all : 0;
@@ -288,6 +297,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (niter > 1) load_q(1, false);
         }
         grid_dependency_wait();     // (the lanes that issued nothing, and a CTA without tiles)
+        grid_launch_dependents();   // the dQ conversion that follows may be set up while this grid drains
         for (int it = 0; it < niter; ++it) {
             if (it + kDoSlots < niter) {     // dV(it) done: its dO slot takes tile it + kDoSlots
                 if (!mbar_wait(bars + B_DOEMPTY + it % kDoSlots, (it / kDoSlots) & 1, abortp, status, ERR_EMPTY)) break;
@@ -722,7 +732,7 @@ cudaError_t launch_bwd(const Problem &p, const void *Q, const void *K, const voi
 }  // namespace
 
 cudaError_t tc_bwd_preprocess(const Problem &p, const void *dO, const void *O, const float *L, float *Lp, float *Dp,
-                              cudaStream_t st)
+                              float *zero_acc, cudaStream_t st)
 {
     const int n_pad = (p.n + 127) / 128 * 128;
     const size_t rows = (size_t)p.BH() * n_pad;
@@ -731,16 +741,9 @@ cudaError_t tc_bwd_preprocess(const Problem &p, const void *dO, const void *O, c
     const size_t rows_per_block = (size_t)wpb * (32 / (D / 8)) * 4;   // warps x rows per pass x passes
     const unsigned grid = (unsigned)((rows + rows_per_block - 1) / rows_per_block);
     LaunchScope scope(MOA_KERNEL_PREPROCESS, st);
-    if (D == 256)
-        bwd_preprocess_kernel<256><<<grid, wpb * 32, 0, st>>>((const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, L,
-                                                              Lp, Dp, p.n, n_pad, rows, p.H, p.so, p.d);
-    else if (D == 64)
-        bwd_preprocess_kernel<64><<<grid, wpb * 32, 0, st>>>((const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, L,
-                                                             Lp, Dp, p.n, n_pad, rows, p.H, p.so, p.d);
-    else
-        bwd_preprocess_kernel<128><<<grid, wpb * 32, 0, st>>>((const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, L,
-                                                              Lp, Dp, p.n, n_pad, rows, p.H, p.so, p.d);
-    return cudaGetLastError();
+    const auto kernel = D == 256 ? bwd_preprocess_kernel<256> : D == 64 ? bwd_preprocess_kernel<64> : bwd_preprocess_kernel<128>;
+    return launch_dependent(kernel, dim3(grid), dim3(wpb * 32), (size_t)0, st, (const __nv_bfloat16 *)dO, (const __nv_bfloat16 *)O, L,
+                            Lp, Dp, zero_acc, p.n, n_pad, rows, p.H, p.so, p.d);
 }
 
 cudaError_t tc_bwd_kv(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,

@@ -156,10 +156,15 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             mbar_arrive_expect_tx(bars + W_DOFULL, 4 * SM::kBoxQ);
             for (int b = 0; b < 4; ++b) tma_load_4d(sdO + b * SM::kBoxQ, &mapdO, bars + W_DOFULL, 64 * b, q0, qh + hq0, bb);
         };
+        // (K, V, Q and dO are the call's inputs; -L, -D and the cleared accumulator come from the kernel in front)
         if (lane == 0 && niter > 0) {
-            load_qown(0);
             load_qoth(0);
             load_do(0);
+        }
+        grid_dependency_wait();
+        grid_launch_dependents();
+        if (lane == 0 && niter > 0) {
+            load_qown(0);
             if (niter > 1) load_qown(1);
         }
         // Refills, in the order in which the commits they wait for happen: the other half of Q_{it+1} when S(it) has
@@ -268,6 +273,7 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     } else if (warp >= kReduceWarp0) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
         // ------------------------------------------------- dQ warps: lanes are the 128 columns of this pass's d-half
+        grid_dependency_wait();      // the accumulator these warps add into was cleared by the kernel in front
         const int lane_row = 32 * (warp % 4) + lane;
         const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp % 4)) << 16);
         const bool col_exists = 128 * pass + lane_row < d;      // (the accumulator row is 256 wide; columns past d stay zero)
@@ -453,7 +459,6 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
         !make_tensor_map_4d_strided(&mdk, dK, bf, 2, p.B, hkv, p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64) ||
         !make_tensor_map_4d_strided(&mdv, dV, bf, 2, p.B, hkv, p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64))
         return cudaErrorInvalidValue;
-    auto kernel = tc_bwd_wide_kernel<kGrouped>;
     constexpr int kSmem = WideSmem::kTotal;
     cudaError_t e = allow_smem<tc_bwd_wide_kernel<kGrouped>>(kSmem);
     if (e != cudaSuccess) return e;
@@ -463,10 +468,9 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
     pkv.H = hkv;
     pkv.Hkv = 0;
     // two CTAs (the two halves of d) per (K/V head, key tile), adjacent in the grid: they share every load in L2
-    kernel<<<(unsigned)(2 * nkt * p.BHkv()), kThreads, kSmem, st>>>(
+    return launch_dependent(tc_bwd_wide_kernel<kGrouped>, dim3((unsigned)(2 * nkt * p.BHkv())), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mdo, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.d, p.causal, p.scale, p.scale * kLog2e, nkt,
         heads_per_group(pkv, nkt), p.group(), hkv, device_status_ptr());
-    return cudaGetLastError();
 }
 
 }  // namespace

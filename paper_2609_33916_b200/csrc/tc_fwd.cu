@@ -128,6 +128,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         mbar_init(bars + F_KFULL, 1u);
         mbar_init(bars + F_KFULL + 1, 1u);
         fence_mbar_init();
+        grid_dependency_wait();
         if (early_k > 0) {
             mbar_arrive_expect_tx(bars + F_Q, KC * kTileBytes);
             for (int b = 0; b < KC * kBoxes; ++b) tma_load_4d(sQ + b * kBoxBytes, &mapQ, bars + F_Q, 64 * b, q0, hq, bb);
@@ -143,6 +144,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         mbar_init(bars + F_VFULL, 1u);
         mbar_init(bars + F_VFULL + 1, 1u);
         fence_mbar_init();
+        grid_dependency_wait();
         for (int j = 0; j < early_v; ++j) {
             mbar_arrive_expect_tx(bars + F_VFULL + j, kTileBytes);
             for (int b = 0; b < kBoxes; ++b)
@@ -163,6 +165,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_dependency_wait();
+    // Short launches let the next kernel set itself up from the start (B1 H32 n512 causal 34.8 -> 31.0 us per fused call); long ones
+    // only as they end: there the set-up is nothing, and B1 H16 n16384 took 1.2 % longer with the early trigger.
+    if (gridDim.x <= 512) grid_launch_dependents();
     const uint32_t tbase = *tmem_base_p;
     const int nkt = (*abortp == 0) ? nkt_want : 0;   // misaligned shared memory: every role is a no-op
 
@@ -411,7 +417,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             const uint4 *src = reinterpret_cast<const uint4 *>(prep.dO + prep.so.at(bb, hq, row) + (D / 2) * h);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k)      // columns past the head dimension count as zeros
-                dov[k] = (D / 2) * h + 8 * k < prep.d ? __ldg(src + k) : make_uint4(0u, 0u, 0u, 0u);
+                dov[k] = (D / 2) * h + 8 * k < prep.d ? src[k] : make_uint4(0u, 0u, 0u, 0u);
         }
         float dpart = 0.f;
         xch[h * 128 + lane_row] = make_float2(m_used, l);
@@ -505,11 +511,10 @@ cudaError_t launch_fwd(const Problem &p, const void *Q, const void *K, const voi
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + BM - 1) / BM;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    tc_fwd_kernel<D, KC><<<(unsigned)(nqt * p.BH() * KC), kThreads, kSmem, st>>>(
+    return launch_dependent(tc_fwd_kernel<D, KC>, dim3((unsigned)(nqt * p.BH() * KC)), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mo, L, p.n, p.causal, p.scale * kLog2e, nqt, heads_per_group(p, nqt), p.group(), p.H,
         FwdSplit{p.n, 1, (p.n + BN - 1) / BN}, fb.zero_acc,
         FwdPrep{(const __nv_bfloat16 *)fb.dO, fb.Lp, fb.Dp, nqt * BM, p.so, p.d}, device_status_ptr());
-    return cudaGetLastError();
 }
 
 // Decode through the forward kernel: the G query heads that share a K/V head are the query rows of
@@ -531,10 +536,9 @@ cudaError_t launch_fwd_decode(int B, int Hkv, int G, int n, float scale, const v
     cudaError_t e = allow_smem<tc_fwd_kernel<D, 1>>(kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    tc_fwd_kernel<D, 1><<<(unsigned)(B * Hkv * splits), kThreads, kSmem, st>>>(
+    return launch_dependent(tc_fwd_kernel<D, 1>, dim3((unsigned)(B * Hkv * splits)), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mo, L_part, n, 0, scale * kLog2e, 1, 1, 1, Hkv, FwdSplit{G, splits, tiles_per_split},
         nullptr, FwdPrep{nullptr, nullptr, nullptr, 0, Strides{0, 0, 0}, D}, device_status_ptr());
-    return cudaGetLastError();
 }
 
 }  // namespace

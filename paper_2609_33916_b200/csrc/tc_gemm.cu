@@ -168,6 +168,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     __syncthreads();
     if (kPair) cluster_sync_all();       // the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after();
+    grid_dependency_wait();
+    grid_launch_dependents();
     const uint32_t tbase = *tmem_slot;
 
     if (warp == 0 && lane == 0) {
@@ -567,28 +569,9 @@ cudaError_t launch_gemm_as(const Operand &A0, const Operand &B0, const Operand *
     // persistent grid: one CTA per SM, or as many clusters of two as the device can hold at once
     const int sms = device_info().sms, pairs = kPair ? max_active_pairs(kernel, kSmem) : 0;
     const int ctas = kPair ? 2 * (tiles < pairs ? tiles : pairs) : (tiles < sms ? tiles : sms);
-    if (!kPair) {
-        kernel<<<ctas, kGemmThreads, kSmem, st>>>(ma0, mb0, ma1, mb1, mc[0], mc[1], mc[2], mc[3], M, N, K, nparts, nbatch,
-                                                  a_blocked ? 1 : 0, b_blocked ? 1 : 0, has_res ? 1 : 0, (int)group_rows,
-                                                  device_status_ptr());
-        return cudaGetLastError();
-    }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = kSmem;
-    cfg.stream = st;
-    if (kPair) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, kernel, ma0, mb0, ma1, mb1, mc[0], mc[1], mc[2], mc[3], M, N, K, nparts, nbatch,
-                              a_blocked ? 1 : 0, b_blocked ? 1 : 0, has_res ? 1 : 0, (int)group_rows, device_status_ptr());
+    return launch_cluster(kernel, kPair ? 2u : 1u, dim3((unsigned)ctas), dim3(kGemmThreads), (size_t)kSmem, st, ma0, mb0, ma1, mb1, mc[0],
+                          mc[1], mc[2], mc[3], M, N, K, nparts, nbatch, a_blocked ? 1 : 0, b_blocked ? 1 : 0, has_res ? 1 : 0,
+                          (int)group_rows, device_status_ptr());
 }
 
 // Pairs of CTAs (tiles of 256 rows, half the B traffic per SM) by default; single CTAs where pairs would need more
