@@ -111,6 +111,9 @@ size_t decode_workspace_bytes(const DecodeProblem &p, int dtype);    // partial 
 cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const void *K, const void *V, void *out,
                         float *lse, void *ws, cudaStream_t st);
 
+// counters of a merge by the last CTA to zero, in stream order
+cudaError_t decode_clear(unsigned int *counters, int count, cudaStream_t st);
+
 // Host-side launch counter (moa_launch_count).
 void count_launch(int k = 1);
 

@@ -14,8 +14,11 @@
 //     butterfly over the lanes of the row;
 //   * online softmax per lane group (exp2, running max and sum), out += p * v on the lane's own
 //     elements of the V row: no further exchange inside the loop;
-//   * at the end the lane groups of a warp, the warps of the CTA (through shared memory) and,
-//     in a second tiny kernel, the CTAs of a head are merged by their running maxima.
+//   * at the end the lane groups of a warp, the warps of the CTA (through shared memory) and the CTAs
+//     of a head are merged by their running maxima: up to eight CTAs are a cluster and read each other's
+//     shared memory (one launch, nothing through global memory); more of them leave partial results in the
+//     workspace and the last one to finish merges, told by a counter that a one-block kernel in front has
+//     cleared -- the streaming starts without waiting for it.
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -25,6 +28,7 @@ namespace {
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
 constexpr int kUnroll = 4;
+constexpr int kMaxCluster = 8;      // segments of a head that are one cluster (the portable size)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -126,10 +130,10 @@ struct DecodeState {
         }
     }
 
-    // Merge the lane groups of the warp, then the warps of the CTA through `sm` ([warp][g][D + 2]
-    // floats), and write this segment's partial result: part_o [splits][B*H][D], part_ml [splits][B*H][2].
-    __device__ void finish(float *sm, int warp, int lane, int nwarps, int gcount, size_t head0, int split, size_t BH,
-                           float *part_o, float *part_ml, int nthreads)
+    // Merge the lane groups of the warp, then the warps of the CTA through `sm` ([warp][g][D + 2] floats); put(g, c, o, m, l)
+    // receives this segment's unnormalised output column, running maximum and sum.
+    template <typename Put>
+    __device__ void finish(float *sm, int warp, int lane, int nwarps, int gcount, int nthreads, Put put)
     {
         const int sub = lane / LPR, l = lane % LPR;
 #pragma unroll
@@ -173,9 +177,7 @@ struct DecodeState {
                 o = fmaf(src[c], a, o);
                 ls = fmaf(src[D + 1], a, ls);
             }
-            const size_t at = (size_t)split * BH + head0 + g;
-            part_o[at * D + c] = o;
-            if (c == 0) { part_ml[at * 2] = mx; part_ml[at * 2 + 1] = ls; }
+            put(g, c, o, mx, ls);
         }
     }
 };
@@ -267,6 +269,68 @@ __device__ __forceinline__ void merge_if_last(unsigned int *counters, const Deco
     for (int g = 0; g < job.gcount; ++g) merge_head<T, D>(part_o, part_ml, out, lse, splits, BH, job.head0 + g, sh);
 }
 
+__device__ __forceinline__ float cluster_load(const float *mine, uint32_t rank)      // the same word of another CTA's shared memory
+{
+    const uint32_t at = ptx::mapa_u32(ptx::smem_u32(mine), rank);
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+
+// The end of a segment: merge the CTA's warps and then the CTAs of the head (`sm`: kWarps * GC * (D + 2) floats and room for
+// the merge behind them).
+template <typename T, int D, int GC>
+__device__ __forceinline__ void finish_segment(DecodeState<T, D, GC> &st, const DecodeJob &job, float *sm, int warp, int lane, int nthreads,
+                                               int clustered, int splits, size_t BH, float *part_o, float *part_ml, T *out, float *lse,
+                                               unsigned int *counters)
+{
+    constexpr int kStride = D + 2;
+    if (!clustered) {
+        ptx::grid_dependency_wait();       // the counters are clear (and whatever read the workspace before has finished)
+        ptx::grid_launch_dependents();
+        st.finish(sm, warp, lane, kWarps, job.gcount, nthreads, [&](int g, int c, float o, float mx, float ls) {
+            const size_t at = (size_t)job.split * BH + job.head0 + g;       // part_o [splits][B*H][D], part_ml [splits][B*H][2]
+            part_o[at * D + c] = o;
+            if (c == 0) { part_ml[at * 2] = mx; part_ml[at * 2 + 1] = ls; }
+        });
+        merge_if_last<T, D>(counters, job, splits, BH, part_o, part_ml, out, lse, sm);
+        return;
+    }
+    float *seg = sm + kWarps * GC * kStride;       // this segment's result, [g][D + 2]
+    st.finish(sm, warp, lane, kWarps, job.gcount, nthreads, [&](int g, int c, float o, float mx, float ls) {
+        seg[g * kStride + c] = o;
+        if (c == 0) { seg[g * kStride + D] = mx; seg[g * kStride + D + 1] = ls; }
+    });
+    if (splits > 1) ptx::cluster_sync_all();
+    else __syncthreads();
+    // the ranks share the columns of the group's heads; segments are added in rank order
+    for (int idx = job.split * nthreads + (int)threadIdx.x; idx < job.gcount * D; idx += splits * nthreads) {
+        const int g = idx / D, c = idx - g * D;
+        const float *at = seg + g * kStride;
+        float mt = -INFINITY, o = 0.f, ls = 0.f;
+        for (int k = 0; k < splits; ++k) mt = fmaxf(mt, cluster_load(at + D, k));
+        for (int k = 0; k < splits; ++k) {
+            const float a = exp2f(cluster_load(at + D, k) - mt);
+            o = fmaf(cluster_load(at + c, k), a, o);
+            ls = fmaf(cluster_load(at + D + 1, k), a, ls);
+        }
+        const size_t head = job.head0 + g;
+        out[head * D + c] = from_float<T>(o / ls);
+        if (lse && c == 0) lse[head] = (mt + log2f(ls)) * kLn2;
+    }
+    __syncwarp();
+    if (splits > 1) ptx::cluster_sync_all();       // nobody leaves while another CTA may still read its shared memory
+}
+
+// Clears the counters of the merge by the last CTA.  A kernel, not a memset: the streaming kernel is its programmatic dependent
+// and waits for it only before it publishes its partial results.
+__global__ void __launch_bounds__(256) decode_clear_kernel(unsigned int *__restrict__ counters, int count)
+{
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    for (int i = threadIdx.x; i < count; i += blockDim.x) counters[i] = 0u;
+}
+
 // ---- variant 1: rows straight from global memory into registers (16-byte streaming loads, kUnroll row
 // groups of K and of V in flight per warp).  Few registers when the group is small, so several CTAs
 // per SM keep enough bytes in flight: used for one or two query heads per K/V head.
@@ -274,9 +338,15 @@ template <typename T, int D, int GC>
 __global__ void __launch_bounds__(kThreads)
 decode_split_kernel(const T *__restrict__ q, const T *__restrict__ K, const T *__restrict__ V,
                     float *__restrict__ part_o, float *__restrict__ part_ml, T *__restrict__ out, float *__restrict__ lse,
-                    unsigned int *__restrict__ counters,
+                    unsigned int *__restrict__ counters, int clustered,
                     int n, int H, int Hkv, int group, int splits, int keys_per_split, size_t BH, float scale_log2)
 {
+    // in a cluster this is the call's first kernel; otherwise the clearing kernel in front of it is
+    if (clustered) {
+        ptx::grid_dependency_wait();
+        ptx::grid_launch_dependents();
+    }
+    q = ptx::after_wait(q); K = ptx::after_wait(K); V = ptx::after_wait(V);
     using State = DecodeState<T, D, GC>;
     constexpr int E = State::E, LPR = State::LPR, RPW = State::RPW;
     const DecodeJob job(splits, GC, group, H, Hkv, n, keys_per_split);
@@ -301,8 +371,7 @@ decode_split_kernel(const T *__restrict__ q, const T *__restrict__ K, const T *_
         st.template consume<kUnroll>(kraw, vraw, live);
     }
     extern __shared__ float sm[];
-    st.finish(sm, warp, lane, kWarps, job.gcount, job.head0, job.split, BH, part_o, part_ml, kThreads);
-    merge_if_last<T, D>(counters, job, splits, BH, part_o, part_ml, out, lse, sm);
+    finish_segment<T, D, GC>(st, job, sm, warp, lane, kThreads, clustered, splits, BH, part_o, part_ml, out, lse, counters);
 }
 
 // ---- variant 2: the cache segment streams through a shared-memory ring filled by bulk copies (a tile
@@ -323,7 +392,7 @@ template <typename T, int D, int GC>
 __global__ void __launch_bounds__(kRingThreads, 1)
 decode_ring_kernel(const T *__restrict__ q, const T *__restrict__ K, const T *__restrict__ V,
                    float *__restrict__ part_o, float *__restrict__ part_ml, T *__restrict__ out, float *__restrict__ lse,
-                   unsigned int *__restrict__ counters,
+                   unsigned int *__restrict__ counters, int clustered,
                    int n, int H, int Hkv, int group, int splits, int keys_per_split, size_t BH, float scale_log2,
                    unsigned int *status)
 {
@@ -348,6 +417,11 @@ decode_ring_kernel(const T *__restrict__ q, const T *__restrict__ K, const T *__
         fence_mbar_init();
     }
     __syncthreads();
+    if (clustered) {       // (as in the kernel above)
+        grid_dependency_wait();
+        grid_launch_dependents();
+    }
+    q = after_wait(q);
     State st;
     if (warp == kWarps) {
         // ------------------------------------------------------------------ producer
@@ -393,9 +467,8 @@ decode_ring_kernel(const T *__restrict__ q, const T *__restrict__ K, const T *__
     }
     __syncthreads();       // every consumer is done with the ring: reuse its start for the merge
     if (warp == kWarps) st.init(q + job.head0 * D, 0, 0, 0.f);     // the producer warp holds no state
-    st.finish(reinterpret_cast<float *>(ring), warp, lane, kWarps, job.gcount, job.head0, job.split, BH, part_o,
-              part_ml, kRingThreads);
-    merge_if_last<T, D>(counters, job, splits, BH, part_o, part_ml, out, lse, reinterpret_cast<float *>(ring));
+    finish_segment<T, D, GC>(st, job, reinterpret_cast<float *>(ring), warp, lane, kRingThreads, clustered, splits, BH, part_o, part_ml, out,
+                             lse, counters);
 }
 
 // Merge for the tensor-core route: O_part [splits*B, Hkv, G, D] bf16 (each normalised over its own
@@ -407,6 +480,9 @@ decode_merge_tc_kernel(const __nv_bfloat16 *__restrict__ O_part, const float *__
 {
     constexpr int kStripes = 256 / D;
     __shared__ float sh_o[kStripes][D], sh_m[kStripes], sh_l[kStripes];
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    O_part = ptx::after_wait(O_part); L_part = ptx::after_wait(L_part);
     const int head = blockIdx.x;                      // b * H + kvh * G + g
     const int H = Hkv * G;
     const int b = head / H, hq = head - b * H, kvh = hq / G, g = hq - kvh * G;
@@ -440,6 +516,16 @@ decode_merge_tc_kernel(const __nv_bfloat16 *__restrict__ O_part, const float *__
     }
 }
 
+}  // namespace
+
+cudaError_t decode_clear(unsigned int *counters, int count, cudaStream_t st)
+{
+    LaunchScope scope(MOA_KERNEL_OTHER, st);
+    return launch_dependent(decode_clear_kernel, dim3(1), dim3(256), (size_t)0, st, counters, count);
+}
+
+namespace {
+
 int group_chunk(int group) { return group >= 8 ? 8 : group >= 4 ? 4 : group >= 2 ? 2 : 1; }
 
 template <typename T, int D, int GC>
@@ -449,29 +535,31 @@ cudaError_t launch_split(const DecodeProblem &p, const void *q, const void *K, c
 {
     const int group = p.H / p.Hkv;
     dim3 grid((unsigned)(p.B * p.Hkv * splits), (unsigned)((group + GC - 1) / GC));
-    size_t merge_smem = (size_t)kWarps * GC * (D + 2) * sizeof(float);       // warps' states; then the stripes of merge_head
+    // warps' states and this segment's result; or the stripes of merge_head
+    size_t merge_smem = (size_t)(kWarps + 1) * GC * (D + 2) * sizeof(float);
     if (merge_smem < (size_t)(256 / D) * (D + 2) * sizeof(float)) merge_smem = (size_t)(256 / D) * (D + 2) * sizeof(float);
-    // one counter per (K/V head, chunk of query heads): the last of its CTAs to finish merges
-    cudaError_t ce = cudaMemsetAsync(counters, 0, (size_t)p.B * p.Hkv * grid.y * sizeof(unsigned int), st);
-    if (ce != cudaSuccess) return ce;
+    const int clustered = splits <= kMaxCluster ? 1 : 0;
+    if (!clustered) {       // one counter per (K/V head, chunk of query heads): the last of its CTAs to finish merges
+        const cudaError_t ce = decode_clear(counters, (int)(p.B * p.Hkv * grid.y), st);
+        if (ce != cudaSuccess) return ce;
+    }
+    const unsigned cluster = clustered ? (unsigned)splits : 1u;
     LaunchScope scope(MOA_KERNEL_OTHER, st);
     if (GC >= 4) {
         constexpr int kStages = Ring<T, D>::kStages;
-        const size_t smem = (size_t)kStages * 2 * kTileRows * D * sizeof(T) + 2 * kStages * sizeof(uint64_t) + 16;
-        cudaError_t e = allow_smem<decode_ring_kernel<T, D, GC>>(smem > merge_smem ? smem : merge_smem);
+        const size_t ring_smem = (size_t)kStages * 2 * kTileRows * D * sizeof(T) + 2 * kStages * sizeof(uint64_t) + 16;
+        const size_t smem = ring_smem > merge_smem ? ring_smem : merge_smem;
+        cudaError_t e = allow_smem<decode_ring_kernel<T, D, GC>>(smem);
         if (e != cudaSuccess) return e;
-        decode_ring_kernel<T, D, GC><<<grid, kRingThreads, smem > merge_smem ? smem : merge_smem, st>>>(
-            (const T *)q, (const T *)K, (const T *)V, part_o, part_ml, (T *)out, lse, counters, p.n, p.H, p.Hkv, group, splits,
-            keys_per_split, (size_t)p.B * p.H, p.scale * kLog2e, device_status_ptr());
-        return cudaGetLastError();
+        return launch_cluster(decode_ring_kernel<T, D, GC>, cluster, grid, dim3(kRingThreads), smem, st, (const T *)q, (const T *)K,
+                              (const T *)V, part_o, part_ml, (T *)out, lse, counters, clustered, p.n, p.H, p.Hkv, group, splits,
+                              keys_per_split, (size_t)p.B * p.H, p.scale * kLog2e, device_status_ptr());
     }
     cudaError_t e = allow_smem<decode_split_kernel<T, D, GC>>(merge_smem);
     if (e != cudaSuccess) return e;
-    decode_split_kernel<T, D, GC><<<grid, kThreads, merge_smem, st>>>((const T *)q, (const T *)K, (const T *)V, part_o,
-                                                                      part_ml, (T *)out, lse, counters, p.n, p.H, p.Hkv,
-                                                                      group, splits, keys_per_split, (size_t)p.B * p.H,
-                                                                      p.scale * kLog2e);
-    return cudaGetLastError();
+    return launch_cluster(decode_split_kernel<T, D, GC>, cluster, grid, dim3(kThreads), merge_smem, st, (const T *)q, (const T *)K,
+                          (const T *)V, part_o, part_ml, (T *)out, lse, counters, clustered, p.n, p.H, p.Hkv, group, splits, keys_per_split,
+                          (size_t)p.B * p.H, p.scale * kLog2e);
 }
 
 template <typename T, int D>
@@ -484,7 +572,6 @@ cudaError_t launch_decode(const DecodeProblem &p, const void *q, const void *K, 
     float *part_o = ws, *part_ml = ws + (size_t)splits * BH * D;
     unsigned int *counters = reinterpret_cast<unsigned int *>(part_ml + (size_t)splits * BH * 2);
     const int gc = group_chunk(p.H / p.Hkv);
-    // the merge of a head's segments is done by the last of its CTAs to finish (no merge launch)
     return gc == 8 ? launch_split<T, D, 8>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st)
          : gc == 4 ? launch_split<T, D, 4>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st)
          : gc == 2 ? launch_split<T, D, 2>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st)
@@ -526,18 +613,23 @@ static void decode_tc_splits(const DecodeProblem &p, int *splits, int *tiles_per
     *splits = (nkt + tps - 1) / tps;          // every segment has at least one tile
 }
 
-// Segments of the cache per K/V head: enough CTAs to fill the GPU a few times over, each with at
-// least 256 keys.
+// Segments of the cache per K/V head: enough CTAs to fill the GPU a few times over, each with at least 128 keys (one round of
+// loads of the bf16 d = 64 kernel; with 256 a short cache left half of the SMs idle: B1 H16 n1000 8.2 -> 5.3 us) or, in the
+// ring kernel, of which an SM holds one CTA, 256 (with 128: fp32 groups of 8 over 4359 keys 54 -> 66 us).  Up to eight
+// segments, a power of two, are one cluster.
 int decode_splits(const DecodeProblem &p)
 {
     const int group = p.H / p.Hkv;
-    const int gc = group >= 8 ? 8 : group >= 4 ? 4 : group >= 2 ? 2 : 1;
+    const int gc = group_chunk(group);
     const long long ctas_per_split = (long long)p.B * p.Hkv * ((group + gc - 1) / gc);
     long long s = (4LL * device_info().sms + ctas_per_split - 1) / ctas_per_split;
-    const long long cap = (p.n + 255) / 256;
+    const long long least = gc >= 4 ? 256 : 128, cap = (p.n + least - 1) / least;
     if (s > cap) s = cap;
     if (s < 1) s = 1;
     if (s > 1024) s = 1024;
+    if (s <= kMaxCluster)
+        for (int c = 1; c <= kMaxCluster; c *= 2)
+            if (c >= s) { s = c; break; }
     return (int)s;
 }
 
@@ -566,13 +658,9 @@ cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const 
         cudaError_t e = tc_fwd_decode(p.B, p.Hkv, G, p.n, p.d, p.scale, q, K, V, O_part, L_part, splits, tps, st);
         if (e != cudaSuccess) return e;
         LaunchScope scope(MOA_KERNEL_OTHER, st);
-        if (p.d == 64)
-            decode_merge_tc_kernel<64><<<(unsigned)(p.B * p.H), 256, 0, st>>>((const __nv_bfloat16 *)O_part, L_part,
-                                                                              (__nv_bfloat16 *)out, lse, splits, p.B, p.Hkv, G);
-        else
-            decode_merge_tc_kernel<128><<<(unsigned)(p.B * p.H), 256, 0, st>>>((const __nv_bfloat16 *)O_part, L_part,
-                                                                               (__nv_bfloat16 *)out, lse, splits, p.B, p.Hkv, G);
-        return cudaGetLastError();
+        return launch_dependent(p.d == 64 ? decode_merge_tc_kernel<64> : decode_merge_tc_kernel<128>, dim3((unsigned)(p.B * p.H)), dim3(256),
+                                (size_t)0, st, (const __nv_bfloat16 *)O_part, (const float *)L_part, (__nv_bfloat16 *)out, lse, splits, p.B,
+                                p.Hkv, G);
     }
     float *wsf = (float *)ws;
     if (dtype == MOA_F32) {
