@@ -95,6 +95,30 @@ inline int heads_per_group(const Problem &p, int tiles)
     return (int)g;
 }
 
+// CTAs that share a key tile of the backward (a cluster; each takes a contiguous part of the tile's query tiles and the partial
+// dK, dV are added through distributed shared memory).  One CTA per key tile leaves SMs idle when there are few tiles, and with
+// shared K/V heads or the causal mask the longest tile alone can outlast the average SM's share by far.  Estimated in units
+// of one query tile: a CTA costs `fixed` beside its tiles, a merge `merge` more; equal jobs go in rounds, causal ones longest first,
+// which packs to within a part of an average job.  A cluster has to beat the next smaller one by 5 %.
+//   jobs: key tiles of all K/V heads (times the passes over d); longest, total: query tiles of the longest job, of all jobs
+inline int bwd_split(long long jobs, long long longest, long long total, bool causal, double fixed, double merge)
+{
+    const double sms = device_info().sms;
+    int best = 1;
+    double best_cost = 0;
+    for (int s = 1; s <= 8; s *= 2) {
+        if (s > 1 && (longest < s || jobs * s > 8 * (long long)sms)) break;
+        const double slots = s <= 2 ? sms : s == 4 ? 0.9 * sms : 0.85 * sms;     // (clusters of 4 and 8 leave SMs of a GPC over)
+        const double extra = fixed + (s > 1 ? merge : 0.0), job = (double)longest / s + extra;
+        const double avg = ((double)total + (double)jobs * s * extra) / slots, mean = (double)total / (jobs * s) + extra;
+        const long long n = jobs * s, rounds = (n + (long long)slots - 1) / (long long)slots;
+        const double even = (double)rounds * job, packed = avg + 0.5 * mean;
+        const double cost = causal ? (job > packed ? job : packed < even ? packed : even) : even;
+        if (s == 1 || cost < 0.95 * best_cost) { best = s; best_cost = cost; }
+    }
+    return best;
+}
+
 // Decode through the tensor-core forward kernel (tc_fwd.cu): the G query heads of a K/V head are
 // the rows of one query tile, the cache is split among CTAs; partial results to be merged.
 cudaError_t tc_fwd_decode(int B, int Hkv, int G, int n, int d, float scale, const void *q, const void *K, const void *V,
@@ -232,7 +256,9 @@ cudaError_t tc_bwd_preprocess(const Problem &p, const void *dO, const void *O, c
 // (fp32 [B,H,n,kernel_d(d)], pre-zeroed); dQacc == nullptr skips the dQ contraction altogether
 cudaError_t tc_bwd_kv(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
                       const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, int dq_bulk,
-                      cudaStream_t st);   // dq_bulk: TMA bulk add-reduce instead of red.global (d = 128 only)
+                      bool share, cudaStream_t st);   // dq_bulk: TMA bulk add-reduce instead of red.global (d <= 128 only)
+// share: several CTAs may share a key tile (bwd_split).  MOA_DQ_AUTO only: the dq_modes a caller names are for comparing the
+// strategies, all on the same one-CTA-per-key-tile form (and its bits of dK, dV, which the paired form reproduces).
 
 // The same on pairs of CTAs (tc_bwd_pair.cu; the 128-column kernel only), and whether tc_bwd_kv hands such
 // problems to it (moa_bwd_pair_mode; environment variable MOA_BWD_PAIR=1 for the initial mode; default: no)
@@ -245,7 +271,7 @@ int bwd_pair_mode(int set);      // set < 0: query; returns the mode in force be
 // Head dimensions 136..256 (tc_bwd_wide.cu): tiles of 128 keys x 64 queries, two passes over the halves of d; dQ by
 // red.global into dQacc (fp32 [B,H,n,256], pre-zeroed)
 cudaError_t tc_bwd_kv_wide(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
-                           const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, cudaStream_t st);
+                           const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st);
 
 // atomic-free query-parallel dQ pass on the tensor cores (tc_dq.cu); writes dQ (bf16) directly
 cudaError_t tc_bwd_dq(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,

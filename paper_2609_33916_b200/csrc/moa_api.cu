@@ -298,12 +298,12 @@ moa_status run_bwd(const moa_attn_desc *d, const void *Q, const void *K, const v
     if (use_tc_bwd(d)) {
         if (!prepared) MOA_TRY(tc_bwd_preprocess(p, dO, O, L, Lp, Dv, mode == MOA_DQ_SEPARATE_PASS ? nullptr : dQacc, st));
         if (mode == MOA_DQ_SEPARATE_PASS) {
-            MOA_TRY(tc_bwd_kv(p, Q, K, V, dO, Lp, Dv, dK, dV, nullptr, 0, st));
+            MOA_TRY(tc_bwd_kv(p, Q, K, V, dO, Lp, Dv, dK, dV, nullptr, 0, false, st));
             MOA_TRY(tc_bwd_dq(p, Q, K, V, dO, Lp, Dv, dQ, st));
             return MOA_OK;
         }
         const int acc_ld = kernel_d(p.d);
-        MOA_TRY(tc_bwd_kv(p, Q, K, V, dO, Lp, Dv, dK, dV, dQacc, mode == MOA_DQ_BULK_REDUCE, st));
+        MOA_TRY(tc_bwd_kv(p, Q, K, V, dO, Lp, Dv, dK, dV, dQacc, mode == MOA_DQ_BULK_REDUCE, d->dq_mode == MOA_DQ_AUTO, st));
         if (!p.contiguous_bhnd() || acc_ld != p.d) MOA_TRY(convert_f32_to_bf16_rows(dQacc, acc_ld, dQ, p.B, p.H, p.n, p.d, p.sq, p.scale, st));
         else MOA_TRY(convert_f32_to_bf16(dQacc, dQ, elems, p.scale, st));
         return MOA_OK;

@@ -364,6 +364,22 @@ __device__ __forceinline__ void tma_load_4d_pair(void *dst, const CUtensorMap *m
         ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z), "r"(w)
         : "memory");
 }
+// v = mul * (sum over the CTAs of the cluster, in rank order, of the 8 floats at the shared-memory addresses a, b)
+__device__ __forceinline__ void sum_split(uint32_t a, uint32_t b, int split, float mul, float (&v)[8])
+{
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = 0.f;
+    for (int k = 0; k < split; ++k) {
+        float x[8];
+        const uint32_t ra = mapa_u32(a, (uint32_t)k), rb = mapa_u32(b, (uint32_t)k);
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(ra) : "memory");
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]) : "r"(rb) : "memory");
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] += x[e];
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] *= mul;
+}
 // Arrival on a barrier of any CTA of the cluster that publishes this thread's earlier writes (also those to the other
 // CTA's shared memory) to whoever waits on it with cluster scope
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr)

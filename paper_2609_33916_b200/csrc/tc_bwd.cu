@@ -162,6 +162,13 @@ struct BwdSmem {
     static constexpr int kTotal = offBar + 192;
 };
 
+// kSplit: where the merged dK, dV go
+struct SplitOut {
+    __nv_bfloat16 *dK, *dV;
+    Strides skv;
+    int d;               // columns of a row in memory
+};
+
 // Barrier slots inside the shared-memory barrier block
 enum {
     B_KV = 0, B_QFULL = 1 /*2*/, B_QEMPTY = 3 /*2*/, B_DOFULL = 5 /*2*/, B_DOEMPTY = 7 /*2*/,
@@ -169,7 +176,7 @@ enum {
     B_EPI = 19 /*dK, dV tiles staged in shared memory*/, B_COUNT = 20
 };
 
-template <int D, bool kBulk, bool kGrouped>
+template <int D, bool kBulk, bool kGrouped, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapdO,
@@ -177,7 +184,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
               const __grid_constant__ CUtensorMap mapdV, const float *__restrict__ Lp, const float *__restrict__ Dp,
               float *__restrict__ dQacc,
               int n, int n_pad, int causal, float scale, float scale_log2, int nkt, int hpg, int group,
-              int Hkv, int skip_dq, unsigned int *status)
+              int Hkv, int skip_dq, unsigned int *status, int split, SplitOut out)
 {
     using SM = BwdSmem<D, kBulk>;
     constexpr int kDoSlots = SM::kDoSlots;
@@ -204,7 +211,10 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     int bh, kt;                               // causal: key tile 0 has the most query tiles and goes first
-    job_from_block((int)blockIdx.x, nkt, (int)gridDim.x / nkt, hpg, bh, kt);
+    // kSplit: the `split` CTAs of a cluster share the key tile, each takes a contiguous part of its query tiles
+    const int rank = kSplit ? (int)cluster_ctarank() : 0;
+    if (kSplit) job_from_block((int)blockIdx.x / split, nkt, (int)gridDim.x / split / nkt, hpg, bh, kt);
+    else job_from_block((int)blockIdx.x, nkt, (int)gridDim.x / nkt, hpg, bh, kt);
     const int k0 = kt * 128;
     const int nqt = n_pad / 128;
     const int i_begin = causal ? kt : 0;
@@ -216,7 +226,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     // [B*H, ...] arrays (L', D, the dQ accumulator)
     const int bb = bh / Hkv, hk = bh - bb * Hkv;
     const int hq0 = hk * (kGrouped ? group : 1) - bh * (kGrouped ? group : 1);   // query head in batch = flat index + hq0
-    const int niter_all = (kGrouped ? group : 1) * (nqt - i_begin);
+    const int niter_tile = (kGrouped ? group : 1) * (nqt - i_begin);
+    const int it0 = kSplit ? niter_tile * rank / split : 0;                 // this CTA's first query tile of the job
+    const int niter_all = kSplit ? niter_tile * (rank + 1) / split - it0 : niter_tile;
     // (query head, query tile) of consecutive iterations, advanced without a division: each role
     // keeps a walker of its own, in step with the iterations it handles.  kGrouped = false (one K/V
     // head per query head) compiles to the plain tile counter.
@@ -228,7 +240,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (kGrouped && qi == end) { qi = first; ++qh; }
         }
     };
-    const TileWalk walk0{kGrouped ? bh * group : bh, i_begin, i_begin, nqt};
+    const int head0 = kGrouped && kSplit ? it0 / (nqt - i_begin) : 0;       // query heads of the group in front of it
+    const TileWalk walk0{(kGrouped ? bh * group : bh) + head0, i_begin + it0 - head0 * (nqt - i_begin), i_begin, nqt};
 
     if (tid == 0) {
         for (int b = 0; b < B_COUNT; ++b) {
@@ -470,9 +483,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                         if (leader && stage_ok && mbar_wait(bars + B_STGFULL + st, (g >> 1) & 1, abortp, status, ERR_STAGE)) {
                             // (query head, tile) of this iteration: recomputed here, by the one thread that
                             // needs them, rather than kept live beside the 128 registers of the tile
-                            const int nq_per = nqt - i_begin;
-                            const int hh = kGrouped ? it / nq_per : 0;
-                            tma_reduce_add_3d(&mapdQ, stage, 0, (i_begin + it - hh * nq_per) * 128 + 32 * c,
+                            const int nq_per = nqt - i_begin, at = it0 + it;
+                            const int hh = kGrouped ? at / nq_per : 0;
+                            tma_reduce_add_3d(&mapdQ, stage, 0, (i_begin + at - hh * nq_per) * 128 + 32 * c,
                                               (kGrouped ? bh * group : bh) + hh);
                             bulk_commit();
                         }
@@ -633,7 +646,35 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
           }
             if (it + 1 < niter) ok = p_phase(it + 1);
         }
-        if (ok && mbar_wait(bars + B_DQ, (niter - 1) & 1, abortp, status, ERR_DQ) &&
+        if (kSplit) {
+            // partial dV, dK of this CTA's query tiles, as floats over the K, V and Q tiles, which are no longer read: rows of
+            // D floats, 16-byte chunks swizzled by the row (a thread owns a row)
+            const bool done = ok && mbar_wait(bars + B_DQ, (niter - 1) & 1, abortp, status, ERR_DQ) &&
+                (!kDKfromSmem || mbar_wait(bars + B_QEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, ERR_DQ));
+            tc_fence_after();
+#pragma unroll 1
+            for (int which = 0; which < 2; ++which) {
+                const uint32_t col = (which == 0 ? colDV : colDK) + (D / 2) * wg;
+                uint8_t *row = sm + which * (128 * D * 4) + lane_row * (D * 4);
+#pragma unroll 1
+                for (int c = 0; c < D / 2; c += 32) {
+                    uint32_t r[32];
+                    if (__all_sync(0xffffffffu, done)) {
+                        tmem_ld(lane_addr + col + c, r);
+                        tc_wait_ld();
+                    } else {              // (a CTA without query tiles adds nothing)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = 0u;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4) {
+                        const int chunk = (((D / 2) * wg + c + e) / 4) ^ (lane_row & 7);
+                        *reinterpret_cast<uint4 *>(row + chunk * 16) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
+                    }
+                }
+            }
+        }
+        if (!kSplit && ok && mbar_wait(bars + B_DQ, (niter - 1) & 1, abortp, status, ERR_DQ) &&
             (!kDKfromSmem || mbar_wait(bars + B_QEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, ERR_DQ))) {
             // All UMMAs have completed.  dV and scale*dK go out as bf16 through shared memory (the K and V
             // tiles are no longer read) and TMA stores: a thread owns a row, so direct stores would be 16
@@ -679,6 +720,25 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
+    if (kSplit) {
+        // the ranks add up the partial results, in rank order, 128 / split rows each, and write them out
+        __syncwarp();
+        cluster_sync_all();
+        if (warp < kReduceWarp0) {
+            const int per = 128 / split;
+            for (int i = tid; i < 2 * per * (D / 8); i += 32 * kReduceWarp0) {
+                const int c8 = i % (D / 8), r = rank * per + (i / (D / 8)) % per, which = i / (D / 8) / per;
+                const uint32_t row = smem_u32(sm) + which * (128 * D * 4) + r * (D * 4);
+                float v[8];
+                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), split, which == 0 ? 1.f : scale, v);
+                if (k0 + r < n && 8 * c8 < out.d)
+                    *reinterpret_cast<uint4 *>((which == 0 ? out.dV : out.dK) + out.skv.at(bb, hk, k0 + r) + 8 * c8) =
+                        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
+    }
     if (*abortp && tid == kLoadWarp * 32) {
         // A wait expired: copies this thread asked for may still be on their way into the CTA's shared memory.  It
         // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) before the CTA can leave.  (The other
@@ -688,9 +748,9 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     }
 }
 
-template <int D, bool kBulk, bool kGrouped>
+template <int D, bool kBulk, bool kGrouped, bool kSplit>
 cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
-                       const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, cudaStream_t st)
+                       const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, int split, cudaStream_t st)
 {
     CUtensorMap mq, mk, mv, mdo, mdq, mdk, mdv;
     const uint64_t heads = (uint64_t)p.BH();
@@ -708,7 +768,7 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     if (!make_tensor_map_3d(&mdq, dQacc ? (const void *)dQacc : Q, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, heads, p.n, D, 32, D == 64 ? 32 : D))
         return cudaErrorInvalidValue;
     constexpr int kSmem = BwdSmem<D, kBulk>::kTotal;
-    cudaError_t e = allow_smem<tc_bwd_kernel<D, kBulk, kGrouped>>(kSmem);
+    cudaError_t e = allow_smem<tc_bwd_kernel<D, kBulk, kGrouped, kSplit>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
@@ -716,17 +776,26 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     Problem pkv = p;
     pkv.H = p.kv_heads();
     pkv.Hkv = 0;
-    return launch_dependent(tc_bwd_kernel<D, kBulk, kGrouped>, dim3((unsigned)(nkt * p.BHkv())), dim3(kThreads), (size_t)kSmem, st,
+    return launch_cluster(tc_bwd_kernel<D, kBulk, kGrouped, kSplit>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)),
+                          dim3(kThreads), (size_t)kSmem, st,
                             mq, mk, mv, mdo, mdq, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.causal, p.scale, p.scale * kLog2e, nkt,
-                            heads_per_group(pkv, nkt), p.group(), p.kv_heads(), dQacc == nullptr ? 1 : 0, device_status_ptr());
+                            heads_per_group(pkv, nkt), p.group(), p.kv_heads(), dQacc == nullptr ? 1 : 0, device_status_ptr(),
+                            split, SplitOut{(__nv_bfloat16 *)dK, (__nv_bfloat16 *)dV, p.skv, p.d});
 }
 
 template <int D, bool kBulk>
 cudaError_t launch_bwd(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
-                       const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, cudaStream_t st)
+                       const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st)
 {
-    return p.group() > 1 ? launch_bwd_g<D, kBulk, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st)
-                         : launch_bwd_g<D, kBulk, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
+    if constexpr (kBulk) {        // (AUTO is the bulk reduce at these head dimensions)
+        const long long nkt = (p.n + 127) / 128, jobs = nkt * p.BHkv(), longest = nkt * p.group();
+        const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) / 2 : jobs * longest, p.causal, 2.0, 1.0);
+        if (split > 1)
+            return p.group() > 1 ? launch_bwd_g<D, kBulk, true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
+                                 : launch_bwd_g<D, kBulk, false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
+    }
+    return p.group() > 1 ? launch_bwd_g<D, kBulk, true, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st)
+                         : launch_bwd_g<D, kBulk, false, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st);
 }
 
 }  // namespace
@@ -747,16 +816,17 @@ cudaError_t tc_bwd_preprocess(const Problem &p, const void *dO, const void *O, c
 }
 
 cudaError_t tc_bwd_kv(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
-                      const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, int dq_bulk, cudaStream_t st)
+                      const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, int dq_bulk, bool share,
+                      cudaStream_t st)
 {
     if (p.d < 8 || p.d > 256 || p.d % 8) return cudaErrorInvalidValue;
     const int D = kernel_d(p.d);     // dQacc rows are D floats wide
-    if (D == 256) return dq_bulk ? cudaErrorInvalidValue : tc_bwd_kv_wide(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
+    if (D == 256) return dq_bulk ? cudaErrorInvalidValue : tc_bwd_kv_wide(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
     if (D == 128 && bwd_pair_enabled()) return tc_bwd_kv_pair(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, dq_bulk, st);
-    if (D == 64 && !dq_bulk) return launch_bwd<64, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
-    if (D == 64 && dq_bulk) return launch_bwd<64, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
-    if (D == 128 && !dq_bulk) return launch_bwd<128, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
-    if (D == 128 && dq_bulk) return launch_bwd<128, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
+    if (D == 64 && !dq_bulk) return launch_bwd<64, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
+    if (D == 64 && dq_bulk) return launch_bwd<64, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
+    if (D == 128 && !dq_bulk) return launch_bwd<128, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
+    if (D == 128 && dq_bulk) return launch_bwd<128, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
     return cudaErrorInvalidValue;
 }
 

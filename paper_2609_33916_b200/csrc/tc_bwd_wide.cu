@@ -62,14 +62,15 @@ __device__ __forceinline__ void red_add_f32(float *addr, float a)
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(a) : "memory");
 }
 
-template <bool kGrouped>
+template <bool kGrouped, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                    const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapdO,
                    const __grid_constant__ CUtensorMap mapdK, const __grid_constant__ CUtensorMap mapdV,
                    const float *__restrict__ Lp, const float *__restrict__ Dp, float *__restrict__ dQacc,
                    int n, int n_pad, int d, int causal, float scale, float scale_log2, int nkt, int hpg, int group,
-                   int Hkv, unsigned int *status)
+                   int Hkv, unsigned int *status, int split, __nv_bfloat16 *__restrict__ dK, __nv_bfloat16 *__restrict__ dV,
+                   Strides skv)
 {
     using SM = WideSmem;
     constexpr uint32_t colS = 0, colDP = 64, colDQ = 128, colDV = 192, colDK = 320;
@@ -82,15 +83,19 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     volatile uint32_t *abortp = reinterpret_cast<uint32_t *>(bars + W_COUNT + 1);
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int pass = (int)(blockIdx.x & 1u);             // the d-half whose dV, dK, dQ columns this CTA accumulates
+    // kSplit: the `split` CTAs of a cluster share a pass of a key tile, each takes a contiguous part of its query tiles
+    const int rank = kSplit ? (int)cluster_ctarank() : 0, blk = kSplit ? (int)blockIdx.x / split : (int)blockIdx.x;
+    const int pass = blk & 1;                             // the d-half whose dV, dK, dQ columns this CTA accumulates
     int bh, kt;                                           // causal: key tile 0 has the most query tiles and goes first
-    job_from_block((int)(blockIdx.x >> 1), nkt, (int)(gridDim.x >> 1) / nkt, hpg, bh, kt);
+    job_from_block(blk >> 1, nkt, (int)(gridDim.x >> 1) / (kSplit ? split : 1) / nkt, hpg, bh, kt);
     const int k0 = kt * 128;
     const int nqt = n_pad / BQ;                           // query tiles of 64 rows
     const int i_begin = causal ? 2 * kt : 0;
     const int bb = bh / Hkv, hk = bh - bb * Hkv;
     const int hq0 = hk * (kGrouped ? group : 1) - bh * (kGrouped ? group : 1);   // query head in batch = flat index + hq0
-    const int niter_all = (kGrouped ? group : 1) * (nqt - i_begin);
+    const int niter_tile = (kGrouped ? group : 1) * (nqt - i_begin);
+    const int it0 = kSplit ? niter_tile * rank / split : 0;                 // this CTA's first query tile of the job
+    const int niter_all = kSplit ? niter_tile * (rank + 1) / split - it0 : niter_tile;
     struct TileWalk {
         int qh, qi, first, end;
         __device__ void next()
@@ -99,7 +104,8 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             if (kGrouped && qi == end) { qi = first; ++qh; }
         }
     };
-    const TileWalk walk0{kGrouped ? bh * group : bh, i_begin, i_begin, nqt};
+    const int head0 = kGrouped && kSplit ? it0 / (nqt - i_begin) : 0;       // query heads of the group in front of it
+    const TileWalk walk0{(kGrouped ? bh * group : bh) + head0, i_begin + it0 - head0 * (nqt - i_begin), i_begin, nqt};
 
     if (tid == 0) {
         for (int b = 0; b < W_COUNT; ++b)
@@ -130,9 +136,9 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         }
         const int nq_per = nqt - i_begin;
         auto tile_of = [&](int it, int &qh, int &q0) {
-            const int hh = kGrouped ? it / nq_per : 0;
+            const int at = it0 + it, hh = kGrouped ? at / nq_per : 0;
             qh = (kGrouped ? bh * group : bh) + hh;
-            q0 = (i_begin + it - hh * nq_per) * BQ;
+            q0 = (i_begin + at - hh * nq_per) * BQ;
         };
         auto load_qown = [&](int it) {        // this pass's d-half of Q_it, with -L log2e and -D of its 64 queries
             int qh, q0;
@@ -391,7 +397,33 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
           }
             if (it + 1 < niter) ok = p_phase(it + 1);
         }
-        if (ok && mbar_wait(bars + W_DQ, (niter - 1) & 1, abortp, status, WERR_DQ)) {
+        if (kSplit) {
+            // partial dV[:, pass], dK[:, pass] as floats over the K and V tiles, which are no longer read: rows of 128 floats,
+            // 16-byte chunks swizzled by the row
+            const bool done = ok && mbar_wait(bars + W_DQ, (niter - 1) & 1, abortp, status, WERR_DQ);
+            tc_fence_after();
+#pragma unroll 1
+            for (int which = 0; which < 2; ++which) {
+                uint8_t *row = sm + which * 65536 + lane_row * 512;
+#pragma unroll 1
+                for (int c = 0; c < 64; c += 32) {
+                    uint32_t r[32];
+                    if (__all_sync(0xffffffffu, done)) {
+                        tmem_ld(lane_addr + (which == 0 ? colDV : colDK) + 64 * wg + c, r);
+                        tc_wait_ld();
+                    } else {              // (a CTA without query tiles adds nothing)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) r[e] = 0u;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4) {
+                        const int chunk = ((64 * wg + c + e) / 4) ^ (lane_row & 7);
+                        *reinterpret_cast<uint4 *>(row + chunk * 16) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
+                    }
+                }
+            }
+        }
+        if (!kSplit && ok && mbar_wait(bars + W_DQ, (niter - 1) & 1, abortp, status, WERR_DQ)) {
             // All UMMAs have completed (one issuing thread; dQ is its last product).  dV[:, pass] and scale*dK[:, pass] go
             // out as bf16 through the first two boxes of the V and K tiles (no longer read) and TMA stores; rows past n and
             // columns past d are clipped by the tensor map.
@@ -436,6 +468,25 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
+    if (kSplit) {
+        // the ranks add up the partial results, in rank order, 128 / split rows each, and write them out
+        __syncwarp();
+        cluster_sync_all();
+        if (warp < kReduceWarp0) {
+            const int per = 128 / split;
+            for (int i = tid; i < 2 * per * 16; i += 32 * kReduceWarp0) {
+                const int c8 = i % 16, r = rank * per + (i / 16) % per, which = i / 16 / per, col = 128 * pass + 8 * c8;
+                const uint32_t row = smem_u32(sm) + which * 65536 + r * 512;
+                float v[8];
+                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), split, which == 0 ? 1.f : scale, v);
+                if (k0 + r < n && col < d)
+                    *reinterpret_cast<uint4 *>((which == 0 ? dV : dK) + skv.at(bb, hk, k0 + r) + col) =
+                        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
+    }
     if (*abortp && tid == kLoadWarp * 32) {
         // A wait expired: copies this thread asked for may still be on their way into the CTA's shared memory.  It
         // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) before the CTA can leave.
@@ -444,9 +495,9 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     }
 }
 
-template <bool kGrouped>
+template <bool kGrouped, bool kSplit>
 cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const void *V, const void *dO, const float *Lp,
-                        const float *Dp, void *dK, void *dV, float *dQacc, cudaStream_t st)
+                        const float *Dp, void *dK, void *dV, float *dQacc, int split, cudaStream_t st)
 {
     CUtensorMap mq, mk, mv, mdo, mdk, mdv;
     const auto bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
@@ -460,7 +511,7 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
         !make_tensor_map_4d_strided(&mdv, dV, bf, 2, p.B, hkv, p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64))
         return cudaErrorInvalidValue;
     constexpr int kSmem = WideSmem::kTotal;
-    cudaError_t e = allow_smem<tc_bwd_wide_kernel<kGrouped>>(kSmem);
+    cudaError_t e = allow_smem<tc_bwd_wide_kernel<kGrouped, kSplit>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
@@ -468,19 +519,25 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
     pkv.H = hkv;
     pkv.Hkv = 0;
     // two CTAs (the two halves of d) per (K/V head, key tile), adjacent in the grid: they share every load in L2
-    return launch_dependent(tc_bwd_wide_kernel<kGrouped>, dim3((unsigned)(2 * nkt * p.BHkv())), dim3(kThreads), (size_t)kSmem, st,
+    return launch_cluster(tc_bwd_wide_kernel<kGrouped, kSplit>, (unsigned)split, dim3((unsigned)(2 * nkt * p.BHkv() * split)), dim3(kThreads),
+                          (size_t)kSmem, st,
         mq, mk, mv, mdo, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.d, p.causal, p.scale, p.scale * kLog2e, nkt,
-        heads_per_group(pkv, nkt), p.group(), hkv, device_status_ptr());
+        heads_per_group(pkv, nkt), p.group(), hkv, device_status_ptr(), split, (__nv_bfloat16 *)dK, (__nv_bfloat16 *)dV, p.skv);
 }
 
 }  // namespace
 
 cudaError_t tc_bwd_kv_wide(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
-                           const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, cudaStream_t st)
+                           const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st)
 {
     if (p.d <= 128 || p.d > 256 || p.d % 8 || dQacc == nullptr) return cudaErrorInvalidValue;
-    return p.group() > 1 ? launch_wide<true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st)
-                         : launch_wide<false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, st);
+    const long long nkt = (p.n + 127) / 128, jobs = 2 * nkt * p.BHkv(), longest = 2 * nkt * p.group();     // query tiles of 64
+    const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) : jobs * longest, p.causal, 2.5, 1.5);
+    if (split > 1)
+        return p.group() > 1 ? launch_wide<true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
+                             : launch_wide<false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
+    return p.group() > 1 ? launch_wide<true, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st)
+                         : launch_wide<false, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st);
 }
 
 }  // namespace moa
