@@ -3,11 +3,11 @@
 //
 //   C[M,N] = sum over operand pairs p of  A_p[M,K] * B_p[N,K]^T
 //
-// One persistent CTA per SM walks output tiles of 128 x 256.  Warp 0 is the TMA producer (a ring of
-// stages of 64 K-elements: 16 KB of A, 32 KB of B), warp 1 allocates TMEM and issues the
-// UMMAs (M = 128, N = 256, K = 16 each, four per stage), warps 2-9 are the epilogue (two warps per
-// 32-lane group of TMEM, one column half each).  The two
-// 256-column halves of TMEM alternate between tiles, so the epilogue of a tile runs under the main
+// One persistent CTA per SM walks output tiles of 128 x kN, kN = 256, 128 or 64.  Warp 0 is the TMA producer (a ring of
+// stages of 64 K-elements: 16 KB of A, 128 kN bytes of B), warp 1 allocates TMEM and issues the
+// UMMAs (M = 128, N = kN, K = 16 each, four per stage), warps 2-9 are the epilogue (two warps per
+// 32-lane group of TMEM, one column half each).  Two
+// kN-column accumulators in TMEM alternate between tiles, so the epilogue of a tile runs under the main
 // loop of the next one.  Every wait is bounded (ptx::mbar_wait).
 //
 // kPair: the same roles in each of the two CTAs of a cluster, on tiles of 256 x 256: the CTA of rank 0
@@ -44,26 +44,29 @@ namespace {
 
 using namespace ptx;
 
-constexpr int GM = 128, GN = 256, GK = 64;
+constexpr int GM = 128, GK = 64;
 constexpr int kGemmThreads = 320;                      // producer, issuer, eight epilogue warps
-constexpr int kABytes = GM * GK * 2, kBBytes = GN * GK * 2;
+constexpr int kABytes = GM * GK * 2;
 // A CTA on its own stages 16 KB of A and 32 KB of B per 64 K-elements, four stages (three measured 7-16 % slower: the
 // ring has to cover the L2 latency).  A CTA of a pair stages 16 KB of A and its half of B, 16 KB: six stages.
 // In a pair a stage holds two such blocks (128 K-elements, 64 KB) and the ring has three: one wait and one commit of
 // the issuing thread per eight UMMAs instead of per four (that thread's time per stage is on the critical path: a
 // second commit per stage cost 3-4 %).
-constexpr int kMaxStages = 6;
+// Narrower tiles are for launches whose 256-column tiles would leave SMs idle: less work per SM and a shorter epilogue, at more operand
+// traffic per unit of work; six and eight stages of 32 and 24 KB.
+constexpr int kMaxStages = 8;
 __host__ __device__ constexpr int gemm_sub(bool pair) { return pair ? 2 : 1; }                 // 64-element K blocks per stage
-__host__ __device__ constexpr int gemm_stages(bool pair) { return pair ? 3 : 4; }
-__host__ __device__ constexpr int gemm_sub_bytes(bool pair) { return kABytes + (pair ? kBBytes / 2 : kBBytes); }
-__host__ __device__ constexpr int gemm_stage_bytes(bool pair) { return gemm_sub(pair) * gemm_sub_bytes(pair); }
+__host__ __device__ constexpr int gemm_stages(bool pair, int n) { return pair ? 3 : n == 256 ? 4 : n == 128 ? 6 : 8; }
+__host__ __device__ constexpr int gemm_b_bytes(int n) { return n * GK * 2; }
+__host__ __device__ constexpr int gemm_sub_bytes(bool pair, int n) { return kABytes + (pair ? gemm_b_bytes(n) / 2 : gemm_b_bytes(n)); }
+__host__ __device__ constexpr int gemm_stage_bytes(bool pair, int n) { return gemm_sub(pair) * gemm_sub_bytes(pair, n); }
 constexpr int kMnBox = 64 * GK * 2;                    // one MN-major box: 64 columns x 64 K-rows
 constexpr int kOutBox = 128 * 64 * 2;                  // one staged output chunk: 128 rows x 64 columns, bf16
-__host__ __device__ constexpr int gemm_smem(bool pair)
+__host__ __device__ constexpr int gemm_smem(bool pair, int n)
 {
-    return gemm_stages(pair) * gemm_stage_bytes(pair) + 2 * kOutBox + 1024 /* alignment */ + 256 /* barriers */;
+    return gemm_stages(pair, n) * gemm_stage_bytes(pair, n) + 2 * kOutBox + 1024 /* alignment */ + 256 /* barriers */;
 }
-constexpr int kStages = kMaxStages;                    // barrier slots (the ring uses gemm_stages(pair) of them)
+constexpr int kStages = kMaxStages;                    // barrier slots (the ring uses gemm_stages() of them)
 
 enum { EPI_STORE = 0, EPI_SWIGLU_FWD = 1, EPI_SWIGLU_BWD = 2 };
 enum { G_FULL = 0, G_EMPTY = kStages, G_ACCFULL = 2 * kStages, G_ACCEMPTY = 2 * kStages + 2, G_EPI = 2 * kStages + 4,
@@ -107,22 +110,24 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
     tm = g * kGroup + (r - tn * rows);
 }
 
-template <bool kAMn, bool kBMn, int kEpi, bool kPair>
+template <bool kAMn, bool kBMn, int kEpi, bool kPair, int kN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapB0,
                const __grid_constant__ CUtensorMap mapA1, const __grid_constant__ CUtensorMap mapB1,
                const __grid_constant__ CUtensorMap mapC0, const __grid_constant__ CUtensorMap mapC1,
                const __grid_constant__ CUtensorMap mapC2, const __grid_constant__ CUtensorMap mapC3, int M, int N, int K, int nparts, int nbatch, int a_blocked, int b_blocked, int has_res, int group_rows, unsigned int *status)
 {
-    constexpr bool kDualN = kEpi == EPI_SWIGLU_FWD;         // B tile = 128 rows of map B0 + 128 rows of map B1
-    constexpr int kTileN = kDualN ? 128 : GN;                // output columns a tile covers
+    static_assert(kN == 256 || (!kPair && (kN == 128 || (kN == 64 && kEpi != EPI_SWIGLU_FWD))), "tile widths");
+    constexpr bool kDualN = kEpi == EPI_SWIGLU_FWD;         // B tile = kN / 2 rows of map B0 + kN / 2 rows of map B1
+    constexpr int kTileN = kDualN ? kN / 2 : kN;             // output columns a tile covers
+    constexpr int kBBytes = gemm_b_bytes(kN);
     // Epilogue warps: two per 32-lane group of TMEM; together they fill one 64-column output chunk at a time
     constexpr int kEpiWarps = 8;
     // kPair: the two CTAs of a cluster share tiles of 256 rows: UMMAs of M = 256 issued by the CTA of rank 0 read the
     // A rows and the B half staged in each CTA (this CTA: rows rank*128.. of the tile, B rows rank*128.. of its 256)
     // and write each CTA's accumulator; every CTA runs its own producer and epilogue.
-    constexpr int kSt = gemm_stages(kPair), kStageBytes = gemm_stage_bytes(kPair), kTileM = kPair ? 2 * GM : GM;
-    constexpr int kSub = gemm_sub(kPair), kSubBytes = gemm_sub_bytes(kPair);
+    constexpr int kSt = gemm_stages(kPair, kN), kStageBytes = gemm_stage_bytes(kPair, kN), kTileM = kPair ? 2 * GM : GM;
+    constexpr int kSub = gemm_sub(kPair), kSubBytes = gemm_sub_bytes(kPair, kN);
     const uint32_t rank = kPair ? cluster_ctarank() : 0u;
     const int cta = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, ncta = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     extern __shared__ uint8_t smem_raw[];
@@ -160,7 +165,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             tmem_alloc_pair(tmem_slot, 512);
             tmem_relinquish_pair();
         } else {
-            tmem_alloc(tmem_slot, 512);
+            tmem_alloc(tmem_slot, 2 * kN);
             tmem_relinquish();
         }
     }
@@ -184,7 +189,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             const int second = t >= tiles_one ? 1 : 0;
             tile_coords(t - second * tiles_one, tiles_m, tiles_n, group_rows, tm, tn);
             const int m0 = tm * kTileM + (int)rank * GM, n0 = tn * kTileN;
-            const int nb0 = n0 + ((kPair && !kDualN) ? (int)rank * (GN / 2) : 0);    // first B row this CTA stages
+            const int nb0 = n0 + ((kPair && !kDualN) ? (int)rank * (kN / 2) : 0);    // first B row this CTA stages
             for (int ks = 0; ks < nk_total; ++ks, ++it) {
                 const int s = it % kSt;
                 if (!mbar_wait(bars + G_EMPTY + s, ((it / kSt) & 1) ^ 1, abortp, status, GERR_EMPTY)) { ok = false; break; }
@@ -218,7 +223,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                         load(sb, mb, 0, k0, nb0 / 64);
                     } else {
 #pragma unroll
-                        for (int b = 0; b < (kPair ? 2 : 4); ++b) load(sb + b * kMnBox, mb, nb0 + 64 * b, k0, 0);
+                        for (int b = 0; b < (kPair ? 2 : kN / 64); ++b) load(sb + b * kMnBox, mb, nb0 + 64 * b, k0, 0);
                     }
                 } else if (kDualN) {
                     if (kPair) {                              // rank 0 stages the W1 rows, rank 1 the W3 rows
@@ -236,7 +241,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         mbar_drain(bars, armed);      // copies of this CTA still on their way land before it leaves (bounded)
     } else if (warp == 1 && lane == 0 && rank == 0) {
         // ------------------------------------------------------------------- UMMA issuer
-        constexpr uint32_t idesc = idesc_bf16_f32(kTileM, GN, kAMn ? 1 : 0, kBMn ? 1 : 0);
+        constexpr uint32_t idesc = idesc_bf16_f32(kTileM, kN, kAMn ? 1 : 0, kBMn ? 1 : 0);
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kMnBox, 1024);
         const uint32_t a_hi = (uint32_t)((kAMn ? mn_proto : km_proto) >> 32), b_hi = (uint32_t)((kBMn ? mn_proto : km_proto) >> 32);
         const uint32_t a_lo0 = (uint32_t)(kAMn ? mn_proto : km_proto), b_lo0 = (uint32_t)(kBMn ? mn_proto : km_proto);
@@ -247,7 +252,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             const int buf = ti & 1;
             if (!mbar_wait(bars + G_ACCEMPTY + buf, ((ti >> 1) & 1) ^ 1, abortp, status, GERR_ACCEMPTY)) break;
             tc_fence_after();
-            const uint32_t acc = tbase + (uint32_t)(buf * GN);
+            const uint32_t acc = tbase + (uint32_t)(buf * kN);
             for (int ks = 0; ks < nk_total; ++ks, ++it) {
                 const int s = it % kSt;
                 if (!mbar_wait(bars + G_FULL + s, (it / kSt) & 1, abortp, status, GERR_FULL)) { ok = false; break; }
@@ -362,27 +367,28 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             const int m0 = tm * kTileM + (int)rank * GM, n0 = tn * kTileN;
             if (kEpi == EPI_STORE && has_res && leader) {     // the tile's residual: into L2 while its main loop runs
 #pragma unroll
-                for (int c0 = 0; c0 < GN; c0 += 64) tma_prefetch_3d(&mapC2, n0 + c0, m0, 0);
+                for (int c0 = 0; c0 < kN; c0 += 64) tma_prefetch_3d(&mapC2, n0 + c0, m0, 0);
             }
             if (kEpi == EPI_SWIGLU_BWD && leader) {       // the tile's stored a, u: into L2 while its main loop runs
 #pragma unroll
-                for (int c0 = 0; c0 < GN; c0 += 64) {
+                for (int c0 = 0; c0 < kN; c0 += 64) {
                     tma_prefetch_3d(&mapC2, n0 + c0, m0, 0);
                     tma_prefetch_3d(&mapC3, n0 + c0, m0, 0);
                 }
             }
             if (!mbar_wait(bars + G_ACCFULL + buf, (ti >> 1) & 1, abortp, status, GERR_ACCFULL)) break;
             tc_fence_after();
-            const uint32_t acc = lane_addr + (uint32_t)(buf * GN);
+            const uint32_t acc = lane_addr + (uint32_t)(buf * kN);
+            const int cols = min(kTileN, (N - n0 + 63) / 64 * 64);      // chunks wholly past the last column are not worked on
             if (kEpi == EPI_SWIGLU_FWD) {
 #pragma unroll 1
-                for (int c0 = 0; ok && c0 < 128; c0 += 64) {
+                for (int c0 = 0; ok && c0 < cols; c0 += 64) {
                     const int c = c0 + 32 * half;
                     uint32_t ra[32], ru[32];
                     tmem_ld(acc + c, ra);
-                    tmem_ld(acc + 128 + c, ru);
+                    tmem_ld(acc + kN / 2 + c, ru);
                     tc_wait_ld();
-                    if (c0 == 64) {                       // last read of this accumulator: hand it back early
+                    if (c0 == cols - 64) {                // last read of this accumulator: hand it back early
                         acc_release(buf);
                     }
                     uint32_t pa[16], pu[16], ph[16];
@@ -399,11 +405,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 }
             } else if (kEpi == EPI_STORE) {
 #pragma unroll 1
-                for (int c0 = 0; ok && c0 < GN; c0 += 64) {
+                for (int c0 = 0; ok && c0 < cols; c0 += 64) {
                     uint32_t r[32];
                     tmem_ld(acc + c0 + 32 * half, r);
                     tc_wait_ld();
-                    if (c0 == GN - 64) {                  // last read of this accumulator: hand it back early
+                    if (c0 == cols - 64) {                // last read of this accumulator: hand it back early
                         acc_release(buf);
                     }
                     if (has_res) {
@@ -419,7 +425,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 // Backward gate: per 64-column chunk the stored a and u come into the two staging buffers by TMA, every
                 // thread turns its 32 + 32 values into da, du in place, and the buffers leave by TMA stores.
 #pragma unroll 1
-                for (int c0 = 0; ok && c0 < GN; c0 += 64, ++in_q) {
+                for (int c0 = 0; ok && c0 < cols; c0 += 64, ++in_q) {
                     if (leader) {
                         bulk_wait_read<0>();              // the previous chunk's stores have left both buffers
                         mbar_arm(bars, G_IN, 2 * kOutBox, armed);
@@ -429,7 +435,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                     uint32_t r[32];
                     tmem_ld(acc + c0 + 32 * half, r);
                     tc_wait_ld();
-                    if (c0 == GN - 64) {
+                    if (c0 == cols - 64) {
                         acc_release(buf);
                     }
                     if (!mbar_wait(bars + G_IN, in_q & 1, abortp, status, GERR_IN)) { ok = false; break; }
@@ -476,7 +482,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         cluster_sync_all();
         if (warp == 1) tmem_dealloc_pair(tbase, 512);
     } else if (warp == 1) {
-        tmem_dealloc(tbase, 512);
+        tmem_dealloc(tbase, 2 * kN);
     }
 }
 
@@ -526,7 +532,7 @@ int max_active_pairs(K kernel, int smem)
     return cache[dev] = n;
 }
 
-template <bool kAMn, bool kBMn, int kEpi, bool kPair>
+template <bool kAMn, bool kBMn, int kEpi, bool kPair, int kN>
 // C0..C2: output arrays (row length ldc); unused ones may repeat C0.
 cudaError_t launch_gemm_as(const Operand &A0, const Operand &B0, const Operand *A1, const Operand *B1, void *C0, void *C1,
                         const void *C2, const void *C3, int c_rows, int ldc, int M, int N, int K, cudaStream_t st,
@@ -534,7 +540,7 @@ cudaError_t launch_gemm_as(const Operand &A0, const Operand &B0, const Operand *
 {
     constexpr bool kDualN = kEpi == EPI_SWIGLU_FWD;
     CUtensorMap ma0, mb0, ma1, mb1;
-    const int b_rows = (kDualN || kPair) ? 128 : GN;     // B rows one CTA stages per copy
+    const int b_rows = (kDualN || kPair) ? kN / 2 : kN;     // B rows one CTA stages per copy
     // MN-major operands whose width is a multiple of 64 come in by one blocked copy per stage (try the encode; if the
     // driver refuses the map, or a width has a tail, use one copy per 64-column block)
     const Operand &a1 = A1 ? *A1 : A0, &b1 = B1 ? *B1 : B0;
@@ -549,11 +555,11 @@ cudaError_t launch_gemm_as(const Operand &A0, const Operand &B0, const Operand *
     for (int i = 0; i < 4; ++i)     // [c_rows, ldc] bf16, boxes of 128 rows x 64 columns, 128-byte swizzle
         if (!make_tensor_map_3d(&mc[i], cs[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 1, (uint64_t)c_rows, (uint64_t)ldc, 128, 64))
             return cudaErrorInvalidValue;
-    auto kernel = tc_gemm_kernel<kAMn, kBMn, kEpi, kPair>;
-    constexpr int kSmem = gemm_smem(kPair), kTileM = kPair ? 2 * GM : GM;
-    cudaError_t e = allow_smem<tc_gemm_kernel<kAMn, kBMn, kEpi, kPair>>(kSmem);
+    auto kernel = tc_gemm_kernel<kAMn, kBMn, kEpi, kPair, kN>;
+    constexpr int kSmem = gemm_smem(kPair, kN), kTileN = kDualN ? kN / 2 : kN, kTileM = kPair ? 2 * GM : GM;
+    cudaError_t e = allow_smem<tc_gemm_kernel<kAMn, kBMn, kEpi, kPair, kN>>(kSmem);
     if (e != cudaSuccess) return e;
-    const int tiles = ((M + kTileM - 1) / kTileM) * ((N + (kDualN ? 128 : GN) - 1) / (kDualN ? 128 : GN)) * nbatch;
+    const int tiles = ((M + kTileM - 1) / kTileM) * ((N + kTileN - 1) / kTileN) * nbatch;
     const int nparts = (A1 && !kDualN && nbatch == 1) ? 2 : 1;
     // Groups of 8 tile rows, unless B is too large to stay in L2 between groups (above 48 MB): then groups as tall as
     // keeps their A rows within 32 MB, so that B is swept fewer times (measured: taller groups cost the products with
@@ -590,17 +596,37 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
                         const void *C2, const void *C3, int c_rows, int ldc, int M, int N, int K, cudaStream_t st,
                         int nbatch = 1, bool has_res = false)
 {
-    const int tn = kEpi == EPI_SWIGLU_FWD ? 128 : GN;
-    const long long cols = (N + tn - 1) / tn;
-    const long long pair_tiles = (long long)((M + 2 * GM - 1) / (2 * GM)) * cols * nbatch;
-    const long long single_tiles = (long long)((M + GM - 1) / GM) * cols * nbatch;
-    // pairs unless they would need more waves than single CTAs (tiny M); the two gate GEMMs only when the main loop
-    // outlasts their epilogue
-    const long long sms = device_info().sms, pairs = sms / 2;
-    const bool fits = pair_tiles >= 8 && (pair_tiles + pairs - 1) / pairs <= (single_tiles + sms - 1) / sms;   // (a few tiles: launch-bound)
-    if (gemm_pair_mode() == 2 || (gemm_pair_mode() && fits && (kEpi == EPI_STORE || K >= 1024)))
-        return launch_gemm_as<kAMn, kBMn, kEpi, true>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
-    return launch_gemm_as<kAMn, kBMn, kEpi, false>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+    // Pairs unless they would need more waves than single CTAs (tiny M); the two gate GEMMs only when the main loop outlasts
+    // their epilogue.
+    constexpr bool kDualN = kEpi == EPI_SWIGLU_FWD;
+    const long long sms = device_info().sms, pairs = sms / 2, rows = (M + GM - 1) / GM, K64 = (K + GK - 1) / GK;
+    auto tiles = [&](int n) { return rows * ((N + (kDualN ? n / 2 : n) - 1) / (kDualN ? n / 2 : n)) * nbatch; };
+    const long long pair_tiles = (long long)((M + 2 * GM - 1) / (2 * GM)) * (tiles(256) / rows);
+    const int mode = gemm_pair_mode();
+    const bool fits = pair_tiles >= 8 && (pair_tiles + pairs - 1) / pairs <= (tiles(256) + sms - 1) / sms;   // (a few tiles: launch-bound)
+    const bool pair_ok = mode && fits && (kEpi == EPI_STORE || K >= 1024);
+    // Where the 256-column tiles leave SMs idle, the narrower ones compete: cycles of a K block (UMMAs at 256 columns, its
+    // operands' way from L2 below that), of a chunk of the epilogue, and the rounds the grid takes.
+    constexpr double kChunk = kEpi == EPI_STORE ? 1100 : kEpi == EPI_SWIGLU_FWD ? 2500 : 3500;
+    const double blocks = (double)K64 * ((A1 && !kDualN && nbatch == 1) ? 2 : 1);
+    auto cost = [&](long long t, long long slots, double block, int n) {
+        const double epi = kChunk * (kDualN ? n / 128 : n / 64), main = blocks * block;
+        return (double)((t + slots - 1) / slots) * (main > epi ? main : epi) + epi;
+    };
+    int n = 256;
+    bool pair = mode == 2 || pair_ok;
+    if (mode != 2 && tiles(256) < 2 * sms) {
+        double best = pair ? cost(pair_tiles, pairs, 530, 256) : cost(tiles(256), sms, 520, 256);
+        const double c128 = cost(tiles(128), sms, 400, 128);
+        if (c128 < 0.95 * best) { best = c128; n = 128; pair = false; }
+        const double c64 = kDualN ? 1e30 : cost(tiles(64), sms, 300, 64);
+        if (c64 < 0.95 * best) { n = 64; pair = false; }
+    }
+    if (pair) return launch_gemm_as<kAMn, kBMn, kEpi, true, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+    if constexpr (!kDualN)
+        if (n == 64) return launch_gemm_as<kAMn, kBMn, kEpi, false, 64>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+    if (n == 128) return launch_gemm_as<kAMn, kBMn, kEpi, false, 128>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+    return launch_gemm_as<kAMn, kBMn, kEpi, false, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
 }
 
 }  // namespace

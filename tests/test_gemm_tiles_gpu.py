@@ -1,0 +1,63 @@
+"""Products at the edges of the rule that picks the tile: 64, 128 and 256 columns on single CTAs and pairs, tails in every
+direction, against a float64 product of the same bf16 operands."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rt():
+    torch = pytest.importorskip("torch")
+    from paper_2609_33916_b200 import binding as mb
+    from paper_2609_33916_b200 import build
+    build.build()
+    return torch, mb
+
+
+# M, N, K: one tile | a tail of one chunk | 64 columns, several rows | 128 columns | a pair of CTAs | 256 columns on single CTAs
+SHAPES = [(8, 8, 8), (128, 72, 64), (136, 200, 520), (520, 640, 4096), (1704, 1000, 1024), (2048, 2304, 512), (104, 76808, 64)]
+
+
+@pytest.mark.parametrize("a_layout,b_layout", [(0, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("M,N,K", SHAPES)
+@pytest.mark.parametrize("res", [False, True])
+def test_products(rt, M, N, K, a_layout, b_layout, res):
+    torch, mb = rt
+    gen = torch.Generator(device="cuda").manual_seed(M + N + K)
+    R = lambda *s: torch.randn(s, generator=gen, device="cuda").bfloat16()      # noqa: E731
+    A, B = (R(K, M) if a_layout else R(M, K)), (R(K, N) if b_layout else R(N, K)) * K ** -0.5
+    add = R(M, N) if res else None
+    C = torch.full((M, N), float("nan"), device="cuda", dtype=torch.bfloat16)
+    mb.moa_gemm(mb.make_gemm_desc(M, N, K, a_layout, b_layout), A, B, C, R=add)
+    assert mb.moa_last_device_status() == mb.MOA_OK
+    ref = (A.double().T if a_layout else A.double()) @ (B.double() if b_layout else B.double().T)
+    if res:
+        ref = ref + add.double()
+    # one rounding to bf16 of the result (2^-9 of an element), fp32 sums far below that
+    assert (C.double() - ref).abs().max().item() <= 2 ** -8 * ref.abs().max().item()
+
+
+@pytest.mark.parametrize("n,d,dff", [(8, 64, 72), (300, 128, 1000), (700, 1024, 648), (2100, 256, 2048)])
+def test_gated_mlp_widths(rt, n, d, dff):
+    torch, mb = rt
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    R = lambda *s: torch.randn(s, generator=gen, device="cuda").bfloat16()      # noqa: E731
+    x, W1, W3, W2, dy = R(n, d), R(dff, d) * d ** -0.5, R(dff, d) * d ** -0.5, R(d, dff) * dff ** -0.5, R(n, d)
+    E = lambda *s: torch.full(s, float("nan"), device="cuda", dtype=torch.bfloat16)      # noqa: E731
+    a, u, h, y, dx, dW1, dW3, dW2 = E(n, dff), E(n, dff), E(n, dff), E(n, d), E(n, d), E(dff, d), E(dff, d), E(d, dff)
+    desc = mb.make_mlp_desc(n, d, dff)
+    ws = torch.empty(mb.moa_gated_mlp_workspace_bytes(desc), dtype=torch.uint8, device="cuda")
+    mb.moa_gated_mlp_fwd(desc, x, W1, W3, W2, a, u, h, y)
+    mb.moa_gated_mlp_bwd(desc, x, W1, W3, W2, a, u, h, dy, dx, dW1, dW3, dW2, ws)
+    assert mb.moa_last_device_status() == mb.MOA_OK
+    f = lambda t: t.double()                                                     # noqa: E731
+    ra, ru = f(x) @ f(W1).T, f(x) @ f(W3).T
+    rh = torch.nn.functional.silu(ra) * ru
+    # the backward from the a, u, h that were stored (bf16), as the library has them
+    sa, su = f(a), f(u)
+    s = torch.sigmoid(sa)
+    dh = f(dy) @ f(W2)
+    da, du = dh * su * s * (1 + sa * (1 - s)), dh * sa * s
+    for got, ref in ((a, ra), (u, ru), (h, rh), (y, f(h) @ f(W2).T), (dW2, f(dy).T @ f(h)), (dW1, da.T @ f(x)), (dW3, du.T @ f(x)),
+                     (dx, da @ f(W1) + du @ f(W3))):
+        assert (got.double() - ref).abs().max().item() <= 1e-2 * ref.abs().max().item()
