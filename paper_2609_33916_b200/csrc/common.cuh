@@ -135,6 +135,11 @@ size_t decode_workspace_bytes(const DecodeProblem &p, int dtype);    // partial 
 cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const void *K, const void *V, void *out,
                         float *lse, void *ws, cudaStream_t st);
 
+// groups of query heads on warp-level tensor-core instructions (decode_mma.cu)
+bool decode_uses_mma(const DecodeProblem &p, int dtype);
+size_t decode_mma_workspace_bytes(const DecodeProblem &p);
+cudaError_t decode_mma(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse, void *ws,
+                       cudaStream_t st);
 // counters of a merge by the last CTA to zero, in stream order
 cudaError_t decode_clear(unsigned int *counters, int count, cudaStream_t st);
 

@@ -580,8 +580,8 @@ cudaError_t launch_decode(const DecodeProblem &p, const void *q, const void *K, 
 
 }  // namespace
 
-// Groups of 4 to 128 query heads over a bf16 cache go through the tensor-core forward kernel (the
-// group is its query tile); everything else through the CUDA-core streaming kernels above.
+// Over a bf16 cache, groups of 4 to 16 query heads go through decode_mma.cu and larger ones, up to 128, through the
+// tensor-core forward kernel (the group is its query tile); everything else through the CUDA-core streaming kernels above.
 static bool decode_uses_tc(const DecodeProblem &p, int dtype)
 {
     const int group = p.H / p.Hkv;
@@ -635,6 +635,7 @@ int decode_splits(const DecodeProblem &p)
 
 size_t decode_workspace_bytes(const DecodeProblem &p, int dtype)
 {
+    if (decode_uses_mma(p, dtype)) return decode_mma_workspace_bytes(p);
     if (decode_uses_tc(p, dtype)) {
         int splits, tps;
         decode_tc_splits(p, &splits, &tps);
@@ -648,6 +649,7 @@ size_t decode_workspace_bytes(const DecodeProblem &p, int dtype)
 cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const void *K, const void *V, void *out,
                         float *lse, void *ws, cudaStream_t st)
 {
+    if (decode_uses_mma(p, dtype)) return decode_mma(p, q, K, V, out, lse, ws, st);
     if (decode_uses_tc(p, dtype)) {
         int splits, tps;
         decode_tc_splits(p, &splits, &tps);

@@ -1,0 +1,338 @@
+// Decode attention for bf16 caches shared by groups of 4 to 16 query heads: the scores and the weighted sums of a group on
+// warp-level tensor-core instructions (mma.sync m16n8k16, the queries of a group as the 16 rows), the cache streamed once.
+//
+// HBM-bound: 4 d bytes of cache per key against 4 d G flop; what matters is that every SM streams all the time.  The 128-row
+// tiles of the tcgen05 forward kernel cost a job of that kernel about 3.5 tile times beside its tiles and the jobs go in
+// whole rounds; here
+//   * one CTA per SM takes an equal, contiguous share of all (K/V head, 64-key tile) units, across heads, through one
+//     ring of TMA loads (six stages of 32 KB at d = 128) that never drains at a head's end;
+//   * warp 8 requests the tiles; two groups of four warps take the tiles in turn, a warp 16 keys of its group's tile:
+//     S = q K^T with K rows by ldmatrix, online softmax per warp (rescaled only when a maximum grows by more than 8 in
+//     the log2 domain), O += P V with V by ldmatrix.trans; about a hundred instructions per warp and 16 keys, a tenth of
+//     what the SM can issue in the time HBM takes for them;
+//   * when a CTA's share of a head ends, its eight warps' results are merged through shared memory.  A head that lies in one
+//     CTA's share is written out at once; the others leave fp32 partial results in the workspace (at most two per CTA) and
+//     the CTA that finishes a head last merges them, told by a counter that a one-block kernel in front has cleared.
+// Every wait is bounded; no CTA waits for another.
+#include "common.cuh"
+#include "ptx.cuh"
+#include "tensormap.cuh"
+
+namespace moa {
+namespace {
+
+using namespace ptx;
+
+constexpr int kKeys = 64;                       // keys per tile: 16 per warp of a group
+constexpr int kConsumers = 8, kMmaThreads = 32 * (kConsumers + 1);
+constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
+constexpr float kRescale = 8.f;
+enum : uint32_t { MERR_EMPTY = 0x311, MERR_FULL = 0x312 };
+
+template <int D>
+struct MmaSmem {
+    static constexpr int kBox = kKeys * 128;                     // 64 keys x 64 columns, 128-byte swizzle
+    static constexpr int kTile = D / 64 * kBox;
+    static constexpr int kStages = D == 128 ? 6 : 8;             // even: a stage belongs to one group of warps for good
+    static constexpr int offMerge = kStages * 2 * kTile;         // [8 warps][8 queries][D + 2] floats
+    static constexpr int offBar = offMerge + kConsumers * 8 * (D + 2) * 4;
+    static constexpr int kTotal = offBar + 2 * kStages * 8 + 16;
+};
+
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Units of CTA c: [first_unit(c), first_unit(c + 1)); the CTA that holds unit u.
+__device__ __forceinline__ int first_unit(int units, int c, int ctas) { return (int)((long long)units * c / ctas); }
+__device__ __forceinline__ int cta_of_unit(int units, int u, int ctas)
+{
+    int c = (int)(((long long)u * ctas) / units);
+    while (first_unit(units, c + 1, ctas) <= u) ++c;
+    return c;
+}
+
+// kHi: groups of 9 to 16 (the upper eight rows of the tiles are queries too)
+template <int D, bool kHi>
+__global__ void __launch_bounds__(kMmaThreads, 1)
+decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
+                  const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse,
+                  float *__restrict__ part_o, float *__restrict__ part_ml, unsigned int *__restrict__ counters, int n, int Hkv,
+                  int G, int nt, int units, float scale_log2, unsigned int *status)
+{
+    using S = MmaSmem<D>;
+    constexpr int kRowsLane = kHi ? 2 : 1, kKS = D / 16, kNT = D / 8;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    float *merge = reinterpret_cast<float *>(smem + S::offMerge);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + S::offBar), *empty = full + S::kStages;
+    volatile uint32_t *abortp = reinterpret_cast<uint32_t *>(empty + S::kStages);
+    volatile uint32_t *s_last = abortp + 1;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    const int ctas = (int)gridDim.x, u0 = first_unit(units, blockIdx.x, ctas), u1 = first_unit(units, blockIdx.x + 1, ctas);
+    if (tid == 0) {
+        for (int s = 0; s < S::kStages; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, kConsumers / 2); }
+        *abortp = (smem_u32(smem) & 1023u) ? 1u : 0u;
+        if (*abortp && status) atomicCAS(status, 0u, (unsigned int)MERR_FULL);
+        fence_mbar_init();
+        prefetch_tensormap(&mapK);
+        prefetch_tensormap(&mapV);
+    }
+    __syncthreads();
+    const bool sound = *abortp == 0;
+
+    if (warp == kConsumers) {
+        // ------------------------------------------------------------------ producer
+        // (q, K, V are the call's inputs: the clearing kernel in front has made sure that whatever wrote them is done)
+        if (lane == 0 && sound) {
+            ArmCounts<S::kStages> armed;
+            int head = u0 / nt, t = u0 - head * nt;
+            for (int u = u0; u < u1; ++u) {
+                const int i = u - u0, s = i % S::kStages;
+                if (i >= S::kStages && !mbar_wait(empty + s, (i / S::kStages - 1) & 1, abortp, status, MERR_EMPTY)) break;
+                const int b = head / Hkv, hk = head - b * Hkv;
+                mbar_arm(full, s, 2 * S::kTile, armed);
+                uint8_t *dst = smem + s * 2 * S::kTile;
+                for (int x = 0; x < D / 64; ++x) {
+                    tma_load_4d(dst + x * S::kBox, &mapK, full + s, 64 * x, t * kKeys, hk, b);
+                    tma_load_4d(dst + S::kTile + x * S::kBox, &mapV, full + s, 64 * x, t * kKeys, hk, b);
+                }
+                if (++t == nt) { t = 0; ++head; }
+            }
+            mbar_drain(full, armed);      // copies still on their way land before the CTA leaves (bounded)
+        }
+        grid_dependency_wait();
+        grid_launch_dependents();
+        return;
+    }
+
+    // ---------------------------------------------------------------------- consumers
+    q = after_wait(q);
+    const int grp = warp / 4, w4 = warp % 4, r0 = lane / 4, c0 = (lane % 4) * 2;
+    // lane addresses of ldmatrix inside a tile: K rows as [keys][d], V transposed
+    const uint32_t base = smem_u32(smem);
+    const int krow = 16 * w4 + (lane / 16) * 8 + lane % 8, kch = (lane / 8) & 1;
+    const int vrow = 16 * w4 + ((lane / 8) & 1) * 8 + lane % 8, vch = lane / 16;
+    auto addr = [&](int row, int chunk) {       // 16-byte chunk `chunk` of a row of the tile
+        return (uint32_t)((chunk >> 3) * S::kBox + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
+    };
+    bool waited = false;
+    int u = u0;
+    bool ok = sound;
+    while (u < u1) {
+        const int head = u / nt, t_first = u - head * nt, seg_end = min(u1, (head + 1) * nt);
+        uint32_t qa[kKS][4];
+#pragma unroll
+        for (int ks = 0; ks < kKS; ++ks)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int row = r0 + 8 * (e & 1);
+                qa[ks][e] = ((e & 1) == 0 || kHi) && row < G
+                                ? *reinterpret_cast<const uint32_t *>(q + ((size_t)head * G + row) * D + 16 * ks + c0 + 8 * (e >> 1)) : 0u;
+            }
+        float o[kNT][4], m[kRowsLane], l[kRowsLane];
+#pragma unroll
+        for (int i = 0; i < kNT; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[i][e] = 0.f;
+#pragma unroll
+        for (int i = 0; i < kRowsLane; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+        for (; u < seg_end; ++u) {
+            const int i = u - u0, s = i % S::kStages;
+            if ((i & 1) != grp) continue;                           // the other group's tile (and, kStages being even, stage)
+            if (ok && !mbar_wait(full + s, (i / S::kStages) & 1, abortp, status, MERR_FULL)) ok = false;
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) continue;
+            const uint32_t tk = base + s * 2 * S::kTile, tv = tk + S::kTile;
+            float sc[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sc[j][e] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < kKS; ++ks) {
+                uint32_t kb[4];
+                ldmatrix4(kb, tk + addr(krow, 2 * ks + kch));
+                mma16816(sc[0], qa[ks], kb[0], kb[1]);
+                mma16816(sc[1], qa[ks], kb[2], kb[3]);
+            }
+            const int key0 = (u - head * nt) * kKeys + 16 * w4 + c0;
+            if ((u - head * nt + 1) * kKeys > n)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (key0 + 8 * j + (e & 1) >= n) sc[j][e] = -INFINITY;
+            uint32_t pa[4] = {0u, 0u, 0u, 0u};
+            float mx[kRowsLane];
+            bool grow = false;
+#pragma unroll
+            for (int h = 0; h < kRowsLane; ++h) {
+                mx[h] = fmaxf(fmaxf(sc[0][2 * h], sc[0][2 * h + 1]), fmaxf(sc[1][2 * h], sc[1][2 * h + 1]));
+                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2)) * scale_log2;
+                grow = grow || mx[h] > m[h] + kRescale;
+            }
+            if (__any_sync(0xffffffffu, grow)) {
+#pragma unroll
+                for (int h = 0; h < kRowsLane; ++h) {
+                    const float mn = fmaxf(m[h], mx[h]);
+                    const float a = mn == -INFINITY ? 1.f : ex2(m[h] - mn);
+                    m[h] = mn;
+                    l[h] *= a;
+#pragma unroll
+                    for (int i2 = 0; i2 < kNT; ++i2) { o[i2][2 * h] *= a; o[i2][2 * h + 1] *= a; }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int h = 0; h < kRowsLane; ++h) {
+                    const float ref = m[h] == -INFINITY ? 0.f : m[h];      // (no key visible yet)
+                    const float p0 = ex2(fmaf(sc[j][2 * h], scale_log2, -ref)), p1 = ex2(fmaf(sc[j][2 * h + 1], scale_log2, -ref));
+                    l[h] += p0 + p1;
+                    pa[2 * j + h] = pack_bf16(p0, p1);
+                }
+#pragma unroll
+            for (int nn = 0; nn < kNT / 2; ++nn) {
+                uint32_t vb[4];
+                ldmatrix4_trans(vb, tv + addr(vrow, 2 * nn + vch));
+                mma16816(o[2 * nn], pa, vb[0], vb[1]);
+                mma16816(o[2 * nn + 1], pa, vb[2], vb[3]);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty + s);
+        }
+        // ---- the segment's end: merge the warps, eight queries at a time
+        if (!waited) {
+            grid_dependency_wait();        // the counters are clear, and whatever read the workspace or the outputs before is done
+            grid_launch_dependents();
+            waited = true;
+        }
+        const bool whole = t_first == 0 && seg_end == (head + 1) * nt;
+        const int slot = 2 * (int)blockIdx.x + (t_first == 0 ? 1 : 0);
+        constexpr int kLd = D + 2;
+#pragma unroll
+        for (int h = 0; h < kRowsLane; ++h) {
+            float lt = l[h];
+            lt += __shfl_xor_sync(0xffffffffu, lt, 1);
+            lt += __shfl_xor_sync(0xffffffffu, lt, 2);
+            asm volatile("bar.sync 1, 256;" ::: "memory");          // (the merge before has been read)
+            float *row = merge + (warp * 8 + r0) * kLd;
+#pragma unroll
+            for (int i2 = 0; i2 < kNT; ++i2) *reinterpret_cast<float2 *>(row + 8 * i2 + c0) = make_float2(o[i2][2 * h], o[i2][2 * h + 1]);
+            if (lane % 4 == 0) { row[D] = m[h]; row[D + 1] = lt; }
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            for (int idx = tid; idx < min(8, G - 8 * h) * D; idx += 256) {
+                const int r = idx / D, c = idx - r * D, g = 8 * h + r;
+                float mt = -INFINITY, ot = 0.f, ls = 0.f;
+#pragma unroll
+                for (int w = 0; w < kConsumers; ++w) mt = fmaxf(mt, merge[(w * 8 + r) * kLd + D]);
+                const float ref = mt == -INFINITY ? 0.f : mt;
+#pragma unroll
+                for (int w = 0; w < kConsumers; ++w) {
+                    const float *src = merge + (w * 8 + r) * kLd;
+                    const float a = ex2(src[D] - ref);
+                    ot = fmaf(src[c], a, ot);
+                    ls = fmaf(src[D + 1], a, ls);
+                }
+                if (whole) {
+                    out[((size_t)head * G + g) * D + c] = __float2bfloat16_rn(ot / ls);
+                    if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
+                } else {
+                    part_o[((size_t)slot * G + g) * D + c] = ot;
+                    if (c == 0) { part_ml[((size_t)slot * G + g) * 2] = mt; part_ml[((size_t)slot * G + g) * 2 + 1] = ls; }
+                }
+            }
+        }
+        if (whole) continue;
+        // ---- a head shared by several CTAs: whoever publishes last merges
+        const int ca = cta_of_unit(units, head * nt, ctas), cb = cta_of_unit(units, (head + 1) * nt - 1, ctas);
+        __threadfence();
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (tid == 0) *s_last = atomicAdd(counters + head, 1u) == (unsigned)(cb - ca) ? 1u : 0u;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (*s_last == 0u) continue;
+        __threadfence();
+        for (int idx = tid; idx < G * (D / 4); idx += 256) {
+            const int g = idx / (D / 4), c = (idx - g * (D / 4)) * 4;
+            auto at = [&](int k) { return (size_t)(2 * k + (k == ca ? 1 : 0)) * G + g; };
+            float mt = -INFINITY, ls = 0.f;
+#pragma unroll 8
+            for (int k = ca; k <= cb; ++k) mt = fmaxf(mt, __ldcg(part_ml + at(k) * 2));
+            float4 ot = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+            for (int k = ca; k <= cb; ++k) {
+                const float2 ml = __ldcg(reinterpret_cast<const float2 *>(part_ml + at(k) * 2));
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(part_o + at(k) * D + c));
+                const float a = ex2(ml.x - mt);
+                ls = fmaf(ml.y, a, ls);
+                ot.x = fmaf(v.x, a, ot.x); ot.y = fmaf(v.y, a, ot.y); ot.z = fmaf(v.z, a, ot.z); ot.w = fmaf(v.w, a, ot.w);
+            }
+            const float inv = 1.f / ls;
+            *reinterpret_cast<uint2 *>(out + ((size_t)head * G + g) * D + c) =
+                make_uint2(pack_bf16(ot.x * inv, ot.y * inv), pack_bf16(ot.z * inv, ot.w * inv));
+            if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
+        }
+    }
+    if (!waited) {
+        grid_dependency_wait();
+        grid_launch_dependents();
+    }
+}
+
+template <int D, bool kHi>
+cudaError_t launch(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse, void *ws, cudaStream_t st)
+{
+    using S = MmaSmem<D>;
+    CUtensorMap mk, mv;
+    const auto bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    if (!make_tensor_map_4d(&mk, K, bf, 2, p.B, p.Hkv, p.n, D, false, kKeys, 64) ||
+        !make_tensor_map_4d(&mv, V, bf, 2, p.B, p.Hkv, p.n, D, false, kKeys, 64))
+        return cudaErrorInvalidValue;
+    const int G = p.H / p.Hkv, nt = (p.n + kKeys - 1) / kKeys, heads = p.B * p.Hkv, units = nt * heads, sms = device_info().sms;
+    const int ctas = units < sms ? units : sms;
+    float *part_o = (float *)ws, *part_ml = part_o + (size_t)2 * sms * G * D;
+    unsigned int *counters = reinterpret_cast<unsigned int *>(part_ml + (size_t)2 * sms * G * 2);
+    cudaError_t e = allow_smem<decode_mma_kernel<D, kHi>>(S::kTotal);
+    if (e != cudaSuccess) return e;
+    if ((e = decode_clear(counters, heads, st)) != cudaSuccess) return e;
+    LaunchScope scope(MOA_KERNEL_OTHER, st);
+    return launch_dependent(decode_mma_kernel<D, kHi>, dim3((unsigned)ctas), dim3(kMmaThreads), (size_t)S::kTotal, st, mk, mv,
+                            (const __nv_bfloat16 *)q, (__nv_bfloat16 *)out, lse, part_o, part_ml, counters, p.n, p.Hkv, G, nt, units,
+                            p.scale * kLog2e, device_status_ptr());
+}
+
+}  // namespace
+
+// Groups of 4 to 16 (below, the CUDA-core kernels keep their fp32 weights; above, the group fills the rows of a tcgen05 tile
+// better); the units have to be countable in an int.
+bool decode_uses_mma(const DecodeProblem &p, int dtype)
+{
+    const int G = p.H / p.Hkv;
+    return dtype == MOA_BF16 && G >= 4 && G <= 16 && p.scale > 0.f && ((long long)p.n + kKeys - 1) / kKeys * p.B * p.Hkv < (1LL << 31);
+}
+
+size_t decode_mma_workspace_bytes(const DecodeProblem &p)
+{
+    return (size_t)2 * device_info().sms * (p.H / p.Hkv) * (p.d + 2) * sizeof(float) + (size_t)p.B * p.Hkv * sizeof(unsigned int);
+}
+
+cudaError_t decode_mma(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse, void *ws, cudaStream_t st)
+{
+    const bool hi = p.H / p.Hkv > 8;
+    if (p.d == 64) return hi ? launch<64, true>(p, q, K, V, out, lse, ws, st) : launch<64, false>(p, q, K, V, out, lse, ws, st);
+    if (p.d == 128) return hi ? launch<128, true>(p, q, K, V, out, lse, ws, st) : launch<128, false>(p, q, K, V, out, lse, ws, st);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace moa
