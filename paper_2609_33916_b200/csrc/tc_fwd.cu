@@ -38,6 +38,8 @@
 // tile passes through it KC times -- and the grid has KC CTAs per (head, query tile), each with the V columns and the
 // O columns of one 128-column half (the scores and the softmax are computed KC times; O(n d) memory as before).
 // The backward's per-row inputs are then not prepared here (a CTA holds half of an O row).
+// KL: 16-column steps of the last chunk that hold anything (4 for head dimensions 136..192: 12 UMMAs for the scores instead of 16,
+// and the second pass's products are 64 columns wide).
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tensormap.cuh"
@@ -85,7 +87,7 @@ struct FwdPrep {
     int d;               // columns of a dO row in memory (<= D)
 };
 
-template <int D, int KC>
+template <int D, int KC, int KL>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
@@ -258,7 +260,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 if (c == 0) umma_ss2<false>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
                 else        umma_ss2<true>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
 #pragma unroll
-                for (int ks = 1; ks < D / 16; ++ks) {
+                for (int ks = 1; ks < (c == KC - 1 ? KL : D / 16); ++ks) {
                     const uint32_t off = (uint32_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4);
                     umma_ss2<true>(dcol, q_c + off, km_hi, k_lo + off, km_hi, idesc_s);
                 }
@@ -269,7 +271,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         }
       } else if (warp == 10 && lane == 0) {
         // ------------------------------------------------ UMMA issuer for O += P V (one thread)
-        constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, 0, 1);
+        const uint32_t idesc_pv = KL < D / 16 && pass == KC - 1 ? idesc_bf16_f32(128, 16 * KL, 0, 1) : idesc_bf16_f32(128, D, 0, 1);
         const uint64_t mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);
         const uint32_t mn_hi = (uint32_t)(mn_proto >> 32);
         const uint32_t v_lo0 = (uint32_t)mn_proto + ((smem_u32(sV) >> 4) & 0x3FFFu);
@@ -493,7 +495,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     if (warp == 9) tmem_dealloc(tbase, kTmemCols);
 }
 
-template <int D, int KC>
+template <int D, int KC, int KL>
 cudaError_t launch_fwd(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L,
                        const FwdForBwd &fb, cudaStream_t st)
 {
@@ -507,11 +509,11 @@ cudaError_t launch_fwd(const Problem &p, const void *Q, const void *K, const voi
         !make_tensor_map_4d_strided(&mv, V, bf, 2, p.B, p.kv_heads(), p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64) ||
         !make_tensor_map_4d_strided(&mo, O, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem<tc_fwd_kernel<D, KC>>(kSmem);
+    cudaError_t e = allow_smem<tc_fwd_kernel<D, KC, KL>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + BM - 1) / BM;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_dependent(tc_fwd_kernel<D, KC>, dim3((unsigned)(nqt * p.BH() * KC)), dim3(kThreads), (size_t)kSmem, st,
+    return launch_dependent(tc_fwd_kernel<D, KC, KL>, dim3((unsigned)(nqt * p.BH() * KC)), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mo, L, p.n, p.causal, p.scale * kLog2e, nqt, heads_per_group(p, nqt), p.group(), p.H,
         FwdSplit{p.n, 1, (p.n + BN - 1) / BN}, fb.zero_acc,
         FwdPrep{(const __nv_bfloat16 *)fb.dO, fb.Lp, fb.Dp, nqt * BM, p.so, p.d}, device_status_ptr());
@@ -533,10 +535,10 @@ cudaError_t launch_fwd_decode(int B, int Hkv, int G, int n, float scale, const v
         !make_tensor_map_4d(&mv, V, bf, 2, B, Hkv, n, D, false, 128, 64) ||
         !make_tensor_map_4d(&mo, O_part, bf, 2, (uint64_t)splits * B, Hkv, G, D, false, 128, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem<tc_fwd_kernel<D, 1>>(kSmem);
+    cudaError_t e = allow_smem<tc_fwd_kernel<D, 1, D / 16>>(kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_dependent(tc_fwd_kernel<D, 1>, dim3((unsigned)(B * Hkv * splits)), dim3(kThreads), (size_t)kSmem, st,
+    return launch_dependent(tc_fwd_kernel<D, 1, D / 16>, dim3((unsigned)(B * Hkv * splits)), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mo, L_part, n, 0, scale * kLog2e, 1, 1, 1, Hkv, FwdSplit{G, splits, tiles_per_split},
         nullptr, FwdPrep{nullptr, nullptr, nullptr, 0, Strides{0, 0, 0}, D}, device_status_ptr());
 }
@@ -555,8 +557,9 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
                    const FwdForBwd &fb, cudaStream_t st)
 {
     if (p.d < 8 || p.d > 256 || p.d % 8) return cudaErrorInvalidValue;
-    if (p.d > 128) return launch_fwd<128, 2>(p, Q, K, V, O, L, fb, st);      // two 128-column passes, scores over both chunks
-    return kernel_d(p.d) == 64 ? launch_fwd<64, 1>(p, Q, K, V, O, L, fb, st) : launch_fwd<128, 1>(p, Q, K, V, O, L, fb, st);
+    if (p.d > 192) return launch_fwd<128, 2, 8>(p, Q, K, V, O, L, fb, st);      // two 128-column passes, scores over both chunks
+    if (p.d > 128) return launch_fwd<128, 2, 4>(p, Q, K, V, O, L, fb, st);
+    return kernel_d(p.d) == 64 ? launch_fwd<64, 1, 4>(p, Q, K, V, O, L, fb, st) : launch_fwd<128, 1, 8>(p, Q, K, V, O, L, fb, st);
 }
 
 }  // namespace moa
