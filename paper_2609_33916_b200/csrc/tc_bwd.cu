@@ -36,6 +36,9 @@
 // P^T (bf16) overwrites the front of its fp32 source columns (for D = 64 so does dS^T); for D = 128 the dQ
 // tile reuses the dP^T columns, which are free once the elementwise threads have read dP^T.
 //
+// KL: 16-column steps of the head dimension that hold anything (D / 16, or 6 for 72..96 columns in the 128-column kernel: six
+// UMMAs instead of eight for S^T and for dP^T, dV and dK 96 columns wide).
+//
 // Rows past n need no masking: TMA zero-fills K, V, Q, dO there, the preprocess kernel
 // pads L with +inf (so P = 0) and D with 0, and stores are row-guarded.
 #include "common.cuh"
@@ -176,7 +179,7 @@ enum {
     B_EPI = 19 /*dK, dV tiles staged in shared memory*/, B_COUNT = 20
 };
 
-template <int D, bool kBulk, bool kGrouped, bool kSplit>
+template <int D, bool kBulk, bool kGrouped, bool kSplit, int KL>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapdO,
@@ -327,7 +330,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         // ------------------------------------------------------------------- UMMA issuer
         // Issue order per query tile i:  dP(i), dV(i), S(i+1), dQ(i), dK(i)  (D = 64: dK(i), dQ(i)).
         constexpr uint32_t idesc_st = idesc_bf16_f32(128, 128, 0, 0);   // S^T, dP^T
-        constexpr uint32_t idesc_acc = idesc_bf16_f32(128, D, 0, 1);    // dV, dK: A in TMEM, B MN-major
+        constexpr uint32_t idesc_acc = idesc_bf16_f32(128, 16 * KL, 0, 1);    // dV, dK: A in TMEM, B MN-major
         constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 1, 1);     // dQ: A and B MN-major
         constexpr uint32_t idesc_dqt = idesc_bf16_f32(128, 128, 1, 1);  // dQ^T (D = 128 only)
         // Descriptors are built once and kept as 32-bit halves.  Only the low half (address field)
@@ -350,7 +353,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         auto issue_S = [&](uint32_t q_km) {
             umma_ss2<false>(tbase + colS, k_km, km_hi, q_km, km_hi, idesc_st);
 #pragma unroll
-            for (int ks = 1; ks < D / 16; ++ks)
+            for (int ks = 1; ks < KL; ++ks)
                 umma_ss2<true>(tbase + colS, k_km + koff(ks), km_hi, q_km + koff(ks), km_hi, idesc_st);
             umma_commit(bars + B_S);
         };
@@ -370,7 +373,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (lane == 0) {
                 umma_ss2<false>(tbase + colDP, v_km, km_hi, do_km, km_hi, idesc_st);
 #pragma unroll
-                for (int ks = 1; ks < D / 16; ++ks)
+                for (int ks = 1; ks < KL; ++ks)
                     umma_ss2<true>(tbase + colDP, v_km + koff(ks), km_hi, do_km + koff(ks), km_hi, idesc_st);
                 umma_commit(bars + B_DP);
             }
@@ -748,7 +751,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     }
 }
 
-template <int D, bool kBulk, bool kGrouped, bool kSplit>
+template <int D, bool kBulk, bool kGrouped, bool kSplit, int KL>
 cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
                        const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, int split, cudaStream_t st)
 {
@@ -768,7 +771,7 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     if (!make_tensor_map_3d(&mdq, dQacc ? (const void *)dQacc : Q, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, heads, p.n, D, 32, D == 64 ? 32 : D))
         return cudaErrorInvalidValue;
     constexpr int kSmem = BwdSmem<D, kBulk>::kTotal;
-    cudaError_t e = allow_smem<tc_bwd_kernel<D, kBulk, kGrouped, kSplit>>(kSmem);
+    cudaError_t e = allow_smem<tc_bwd_kernel<D, kBulk, kGrouped, kSplit, KL>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
@@ -776,14 +779,14 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     Problem pkv = p;
     pkv.H = p.kv_heads();
     pkv.Hkv = 0;
-    return launch_cluster(tc_bwd_kernel<D, kBulk, kGrouped, kSplit>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)),
+    return launch_cluster(tc_bwd_kernel<D, kBulk, kGrouped, kSplit, KL>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)),
                           dim3(kThreads), (size_t)kSmem, st,
                             mq, mk, mv, mdo, mdq, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.causal, p.scale, p.scale * kLog2e, nkt,
                             heads_per_group(pkv, nkt), p.group(), p.kv_heads(), dQacc == nullptr ? 1 : 0, device_status_ptr(),
                             split, SplitOut{(__nv_bfloat16 *)dK, (__nv_bfloat16 *)dV, p.skv, p.d});
 }
 
-template <int D, bool kBulk>
+template <int D, bool kBulk, int KL = D / 16>
 cudaError_t launch_bwd(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
                        const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st)
 {
@@ -791,11 +794,11 @@ cudaError_t launch_bwd(const Problem &p, const void *Q, const void *K, const voi
         const long long nkt = (p.n + 127) / 128, jobs = nkt * p.BHkv(), longest = nkt * p.group();
         const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) / 2 : jobs * longest, p.causal, 2.0, 1.0);
         if (split > 1)
-            return p.group() > 1 ? launch_bwd_g<D, kBulk, true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
-                                 : launch_bwd_g<D, kBulk, false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
+            return p.group() > 1 ? launch_bwd_g<D, kBulk, true, true, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
+                                 : launch_bwd_g<D, kBulk, false, true, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
     }
-    return p.group() > 1 ? launch_bwd_g<D, kBulk, true, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st)
-                         : launch_bwd_g<D, kBulk, false, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st);
+    return p.group() > 1 ? launch_bwd_g<D, kBulk, true, false, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st)
+                         : launch_bwd_g<D, kBulk, false, false, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st);
 }
 
 }  // namespace
@@ -826,6 +829,7 @@ cudaError_t tc_bwd_kv(const Problem &p, const void *Q, const void *K, const void
     if (D == 64 && !dq_bulk) return launch_bwd<64, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
     if (D == 64 && dq_bulk) return launch_bwd<64, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
     if (D == 128 && !dq_bulk) return launch_bwd<128, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
+    if (D == 128 && dq_bulk && p.d <= 96) return launch_bwd<128, true, 6>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
     if (D == 128 && dq_bulk) return launch_bwd<128, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, share, st);
     return cudaErrorInvalidValue;
 }

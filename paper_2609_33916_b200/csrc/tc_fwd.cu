@@ -39,7 +39,7 @@
 // O columns of one 128-column half (the scores and the softmax are computed KC times; O(n d) memory as before).
 // The backward's per-row inputs are then not prepared here (a CTA holds half of an O row).
 // KL: 16-column steps of the last chunk that hold anything (4 for head dimensions 136..192: 12 UMMAs for the scores instead of 16,
-// and the second pass's products are 64 columns wide).
+// and the second pass's products are 64 columns wide; 6 for 72..96 in the 128-column kernel).
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tensormap.cuh"
@@ -453,6 +453,9 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                     float v[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(o0[i + u]) * w0 + (has1 ? __uint_as_float(o1[i + u]) * w1 : 0.f);
+                    if (KC == 1 && KL < D / 16 && (D / 2) * h + c + i >= 16 * KL)      // columns no product wrote
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) v[u] = 0.f;
                     if (want_d) {
                         const uint4 g = dov[(c + i) / 8];
                         const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
@@ -559,7 +562,8 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
     if (p.d < 8 || p.d > 256 || p.d % 8) return cudaErrorInvalidValue;
     if (p.d > 192) return launch_fwd<128, 2, 8>(p, Q, K, V, O, L, fb, st);      // two 128-column passes, scores over both chunks
     if (p.d > 128) return launch_fwd<128, 2, 4>(p, Q, K, V, O, L, fb, st);
-    return kernel_d(p.d) == 64 ? launch_fwd<64, 1, 4>(p, Q, K, V, O, L, fb, st) : launch_fwd<128, 1, 8>(p, Q, K, V, O, L, fb, st);
+    if (p.d <= 64) return launch_fwd<64, 1, 4>(p, Q, K, V, O, L, fb, st);
+    return p.d <= 96 ? launch_fwd<128, 1, 6>(p, Q, K, V, O, L, fb, st) : launch_fwd<128, 1, 8>(p, Q, K, V, O, L, fb, st);
 }
 
 }  // namespace moa
