@@ -101,6 +101,32 @@ typedef struct {
 } moa_gemm_desc;
 moa_status moa_gemm(const moa_gemm_desc *desc, const void *A, const void *B, const void *R, void *C, void *stream);
 
+/* ---------------------------------------------------------------------- the block
+ * A whole pre-norm transformer block as one call per direction: the sequence of the calls above with a packed Q/K/V
+ * projection (host work only: a step of a small block spent more time between the calls than in them).
+ *     h1 = RMSNorm(x; g1)    qkv = h1 Wqkv^T ([T, 3 H d], T = B n: its thirds are Q, K, V of a [B,n,3,H,d] array)
+ *     o = attention(Q, K, V)    x2 = x + o Wo^T    h2 = RMSNorm(x2; g2)    y = x2 + gated_mlp(h2)
+ * Every array is [T, H d] unless said otherwise; weights are stored [out,in].  The forward reads x and the weights and writes
+ * the activations; the backward reads those, the weights and dy and writes the gradients.  Workspaces as for the single calls
+ * (attention: MOA_OP_BWD).  The first error of a call of the sequence is returned. */
+typedef struct {
+    int32_t B, n, H, d, d_ff;
+    int32_t causal;
+    float   eps, scale;
+} moa_block_desc;
+typedef struct {
+    const void *x, *g1, *g2, *Wqkv /* [3 H d, H d] */, *Wo, *W1 /* [d_ff, H d] */, *W3, *W2 /* [H d, d_ff] */;
+    void *h1, *qkv /* [T, 3 H d] */, *o, *x2, *h2, *a /* [T, d_ff] */, *u, *h, *y;
+    float *r1 /* [T] */, *r2, *L /* [B,H,n] */;
+    const void *dy;                                                     /* from here on: backward only */
+    void *dh2, *dx2, *dout /* gradient of o */, *dqkv, *dh1, *dx;
+    void *dg1, *dg2, *dWqkv, *dWo, *dW1, *dW3, *dW2;
+    void *norm_ws, *attn_ws, *mlp_ws;
+    size_t norm_ws_bytes, attn_ws_bytes, mlp_ws_bytes;
+} moa_block_arrays;
+moa_status moa_block_fwd(const moa_block_desc *desc, const moa_block_arrays *arrays, void *stream);
+moa_status moa_block_bwd(const moa_block_desc *desc, const moa_block_arrays *arrays, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -29,7 +29,7 @@ EXPORTS = (
     "moa_profile_enable", "moa_profile_read", "moa_attn_bwd_static_scratch", "moa_attn_fused_rowparallel",
     "moa_decode_workspace_bytes", "moa_decode_attn",
     "moa_rmsnorm_workspace_bytes", "moa_rmsnorm_fwd", "moa_rmsnorm_bwd",
-    "moa_gated_mlp_fwd", "moa_gated_mlp_workspace_bytes", "moa_gated_mlp_bwd", "moa_gemm",
+    "moa_gated_mlp_fwd", "moa_gated_mlp_workspace_bytes", "moa_gated_mlp_bwd", "moa_gemm", "moa_block_fwd", "moa_block_bwd",
     "moa_selftest_expired_wait", "moa_bwd_pair_mode",
 )
 
@@ -58,6 +58,17 @@ class moa_gemm_desc(ctypes.Structure):
 
 class moa_mlp_desc(ctypes.Structure):
     _fields_ = [("n", ctypes.c_int32), ("d", ctypes.c_int32), ("d_ff", ctypes.c_int32), ("dtype", ctypes.c_int32)]
+
+
+class moa_block_desc(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int32) for k in ("B", "n", "H", "d", "d_ff", "causal")] + [("eps", ctypes.c_float), ("scale", ctypes.c_float)]
+
+
+class moa_block_arrays(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_void_p) for k in
+                ("x", "g1", "g2", "Wqkv", "Wo", "W1", "W3", "W2", "h1", "qkv", "o", "x2", "h2", "a", "u", "h", "y", "r1", "r2", "L",
+                 "dy", "dh2", "dx2", "dout", "dqkv", "dh1", "dx", "dg1", "dg2", "dWqkv", "dWo", "dW1", "dW3", "dW2",
+                 "norm_ws", "attn_ws", "mlp_ws")] + [(k, ctypes.c_size_t) for k in ("norm_ws_bytes", "attn_ws_bytes", "mlp_ws_bytes")]
 
 
 MOA_KERNEL_KINDS = 6
@@ -118,6 +129,9 @@ def lib() -> ctypes.CDLL:
         L.moa_gemm.argtypes = [ctypes.POINTER(moa_gemm_desc)] + [vp] * 4 + [vp]
         L.moa_gated_mlp_bwd.restype = ctypes.c_int
         L.moa_gated_mlp_bwd.argtypes = [mp] + [vp] * 12 + [vp, sz, vp]
+        for f in (L.moa_block_fwd, L.moa_block_bwd):
+            f.restype = ctypes.c_int
+            f.argtypes = [ctypes.POINTER(moa_block_desc), ctypes.POINTER(moa_block_arrays), vp]
         L.moa_last_device_status.restype = ctypes.c_int
         L.moa_last_device_status.argtypes = [vp]
         L.moa_selftest_expired_wait.restype = ctypes.c_int
@@ -326,6 +340,20 @@ def moa_gated_mlp_bwd(desc, x, W1, W3, W2, a, u, h, dy, dx, dW1, dW3, dW2, ws=No
                                 _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
     if check and s != MOA_OK:
         raise MoaError(s, "moa_gated_mlp_bwd")
+    return s
+
+
+def moa_block_fwd(desc, arrays, stream=None, check=True) -> int:
+    s = lib().moa_block_fwd(ctypes.byref(desc), ctypes.byref(arrays), _stream(stream))
+    if check and s != MOA_OK:
+        raise MoaError(s, "moa_block_fwd")
+    return s
+
+
+def moa_block_bwd(desc, arrays, stream=None, check=True) -> int:
+    s = lib().moa_block_bwd(ctypes.byref(desc), ctypes.byref(arrays), _stream(stream))
+    if check and s != MOA_OK:
+        raise MoaError(s, "moa_block_bwd")
     return s
 
 

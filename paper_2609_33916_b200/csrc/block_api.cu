@@ -126,4 +126,67 @@ moa_status moa_gemm(const moa_gemm_desc *desc, const void *A, const void *B, con
                ? MOA_OK : MOA_ERR_CUDA;
 }
 
+namespace {
+
+// the descriptors of the block's calls
+struct BlockCalls {
+    moa_rmsnorm_desc norm;
+    moa_attn_desc attn;
+    moa_mlp_desc mlp;
+    int T, dm;
+    explicit BlockCalls(const moa_block_desc &b) : norm{}, attn{}, mlp{}, T(b.B * b.n), dm(b.H * b.d)
+    {
+        norm = moa_rmsnorm_desc{T, dm, b.eps, MOA_BF16};
+        attn.B = b.B; attn.H = b.H; attn.n = b.n; attn.d = b.d; attn.causal = b.causal; attn.scale = b.scale;
+        attn.layout = MOA_LAYOUT_STRIDED;
+        const int64_t third[3] = {3LL * dm, b.d, (int64_t)b.n * 3 * dm}, whole[3] = {dm, b.d, (int64_t)b.n * dm};
+        for (int i = 0; i < 3; ++i) { attn.q_stride[i] = attn.kv_stride[i] = third[i]; attn.o_stride[i] = whole[i]; }
+        mlp = moa_mlp_desc{T, dm, b.d_ff, MOA_BF16};
+    }
+    moa_gemm_desc gemm(int M, int N, int K, int a_layout, int b_layout) const { return moa_gemm_desc{M, N, K, a_layout, b_layout, MOA_BF16}; }
+    char *third(void *packed, int i) const { return packed ? (char *)packed + (size_t)i * dm * 2 : nullptr; }
+};
+
+bool block_desc_ok(const moa_block_desc *b, const moa_block_arrays *r)
+{
+    // (products of sizes that have to be countable in an int; everything else is checked by the calls)
+    return b && r && b->B > 0 && b->n > 0 && b->H > 0 && b->d > 0 && b->d_ff > 0 && (long long)b->B * b->n < (1LL << 31) &&
+           3LL * b->H * b->d < (1LL << 31);
+}
+
+}  // namespace
+
+#define MOA_STEP(call) do { const moa_status step = (call); if (step != MOA_OK) return step; } while (0)
+
+moa_status moa_block_fwd(const moa_block_desc *desc, const moa_block_arrays *r, void *stream)
+{
+    if (!block_desc_ok(desc, r)) return MOA_ERR_INVALID_ARG;
+    const BlockCalls c(*desc);
+    MOA_STEP(moa_rmsnorm_fwd(&c.norm, r->x, r->g1, r->h1, r->r1, stream));
+    const moa_gemm_desc proj3 = c.gemm(c.T, 3 * c.dm, c.dm, 0, 0), proj = c.gemm(c.T, c.dm, c.dm, 0, 0);
+    MOA_STEP(moa_gemm(&proj3, r->h1, r->Wqkv, nullptr, r->qkv, stream));
+    MOA_STEP(moa_attn_fwd(&c.attn, c.third(r->qkv, 0), c.third(r->qkv, 1), c.third(r->qkv, 2), r->o, r->L, nullptr, 0, stream));
+    MOA_STEP(moa_gemm(&proj, r->o, r->Wo, r->x, r->x2, stream));
+    MOA_STEP(moa_rmsnorm_fwd(&c.norm, r->x2, r->g2, r->h2, r->r2, stream));
+    return moa_gated_mlp_fwd(&c.mlp, r->h2, r->W1, r->W3, r->W2, r->x2, r->a, r->u, r->h, r->y, stream);
+}
+
+moa_status moa_block_bwd(const moa_block_desc *desc, const moa_block_arrays *r, void *stream)
+{
+    if (!block_desc_ok(desc, r)) return MOA_ERR_INVALID_ARG;
+    const BlockCalls c(*desc);
+    MOA_STEP(moa_gated_mlp_bwd(&c.mlp, r->h2, r->W1, r->W3, r->W2, r->a, r->u, r->h, r->dy, r->dh2, r->dW1, r->dW3, r->dW2, r->mlp_ws,
+                               r->mlp_ws_bytes, stream));
+    MOA_STEP(moa_rmsnorm_bwd(&c.norm, r->x2, r->g2, r->r2, r->dh2, r->dy, r->dx2, r->dg2, r->norm_ws, r->norm_ws_bytes, stream));
+    const moa_gemm_desc wgrad = c.gemm(c.dm, c.dm, c.T, 1, 1), back = c.gemm(c.T, c.dm, c.dm, 0, 1);
+    MOA_STEP(moa_gemm(&wgrad, r->dx2, r->o, nullptr, r->dWo, stream));
+    MOA_STEP(moa_gemm(&back, r->dx2, r->Wo, nullptr, r->dout, stream));
+    MOA_STEP(moa_attn_bwd(&c.attn, c.third(r->qkv, 0), c.third(r->qkv, 1), c.third(r->qkv, 2), r->o, r->L, r->dout, c.third(r->dqkv, 0),
+                          c.third(r->dqkv, 1), c.third(r->dqkv, 2), r->attn_ws, r->attn_ws_bytes, stream));
+    const moa_gemm_desc back3 = c.gemm(c.T, c.dm, 3 * c.dm, 0, 1), wgrad3 = c.gemm(3 * c.dm, c.dm, c.T, 1, 1);
+    MOA_STEP(moa_gemm(&back3, r->dqkv, r->Wqkv, nullptr, r->dh1, stream));
+    MOA_STEP(moa_gemm(&wgrad3, r->dqkv, r->h1, nullptr, r->dWqkv, stream));
+    return moa_rmsnorm_bwd(&c.norm, r->x, r->g1, r->r1, r->dh1, r->dx2, r->dx, r->dg1, r->norm_ws, r->norm_ws_bytes, stream);
+}
+
 }  // extern "C"
