@@ -256,6 +256,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16, warp = tid / 32;
     float *Pw = Vs + BN * LD + warp * BN * LP;      // this warp's P^T: [key][2 R rows]
     ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
     Q = ptx::after_wait(Q); K = ptx::after_wait(K); V = ptx::after_wait(V); dO = ptx::after_wait(dO);
 
     const int rank = split > 1 ? (int)cluster_rank() : 0;
@@ -354,9 +355,6 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     }
     cp_wait<0>();
     __syncthreads();
-    // (only here: the grid leaves slots free, and a successor's CTAs that sit in them from the start skew the balance of its
-    // own work -- B2 H1 n2048 d64: 252 us per fused call with the trigger on top, 219 here)
-    ptx::grid_launch_dependents();
     // partial results into shared memory: O [BM][LD] over Q, then m, l
     float *Om = smem, *Mm = Ks, *Lm = Ks + BM;
 #pragma unroll
@@ -542,6 +540,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
     }
     // (the tiles above are the call's inputs; L, D and the cleared dQ come from the kernel in front)
     ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
     L = ptx::after_wait(L); Dv = ptx::after_wait(Dv);
     for (; q0 < n; q0 += step) {
         if (tid < BM) {
@@ -629,7 +628,6 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
                 }
         }
     }
-    ptx::grid_launch_dependents();       // (late, as in the forward)
     if (split == 1) {
 #pragma unroll
         for (int i = 0; i < R / 2; ++i)
@@ -1022,7 +1020,9 @@ cudaError_t fwd_r(const Problem &p, const void *Q, const void *K, const void *V,
     const cudaError_t e = allow_smem<simt_fwd_kernel<T, R, D>>(S::kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_cluster(simt_fwd_kernel<T, R, D>, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K, (const T *)V,
+    // Not a programmatic dependent where an SM gets more than one CTA: those placed while the kernel in front drains pile up on
+    // the SMs it leaves first (B2 H1 n2048 d64: 252 us per fused call against 219).
+    return launch_cluster_as(tiles * split <= device_info().sms, simt_fwd_kernel<T, R, D>, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K, (const T *)V,
                        (T *)O, L, (const T *)pr.dO, pr.Dv, pr.dQzero, p.n, p.causal, p.scale, nqt, split);
 }
 template <typename T, int D>
