@@ -257,6 +257,10 @@ struct FwdForBwd {
 cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L,
                    const FwdForBwd &fb, cudaStream_t st);
 
+// The same on pairs of query tiles (tc_fwd2.cu; d <= 128), and whether that is the faster form of a problem
+cudaError_t tc_fwd_pairs(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const FwdForBwd &fb, cudaStream_t st);
+bool fwd_pairs_pay(const Problem &p);
+
 // Lp = -L*log2(e) and Dp = -rowsum(dO o O) (negated: fma/add operands), each padded per head to a
 // multiple of 128 rows (-inf / 0 past n)
 // (and, unless zero_acc is null, clears the fp32 accumulator [B*H, n, kernel_d(d)] the backward adds dQ into)

@@ -560,6 +560,7 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
                    const FwdForBwd &fb, cudaStream_t st)
 {
     if (p.d < 8 || p.d > 256 || p.d % 8) return cudaErrorInvalidValue;
+    if (p.d <= 128 && fwd_pairs_pay(p)) return tc_fwd_pairs(p, Q, K, V, O, L, fb, st);
     if (p.d > 192) return launch_fwd<128, 2, 8>(p, Q, K, V, O, L, fb, st);      // two 128-column passes, scores over both chunks
     if (p.d > 128) return launch_fwd<128, 2, 4>(p, Q, K, V, O, L, fb, st);
     if (p.d <= 64) return launch_fwd<64, 1, 4>(p, Q, K, V, O, L, fb, st);
