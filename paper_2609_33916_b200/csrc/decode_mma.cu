@@ -11,9 +11,10 @@
 //     the log2 domain), O += P V with V by ldmatrix.trans; about a hundred instructions per warp and 16 keys, a tenth of
 //     what the SM can issue in the time HBM takes for them;
 //   * when a CTA's share of a head ends, its eight warps' results are merged through shared memory.  A head that lies in one
-//     CTA's share is written out at once; the others leave fp32 partial results in the workspace (at most two per CTA) and
-//     the CTA that finishes a head last merges them, told by a counter that a one-block kernel in front has cleared.
-// Every wait is bounded; no CTA waits for another.
+//     CTA's share is written out at once; the others leave fp32 partial results in the workspace (at most two per CTA) for a
+//     merge kernel, which is set up while this one streams;
+//   * few heads: a cluster of up to eight CTAs per head, merged through distributed shared memory, and no second kernel.
+// Every wait is bounded; no CTA waits for another outside its cluster.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tensormap.cuh"
@@ -67,8 +68,8 @@ template <int D, bool kHi>
 __global__ void __launch_bounds__(kMmaThreads, 1)
 decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
                   const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out, float *__restrict__ lse,
-                  float *__restrict__ part_o, float *__restrict__ part_ml, unsigned int *__restrict__ counters, int n, int Hkv,
-                  int G, int nt, int units, float scale_log2, unsigned int *status)
+                  float *__restrict__ part_o, float *__restrict__ part_ml, int n, int Hkv, int G, int nt, int units, int cl,
+                  float scale_log2, unsigned int *status)
 {
     using S = MmaSmem<D>;
     constexpr int kRowsLane = kHi ? 2 : 1, kKS = D / 16, kNT = D / 8;
@@ -76,9 +77,11 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
     float *merge = reinterpret_cast<float *>(smem + S::offMerge);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + S::offBar), *empty = full + S::kStages;
     volatile uint32_t *abortp = reinterpret_cast<uint32_t *>(empty + S::kStages);
-    volatile uint32_t *s_last = abortp + 1;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int ctas = (int)gridDim.x, u0 = first_unit(units, blockIdx.x, ctas), u1 = first_unit(units, blockIdx.x + 1, ctas);
+    // cl > 0: the CTA of rank r of a cluster takes the r-th part of the cluster's head; otherwise an equal share of all units
+    const int rank = cl ? (int)cluster_ctarank() : 0, ctas = (int)gridDim.x;
+    const int u0 = cl ? (int)blockIdx.x / cl * nt + nt * rank / cl : first_unit(units, blockIdx.x, ctas);
+    const int u1 = cl ? (int)blockIdx.x / cl * nt + nt * (rank + 1) / cl : first_unit(units, blockIdx.x + 1, ctas);
     if (tid == 0) {
         for (int s = 0; s < S::kStages; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, kConsumers / 2); }
         *abortp = (smem_u32(smem) & 1023u) ? 1u : 0u;
@@ -88,11 +91,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
         prefetch_tensormap(&mapV);
     }
     __syncthreads();
+    grid_dependency_wait();
+    grid_launch_dependents();
     const bool sound = *abortp == 0;
 
     if (warp == kConsumers) {
         // ------------------------------------------------------------------ producer
-        // (q, K, V are the call's inputs: the clearing kernel in front has made sure that whatever wrote them is done)
         if (lane == 0 && sound) {
             ArmCounts<S::kStages> armed;
             int head = u0 / nt, t = u0 - head * nt;
@@ -110,8 +114,11 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
             }
             mbar_drain(full, armed);      // copies still on their way land before the CTA leaves (bounded)
         }
-        grid_dependency_wait();
-        grid_launch_dependents();
+        __syncwarp();
+        if (cl > 1) {
+            cluster_sync_all();
+            cluster_sync_all();
+        }
         return;
     }
 
@@ -125,7 +132,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
     auto addr = [&](int row, int chunk) {       // 16-byte chunk `chunk` of a row of the tile
         return (uint32_t)((chunk >> 3) * S::kBox + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
     };
-    bool waited = false;
     int u = u0;
     bool ok = sound;
     while (u < u1) {
@@ -213,14 +219,10 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
             if (lane == 0) mbar_arrive(empty + s);
         }
         // ---- the segment's end: merge the warps, eight queries at a time
-        if (!waited) {
-            grid_dependency_wait();        // the counters are clear, and whatever read the workspace or the outputs before is done
-            grid_launch_dependents();
-            waited = true;
-        }
         const bool whole = t_first == 0 && seg_end == (head + 1) * nt;
         const int slot = 2 * (int)blockIdx.x + (t_first == 0 ? 1 : 0);
         constexpr int kLd = D + 2;
+        float *seg = reinterpret_cast<float *>(smem);      // cluster: this CTA's part, [G][D + 2], over the ring, which is done
 #pragma unroll
         for (int h = 0; h < kRowsLane; ++h) {
             float lt = l[h];
@@ -245,7 +247,10 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
                     ot = fmaf(src[c], a, ot);
                     ls = fmaf(src[D + 1], a, ls);
                 }
-                if (whole) {
+                if (cl > 1) {
+                    seg[g * kLd + c] = ot;
+                    if (c == 0) { seg[g * kLd + D] = mt; seg[g * kLd + D + 1] = ls; }
+                } else if (whole) {
                     out[((size_t)head * G + g) * D + c] = __float2bfloat16_rn(ot / ls);
                     if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
                 } else {
@@ -254,39 +259,64 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
                 }
             }
         }
-        if (whole) continue;
-        // ---- a head shared by several CTAs: whoever publishes last merges
-        const int ca = cta_of_unit(units, head * nt, ctas), cb = cta_of_unit(units, (head + 1) * nt - 1, ctas);
-        __threadfence();
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (tid == 0) *s_last = atomicAdd(counters + head, 1u) == (unsigned)(cb - ca) ? 1u : 0u;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (*s_last == 0u) continue;
-        __threadfence();
-        for (int idx = tid; idx < G * (D / 4); idx += 256) {
-            const int g = idx / (D / 4), c = (idx - g * (D / 4)) * 4;
-            auto at = [&](int k) { return (size_t)(2 * k + (k == ca ? 1 : 0)) * G + g; };
-            float mt = -INFINITY, ls = 0.f;
-#pragma unroll 8
-            for (int k = ca; k <= cb; ++k) mt = fmaxf(mt, __ldcg(part_ml + at(k) * 2));
-            float4 ot = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
-            for (int k = ca; k <= cb; ++k) {
-                const float2 ml = __ldcg(reinterpret_cast<const float2 *>(part_ml + at(k) * 2));
-                const float4 v = __ldcg(reinterpret_cast<const float4 *>(part_o + at(k) * D + c));
-                const float a = ex2(ml.x - mt);
-                ls = fmaf(ml.y, a, ls);
-                ot.x = fmaf(v.x, a, ot.x); ot.y = fmaf(v.y, a, ot.y); ot.z = fmaf(v.z, a, ot.z); ot.w = fmaf(v.w, a, ot.w);
+        if (cl > 1) {       // (the only segment)
+            __syncwarp();
+            cluster_sync_all();
+            auto peer = [&](const float *mine, int k) {
+                float v;
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(mapa_u32(smem_u32(mine), (uint32_t)k)) : "memory");
+                return v;
+            };
+            for (int idx = rank * 256 + tid; idx < G * D; idx += cl * 256) {
+                const int g = idx / D, c = idx - g * D;
+                const float *at = seg + g * kLd;
+                float mt = -INFINITY, ot = 0.f, ls = 0.f;
+                for (int k = 0; k < cl; ++k) mt = fmaxf(mt, peer(at + D, k));
+                for (int k = 0; k < cl; ++k) {
+                    const float a = ex2(peer(at + D, k) - mt);
+                    ot = fmaf(peer(at + c, k), a, ot);
+                    ls = fmaf(peer(at + D + 1, k), a, ls);
+                }
+                out[((size_t)head * G + g) * D + c] = __float2bfloat16_rn(ot / ls);
+                if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
             }
-            const float inv = 1.f / ls;
-            *reinterpret_cast<uint2 *>(out + ((size_t)head * G + g) * D + c) =
-                make_uint2(pack_bf16(ot.x * inv, ot.y * inv), pack_bf16(ot.z * inv, ot.w * inv));
-            if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
+            __syncwarp();
+            cluster_sync_all();       // nobody leaves while another CTA may still read its shared memory
         }
     }
-    if (!waited) {
-        grid_dependency_wait();
-        grid_launch_dependents();
+}
+
+// Heads shared by several CTAs of the kernel above: a block per K/V head adds their partial results in CTA order.
+template <int D>
+__global__ void __launch_bounds__(128)
+decode_mma_merge_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml, __nv_bfloat16 *__restrict__ out,
+                        float *__restrict__ lse, int G, int nt, int units, int ctas)
+{
+    const int head = blockIdx.x, ca = cta_of_unit(units, head * nt, ctas), cb = cta_of_unit(units, (head + 1) * nt - 1, ctas);
+    grid_dependency_wait();
+    grid_launch_dependents();
+    if (ca == cb) return;
+    part_o = after_wait(part_o);
+    part_ml = after_wait(part_ml);
+    for (int idx = threadIdx.x; idx < G * (D / 4); idx += blockDim.x) {
+        const int g = idx / (D / 4), c = (idx - g * (D / 4)) * 4;
+        auto at = [&](int k) { return (size_t)(2 * k + (k == ca ? 1 : 0)) * G + g; };
+        float mt = -INFINITY, ls = 0.f;
+#pragma unroll 8
+        for (int k = ca; k <= cb; ++k) mt = fmaxf(mt, part_ml[at(k) * 2]);
+        float4 ot = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int k = ca; k <= cb; ++k) {
+            const float2 ml = *reinterpret_cast<const float2 *>(part_ml + at(k) * 2);
+            const float4 v = *reinterpret_cast<const float4 *>(part_o + at(k) * D + c);
+            const float a = ex2(ml.x - mt);
+            ls = fmaf(ml.y, a, ls);
+            ot.x = fmaf(v.x, a, ot.x); ot.y = fmaf(v.y, a, ot.y); ot.z = fmaf(v.z, a, ot.z); ot.w = fmaf(v.w, a, ot.w);
+        }
+        const float inv = 1.f / ls;
+        *reinterpret_cast<uint2 *>(out + ((size_t)head * G + g) * D + c) =
+            make_uint2(pack_bf16(ot.x * inv, ot.y * inv), pack_bf16(ot.z * inv, ot.w * inv));
+        if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
     }
 }
 
@@ -300,16 +330,25 @@ cudaError_t launch(const DecodeProblem &p, const void *q, const void *K, const v
         !make_tensor_map_4d(&mv, V, bf, 2, p.B, p.Hkv, p.n, D, false, kKeys, 64))
         return cudaErrorInvalidValue;
     const int G = p.H / p.Hkv, nt = (p.n + kKeys - 1) / kKeys, heads = p.B * p.Hkv, units = nt * heads, sms = device_info().sms;
-    const int ctas = units < sms ? units : sms;
-    float *part_o = (float *)ws, *part_ml = part_o + (size_t)2 * sms * G * D;
-    unsigned int *counters = reinterpret_cast<unsigned int *>(part_ml + (size_t)2 * sms * G * 2);
-    cudaError_t e = allow_smem<decode_mma_kernel<D, kHi>>(S::kTotal);
+    const cudaError_t e = allow_smem<decode_mma_kernel<D, kHi>>(S::kTotal);
     if (e != cudaSuccess) return e;
-    if ((e = decode_clear(counters, heads, st)) != cudaSuccess) return e;
+    // A cluster per head while all of them fit at once, unless its CTAs would stream more than 128 KB beyond an equal share: the merge
+    // kernel costs about what an SM streams in that time.
+    int cl = 0;
+    for (int c = 1; c <= 8 && c <= nt && heads * c <= sms; c *= 2) cl = c;
+    if (cl && ((nt + cl - 1) / cl - (units + sms - 1) / sms) * 2 * S::kTile > 128 * 1024) cl = 0;
+    const int ctas = cl ? heads * cl : units < sms ? units : sms;
+    float *part_o = (float *)ws, *part_ml = part_o + (size_t)2 * sms * G * D;
+    {
+        LaunchScope scope(MOA_KERNEL_OTHER, st);
+        const cudaError_t le = launch_cluster(decode_mma_kernel<D, kHi>, cl > 1 ? (unsigned)cl : 1u, dim3((unsigned)ctas), dim3(kMmaThreads),
+                                              (size_t)S::kTotal, st, mk, mv, (const __nv_bfloat16 *)q, (__nv_bfloat16 *)out, lse, part_o,
+                                              part_ml, p.n, p.Hkv, G, nt, units, cl, p.scale * kLog2e, device_status_ptr());
+        if (le != cudaSuccess || cl) return le;
+    }
     LaunchScope scope(MOA_KERNEL_OTHER, st);
-    return launch_dependent(decode_mma_kernel<D, kHi>, dim3((unsigned)ctas), dim3(kMmaThreads), (size_t)S::kTotal, st, mk, mv,
-                            (const __nv_bfloat16 *)q, (__nv_bfloat16 *)out, lse, part_o, part_ml, counters, p.n, p.Hkv, G, nt, units,
-                            p.scale * kLog2e, device_status_ptr());
+    return launch_dependent(decode_mma_merge_kernel<D>, dim3((unsigned)heads), dim3(128), (size_t)0, st, (const float *)part_o,
+                            (const float *)part_ml, (__nv_bfloat16 *)out, lse, G, nt, units, ctas);
 }
 
 }  // namespace
@@ -324,7 +363,7 @@ bool decode_uses_mma(const DecodeProblem &p, int dtype)
 
 size_t decode_mma_workspace_bytes(const DecodeProblem &p)
 {
-    return (size_t)2 * device_info().sms * (p.H / p.Hkv) * (p.d + 2) * sizeof(float) + (size_t)p.B * p.Hkv * sizeof(unsigned int);
+    return (size_t)2 * device_info().sms * (p.H / p.Hkv) * (p.d + 2) * sizeof(float);
 }
 
 cudaError_t decode_mma(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse, void *ws, cudaStream_t st)

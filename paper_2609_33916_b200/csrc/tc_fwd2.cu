@@ -404,19 +404,21 @@ cudaError_t launch(const Problem &p, const void *Q, const void *K, const void *V
 }  // namespace
 
 // Whether pairs of query tiles finish before single ones (tc_fwd.cu), in units of one key tile of one query tile: a job costs about 8
-// (9 for a pair) beside its tiles; equal jobs go in rounds over the SMs, causal ones longest first.
+// (9 for a pair) beside its tiles; equal jobs go in rounds over the SMs, causal ones longest first.  Forward alone, single / pairs:
+// B2 H16 n4096 d128 causal 141 / 124 us, B1 H16 n16384 1913 / 1845, B4 H8 n1024 d64 24.3 / 19.0, B4 H32 n200 causal 18.0 / 11.3, but
+// B1 H8 n2048 23.5 / 37.7 (64 pairs on 148 SMs) and B1 H32 n512 causal 11.0 / 13.2.
 bool fwd_pairs_pay(const Problem &p)
 {
     const long long sms = device_info().sms, nqt = (p.n + BM - 1) / BM, np = (nqt + 1) / 2, bh = p.BH();
     auto cost = [&](long long jobs, double longest, double total, double fixed) {
         const double even = (double)((jobs + sms - 1) / sms) * (longest + fixed), avg = (total + (double)jobs * fixed) / (double)sms;
-        const double packed = avg + 0.5 * (total / (double)jobs + fixed), last = longest + fixed;
+        const double packed = avg + 0.2 * (total / (double)jobs + fixed), last = longest + fixed;
         return !p.causal ? even : last > packed ? last : packed < even ? packed : even;
     };
     const double total = (double)bh * (p.causal ? nqt * (nqt + 1) / 2 : nqt * nqt);
     const double one = cost(bh * nqt, (double)nqt, total, 8.0);
     const double two = cost(bh * np, (double)(nqt == 1 ? 1 : p.causal ? 2 * nqt - 1 : 2 * nqt), total, 9.0);
-    return two < one;
+    return two < 0.98 * one;
 }
 
 cudaError_t tc_fwd_pairs(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const FwdForBwd &fb, cudaStream_t st)

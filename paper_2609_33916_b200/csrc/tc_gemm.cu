@@ -159,6 +159,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         mbar_init(bars + G_RES + 1, 1);
         *abortp = 0;
         fence_mbar_init();
+        prefetch_tensormap(&mapA0);      // (kernel parameters: nothing to wait for)
+        prefetch_tensormap(&mapB0);
+        prefetch_tensormap(&mapC0);
     }
     if (warp == 1) {
         if (kPair) {
@@ -179,8 +182,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 
     if (warp == 0 && lane == 0) {
         // ------------------------------------------------------------------ TMA producer
-        prefetch_tensormap(&mapA0);
-        prefetch_tensormap(&mapB0);
         ArmCounts<G_COUNT> armed;     // barriers armed for copies into shared memory
         int it = 0;
         bool ok = true;
@@ -469,7 +470,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             }
         }
         if (leader) {
-            bulk_wait<0>();               // every store has completed before the CTA gives up its shared memory
+            bulk_wait_read<0>();          // every store has read its buffer before the CTA gives up its shared memory
             mbar_drain(bars, armed);      // and so has every copy into the staging buffers (bounded)
         }
     }
