@@ -100,10 +100,11 @@ inline int heads_per_group(const Problem &p, int tiles)
 // shared K/V heads or the causal mask the longest tile alone can outlast the average SM's share by far.  Estimated in units
 // of one query tile: a CTA costs `fixed` beside its tiles, a merge `merge` more; equal jobs go in rounds, causal ones longest first,
 // which packs to within a part of an average job.  A cluster has to beat the next smaller one by 5 %.
-//   jobs: key tiles of all K/V heads (times the passes over d); longest, total: query tiles of the longest job, of all jobs
-inline int bwd_split(long long jobs, long long longest, long long total, bool causal, double fixed, double merge)
+//   jobs: key tiles of all K/V heads (times the passes over d); longest, total: query tiles of the longest job, of all jobs;
+//   per_sm: CTAs that an SM holds at once
+inline int bwd_split(long long jobs, long long longest, long long total, bool causal, double fixed, double merge, int per_sm = 1)
 {
-    const double sms = device_info().sms;
+    const double sms = (double)device_info().sms * per_sm;
     int best = 1;
     double best_cost = 0;
     for (int s = 1; s <= 8; s *= 2) {

@@ -996,13 +996,21 @@ convert_rows_kernel(const float *__restrict__ src, int src_ld, __nv_bfloat16 *__
 
 constexpr size_t bwd_smem(int D) { return (size_t)(4 * BM * (D + 1) + 2 * BM * SLD + 2 * BM) * sizeof(float); }
 
-// How many ranks share an output tile: doubled while all CTAs still fit on the chip at once (`slots`), every rank keeps at
-// least one tile of the other axis (`others`), and the cluster stays portable (8).
-int simt_split(long long tiles, int others, long long slots)
+// How many ranks share an output tile (bwd_split's estimate, for `per_sm` CTAs on an SM; set-up and merge are small beside these
+// kernels' tiles).  With the causal mask the longest of B2 H2 n1817 d128's 228 tiles takes twice the average and all run at once, so
+// that clusters of two, in two waves, are faster.
+int simt_split(long long jobs, int own_tiles, int others, int own_rows, int other_rows, bool causal, int per_sm)
 {
-    int s = 1;
-    while (s < 8 && 2 * s <= others && tiles * 2 * s <= slots) s *= 2;
-    return s;
+    // causal: the tiles of the other axis that tile t meets, summed over t (both axes are cut from the same n rows)
+    long long total = (long long)own_tiles * others;
+    if (causal) {
+        total = 0;
+        for (int t = 0; t < own_tiles; ++t) {
+            const long long c = ((long long)(t + 1) * own_rows + other_rows - 1) / other_rows;
+            total += c < others ? c : others;
+        }
+    }
+    return bwd_split(jobs, others, jobs / own_tiles * total, causal, 0.3, 0.3, per_sm);
 }
 
 // Rows per thread: the widest tile (fewest shared-memory loads per multiply-add) whose tiles, shared by clusters as far as
@@ -1013,10 +1021,10 @@ cudaError_t fwd_r(const Problem &p, const void *Q, const void *K, const void *V,
 {
     using S = SimtFwd<R, D>;
     const int nqt = (p.n + S::BM - 1) / S::BM, nkt = (p.n + BN - 1) / BN;
-    const long long tiles = (long long)nqt * p.BH(), slots = (long long)device_info().sms * (R == 8 ? 3 : D == 128 ? 2 : 4);
+    const long long tiles = (long long)nqt * p.BH();
     if (R > 2 && tiles * (nkt < 8 ? nkt : 8) < device_info().sms)
         return fwd_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, O, L, pr, st);
-    const int split = simt_split(tiles, nkt, slots);
+    const int split = simt_split(tiles, nqt, nkt, S::BM, BN, p.causal, R == 8 ? 3 : D == 128 ? 2 : 4);
     const cudaError_t e = allow_smem<simt_fwd_kernel<T, R, D>>(S::kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
@@ -1038,10 +1046,10 @@ cudaError_t bwd_kv_r(const Problem &p, const void *Q, const void *K, const void 
 {
     using S = SimtBwd<R, D>;
     const int nkt = (p.n + S::BN - 1) / S::BN, nqt = (p.n + S::BM - 1) / S::BM;
-    const long long tiles = (long long)nkt * p.BH(), slots = 2LL * device_info().sms;
+    const long long tiles = (long long)nkt * p.BH();
     if (R > 2 && tiles * (nqt < 8 ? nqt : 8) < device_info().sms)
         return bwd_kv_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, dO, L, Dv, dK, dV, dQacc, st);
-    const int split = simt_split(tiles, nqt, slots);
+    const int split = simt_split(tiles, nkt, nqt, S::BN, S::BM, p.causal, 2);
     const cudaError_t e = allow_smem<simt_bwd_kv_kernel<T, R, D>>(S::kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
