@@ -332,11 +332,11 @@ cudaError_t launch(const DecodeProblem &p, const void *q, const void *K, const v
     const int G = p.H / p.Hkv, nt = (p.n + kKeys - 1) / kKeys, heads = p.B * p.Hkv, units = nt * heads, sms = device_info().sms;
     const cudaError_t e = allow_smem<decode_mma_kernel<D, kHi>>(S::kTotal);
     if (e != cudaSuccess) return e;
-    // A cluster per head while all of them fit at once, unless its CTAs would stream more than 128 KB beyond an equal share: the merge
+    // A cluster per head while all of them fit at once, unless its CTAs would stream more than 192 KB beyond an equal share: the merge
     // kernel costs about what an SM streams in that time.
     int cl = 0;
     for (int c = 1; c <= 8 && c <= nt && heads * c <= sms; c *= 2) cl = c;
-    if (cl && ((nt + cl - 1) / cl - (units + sms - 1) / sms) * 2 * S::kTile > 128 * 1024) cl = 0;
+    if (cl && ((nt + cl - 1) / cl - (units + sms - 1) / sms) * 2 * S::kTile > 192 * 1024) cl = 0;
     const int ctas = cl ? heads * cl : units < sms ? units : sms;
     float *part_o = (float *)ws, *part_ml = part_o + (size_t)2 * sms * G * D;
     {

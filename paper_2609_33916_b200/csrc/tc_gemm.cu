@@ -53,13 +53,14 @@ constexpr int kABytes = GM * GK * 2;
 // the issuing thread per eight UMMAs instead of per four (that thread's time per stage is on the critical path: a
 // second commit per stage cost 3-4 %).
 // Narrower tiles are for launches whose 256-column tiles would leave SMs idle: less work per SM and a shorter epilogue, at more operand
-// traffic per unit of work; six and eight stages of 32 and 24 KB.
-constexpr int kMaxStages = 8;
-__host__ __device__ constexpr int gemm_sub(bool pair) { return pair ? 2 : 1; }                 // 64-element K blocks per stage
-__host__ __device__ constexpr int gemm_stages(bool pair, int n) { return pair ? 3 : n == 256 ? 4 : n == 128 ? 6 : 8; }
+// traffic per unit of work.  Their stages hold two K blocks as well: a wait, four short UMMAs and a commit take the issuing thread 640
+// cycles a block whatever the width, so that with one block per stage they gained nothing.
+constexpr int kMaxStages = 6;
+__host__ __device__ constexpr int gemm_sub(bool pair, int n) { return pair || n < 256 ? 2 : 1; }       // 64-element K blocks per stage
+__host__ __device__ constexpr int gemm_stages(bool pair, int n) { return pair ? 3 : n == 256 ? 4 : n == 128 ? 3 : 4; }
 __host__ __device__ constexpr int gemm_b_bytes(int n) { return n * GK * 2; }
 __host__ __device__ constexpr int gemm_sub_bytes(bool pair, int n) { return kABytes + (pair ? gemm_b_bytes(n) / 2 : gemm_b_bytes(n)); }
-__host__ __device__ constexpr int gemm_stage_bytes(bool pair, int n) { return gemm_sub(pair) * gemm_sub_bytes(pair, n); }
+__host__ __device__ constexpr int gemm_stage_bytes(bool pair, int n) { return gemm_sub(pair, n) * gemm_sub_bytes(pair, n); }
 constexpr int kMnBox = 64 * GK * 2;                    // one MN-major box: 64 columns x 64 K-rows
 constexpr int kOutBox = 128 * 64 * 2;                  // one staged output chunk: 128 rows x 64 columns, bf16
 __host__ __device__ constexpr int gemm_smem(bool pair, int n)
@@ -127,7 +128,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     // A rows and the B half staged in each CTA (this CTA: rows rank*128.. of the tile, B rows rank*128.. of its 256)
     // and write each CTA's accumulator; every CTA runs its own producer and epilogue.
     constexpr int kSt = gemm_stages(kPair, kN), kStageBytes = gemm_stage_bytes(kPair, kN), kTileM = kPair ? 2 * GM : GM;
-    constexpr int kSub = gemm_sub(kPair), kSubBytes = gemm_sub_bytes(kPair, kN);
+    constexpr int kSub = gemm_sub(kPair, kN), kSubBytes = gemm_sub_bytes(kPair, kN);
     const uint32_t rank = kPair ? cluster_ctarank() : 0u;
     const int cta = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, ncta = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     extern __shared__ uint8_t smem_raw[];
@@ -260,25 +261,25 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 tc_fence_after();
                 const uint32_t a_lo = a_lo0 + ((smem_u32(sm + s * kStageBytes) >> 4) & 0x3FFFu);
                 const uint32_t b_lo = b_lo0 + ((smem_u32(sm + s * kStageBytes + kABytes) >> 4) & 0x3FFFu);
-                if (kPair) {
 #pragma unroll
-                    for (int sub = 0; sub < kSub; ++sub) {
-                        const uint32_t a_s = a_lo + (uint32_t)(sub * (kSubBytes >> 4)), b_s = b_lo + (uint32_t)(sub * (kSubBytes >> 4));
-                        if (ks == 0 && sub == 0) umma_ss2_pair<false>(acc, a_s, a_hi, b_s, b_hi, idesc);
-                        else                     umma_ss2_pair<true>(acc, a_s, a_hi, b_s, b_hi, idesc);
-#pragma unroll
-                        for (int q = 1; q < GK / 16; ++q)
-                            umma_ss2_pair<true>(acc, a_s + q * a_step, a_hi, b_s + q * b_step, b_hi, idesc);
+                for (int sub = 0; sub < kSub; ++sub) {
+                    const uint32_t a_s = a_lo + (uint32_t)(sub * (kSubBytes >> 4)), b_s = b_lo + (uint32_t)(sub * (kSubBytes >> 4));
+                    if (ks == 0 && sub == 0) {
+                        if (kPair) umma_ss2_pair<false>(acc, a_s, a_hi, b_s, b_hi, idesc);
+                        else       umma_ss2<false>(acc, a_s, a_hi, b_s, b_hi, idesc);
+                    } else {
+                        if (kPair) umma_ss2_pair<true>(acc, a_s, a_hi, b_s, b_hi, idesc);
+                        else       umma_ss2<true>(acc, a_s, a_hi, b_s, b_hi, idesc);
                     }
-                    umma_commit_pair(bars + G_EMPTY + s);     // frees the stage in both CTAs
-                } else {
-                    if (ks == 0) umma_ss2<false>(acc, a_lo, a_hi, b_lo, b_hi, idesc);
-                    else         umma_ss2<true>(acc, a_lo, a_hi, b_lo, b_hi, idesc);
 #pragma unroll
-                    for (int q = 1; q < GK / 16; ++q)
-                        umma_ss2<true>(acc, a_lo + q * a_step, a_hi, b_lo + q * b_step, b_hi, idesc);
-                    umma_commit(bars + G_EMPTY + s);          // the stage is free once these UMMAs have read it
+                    for (int q = 1; q < GK / 16; ++q) {
+                        if (kPair) umma_ss2_pair<true>(acc, a_s + q * a_step, a_hi, b_s + q * b_step, b_hi, idesc);
+                        else       umma_ss2<true>(acc, a_s + q * a_step, a_hi, b_s + q * b_step, b_hi, idesc);
+                    }
                 }
+                // the stage is free (in both CTAs of a pair) once these UMMAs have read it
+                if (kPair) umma_commit_pair(bars + G_EMPTY + s);
+                else       umma_commit(bars + G_EMPTY + s);
             }
             if (ok) {
                 if (kPair) umma_commit_pair(bars + G_ACCFULL + buf);
@@ -618,9 +619,9 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
     bool pair = mode == 2 || pair_ok;
     if (mode != 2 && tiles(256) < 2 * sms) {
         double best = pair ? cost(pair_tiles, pairs, 530, 256) : cost(tiles(256), sms, 520, 256);
-        const double c128 = cost(tiles(128), sms, 400, 128);
+        const double c128 = cost(tiles(128), sms, 360, 128);
         if (c128 < 0.95 * best) { best = c128; n = 128; pair = false; }
-        const double c64 = kDualN ? 1e30 : cost(tiles(64), sms, 300, 64);
+        const double c64 = kDualN ? 1e30 : cost(tiles(64), sms, 290, 64);
         if (c64 < 0.95 * best) { n = 64; pair = false; }
     }
     if (pair) return launch_gemm_as<kAMn, kBMn, kEpi, true, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
