@@ -546,17 +546,26 @@ cudaError_t launch_gemm_as(const Operand &A0, const Operand &B0, const Operand *
     // MN-major operands whose width is a multiple of 64 come in by one blocked copy per stage (try the encode; if the
     // driver refuses the map, or a width has a tail, use one copy per 64-column block)
     const Operand &a1 = A1 ? *A1 : A0, &b1 = B1 ? *B1 : B0;
+    // (maps that repeat another one are copied, not looked up again: a launch of a small product is host time)
     bool a_blocked = kAMn && A0.cols % 64 == 0 && a1.cols % 64 == 0;
     bool b_blocked = kBMn && B0.cols % 64 == 0 && b1.cols % 64 == 0;
-    if (a_blocked && !(operand_map(&ma0, A0, true, GM, true) && operand_map(&ma1, a1, true, GM, true))) a_blocked = false;
-    if (b_blocked && !(operand_map(&mb0, B0, true, b_rows, true) && operand_map(&mb1, b1, true, b_rows, true))) b_blocked = false;
-    if (!a_blocked && (!operand_map(&ma0, A0, kAMn, GM) || !operand_map(&ma1, a1, kAMn, GM))) return cudaErrorInvalidValue;
-    if (!b_blocked && (!operand_map(&mb0, B0, kBMn, b_rows) || !operand_map(&mb1, b1, kBMn, b_rows))) return cudaErrorInvalidValue;
+    auto pair_of = [](CUtensorMap &m0, CUtensorMap &m1, const Operand &o0, const Operand *o1, bool mn, int rows, bool blocked) {
+        if (!operand_map(&m0, o0, mn, rows, blocked)) return false;
+        if (o1) return operand_map(&m1, *o1, mn, rows, blocked);
+        m1 = m0;
+        return true;
+    };
+    if (a_blocked && !pair_of(ma0, ma1, A0, A1, true, GM, true)) a_blocked = false;
+    if (b_blocked && !pair_of(mb0, mb1, B0, B1, true, b_rows, true)) b_blocked = false;
+    if (!a_blocked && !pair_of(ma0, ma1, A0, A1, kAMn, GM, false)) return cudaErrorInvalidValue;
+    if (!b_blocked && !pair_of(mb0, mb1, B0, B1, kBMn, b_rows, false)) return cudaErrorInvalidValue;
     CUtensorMap mc[4];
-    const void *cs[4] = {C0, C1 ? C1 : C0, C2 ? C2 : C0, C3 ? C3 : C0};
-    for (int i = 0; i < 4; ++i)     // [c_rows, ldc] bf16, boxes of 128 rows x 64 columns, 128-byte swizzle
-        if (!make_tensor_map_3d(&mc[i], cs[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 1, (uint64_t)c_rows, (uint64_t)ldc, 128, 64))
+    const void *cs[4] = {C0, C1, C2, C3};
+    for (int i = 0; i < 4; ++i) {     // [c_rows, ldc] bf16, boxes of 128 rows x 64 columns, 128-byte swizzle
+        if (i > 0 && !cs[i]) mc[i] = mc[0];
+        else if (!make_tensor_map_3d(&mc[i], cs[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 1, (uint64_t)c_rows, (uint64_t)ldc, 128, 64))
             return cudaErrorInvalidValue;
+    }
     auto kernel = tc_gemm_kernel<kAMn, kBMn, kEpi, kPair, kN>;
     constexpr int kSmem = gemm_smem(kPair, kN), kTileN = kDualN ? kN / 2 : kN, kTileM = kPair ? 2 * GM : GM;
     cudaError_t e = allow_smem<tc_gemm_kernel<kAMn, kBMn, kEpi, kPair, kN>>(kSmem);
