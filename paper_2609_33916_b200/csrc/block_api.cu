@@ -144,6 +144,18 @@ struct BlockCalls {
         mlp = moa_mlp_desc{T, dm, b.d_ff, MOA_BF16};
     }
     moa_gemm_desc gemm(int M, int N, int K, int a_layout, int b_layout) const { return moa_gemm_desc{M, N, K, a_layout, b_layout, MOA_BF16}; }
+    // two products that do not depend on each other
+    moa_status two(const moa_gemm_desc &g, const void *A, const void *B, void *C, const moa_gemm_desc &h, const void *D, const void *E, void *F,
+                   void *stream) const
+    {
+        for (const void *p : {A, B, (const void *)C, D, E, (const void *)F})
+            if (!p || !aligned16(p)) return MOA_ERR_INVALID_ARG;
+        if (dm % 8 != 0) return MOA_ERR_UNSUPPORTED;
+        const moa_status s = check_device_arch();
+        if (s != MOA_OK) return s;
+        return gemm_bf16_two(GemmArgs{g.a_layout, g.b_layout, g.M, g.N, g.K, A, B, C}, GemmArgs{h.a_layout, h.b_layout, h.M, h.N, h.K, D, E, F},
+                             (cudaStream_t)stream) == cudaSuccess ? MOA_OK : MOA_ERR_CUDA;
+    }
     char *third(void *packed, int i) const { return packed ? (char *)packed + (size_t)i * dm * 2 : nullptr; }
 };
 
@@ -178,14 +190,10 @@ moa_status moa_block_bwd(const moa_block_desc *desc, const moa_block_arrays *r, 
     MOA_STEP(moa_gated_mlp_bwd(&c.mlp, r->h2, r->W1, r->W3, r->W2, r->a, r->u, r->h, r->dy, r->dh2, r->dW1, r->dW3, r->dW2, r->mlp_ws,
                                r->mlp_ws_bytes, stream));
     MOA_STEP(moa_rmsnorm_bwd(&c.norm, r->x2, r->g2, r->r2, r->dh2, r->dy, r->dx2, r->dg2, r->norm_ws, r->norm_ws_bytes, stream));
-    const moa_gemm_desc wgrad = c.gemm(c.dm, c.dm, c.T, 1, 1), back = c.gemm(c.T, c.dm, c.dm, 0, 1);
-    MOA_STEP(moa_gemm(&wgrad, r->dx2, r->o, nullptr, r->dWo, stream));
-    MOA_STEP(moa_gemm(&back, r->dx2, r->Wo, nullptr, r->dout, stream));
+    MOA_STEP(c.two(c.gemm(c.dm, c.dm, c.T, 1, 1), r->dx2, r->o, r->dWo, c.gemm(c.T, c.dm, c.dm, 0, 1), r->dx2, r->Wo, r->dout, stream));
     MOA_STEP(moa_attn_bwd(&c.attn, c.third(r->qkv, 0), c.third(r->qkv, 1), c.third(r->qkv, 2), r->o, r->L, r->dout, c.third(r->dqkv, 0),
                           c.third(r->dqkv, 1), c.third(r->dqkv, 2), r->attn_ws, r->attn_ws_bytes, stream));
-    const moa_gemm_desc back3 = c.gemm(c.T, c.dm, 3 * c.dm, 0, 1), wgrad3 = c.gemm(3 * c.dm, c.dm, c.T, 1, 1);
-    MOA_STEP(moa_gemm(&back3, r->dqkv, r->Wqkv, nullptr, r->dh1, stream));
-    MOA_STEP(moa_gemm(&wgrad3, r->dqkv, r->h1, nullptr, r->dWqkv, stream));
+    MOA_STEP(c.two(c.gemm(c.T, c.dm, 3 * c.dm, 0, 1), r->dqkv, r->Wqkv, r->dh1, c.gemm(3 * c.dm, c.dm, c.T, 1, 1), r->dqkv, r->h1, r->dWqkv, stream));
     return moa_rmsnorm_bwd(&c.norm, r->x, r->g1, r->r1, r->dh1, r->dx2, r->dx, r->dg1, r->norm_ws, r->norm_ws_bytes, stream);
 }
 

@@ -234,6 +234,12 @@ cudaError_t gated_mlp_fwd(int n, int d, int dff, const void *x, const void *W1, 
 // C[M,N] = A B^T (+ R): A given as [M,K] (a_mn = 0) or [K,M] (a_mn = 1), B as [N,K] (b_mn = 0) or [K,N] (b_mn = 1); bf16
 cudaError_t gemm_bf16(int a_mn, int b_mn, int M, int N, int K, const void *A, const void *B, const void *R, void *C,
                       cudaStream_t st);
+struct GemmArgs {
+    int a_mn, b_mn, M, N, K;
+    const void *A, *B;
+    void *C;
+};
+cudaError_t gemm_bf16_two(const GemmArgs &x, const GemmArgs &y, cudaStream_t st);      // one launch where both are small
 cudaError_t gated_mlp_bwd(int n, int d, int dff, const void *x, const void *W1, const void *W3, const void *W2,
                           const void *a, const void *u, const void *h, const void *dy, void *da, void *du,
                           void *dx, void *dW1, void *dW3, void *dW2, cudaStream_t st);

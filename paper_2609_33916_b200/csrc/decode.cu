@@ -202,12 +202,12 @@ struct DecodeJob {
 
 // Merge of the segments of a group's heads, normalise, write out (and the natural-log lse).  An item is four columns of a head; the
 // items of all heads run side by side, and where they leave threads over, several threads (stripes) share an item's segments and are
-// merged through `sh` (kMergeFloats floats).  (One head after the other took 2 us each: fp32 groups of 8 over 4359 keys 52 -> XX us.)
+// merged through `sh` (kMergeFloats floats).  (One head after the other took 2 us each: B5 H16 H_kv2 n2164 d64 fp32 22.5 -> 13.6 us.)
 // Called by every thread of a CTA of at least 256 threads; threads past 256 only take part in the barriers.  The partial
 // results are read with ld.global.cg: other CTAs wrote them.
 constexpr int kMergeFloats = 256 * 6;
 template <typename T, int D>
-__device__ __forceinline__ void merge_heads(const float *__restrict__ part_o, const float *__restrict__ part_ml,
+__device__ __noinline__ void merge_heads(const float *__restrict__ part_o, const float *__restrict__ part_ml,
                                             T *__restrict__ out, float *__restrict__ lse, int splits, size_t BH, size_t head0, int gcount,
                                             float *sh)
 {
@@ -344,8 +344,9 @@ __global__ void __launch_bounds__(256) decode_clear_kernel(unsigned int *__restr
 // ---- variant 1: rows straight from global memory into registers (16-byte streaming loads, kUnroll row
 // groups of K and of V in flight per warp).  Few registers when the group is small, so several CTAs
 // per SM keep enough bytes in flight: used for one or two query heads per K/V head.
+// (One head: at most 64 registers, four CTAs per SM; six more cost a third of the bytes in flight: B7 H32 n2557 d128 53 -> 64 us.)
 template <typename T, int D, int GC>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, GC == 1 ? 4 : GC == 2 && sizeof(T) == 4 ? 3 : 1)
 decode_split_kernel(const T *__restrict__ q, const T *__restrict__ K, const T *__restrict__ V,
                     float *__restrict__ part_o, float *__restrict__ part_ml, T *__restrict__ out, float *__restrict__ lse,
                     unsigned int *__restrict__ counters, int clustered,

@@ -488,6 +488,197 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     }
 }
 
+// Several products C = A B^T (one or two operand pairs, any storage order) as ONE launch of single CTAs: what the backward of a small block needs
+// next to each other.  A launch costs such a product 5 us beside its K blocks and leaves most SMs idle; here the tiles of all of them are
+// walked by one grid.  Same roles, ring and epilogue as tc_gemm_kernel, the operand layouts taken from the job at run time.
+constexpr int kMaxJobs = 4;
+struct GroupJob {
+    CUtensorMap A[2], B[2], C;
+    int M, N, K, nparts, a_mn, b_mn, a_blocked, b_blocked, tile0 /* number of the job's first tile */;
+};
+struct GroupJobs {
+    GroupJob j[kMaxJobs];
+    int count, tiles;
+};
+
+template <int kN>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *status)
+{
+    constexpr int kEpiWarps = 8;
+    constexpr int kSt = gemm_stages(false, kN), kStageBytes = gemm_stage_bytes(false, kN), kSub = gemm_sub(false, kN), kSubBytes = gemm_sub_bytes(false, kN);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t *sout = sm + kSt * kStageBytes;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sout + 2 * kOutBox);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + G_COUNT);
+    volatile uint32_t *abortp = tmem_slot + 1;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    if (tid == 0) {
+        for (int i = 0; i < kStages; ++i) {
+            mbar_init(bars + G_FULL + i, 1);
+            mbar_init(bars + G_EMPTY + i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bars + G_ACCFULL + i, 1);
+            mbar_init(bars + G_ACCEMPTY + i, 32 * kEpiWarps);
+        }
+        mbar_init(bars + G_EPI, 32 * kEpiWarps);
+        *abortp = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, 2 * kN);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const uint32_t tbase = *tmem_slot;
+    const int cta = (int)blockIdx.x, ncta = (int)gridDim.x, tiles = jobs.tiles;
+    // the job of a tile (tiles are walked in ascending order) and the tile's place in it
+    auto job_of = [&](int t, int &jx, int &m0, int &n0) {
+        while (jx + 1 < jobs.count && t >= jobs.j[jx + 1].tile0) ++jx;
+        const GroupJob &J = jobs.j[jx];
+        int tm, tn;
+        tile_coords(t - J.tile0, (J.M + GM - 1) / GM, (J.N + kN - 1) / kN, 8, tm, tn);
+        m0 = tm * GM;
+        n0 = tn * kN;
+    };
+    auto stages_of = [&](const GroupJob &J) { return (J.K + GK * kSub - 1) / (GK * kSub); };      // per operand pair
+
+    if (warp == 0 && lane == 0) {
+        // ------------------------------------------------------------------ TMA producer
+        ArmCounts<G_COUNT> armed;
+        int it = 0, jx = 0;
+        bool ok = true;
+        for (int t = cta; ok && t < tiles; t += ncta) {
+            int m0, n0;
+            job_of(t, jx, m0, n0);
+            const GroupJob &J = jobs.j[jx];
+            const int nk = stages_of(J);
+            for (int ks = 0; ks < nk * J.nparts; ++ks, ++it) {
+                const int s = it % kSt, part = ks / nk;
+                if (!mbar_wait(bars + G_EMPTY + s, ((it / kSt) & 1) ^ 1, abortp, status, GERR_EMPTY)) { ok = false; break; }
+                uint64_t *full = bars + G_FULL + s;
+                mbar_arm(bars, G_FULL + s, kStageBytes, armed);
+                const CUtensorMap *ma = &J.A[part], *mb = &J.B[part];
+#pragma unroll
+                for (int sub = 0; sub < kSub; ++sub) {
+                    const int k0 = ((ks - part * nk) * kSub + sub) * GK;
+                    uint8_t *sa = sm + s * kStageBytes + sub * kSubBytes, *sb = sa + kABytes;
+                    if (!J.a_mn) {
+                        tma_load_3d(sa, ma, full, k0, m0, 0);
+                    } else if (J.a_blocked) {
+                        tma_load_3d(sa, ma, full, 0, k0, m0 / 64);
+                    } else {
+                        tma_load_3d(sa, ma, full, m0, k0, 0);
+                        tma_load_3d(sa + kMnBox, ma, full, m0 + 64, k0, 0);
+                    }
+                    if (!J.b_mn) {
+                        tma_load_3d(sb, mb, full, k0, n0, 0);
+                    } else if (J.b_blocked) {
+                        tma_load_3d(sb, mb, full, 0, k0, n0 / 64);
+                    } else {
+#pragma unroll
+                        for (int b = 0; b < kN / 64; ++b) tma_load_3d(sb + b * kMnBox, mb, full, n0 + 64 * b, k0, 0);
+                    }
+                }
+            }
+        }
+        mbar_drain(bars, armed);      // copies of this CTA still on their way land before it leaves (bounded)
+    } else if (warp == 1 && lane == 0) {
+        // ------------------------------------------------------------------- UMMA issuer
+        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kMnBox, 1024);
+        int it = 0, ti = 0, jx = 0;
+        bool ok = true;
+        for (int t = cta; ok && t < tiles; t += ncta, ++ti) {
+            int m0, n0;
+            job_of(t, jx, m0, n0);
+            const GroupJob &J = jobs.j[jx];
+            const uint64_t ap = J.a_mn ? mn_proto : km_proto, bp = J.b_mn ? mn_proto : km_proto;
+            const uint32_t a_hi = (uint32_t)(ap >> 32), b_hi = (uint32_t)(bp >> 32), a_lo0 = (uint32_t)ap, b_lo0 = (uint32_t)bp;
+            const uint32_t a_step = (J.a_mn ? 2048 : 32) >> 4, b_step = (J.b_mn ? 2048 : 32) >> 4, idesc = idesc_bf16_f32(GM, kN, J.a_mn, J.b_mn);
+            const int nk_total = stages_of(J) * J.nparts, buf = ti & 1;
+            if (!mbar_wait(bars + G_ACCEMPTY + buf, ((ti >> 1) & 1) ^ 1, abortp, status, GERR_ACCEMPTY)) break;
+            tc_fence_after();
+            const uint32_t acc = tbase + (uint32_t)(buf * kN);
+            for (int ks = 0; ks < nk_total; ++ks, ++it) {
+                const int s = it % kSt;
+                if (!mbar_wait(bars + G_FULL + s, (it / kSt) & 1, abortp, status, GERR_FULL)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t a_lo = a_lo0 + ((smem_u32(sm + s * kStageBytes) >> 4) & 0x3FFFu);
+                const uint32_t b_lo = b_lo0 + ((smem_u32(sm + s * kStageBytes + kABytes) >> 4) & 0x3FFFu);
+#pragma unroll
+                for (int sub = 0; sub < kSub; ++sub) {
+                    const uint32_t a_s = a_lo + (uint32_t)(sub * (kSubBytes >> 4)), b_s = b_lo + (uint32_t)(sub * (kSubBytes >> 4));
+                    if (ks == 0 && sub == 0) umma_ss2<false>(acc, a_s, a_hi, b_s, b_hi, idesc);
+                    else                     umma_ss2<true>(acc, a_s, a_hi, b_s, b_hi, idesc);
+#pragma unroll
+                    for (int q = 1; q < GK / 16; ++q) umma_ss2<true>(acc, a_s + q * a_step, a_hi, b_s + q * b_step, b_hi, idesc);
+                }
+                umma_commit(bars + G_EMPTY + s);
+            }
+            if (ok) umma_commit(bars + G_ACCFULL + buf);
+        }
+    } else if (warp >= 2 && warp < 2 + kEpiWarps) {
+        // ---------------------------------------------------------------------- epilogue (as in tc_gemm_kernel, EPI_STORE)
+        const int lane_row = 32 * (warp % 4) + lane, half = (warp - 2) / 4;
+        const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp % 4)) << 16);
+        const bool leader = tid == 64;
+        uint32_t epi_phase = 0, chunk_q = 0;
+        auto epi_sync = [&]() -> bool {
+            mbar_arrive(bars + G_EPI);
+            const bool r = mbar_wait(bars + G_EPI, epi_phase & 1, abortp, status, GERR_EPI);
+            ++epi_phase;
+            return r;
+        };
+        bool ok = true;
+        int ti = 0, jx = 0;
+        for (int t = cta; ok && t < tiles; t += ncta, ++ti) {
+            int m0, n0;
+            job_of(t, jx, m0, n0);
+            const GroupJob &J = jobs.j[jx];
+            const int buf = ti & 1, cols = min(kN, (J.N - n0 + 63) / 64 * 64);
+            if (!mbar_wait(bars + G_ACCFULL + buf, (ti >> 1) & 1, abortp, status, GERR_ACCFULL)) break;
+            tc_fence_after();
+            const uint32_t acc = lane_addr + (uint32_t)(buf * kN);
+#pragma unroll 1
+            for (int c0 = 0; ok && c0 < cols; c0 += 64, ++chunk_q) {
+                uint32_t r[32];
+                tmem_ld(acc + c0 + 32 * half, r);
+                tc_wait_ld();
+                if (c0 == cols - 64) {                    // last read of this accumulator: hand it back early
+                    tc_fence_before();
+                    mbar_arrive(bars + G_ACCEMPTY + buf);
+                }
+                uint8_t *out = sout + (chunk_q & 1) * kOutBox;
+                if (leader) bulk_wait_read<1>();          // the store issued two chunks ago has left this buffer
+                if (!epi_sync()) { ok = false; break; }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) w[e] = pack_bf16(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1]));
+                    *reinterpret_cast<uint4 *>(out + lane_row * 128 + (((half * 4 + j) ^ (lane_row & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+                fence_proxy_async_smem();
+                if (!epi_sync()) { ok = false; break; }
+                if (leader) {
+                    tma_store_3d(&J.C, out, n0 + c0, m0, 0);
+                    bulk_commit();
+                }
+            }
+        }
+        if (leader) bulk_wait_read<0>();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tbase, 2 * kN);
+}
+
 struct Operand {
     const void *p;
     int rows, cols;          // the array as stored: [rows, cols] row-major
@@ -640,7 +831,80 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
     return launch_gemm_as<kAMn, kBMn, kEpi, false, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
 }
 
+// One product of a group
+struct Product {
+    Operand A0, B0;
+    const Operand *A1, *B1;      // second operand pair (null: none)
+    void *C;                     // [M, N]
+    int M, N, K, a_mn, b_mn;
+    long long tiles(int n) const { return (long long)((M + GM - 1) / GM) * ((N + n - 1) / n); }
+};
+
+template <int kN>
+cudaError_t launch_group_n(const Product *p, int count, cudaStream_t st)
+{
+    GroupJobs g;
+    int tiles = 0;
+    for (int i = 0; i < count; ++i) {
+        GroupJob &j = g.j[i];
+        const Operand &a1 = p[i].A1 ? *p[i].A1 : p[i].A0, &b1 = p[i].B1 ? *p[i].B1 : p[i].B0;
+        j.M = p[i].M; j.N = p[i].N; j.K = p[i].K; j.nparts = p[i].A1 ? 2 : 1; j.a_mn = p[i].a_mn; j.b_mn = p[i].b_mn;
+        j.tile0 = tiles;
+        tiles += (int)p[i].tiles(kN);
+        auto maps = [](CUtensorMap *m, const Operand &o0, const Operand &o1, bool two, int mn, int rows, int &blocked) {
+            blocked = mn && o0.cols % 64 == 0 && o1.cols % 64 == 0;
+            for (int tries = 0; tries < 2; ++tries, blocked = 0) {
+                if (operand_map(m, o0, mn != 0, rows, blocked != 0) && (!two || operand_map(m + 1, o1, mn != 0, rows, blocked != 0))) return true;
+                if (!blocked) return false;
+            }
+            return false;
+        };
+        if (!maps(j.A, p[i].A0, a1, p[i].A1 != nullptr, j.a_mn, GM, j.a_blocked) || !maps(j.B, p[i].B0, b1, p[i].A1 != nullptr, j.b_mn, kN, j.b_blocked) ||
+            !make_tensor_map_3d(&j.C, p[i].C, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 1, (uint64_t)p[i].M, (uint64_t)p[i].N, 128, 64))
+            return cudaErrorInvalidValue;
+        if (!p[i].A1) { j.A[1] = j.A[0]; j.B[1] = j.B[0]; }
+    }
+    for (int i = count; i < kMaxJobs; ++i) g.j[i] = g.j[0];
+    g.count = count;
+    g.tiles = tiles;
+    constexpr int kSmem = gemm_smem(false, kN);
+    const cudaError_t e = allow_smem<tc_gemm_group_kernel<kN>>(kSmem);
+    if (e != cudaSuccess) return e;
+    const int sms = device_info().sms;
+    LaunchScope scope(MOA_KERNEL_OTHER, st);
+    return launch_dependent(tc_gemm_group_kernel<kN>, dim3((unsigned)(tiles < sms ? tiles : sms)), dim3(kGemmThreads), (size_t)kSmem, st, g,
+                            device_status_ptr());
+}
+
+// Whether `count` products go out as one launch: while their 128-column tiles fit on the SMs at once (then no wider tile and no pair
+// would have been faster for any of them), and MOA_GEMM_PAIR does not ask for pairs.
+bool group_fits(const Product *p, int count)
+{
+    long long t = 0;
+    for (int i = 0; i < count; ++i) t += p[i].tiles(128);
+    return gemm_pair_mode() != 2 && t <= device_info().sms;
+}
+cudaError_t launch_group(const Product *p, int count, cudaStream_t st)
+{
+    long long t = 0;
+    for (int i = 0; i < count; ++i) t += p[i].tiles(64);
+    return t <= device_info().sms ? launch_group_n<64>(p, count, st) : launch_group_n<128>(p, count, st);
+}
+
 }  // namespace
+
+// Two products of gemm_bf16 that do not depend on each other
+cudaError_t gemm_bf16_two(const GemmArgs &x, const GemmArgs &y, cudaStream_t st)
+{
+    auto product = [](const GemmArgs &g) {
+        return Product{Operand{g.A, g.a_mn ? g.K : g.M, g.a_mn ? g.M : g.K}, Operand{g.B, g.b_mn ? g.K : g.N, g.b_mn ? g.N : g.K}, nullptr, nullptr, g.C,
+                       g.M, g.N, g.K, g.a_mn, g.b_mn};
+    };
+    const Product two[2] = {product(x), product(y)};
+    if (group_fits(two, 2)) return launch_group(two, 2, st);
+    const cudaError_t e = gemm_bf16(x.a_mn, x.b_mn, x.M, x.N, x.K, x.A, x.B, nullptr, x.C, st);
+    return e != cudaSuccess ? e : gemm_bf16(y.a_mn, y.b_mn, y.M, y.N, y.K, y.A, y.B, nullptr, y.C, st);
+}
 
 // C[M,N] = A B^T (+ R): A given as [M,K] (a_mn = 0) or [K,M] (a_mn = 1), B as [N,K] (b_mn = 0) or [K,N] (b_mn = 1)
 cudaError_t gemm_bf16(int a_mn, int b_mn, int M, int N, int K, const void *A, const void *B, const void *R, void *C,
@@ -673,6 +937,10 @@ cudaError_t gated_mlp_bwd(int n, int d, int dff, const void *x, const void *W1, 
     // dh = dy W2 (W2 [d,d_ff] read as the MN-major B operand), gate backward in the epilogue -> da, du
     cudaError_t e = launch_gemm<false, true, EPI_SWIGLU_BWD>(DY, w2, nullptr, nullptr, da, du, a, u, n, dff, n, dff, d, st);
     if (e != cudaSuccess) return e;
+    // small: the four products that follow as one launch
+    const Product rest[4] = {{DY, Hh, nullptr, nullptr, dW2, d, dff, n, 1, 1}, {DA, X, nullptr, nullptr, dW1, dff, d, n, 1, 1},
+                             {DU, X, nullptr, nullptr, dW3, dff, d, n, 1, 1}, {DA, w1, &DU, &w3, dx, n, d, dff, 0, 1}};
+    if (group_fits(rest, 4)) return launch_group(rest, 4, st);
     // dW2 [d,d_ff] = dy^T h: both operands read transposed (K = tokens)
     if ((e = launch_gemm<true, true, EPI_STORE>(DY, Hh, nullptr, nullptr, dW2, nullptr, nullptr, nullptr, d, dff, d, dff, n, st)) !=
         cudaSuccess)

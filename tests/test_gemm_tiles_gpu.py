@@ -61,3 +61,29 @@ def test_gated_mlp_widths(rt, n, d, dff):
     for got, ref in ((a, ra), (u, ru), (h, rh), (y, f(h) @ f(W2).T), (dW2, f(dy).T @ f(h)), (dW1, da.T @ f(x)), (dW3, du.T @ f(x)),
                      (dx, da @ f(W1) + du @ f(W3))):
         assert (got.double() - ref).abs().max().item() <= 1e-2 * ref.abs().max().item()
+
+
+@pytest.mark.parametrize("B,n,H,d,dff", [(1, 40, 1, 64, 72), (2, 186, 4, 128, 1360), (1, 700, 8, 64, 1024), (1, 1613, 16, 64, 1000)])
+def test_block_products_side_by_side(rt, B, n, H, d, dff):
+    """The products a block's backward may launch together, against the block's three-projection form, which makes every call by itself:
+    same sums in the same order, so the same weight gradients up to the atomics in dQ."""
+    torch, mb = rt
+    from paper_2609_33916_b200.block import TransformerBlock
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    dm = H * d
+    R = lambda *s: torch.randn(s, generator=gen, device="cuda").bfloat16()      # noqa: E731
+    w = {k: R(dm, dm) * dm ** -0.5 for k in ("Wq", "Wk", "Wv", "Wo")}
+    w.update(W1=R(dff, dm) * dm ** -0.5, W3=R(dff, dm) * dm ** -0.5, W2=R(dm, dff) * dff ** -0.5, g1=1 + 0.25 * R(dm), g2=1 + 0.25 * R(dm))
+    x, dy = R(B * n, dm), R(B * n, dm)
+    out = []
+    for packed in (True, False):
+        blk = TransformerBlock(torch, B, n, H, d, dff, True, packed_qkv=packed)
+        wp = blk.prepare_weights(w)
+        blk.forward(x, wp)
+        dx, g = blk.backward(x, wp, dy)
+        assert mb.moa_last_device_status() == mb.MOA_OK
+        out.append({"y": blk.y.double(), "dx": dx.double(), **{k: v.double() for k, v in g.items()}})
+    for k in ("y", "W1", "W2", "W3", "g2", "Wo"):
+        assert torch.equal(out[0][k], out[1][k]), k
+    for k in ("dx", "Wq", "Wk", "Wv", "g1"):      # bf16 results of dQ sums in another order (and dh1 as one sum of three)
+        assert (out[0][k] - out[1][k]).abs().max().item() <= 1.6e-2 * out[1][k].abs().max().item(), k
