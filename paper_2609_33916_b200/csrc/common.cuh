@@ -289,8 +289,10 @@ cudaError_t tc_bwd_kv_pair(const Problem &p, const void *Q, const void *K, const
 bool bwd_pair_enabled();
 int bwd_pair_mode(int set);      // set < 0: query; returns the mode in force before the call
 
-// Head dimensions 136..256 (tc_bwd_wide.cu): tiles of 128 keys x 64 queries, two passes over the halves of d; dQ by
-// red.global into dQacc (fp32 [B,H,n,256], pre-zeroed)
+// Head dimensions 136..192 in one pass (tc_bwd_192.cu) and 200..256 in two passes over the halves of d (tc_bwd_wide.cu): tiles of 128
+// keys x 64 queries; dQ by red.global into dQacc (fp32 [B,H,n,256], pre-zeroed)
+cudaError_t tc_bwd_kv_192(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
+                          const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st);
 cudaError_t tc_bwd_kv_wide(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
                            const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st);
 

@@ -1,4 +1,4 @@
-// Backward attention for head dimensions 136..256 on the sm_100a tensor cores, bf16 in, fp32 accumulate.
+// Backward attention for head dimensions 200..256 on the sm_100a tensor cores, bf16 in, fp32 accumulate.
 //
 // Same mathematics, the same key-tile-parallel structure and the same one-writer rule for dK and dV as tc_bwd.cu
 // (the paper's (b,ic)-parallel GV pass, applied to GK as well).  What changes is the tiling, because neither TMEM
@@ -14,13 +14,11 @@
 // Shared memory: K 64 KB + V 64 KB + Q 48 KB + dO 32 KB + dS^T 16 KB = 224 KB; dQ leaves as red.global.add.f32 from
 // registers (one warp-wide instruction = 32 consecutive floats of one dQ row), there is no room for a staging tile.
 // Per query tile i: dP(i), dV(i), S(i+1), dK(i), dQ(i), issued by one thread; roles as in tc_bwd.cu.
-// Head dimensions below 256 (192, ...) run with the missing columns zero-filled by the loads and dropped by the stores; up to
-// 192 (NB = 3 boxes of 64 columns) the fourth box is neither loaded nor multiplied: 12 UMMAs instead of 16 for S^T and for dP^T,
-// and the second pass accumulates 64 columns of dV and dK.
+// Head dimensions below 256 run with the missing columns zero-filled by the loads and dropped by the stores; up to 192 they
+// fit one pass (tc_bwd_192.cu).
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tensormap.cuh"
-#include <type_traits>
 
 namespace moa {
 namespace {
@@ -65,7 +63,7 @@ __device__ __forceinline__ void red_add_f32(float *addr, float a)
     asm volatile("red.global.add.f32 [%0], %1;" ::"l"(addr), "f"(a) : "memory");
 }
 
-template <bool kGrouped, bool kSplit, int NB>
+template <bool kGrouped, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                    const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapdO,
@@ -137,7 +135,6 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 tma_load_4d(sV + b * SM::kBoxK, &mapV, bars + W_KV, 64 * b, k0, hk, bb);
             }
         }
-        const int own = pass == 0 ? 2 : NB - 2;     // 64-column boxes of this pass's d-half
         const int nq_per = nqt - i_begin;
         auto tile_of = [&](int it, int &qh, int &q0) {
             const int at = it0 + it, hh = kGrouped ? at / nq_per : 0;
@@ -149,22 +146,22 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             tile_of(it, qh, q0);
             const int s = it & 1;
             uint8_t *dst = sQ + (1 + s) * SM::kHalf;
-            mbar_arrive_expect_tx(bars + W_QOWN + s, own * SM::kBoxQ + 512);
-            for (int b = 0; b < own; ++b) tma_load_4d(dst + b * SM::kBoxQ, &mapQ, bars + W_QOWN + s, 128 * pass + 64 * b, q0, qh + hq0, bb);
+            mbar_arrive_expect_tx(bars + W_QOWN + s, SM::kHalf + 512);
+            for (int b = 0; b < 2; ++b) tma_load_4d(dst + b * SM::kBoxQ, &mapQ, bars + W_QOWN + s, 128 * pass + 64 * b, q0, qh + hq0, bb);
             bulk_load_1d(sL + s * 64, Lp + (size_t)qh * n_pad + q0, 256, bars + W_QOWN + s);
             bulk_load_1d(sD + s * 64, Dp + (size_t)qh * n_pad + q0, 256, bars + W_QOWN + s);
         };
         auto load_qoth = [&](int it) {        // the other d-half of Q_it (read by S(it) only)
             int qh, q0;
             tile_of(it, qh, q0);
-            mbar_arrive_expect_tx(bars + W_QOTH, (NB - own) * SM::kBoxQ);
-            for (int b = 0; b < NB - own; ++b) tma_load_4d(sQ + b * SM::kBoxQ, &mapQ, bars + W_QOTH, 128 * (1 - pass) + 64 * b, q0, qh + hq0, bb);
+            mbar_arrive_expect_tx(bars + W_QOTH, SM::kHalf);
+            for (int b = 0; b < 2; ++b) tma_load_4d(sQ + b * SM::kBoxQ, &mapQ, bars + W_QOTH, 128 * (1 - pass) + 64 * b, q0, qh + hq0, bb);
         };
         auto load_do = [&](int it) {          // dO_it, all 256 columns
             int qh, q0;
             tile_of(it, qh, q0);
-            mbar_arrive_expect_tx(bars + W_DOFULL, NB * SM::kBoxQ);
-            for (int b = 0; b < NB; ++b) tma_load_4d(sdO + b * SM::kBoxQ, &mapdO, bars + W_DOFULL, 64 * b, q0, qh + hq0, bb);
+            mbar_arrive_expect_tx(bars + W_DOFULL, 4 * SM::kBoxQ);
+            for (int b = 0; b < 4; ++b) tma_load_4d(sdO + b * SM::kBoxQ, &mapdO, bars + W_DOFULL, 64 * b, q0, qh + hq0, bb);
         };
         // (K, V, Q and dO are the call's inputs; -L, -D and the cleared accumulator come from the kernel in front)
         if (lane == 0 && niter > 0) {
@@ -196,8 +193,7 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
       } else if (warp == kMmaWarp && lane == 0) {
         // ------------------------------------------------------------------- UMMA issuer (one thread)
         constexpr uint32_t idesc_st = idesc_bf16_f32(128, 64, 0, 0);     // S^T, dP^T: 128 keys x 64 queries
-        // dV, dK: A in TMEM, B MN-major, the columns of d of this pass
-        const uint32_t idesc_acc = NB == 3 && pass == 1 ? idesc_bf16_f32(128, 64, 0, 1) : idesc_bf16_f32(128, 128, 0, 1);
+        constexpr uint32_t idesc_acc = idesc_bf16_f32(128, 128, 0, 1);   // dV, dK: A in TMEM, B MN-major, 128 columns of d
         constexpr uint32_t idesc_dq = idesc_bf16_f32(128, 64, 1, 1);     // dQ^T: 128 columns of d x 64 queries
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024);
         const uint64_t mnq_proto = smem_desc_sw128(0, SM::kBoxQ, 1024);  // MN-major over boxes of 64 rows (Q, dO, dS^T)
@@ -217,7 +213,7 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         auto issue_S = [&](int it) {
             const uint32_t qown_km = qown_km0 + (uint32_t)(it & 1) * kHalfF;
 #pragma unroll
-            for (int bx = 0; bx < NB; ++bx) {
+            for (int bx = 0; bx < 4; ++bx) {
                 const uint32_t a = k_km + (uint32_t)((bx * SM::kBoxK) >> 4);
                 const uint32_t b = ((bx >> 1) == pass ? qown_km : qoth_km) + (uint32_t)(((bx & 1) * SM::kBoxQ) >> 4);
 #pragma unroll
@@ -239,7 +235,7 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             if (!mbar_wait(bars + W_DOFULL, it & 1, abortp, status, WERR_FULL)) break;
             tc_fence_after();
 #pragma unroll
-            for (int bx = 0; bx < NB; ++bx) {      // dP^T(it) = V dO_it^T over the whole head dimension
+            for (int bx = 0; bx < 4; ++bx) {       // dP^T(it) = V dO_it^T over all 256 columns
                 const uint32_t a = v_km + (uint32_t)((bx * SM::kBoxK) >> 4), b = do_km + (uint32_t)((bx * SM::kBoxQ) >> 4);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -500,7 +496,7 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     }
 }
 
-template <bool kGrouped, bool kSplit, int NB>
+template <bool kGrouped, bool kSplit>
 cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const void *V, const void *dO, const float *Lp,
                         const float *Dp, void *dK, void *dV, float *dQacc, int split, cudaStream_t st)
 {
@@ -516,7 +512,7 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
         !make_tensor_map_4d_strided(&mdv, dV, bf, 2, p.B, hkv, p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64))
         return cudaErrorInvalidValue;
     constexpr int kSmem = WideSmem::kTotal;
-    cudaError_t e = allow_smem<tc_bwd_wide_kernel<kGrouped, kSplit, NB>>(kSmem);
+    cudaError_t e = allow_smem<tc_bwd_wide_kernel<kGrouped, kSplit>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nkt = (p.n + 127) / 128;
     LaunchScope scope(MOA_KERNEL_BWD_KV, st);
@@ -524,7 +520,7 @@ cudaError_t launch_wide(const Problem &p, const void *Q, const void *K, const vo
     pkv.H = hkv;
     pkv.Hkv = 0;
     // two CTAs (the two halves of d) per (K/V head, key tile), adjacent in the grid: they share every load in L2
-    return launch_cluster(tc_bwd_wide_kernel<kGrouped, kSplit, NB>, (unsigned)split, dim3((unsigned)(2 * nkt * p.BHkv() * split)), dim3(kThreads),
+    return launch_cluster(tc_bwd_wide_kernel<kGrouped, kSplit>, (unsigned)split, dim3((unsigned)(2 * nkt * p.BHkv() * split)), dim3(kThreads),
                           (size_t)kSmem, st,
         mq, mk, mv, mdo, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.d, p.causal, p.scale, p.scale * kLog2e, nkt,
         heads_per_group(pkv, nkt), p.group(), hkv, device_status_ptr(), split, (__nv_bfloat16 *)dK, (__nv_bfloat16 *)dV, p.skv);
@@ -538,15 +534,11 @@ cudaError_t tc_bwd_kv_wide(const Problem &p, const void *Q, const void *K, const
     if (p.d <= 128 || p.d > 256 || p.d % 8 || dQacc == nullptr) return cudaErrorInvalidValue;
     const long long nkt = (p.n + 127) / 128, jobs = 2 * nkt * p.BHkv(), longest = 2 * nkt * p.group();     // query tiles of 64
     const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) : jobs * longest, p.causal, 2.5, 1.5);
-    auto run = [&](auto nb) {
-        constexpr int NB = decltype(nb)::value;
-        if (split > 1)
-            return p.group() > 1 ? launch_wide<true, true, NB>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
-                                 : launch_wide<false, true, NB>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
-        return p.group() > 1 ? launch_wide<true, false, NB>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st)
-                             : launch_wide<false, false, NB>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st);
-    };
-    return p.d <= 192 ? run(std::integral_constant<int, 3>()) : run(std::integral_constant<int, 4>());
+    if (split > 1)
+        return p.group() > 1 ? launch_wide<true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
+                             : launch_wide<false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
+    return p.group() > 1 ? launch_wide<true, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st)
+                         : launch_wide<false, false>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, 1, st);
 }
 
 }  // namespace moa

@@ -45,3 +45,19 @@ def test_shared_key_tiles(H, B, Hq, Hkv, n, d, causal, op, layout):
     f = H.f64_inputs(inp, "bf16")
     ref = oracle.attn_fwd_bwd_gqa(f["Q"], f["K"], f["V"], f["dO"], causal, scale)
     H.assert_close(got, ref, H.TOL_BF16, tag=f"H{Hq}/{Hkv} n{n} d{d}")
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,causal", [(2, 40, 40, 64, 136, False), (2, 40, 40, 65, 192, True), (3, 60, 60, 200, 160, True),
+                                                 (2, 80, 40, 129, 192, False), (1, 160, 160, 128, 184, True), (1, 8, 1, 700, 192, False),
+                                                 (1, 3, 3, 1000, 144, True)])
+@pytest.mark.parametrize("op,dq_mode,layout", [("fused", 0, 0), ("split", 1, 1)])
+def test_one_pass_backward_up_to_192(H, B, Hq, Hkv, n, d, causal, op, dq_mode, layout):
+    """136..192 columns: one and several CTAs per key tile, one and many query tiles, every number of columns in the last box."""
+    q = mi.make_inputs(B, Hq, n, d, 800 + n, "bf16")
+    kv = mi.make_inputs(B, Hkv, n, d, 1800 + n, "bf16")
+    inp = {"Q": q["Q"], "dO": q["dO"], "K": kv["K"], "V": kv["V"]}
+    scale = 1.0 / math.sqrt(d)
+    got = H.run_library(inp, "bf16", causal, scale, op=op, layout=layout, dq_mode=dq_mode)
+    f = H.f64_inputs(inp, "bf16")
+    ref = oracle.attn_fwd_bwd_gqa(f["Q"], f["K"], f["V"], f["dO"], causal, scale)
+    H.assert_close(got, ref, H.TOL_BF16, tag=f"H{Hq}/{Hkv} n{n} d{d}")
