@@ -44,9 +44,8 @@
  *  - Supported: d in {64, 128} everywhere; on the bf16 tensor-core kernels also every
  *    other multiple of 8 up to 256 (d = 96, 80, 32, 192, ...: the head runs in the 64-,
  *    128- or 256-column kernel, TMA zero-fills the missing columns on load and drops
- *    them on store; not with materialize = 1).  Above 128 the forward accumulates the
- *    scores over two 128-column chunks and the backward works on 128 x 64 tiles in two
- *    passes over the halves of d; there dq_mode is MOA_DQ_AUTO or MOA_DQ_RED
+ *    them on store; not with materialize = 1).  Above 128 the backward works on 128 x 64
+ *    tiles, above 192 in two passes over the halves of d; there (d > 128) dq_mode is MOA_DQ_AUTO or MOA_DQ_RED
  *    (BULK_REDUCE and SEPARATE_PASS give MOA_ERR_UNSUPPORTED).  Any n >= 1 and B, H >= 1 (B*H <= 2^20 and
  *    ceil(n/64)*B*H < 2^31, else MOA_ERR_UNSUPPORTED); n need not be a multiple
  *    of the tile size.

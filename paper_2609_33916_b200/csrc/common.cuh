@@ -52,7 +52,7 @@ struct Problem {
 // Head dimension the tensor-core kernels are compiled for: a head of d columns (a multiple of 8, so
 // that rows stay 16-byte aligned) runs in the 64-, 128- or 256-column kernels; the TMA loads fill the
 // columns past d with zeros and the TMA stores drop them, which leaves every result unchanged.
-// 256: the two-pass kernels for head dimensions 136..256 (tc_fwd.cu with KC = 2, tc_bwd_wide.cu).
+// 256: the kernels for head dimensions 136..256 (tc_fwd_wide.cu, tc_bwd_192.cu, tc_bwd_wide.cu).
 inline int kernel_d(int d) { return d <= 64 ? 64 : d <= 128 ? 128 : 256; }
 
 // Block order of the tile-parallel kernels.  Heads are taken in groups of `hpg`; inside a group
@@ -267,6 +267,9 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
 // The same on pairs of query tiles (tc_fwd2.cu; d <= 128), and whether that is the faster form of a problem
 cudaError_t tc_fwd_pairs(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const FwdForBwd &fb, cudaStream_t st);
 bool fwd_pairs_pay(const Problem &p);
+
+// Head dimensions 136..256 (tc_fwd_wide.cu)
+cudaError_t tc_fwd_wide(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const FwdForBwd &fb, cudaStream_t st);
 
 // Lp = -L*log2(e) and Dp = -rowsum(dO o O) (negated: fma/add operands), each padded per head to a
 // multiple of 128 rows (-inf / 0 past n)

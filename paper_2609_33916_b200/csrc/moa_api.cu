@@ -446,8 +446,7 @@ moa_status moa_attn_fused_fwd_bwd(const moa_attn_desc *desc, const void *Q, cons
     // tensor-core path with an atomic dQ mode: the forward clears the accumulator its backward adds into
     // and writes the backward's per-row inputs (-L log2e, -D) from the fp32 O it holds
     FwdForBwd fb;
-    // (head dimensions above 128: a forward CTA holds half of an O row, so the backward prepares its own inputs)
-    const bool both_tc = use_tc_fwd(desc) && use_tc_bwd(desc) && kernel_d(desc->d) <= 128;
+    const bool both_tc = use_tc_fwd(desc) && use_tc_bwd(desc);
     if (both_tc) {
         const BwdWorkspace w = bwd_workspace(desc);
         fb.Dp = (float *)ws;
