@@ -364,18 +364,43 @@ __device__ __forceinline__ void tma_load_4d_pair(void *dst, const CUtensorMap *m
         ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar_cluster_addr), "r"(x), "r"(y), "r"(z), "r"(w)
         : "memory");
 }
-// v = mul * (sum over the CTAs of the cluster, in rank order, of the 8 floats at the shared-memory addresses a, b)
-__device__ __forceinline__ void sum_split(uint32_t a, uint32_t b, int split, float mul, float (&v)[8])
+// What CTA `rank` of the cluster has at the shared-memory address `a` of this CTA, or `other` where there is no such rank.  Predicated,
+// not branched around, so that an unrolled loop over the ranks has all its loads in flight: a remote load takes several hundred
+// cycles.
+constexpr int kMaxRanks = 8;      // of the clusters whose CTAs merge partial results
+__device__ __forceinline__ float peer_f1(uint32_t a, int rank, int ranks, float other)
+{
+    float v;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "setp.lt.s32 p, %2, %3;\n\tmov.f32 %0, %4;\n\t"
+        "@p mapa.shared::cluster.u32 t, %1, %2;\n\t@p ld.shared::cluster.f32 %0, [t];\n\t}"
+        : "=&f"(v) : "r"(a), "r"(rank), "r"(ranks), "f"(other) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 peer_f4(uint32_t a, int rank, int ranks)      // (zeros where there is no such rank)
+{
+    float4 v;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "setp.lt.s32 p, %5, %6;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\tmov.f32 %2, 0f00000000;\n\tmov.f32 %3, 0f00000000;\n\t"
+        "@p mapa.shared::cluster.u32 t, %4, %5;\n\t@p ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [t];\n\t}"
+        : "=&f"(v.x), "=&f"(v.y), "=&f"(v.z), "=&f"(v.w) : "r"(a), "r"(rank), "r"(ranks) : "memory");
+    return v;
+}
+// v = mul * (sum over the `split` CTAs of the cluster, a power of two of at least 2, of the 8 floats at the shared-memory addresses a, b).
+// Rank r begins with its own and goes round from there: with all of them reading rank 0, then rank 1, ... one SM at a time
+// served the whole cluster.
+__device__ __forceinline__ void sum_split(uint32_t a, uint32_t b, int rank, int split, float mul, float (&v)[8])
 {
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = 0.f;
-    for (int k = 0; k < split; ++k) {
-        float x[8];
-        const uint32_t ra = mapa_u32(a, (uint32_t)k), rb = mapa_u32(b, (uint32_t)k);
-        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(ra) : "memory");
-        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]) : "r"(rb) : "memory");
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] += x[e];
+#pragma unroll 1
+    for (int k = rank; k < rank + split; k += 2) {
+        const int k0 = k & (split - 1), k1 = (k + 1) & (split - 1);
+        const float4 x0 = peer_f4(a, k0, split), y0 = peer_f4(b, k0, split), x1 = peer_f4(a, k1, split), y1 = peer_f4(b, k1, split);
+        v[0] += x0.x + x1.x; v[1] += x0.y + x1.y; v[2] += x0.z + x1.z; v[3] += x0.w + x1.w;
+        v[4] += y0.x + y1.x; v[5] += y0.y + y1.y; v[6] += y0.z + y1.z; v[7] += y0.w + y1.w;
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] *= mul;

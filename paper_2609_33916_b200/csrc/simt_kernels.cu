@@ -211,25 +211,6 @@ __device__ __forceinline__ void cluster_barrier()
 {
     asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 }
-// address of `p` (this CTA's shared memory) in the CTA of rank r, and loads from there
-__device__ __forceinline__ uint32_t remote(const void *p, uint32_t r)
-{
-    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), d;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(r));
-    return d;
-}
-__device__ __forceinline__ float4 remote_f4(uint32_t a)
-{
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-    return v;
-}
-__device__ __forceinline__ float remote_f1(uint32_t a)
-{
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-    return v;
-}
 
 // ------------------------------------------------------------------------- forward
 // CTA: BM = 8 R query rows; a warp has 2 R rows to itself, a thread R rows x 4 keys of the score tile and R rows x D / 16
@@ -375,15 +356,24 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     const int per = BM / split;        // rows this rank finishes
     for (int r = tid / LPR; r < per; r += SNT / LPR) {
         const int rr = rank * per + r, row = q0 + rr, c = (tid % LPR) * 4;
-        float mt = -INFINITY;
-        for (int k = 0; k < split; ++k) mt = fmaxf(mt, remote_f1(remote(Mm + rr, k)));
+        float mt = -INFINITY, mk[ptx::kMaxRanks], lk[ptx::kMaxRanks];
+        float4 vk[ptx::kMaxRanks];
+#pragma unroll
+        for (int k = 0; k < ptx::kMaxRanks; ++k) {
+            mk[k] = ptx::peer_f1(ptx::smem_u32(Mm + rr), k, split, -INFINITY);
+            lk[k] = ptx::peer_f1(ptx::smem_u32(Lm + rr), k, split, 0.f);
+            vk[k] = ptx::peer_f4(ptx::smem_u32(Om + rr * LD + c), k, split);
+        }
+#pragma unroll
+        for (int k = 0; k < ptx::kMaxRanks; ++k) mt = fmaxf(mt, mk[k]);
         const float ref = mt == -INFINITY ? 0.f : mt;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         float lt = 0.f;
-        for (int k = 0; k < split; ++k) {
-            const float w = expf(remote_f1(remote(Mm + rr, k)) - ref);
-            const float4 v = remote_f4(remote(Om + rr * LD + c, k));
-            lt = fmaf(remote_f1(remote(Lm + rr, k)), w, lt);
+#pragma unroll
+        for (int k = 0; k < ptx::kMaxRanks; ++k) {      // (a rank that does not exist has weight 0)
+            const float w = expf(mk[k] - ref);
+            const float4 v = vk[k];
+            lt = fmaf(lk[k], w, lt);
             a.x = fmaf(v.x, w, a.x); a.y = fmaf(v.y, w, a.y); a.z = fmaf(v.z, w, a.z); a.w = fmaf(v.w, w, a.w);
         }
         const bool live = row < n;
@@ -670,10 +660,17 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
         const int rr = rank * per + r, row = k0 + rr, c = (tid % LPR) * 4;
         if (row >= n) continue;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), g = a;
-        for (int k = 0; k < split; ++k) {
-            const float4 x = remote_f4(remote(Qs + rr * LD + c, k)), y = remote_f4(remote(dOs + rr * LD + c, k));
-            a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
-            g.x += y.x; g.y += y.y; g.z += y.z; g.w += y.w;
+        const uint32_t at_k = ptx::smem_u32(Qs + rr * LD + c), at_v = ptx::smem_u32(dOs + rr * LD + c);
+#pragma unroll 1
+        for (int k0 = 0; k0 < split; k0 += 4) {
+            float4 x[4], y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) { x[u] = ptx::peer_f4(at_k, k0 + u, split); y[u] = ptx::peer_f4(at_v, k0 + u, split); }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a.x += x[u].x; a.y += x[u].y; a.z += x[u].z; a.w += x[u].w;
+                g.x += y[u].x; g.y += y[u].y; g.z += y[u].z; g.w += y[u].w;
+            }
         }
         if (dK) store4(dK + (size_t)row * D + c, a);
         store4(dV + (size_t)row * D + c, g);

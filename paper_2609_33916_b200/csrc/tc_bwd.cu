@@ -724,16 +724,16 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
     if (kSplit) {
-        // the ranks add up the partial results, in rank order, 128 / split rows each, and write them out
+        // the ranks add up the partial results, 128 / split rows each, and write them out
         __syncwarp();
         cluster_sync_all();
-        if (warp < kReduceWarp0) {
+        if (warp < kLoadWarp) {
             const int per = 128 / split;
-            for (int i = tid; i < 2 * per * (D / 8); i += 32 * kReduceWarp0) {
+            for (int i = tid; i < 2 * per * (D / 8); i += 32 * kLoadWarp) {
                 const int c8 = i % (D / 8), r = rank * per + (i / (D / 8)) % per, which = i / (D / 8) / per;
                 const uint32_t row = smem_u32(sm) + which * (128 * D * 4) + r * (D * 4);
                 float v[8];
-                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), split, which == 0 ? 1.f : scale, v);
+                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), rank, split, which == 0 ? 1.f : scale, v);
                 if (k0 + r < n && 8 * c8 < out.d)
                     *reinterpret_cast<uint4 *>((which == 0 ? out.dV : out.dK) + out.skv.at(bb, hk, k0 + r) + 8 * c8) =
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
@@ -792,7 +792,8 @@ cudaError_t launch_bwd(const Problem &p, const void *Q, const void *K, const voi
 {
     if constexpr (kBulk) {        // (AUTO is the bulk reduce at these head dimensions)
         const long long nkt = (p.n + 127) / 128, jobs = nkt * p.BHkv(), longest = nkt * p.group();
-        const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) / 2 : jobs * longest, p.causal, 2.0, 1.0);
+        const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) / 2 : jobs * longest, p.causal, 2.0, 2.5);
+        // (both sides, d = 128: 8 tiles per job 30.8 us alone, 28.1 in pairs; 4 tiles 21.3 alone, 22.7 in pairs; 3 tiles 17.3, 20.3)
         if (split > 1)
             return p.group() > 1 ? launch_bwd_g<D, kBulk, true, true, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
                                  : launch_bwd_g<D, kBulk, false, true, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);

@@ -1,7 +1,7 @@
 // Backward attention for head dimensions 136..192 on the sm_100a tensor cores, bf16 in, fp32 accumulate: the whole head dimension in
 // ONE pass.  (tc_bwd_wide.cu, which runs 200..256, computes the scores and dP in each of two passes over the halves of d; run on 192
 // columns, 40 UMMAs per pass and 64-query tile against 56 here for both, and its loop is bound by the chain of hand-offs, which
-// is paid once here: B1 H16 H_kv4 n3001 causal backward 360 -> XX us.)
+// is paid once here: B1 H16 H_kv4 n3001 causal backward 385 -> 279 us, B1 H8 n8192 2108 -> 1420 us.)
 //
 // Same mathematics, the same key-tile-parallel structure and the same one-writer rule for dK and dV as tc_bwd.cu.  CTA = 128 keys of one
 // K/V head (or, kSplit, its part of their query tiles); query tiles of 64 rows.
@@ -69,7 +69,7 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                    const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapdO,
                    const __grid_constant__ CUtensorMap mapdK, const __grid_constant__ CUtensorMap mapdV,
                    const float *__restrict__ Lp, const float *__restrict__ Dp, float *__restrict__ dQacc,
-                   int n, int n_pad, int d, int causal, float scale, float scale_log2, int nkt, int hpg, int group,
+                   int n, int n_pad, int d, int causal, float scale, float scale_log2, int nkt, int nqt /*tiles of 64 rows*/, int hpg, int group,
                    int Hkv, unsigned int *status, int split, __nv_bfloat16 *__restrict__ dK, __nv_bfloat16 *__restrict__ dV,
                    Strides skv)
 {
@@ -89,7 +89,6 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     int bh, kt;                                           // causal: key tile 0 has the most query tiles and goes first
     job_from_block(blk, nkt, (int)gridDim.x / (kSplit ? split : 1) / nkt, hpg, bh, kt);
     const int k0 = kt * 128;
-    const int nqt = n_pad / BQ;                           // query tiles of 64 rows
     const int i_begin = causal ? 2 * kt : 0;
     const int bb = bh / Hkv, hk = bh - bb * Hkv;
     const int hq0 = hk * (kGrouped ? group : 1) - bh * (kGrouped ? group : 1);   // query head in batch = flat index + hq0
@@ -439,16 +438,16 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
     if (kSplit) {
-        // the ranks add up the partial results, in rank order, 128 / split rows each, and write them out
+        // the ranks add up the partial results, 128 / split rows each, and write them out
         __syncwarp();
         cluster_sync_all();
-        if (warp < kReduceWarp0) {
+        if (warp < kLoadWarp) {
             const int per = 128 / split;
-            for (int i = tid; i < 2 * per * 8 * NB; i += 32 * kReduceWarp0) {
+            for (int i = tid; i < 2 * per * 8 * NB; i += 32 * kLoadWarp) {
                 const int c8 = i % (8 * NB), r = rank * per + (i / (8 * NB)) % per, which = i / (8 * NB) / per;
                 const uint32_t row = smem_u32(sm) + which * SM::kPart + r * (64 * NB * 4);
                 float v[8];
-                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), split, which == 0 ? 1.f : scale, v);
+                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), rank, split, which == 0 ? 1.f : scale, v);
                 if (k0 + r < n && 8 * c8 < d)
                     *reinterpret_cast<uint4 *>((which == 0 ? dV : dK) + skv.at(bb, hk, k0 + r) + 8 * c8) =
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
@@ -490,7 +489,7 @@ cudaError_t launch_192(const Problem &p, const void *Q, const void *K, const voi
     pkv.Hkv = 0;
     return launch_cluster(tc_bwd192_kernel<kGrouped, kSplit>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)), dim3(kThreads),
                           (size_t)kSmem, st,
-        mq, mk, mv, mdo, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.d, p.causal, p.scale, p.scale * kLog2e, nkt,
+        mq, mk, mv, mdo, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.d, p.causal, p.scale, p.scale * kLog2e, nkt, (p.n + BQ - 1) / BQ,
         heads_per_group(pkv, nkt), p.group(), hkv, device_status_ptr(), split, (__nv_bfloat16 *)dK, (__nv_bfloat16 *)dV, p.skv);
 }
 
@@ -500,8 +499,10 @@ cudaError_t tc_bwd_kv_192(const Problem &p, const void *Q, const void *K, const 
                           const float *Lp, const float *Dp, void *dK, void *dV, float *dQacc, bool share, cudaStream_t st)
 {
     if (p.d <= 128 || p.d > 192 || p.d % 8 || dQacc == nullptr) return cudaErrorInvalidValue;
-    const long long nkt = (p.n + 127) / 128, jobs = nkt * p.BHkv(), longest = 2 * nkt * p.group();     // query tiles of 64
-    const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) : jobs * longest, p.causal, 2.5, 1.5);
+    const long long nkt = (p.n + 127) / 128, nqt = (p.n + BQ - 1) / BQ, jobs = nkt * p.BHkv(), longest = nqt * p.group();     // query tiles of 64
+    const long long total = p.causal ? (nkt * nqt - nkt * (nkt - 1)) * p.BHkv() * p.group() : jobs * longest;
+    const int split = !share ? 1 : bwd_split(jobs, longest, total, p.causal, 2.5, 3.0);
+    // (both sides: 16 tiles per job 54.7 us alone, 43.1 in pairs; 8 tiles 34.2 and 31.4; 5 tiles 26.2 and 28.2)
     if (split > 1)
         return p.group() > 1 ? launch_192<true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
                              : launch_192<false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);

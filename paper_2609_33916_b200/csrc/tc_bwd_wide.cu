@@ -470,16 +470,16 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     __syncthreads();
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
     if (kSplit) {
-        // the ranks add up the partial results, in rank order, 128 / split rows each, and write them out
+        // the ranks add up the partial results, 128 / split rows each, and write them out
         __syncwarp();
         cluster_sync_all();
-        if (warp < kReduceWarp0) {
+        if (warp < kLoadWarp) {
             const int per = 128 / split;
-            for (int i = tid; i < 2 * per * 16; i += 32 * kReduceWarp0) {
+            for (int i = tid; i < 2 * per * 16; i += 32 * kLoadWarp) {
                 const int c8 = i % 16, r = rank * per + (i / 16) % per, which = i / 16 / per, col = 128 * pass + 8 * c8;
                 const uint32_t row = smem_u32(sm) + which * 65536 + r * 512;
                 float v[8];
-                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), split, which == 0 ? 1.f : scale, v);
+                sum_split(row + (((2 * c8) ^ (r & 7)) << 4), row + (((2 * c8 + 1) ^ (r & 7)) << 4), rank, split, which == 0 ? 1.f : scale, v);
                 if (k0 + r < n && col < d)
                     *reinterpret_cast<uint4 *>((which == 0 ? dV : dK) + skv.at(bb, hk, k0 + r) + col) =
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
@@ -533,7 +533,8 @@ cudaError_t tc_bwd_kv_wide(const Problem &p, const void *Q, const void *K, const
 {
     if (p.d <= 128 || p.d > 256 || p.d % 8 || dQacc == nullptr) return cudaErrorInvalidValue;
     const long long nkt = (p.n + 127) / 128, jobs = 2 * nkt * p.BHkv(), longest = 2 * nkt * p.group();     // query tiles of 64
-    const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) : jobs * longest, p.causal, 2.5, 1.5);
+    const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) : jobs * longest, p.causal, 2.5, 3.0);
+    // (both sides, d = 256: 64 tiles per job 176 us alone, 100 in pairs, 64 in fours; 7 tiles 27.1 alone, 25.5 in pairs)
     if (split > 1)
         return p.group() > 1 ? launch_wide<true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
                              : launch_wide<false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);
