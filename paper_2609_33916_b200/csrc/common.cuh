@@ -109,7 +109,8 @@ inline int bwd_split(long long jobs, long long longest, long long total, bool ca
     double best_cost = 0;
     for (int s = 1; s <= 8; s *= 2) {
         if (s > 1 && (longest < s || jobs * s > 8 * (long long)sms)) break;
-        const double slots = s <= 2 ? sms : s == 4 ? 0.9 * sms : 0.85 * sms;     // (clusters of 4 and 8 leave SMs of a GPC over)
+        // (clusters of 4 and 8 leave SMs of a GPC over; less so where an SM holds several CTAs)
+        const double slots = s <= 2 ? sms : s == 4 ? (per_sm > 1 ? 1.0 : 0.9) * sms : (per_sm > 1 ? 0.89 : 0.85) * sms;
         const double extra = fixed + (s > 1 ? merge : 0.0), job = (double)longest / s + extra;
         const double avg = ((double)total + (double)jobs * s * extra) / slots, mean = (double)total / (jobs * s) + extra;
         const long long n = jobs * s, rounds = (n + (long long)slots - 1) / (long long)slots;

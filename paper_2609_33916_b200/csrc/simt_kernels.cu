@@ -58,6 +58,7 @@ __device__ __forceinline__ float group16_sum(float v)
 //     of the other axis in turn, and their partial results are added through distributed shared memory, in rank order.
 constexpr int SNT = 128;         // threads per CTA: lane tx = tid % 16 along columns, ty = tid / 16 along rows
 constexpr int STY = SNT / 16;
+constexpr float kLazyMax = 5.f;  // (e^5: far from where fp32 sums of such terms would lose anything)
 
 __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool live)
 {
@@ -277,11 +278,14 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         if (more) tile_in<T, BN, D>(Ks, K, k0 + step, n);      // runs under the softmax and the P V product
         cp_commit();
         const bool mask = k0 + BN > n || (causal && k0 + BN - 1 > q0);
-        uint64_t al[R / 2];
+        // A row's reference is raised only when a score exceeds it by more than kLazyMax, so that most tiles pass without the
+        // exchange of maxima between lanes and the rescaling of O; row sums stay per lane until the end.
+        float mx[R];
+        bool grow = false;
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             const int row = q0 + ty * R + i;
-            float mx = -INFINITY;
+            mx[i] = -INFINITY;
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 float v = s[i][b] * scale;
@@ -290,26 +294,36 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
                     if (col >= n || (causal && col > row)) v = -INFINITY;
                 }
                 s[i][b] = v;
-                mx = fmaxf(mx, v);
+                mx[i] = fmaxf(mx[i], v);
             }
-            mx = group16_max(mx);
-            const float mn = fmaxf(m[i], mx);
-            const float ref = mn == -INFINITY ? 0.f : mn;      // no key visible so far
-            const float alpha = expf(m[i] - ref);
-            float sum = 0.f;
+            grow |= mx[i] > m[i] + kLazyMax;
+        }
+        if (__any_sync(0xffffffffu, grow)) {
+            uint64_t al[R / 2];
+#pragma unroll
+            for (int i = 0; i < R; i += 2) {
+                float alpha[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float mn = fmaxf(m[i + e], group16_max(mx[i + e]));
+                    alpha[e] = expf(m[i + e] - (mn == -INFINITY ? 0.f : mn));
+                    l[i + e] *= alpha[e];
+                    m[i + e] = mn;
+                }
+                al[i / 2] = ptx::pack_f32x2(alpha[0], alpha[1]);
+            }
+#pragma unroll
+            for (int i = 0; i < R / 2; ++i)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) o[i][c] = ptx::mul_f32x2(o[i][c], al[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const float ref = m[i] == -INFINITY ? 0.f : m[i];      // (-inf: no key visible so far)
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 s[i][b] = expf(s[i][b] - ref);
-                sum += s[i][b];
-            }
-            l[i] = l[i] * alpha + group16_sum(sum);
-            m[i] = mn;
-            if (i & 1) {
-                float other, none;
-                ptx::unpack_f32x2(al[i / 2], other, none);
-                al[i / 2] = ptx::pack_f32x2(other, alpha);
-            } else {
-                al[i / 2] = ptx::pack_f32x2(alpha, 0.f);
+                l[i] += s[i][b];
             }
         }
 #pragma unroll
@@ -323,10 +337,6 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
                     *reinterpret_cast<float4 *>(dst + i) = make_float4(s[i][b], s[i + 1][b], s[i + 2][b], s[i + 3][b]);
             }
         }
-#pragma unroll
-        for (int i = 0; i < R / 2; ++i)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) o[i][c] = ptx::mul_f32x2(o[i][c], al[i]);
         cp_wait<1>();                 // V is here; the next K may still be on its way
         __syncthreads();              // (also: every lane's part of P^T is written)
         add_rows<R, BN, D>(o, Pw, LP, (ty % 2) * R, Vs, tx);
@@ -347,14 +357,16 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
             *reinterpret_cast<float4 *>(Om + (ty * R + 2 * i) * LD + 64 * v + 4 * tx) = e;
             *reinterpret_cast<float4 *>(Om + (ty * R + 2 * i + 1) * LD + 64 * v + 4 * tx) = od;
         }
-    if (tx == 0)
 #pragma unroll
-        for (int i = 0; i < R; ++i) { Mm[ty * R + i] = m[i]; Lm[ty * R + i] = l[i]; }
+    for (int i = 0; i < R; ++i) {
+        const float li = group16_sum(l[i]);
+        if (tx == 0) { Mm[ty * R + i] = m[i]; Lm[ty * R + i] = li; }
+    }
     if (split > 1) cluster_barrier();
     else __syncthreads();
     constexpr int LPR = D / 4;         // lanes per row, 16 bytes each
-    const int per = BM / split;        // rows this rank finishes
-    for (int r = tid / LPR; r < per; r += SNT / LPR) {
+    const int per = (BM + split - 1) / split;        // rows this rank finishes (the last rank: what is left)
+    for (int r = tid / LPR; r < per && rank * per + r < BM; r += SNT / LPR) {
         const int rr = rank * per + r, row = q0 + rr, c = (tid % LPR) * 4;
         float mt = -INFINITY, mk[ptx::kMaxRanks], lk[ptx::kMaxRanks];
         float4 vk[ptx::kMaxRanks];
@@ -655,8 +667,8 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
         }
     cluster_barrier();
     constexpr int LPR = D / 4;
-    const int per = BN / split;
-    for (int r = tid / LPR; r < per; r += SNT / LPR) {
+    const int per = (BN + split - 1) / split;
+    for (int r = tid / LPR; r < per && rank * per + r < BN; r += SNT / LPR) {
         const int rr = rank * per + r, row = k0 + rr, c = (tid % LPR) * 4;
         if (row >= n) continue;
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), g = a;
@@ -993,21 +1005,32 @@ convert_rows_kernel(const float *__restrict__ src, int src_ld, __nv_bfloat16 *__
 
 constexpr size_t bwd_smem(int D) { return (size_t)(4 * BM * (D + 1) + 2 * BM * SLD + 2 * BM) * sizeof(float); }
 
-// How many ranks share an output tile (bwd_split's estimate, for `per_sm` CTAs on an SM; set-up and merge are small beside these
-// kernels' tiles).  With the causal mask the longest of B2 H2 n1817 d128's 228 tiles takes twice the average and all run at once, so
-// that clusters of two, in two waves, are faster.
+// How many ranks share an output tile; set-up and merge are small beside these kernels' tiles.
+// Equal tiles (no causal mask): one CTA alone brings an SM to 82 % of what any number of them reach, so k CTAs on an SM take 0.82 k times
+// as long as one, together or in turn, and the time is that of the fullest SM.  Any number of ranks up to 8: B2 H1 n2048 d64's 64 tiles
+// take 156, 82, 94, 70, 85, 75, 82, 76 us with 1 ... 8 ranks (estimate 32, 16.5, 18.9, 13.9, 18.5, 16, 18.5, 14.8 tiles).
+// Causal: the longest job against the packing of all of them (bwd_split for `per_sm` CTAs on an SM; B2 H2 n1817 d128: 207, 146, 126, 152
+// us with 1, 2, 4, 8).
 int simt_split(long long jobs, int own_tiles, int others, int own_rows, int other_rows, bool causal, int per_sm)
 {
-    // causal: the tiles of the other axis that tile t meets, summed over t (both axes are cut from the same n rows)
-    long long total = (long long)own_tiles * others;
     if (causal) {
-        total = 0;
+        // the tiles of the other axis that tile t meets, summed over t (both axes are cut from the same n rows)
+        long long total = 0;
         for (int t = 0; t < own_tiles; ++t) {
             const long long c = ((long long)(t + 1) * own_rows + other_rows - 1) / other_rows;
             total += c < others ? c : others;
         }
+        return bwd_split(jobs, others, jobs / own_tiles * total, true, 0.2, 0.1, per_sm);
     }
-    return bwd_split(jobs, others, jobs / own_tiles * total, causal, 0.3, 0.3, per_sm);
+    const long long sms = device_info().sms;
+    int best = 1;
+    double best_cost = 0;
+    for (int s = 1; s <= 8 && s <= others; ++s) {
+        const long long k = (jobs * s + sms - 1) / sms;
+        const double cost = ((others + s - 1) / s + (s > 1 ? 0.5 : 0.3)) * (k > 1 ? 0.82 * k : 1.0);
+        if (s == 1 || cost < 0.95 * best_cost) { best = s; best_cost = cost; }
+    }
+    return best;
 }
 
 // Rows per thread: the widest tile (fewest shared-memory loads per multiply-add) whose tiles, shared by clusters as far as
