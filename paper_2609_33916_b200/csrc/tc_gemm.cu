@@ -21,6 +21,12 @@
 // operand layout 1240-1340 -> 1350-1530 TFLOP/s; launches of a few tiles, and shapes whose M is so
 // small that pairs would need more waves, stay on single CTAs.
 //
+// A small product is bound by what a launch does once: in a chain of dependent launches of 512 x 64 x 64 the first load went out 0.9 us
+// after the kernel in front was done and the CTA left 1.3 us after its last store was issued.  The place of the first tile is worked out in
+// front of the wait for that kernel, K blocks past K are not loaded, the residual (and the gate's stored a, u) are requested
+// while the main loop runs, and copies are only waited for at the end if a wait has expired (in every other case each of them has been waited
+// for): 5.4 -> 3.3 us per launch, and 8192 x 2048 x 2048 53.6 -> 49.7 us.
+//
 // Operand storage is a template choice per operand, because the backward's GEMMs read the same
 // arrays transposed:
 //   K-major  : the array is [rows = M or N, K] row-major; one TMA box of 64 K-elements x rows.
@@ -144,6 +150,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     // map C0), so that their tiles share the waves of the persistent grid
     const int tiles_one = tiles_m * tiles_n, tiles = tiles_one * nbatch;
     const int nk = (K + GK * kSub - 1) / (GK * kSub), nk_total = nk * nparts;     // stages per operand pair
+    const int tail = (K + GK - 1) / GK - (nk - 1) * kSub;                         // K blocks of a pair's last stage
+    int armed = 0;       // loads this thread armed a barrier for: stages (the producer), staging buffers (the epilogue's leader)
 
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) {
@@ -177,38 +185,51 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     __syncthreads();
     if (kPair) cluster_sync_all();       // the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after();
-    grid_dependency_wait();
-    grid_launch_dependents();
     const uint32_t tbase = *tmem_slot;
+    const bool producer = warp == 0 && lane == 0;
+    if (!producer) {
+        grid_dependency_wait();
+        grid_launch_dependents();
+    }
 
-    if (warp == 0 && lane == 0) {
+    if (producer) {
         // ------------------------------------------------------------------ TMA producer
-        ArmCounts<G_COUNT> armed;     // barriers armed for copies into shared memory
-        int it = 0;
+        int it = 0, tm = 0, tn = 0, second = 0;
         bool ok = true;
-        for (int t = cta; ok && t < tiles; t += ncta) {
-            int tm, tn;
-            const int second = t >= tiles_one ? 1 : 0;
+        auto place = [&](int t) {
+            second = t >= tiles_one ? 1 : 0;
             tile_coords(t - second * tiles_one, tiles_m, tiles_n, group_rows, tm, tn);
+        };
+        // (the divisions of the first tile's place run in front of the wait: behind it they were 0.6 us of a small product's 5)
+        if (cta < tiles) place(cta);
+        grid_dependency_wait();
+        grid_launch_dependents();
+        for (int t = cta; ok && t < tiles; t += ncta) {
+            if (t != cta) place(t);
             const int m0 = tm * kTileM + (int)rank * GM, n0 = tn * kTileN;
             const int nb0 = n0 + ((kPair && !kDualN) ? (int)rank * (kN / 2) : 0);    // first B row this CTA stages
+            int part = 0, kstage = 0;
             for (int ks = 0; ks < nk_total; ++ks, ++it) {
                 const int s = it % kSt;
-                if (!mbar_wait(bars + G_EMPTY + s, ((it / kSt) & 1) ^ 1, abortp, status, GERR_EMPTY)) { ok = false; break; }
-                const int part = ks / nk;
+                if (it >= kSt && !mbar_wait(bars + G_EMPTY + s, ((it / kSt) & 1) ^ 1, abortp, status, GERR_EMPTY)) { ok = false; break; }
+                const int nsub = kstage == nk - 1 ? tail : kSub, kbase = kstage * kSub * GK;
                 const CUtensorMap *ma = (part || second) ? &mapA1 : &mapA0;
                 const CUtensorMap *mb = ((part || second) && !kDualN) ? &mapB1 : &mapB0;
                 uint64_t *full = bars + G_FULL + s;
                 // a pair: the copies of both CTAs complete on the barrier of rank 0, which its producer arms for both
                 const uint32_t full_pair = kPair ? mapa_u32(smem_u32(full), 0) : 0u;
-                if (!kPair || rank == 0) mbar_arm(bars, G_FULL + s, (kPair ? 2 : 1) * kStageBytes, armed);
+                if (!kPair || rank == 0) {
+                    mbar_arrive_expect_tx(full, (uint32_t)((kPair ? 2 : 1) * nsub * kSubBytes));
+                    ++armed;
+                }
                 auto load = [&](void *dst, const CUtensorMap *m, int x, int y, int z) {
                     if (kPair) tma_load_3d_pair(dst, m, full_pair, x, y, z);
                     else tma_load_3d(dst, m, full, x, y, z);
                 };
 #pragma unroll
-              for (int sub = 0; sub < kSub; ++sub) {          // (a block past K is filled with zeros by the copy)
-                const int k0 = ((ks - part * nk) * kSub + sub) * GK;
+              for (int sub = 0; sub < kSub; ++sub) {          // (what lies past K in a block is filled with zeros by the copy)
+                if (sub >= nsub) break;
+                const int k0 = kbase + sub * GK;
                 uint8_t *sa = sm + s * kStageBytes + sub * kSubBytes, *sb = sa + kABytes;
                 if (kAMn) {
                     if (a_blocked) {                          // one copy: (64 columns, K rows, column blocks)
@@ -238,9 +259,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                     load(sb, mb, k0, nb0, 0);
                 }
               }
+                if (++kstage == nk) { kstage = 0; ++part; }
             }
         }
-        mbar_drain(bars, armed);      // copies of this CTA still on their way land before it leaves (bounded)
     } else if (warp == 1 && lane == 0 && rank == 0) {
         // ------------------------------------------------------------------- UMMA issuer
         constexpr uint32_t idesc = idesc_bf16_f32(kTileM, kN, kAMn ? 1 : 0, kBMn ? 1 : 0);
@@ -255,14 +276,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             if (!mbar_wait(bars + G_ACCEMPTY + buf, ((ti >> 1) & 1) ^ 1, abortp, status, GERR_ACCEMPTY)) break;
             tc_fence_after();
             const uint32_t acc = tbase + (uint32_t)(buf * kN);
+            int kstage = 0;
             for (int ks = 0; ks < nk_total; ++ks, ++it) {
                 const int s = it % kSt;
+                const bool last = ++kstage == nk;
+                if (last) kstage = 0;
                 if (!mbar_wait(bars + G_FULL + s, (it / kSt) & 1, abortp, status, GERR_FULL)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t a_lo = a_lo0 + ((smem_u32(sm + s * kStageBytes) >> 4) & 0x3FFFu);
                 const uint32_t b_lo = b_lo0 + ((smem_u32(sm + s * kStageBytes + kABytes) >> 4) & 0x3FFFu);
 #pragma unroll
                 for (int sub = 0; sub < kSub; ++sub) {
+                    if (sub > 0 && last && sub >= tail) break;
                     const uint32_t a_s = a_lo + (uint32_t)(sub * (kSubBytes >> 4)), b_s = b_lo + (uint32_t)(sub * (kSubBytes >> 4));
                     if (ks == 0 && sub == 0) {
                         if (kPair) umma_ss2_pair<false>(acc, a_s, a_hi, b_s, b_hi, idesc);
@@ -297,7 +322,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         const int half = (warp - 2) / 4;                           // which 32 columns of a 64-column chunk
         const bool leader = tid == 64;
         uint32_t epi_phase = 0, chunk_q = 0, in_q = 0;
-        ArmCounts<G_COUNT> armed;     // barriers the leader armed for copies into the staging buffers
         bool ok = true;
         // hands an accumulator back to the issuer (a pair: to the issuer in the CTA of rank 0)
         const uint32_t accempty_pair = kPair ? mapa_u32(smem_u32(bars + G_ACCEMPTY), 0) : 0u;
@@ -331,15 +355,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             ++chunk_q;
             return true;
         };
-        // the same with a residual: the chunk of R comes into the staging buffer by TMA, every thread adds its 32
-        // values in place, and the buffer leaves by a TMA store
-        auto stage_store_res = [&](const CUtensorMap *map, const uint32_t (&racc)[32], int col0, int row0) -> bool {
+        // the same with a residual: the chunk of R comes into the staging buffer by TMA (requested a chunk ahead, a tile's first
+        // before its main loop has finished), every thread adds its 32 values in place, and the buffer leaves by a TMA store
+        auto load_res = [&](uint32_t q, int col0, int row0) {          // (leader; the buffer's last store has been read)
+            mbar_arrive_expect_tx(bars + G_RES + (q & 1), kOutBox);
+            ++armed;
+            tma_load_3d(sout + (q & 1) * kOutBox, &mapC2, bars + G_RES + (q & 1), col0, row0, 0);
+        };
+        auto stage_store_res = [&](const CUtensorMap *map, const uint32_t (&racc)[32], int col0, int row0, bool more) -> bool {
             const uint32_t b = chunk_q & 1;
             uint8_t *buf = sout + b * kOutBox;
-            if (leader) {
-                bulk_wait_read<1>();                                   // the store issued two chunks ago has left this buffer
-                mbar_arm(bars, G_RES + (int)b, kOutBox, armed);
-                tma_load_3d(buf, &mapC2, bars + G_RES + b, col0, row0, 0);
+            if (leader && more) {
+                bulk_wait_read<0>();                                   // the store of the last chunk has left the other buffer
+                load_res(chunk_q + 1, col0 + 64, row0);
             }
             if (!mbar_wait(bars + G_RES + b, (chunk_q >> 1) & 1, abortp, status, GERR_RES)) return false;
 #pragma unroll
@@ -367,13 +395,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             tile_coords(t - second * tiles_one, tiles_m, tiles_n, group_rows, tm, tn);
             const int buf = ti & 1;
             const int m0 = tm * kTileM + (int)rank * GM, n0 = tn * kTileN;
-            if (kEpi == EPI_STORE && has_res && leader) {     // the tile's residual: into L2 while its main loop runs
+            if (kEpi == EPI_STORE && has_res && leader) {     // the tile's residual, while its main loop runs: the first chunk, the rest into L2
+                bulk_wait_read<1>();
+                load_res(chunk_q, n0, m0);
 #pragma unroll
-                for (int c0 = 0; c0 < kN; c0 += 64) tma_prefetch_3d(&mapC2, n0 + c0, m0, 0);
+                for (int c0 = 64; c0 < kN; c0 += 64) tma_prefetch_3d(&mapC2, n0 + c0, m0, 0);
             }
-            if (kEpi == EPI_SWIGLU_BWD && leader) {       // the tile's stored a, u: into L2 while its main loop runs
+            auto load_gate = [&](int c0) {                    // (leader)
+                bulk_wait_read<0>();                          // the previous chunk's stores have left both buffers
+                mbar_arrive_expect_tx(bars + G_IN, 2 * kOutBox);
+                ++armed;
+                tma_load_3d(sout, &mapC2, bars + G_IN, n0 + c0, m0, 0);
+                tma_load_3d(sout + kOutBox, &mapC3, bars + G_IN, n0 + c0, m0, 0);
+            };
+            if (kEpi == EPI_SWIGLU_BWD && leader) {       // the tile's stored a, u, while its main loop runs: likewise
+                load_gate(0);
 #pragma unroll
-                for (int c0 = 0; c0 < kN; c0 += 64) {
+                for (int c0 = 64; c0 < kN; c0 += 64) {
                     tma_prefetch_3d(&mapC2, n0 + c0, m0, 0);
                     tma_prefetch_3d(&mapC3, n0 + c0, m0, 0);
                 }
@@ -415,7 +453,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                         acc_release(buf);
                     }
                     if (has_res) {
-                        ok = stage_store_res(&mapC0, r, n0 + c0, m0);
+                        ok = stage_store_res(&mapC0, r, n0 + c0, m0, c0 + 64 < cols);
                     } else {
                         uint32_t pc[16];
 #pragma unroll
@@ -428,12 +466,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 // thread turns its 32 + 32 values into da, du in place, and the buffers leave by TMA stores.
 #pragma unroll 1
                 for (int c0 = 0; ok && c0 < cols; c0 += 64, ++in_q) {
-                    if (leader) {
-                        bulk_wait_read<0>();              // the previous chunk's stores have left both buffers
-                        mbar_arm(bars, G_IN, 2 * kOutBox, armed);
-                        tma_load_3d(sout, &mapC2, bars + G_IN, n0 + c0, m0, 0);
-                        tma_load_3d(sout + kOutBox, &mapC3, bars + G_IN, n0 + c0, m0, 0);
-                    }
+                    if (leader && c0 > 0) load_gate(c0);
                     uint32_t r[32];
                     tmem_ld(acc + c0 + 32 * half, r);
                     tc_wait_ld();
@@ -470,13 +503,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 }
             }
         }
-        if (leader) {
-            bulk_wait_read<0>();          // every store has read its buffer before the CTA gives up its shared memory
-            mbar_drain(bars, armed);      // and so has every copy into the staging buffers (bounded)
-        }
+        if (leader) bulk_wait_read<0>();          // every store has read its buffer before the CTA gives up its shared memory
     }
     tc_fence_before();
+    __syncwarp();
     __syncthreads();
+    if (*abortp) {      // a wait expired somewhere: copies still on their way land before the CTA leaves (bounded)
+        if (producer)
+            for (int s = 0; s < kSt; ++s) mbar_drain_one(bars + G_FULL + s, armed > s ? (armed - s + kSt - 1) / kSt : 0);
+        if (tid == 64 && kEpi == EPI_STORE)
+            for (int b = 0; b < 2; ++b) mbar_drain_one(bars + G_RES + b, armed > b ? (armed - b + 1) / 2 : 0);
+        if (tid == 64 && kEpi == EPI_SWIGLU_BWD) mbar_drain_one(bars + G_IN, armed);
+    }
     if (kPair) {
         // neither CTA leaves, or frees its TMEM, while the other may still read its shared memory, write its
         // accumulator or arrive on its barriers
@@ -489,7 +527,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 }
 
 // Several products C = A B^T (one or two operand pairs, any storage order) as ONE launch of single CTAs: what the backward of a small block needs
-// next to each other.  A launch costs such a product 5 us beside its K blocks and leaves most SMs idle; here the tiles of all of them are
+// next to each other.  A launch costs such a product 3 us beside its K blocks and leaves most SMs idle; here the tiles of all of them are
 // walked by one grid.  Same roles, ring and epilogue as tc_gemm_kernel, the operand layouts taken from the job at run time.
 constexpr int kMaxJobs = 4;
 struct GroupJob {
@@ -534,8 +572,6 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    grid_dependency_wait();
-    grid_launch_dependents();
     const uint32_t tbase = *tmem_slot;
     const int cta = (int)blockIdx.x, ncta = (int)gridDim.x, tiles = jobs.tiles;
     // the job of a tile (tiles are walked in ascending order) and the tile's place in it
@@ -549,25 +585,43 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
     };
     auto stages_of = [&](const GroupJob &J) { return (J.K + GK * kSub - 1) / (GK * kSub); };      // per operand pair
 
-    if (warp == 0 && lane == 0) {
+    auto tail_of = [&](const GroupJob &J) { return (J.K + GK - 1) / GK - (stages_of(J) - 1) * kSub; };   // K blocks of a pair's last stage
+    const bool producer = warp == 0 && lane == 0;
+    int armed = 0;       // stages the producer armed
+    if (!producer) {
+        grid_dependency_wait();
+        grid_launch_dependents();
+    }
+
+    if (producer) {
         // ------------------------------------------------------------------ TMA producer
-        ArmCounts<G_COUNT> armed;
-        int it = 0, jx = 0;
+        int it = 0, jx = 0, m0 = 0, n0 = 0;
         bool ok = true;
+        if (cta < tiles) {                // in front of the wait: where the first tile is, and its maps
+            job_of(cta, jx, m0, n0);
+            prefetch_tensormap(&jobs.j[jx].A[0]);
+            prefetch_tensormap(&jobs.j[jx].B[0]);
+            prefetch_tensormap(&jobs.j[jx].C);
+        }
+        grid_dependency_wait();
+        grid_launch_dependents();
         for (int t = cta; ok && t < tiles; t += ncta) {
-            int m0, n0;
-            job_of(t, jx, m0, n0);
+            if (t != cta) job_of(t, jx, m0, n0);
             const GroupJob &J = jobs.j[jx];
-            const int nk = stages_of(J);
+            const int nk = stages_of(J), tail = tail_of(J);
+            int part = 0, kstage = 0;
             for (int ks = 0; ks < nk * J.nparts; ++ks, ++it) {
-                const int s = it % kSt, part = ks / nk;
-                if (!mbar_wait(bars + G_EMPTY + s, ((it / kSt) & 1) ^ 1, abortp, status, GERR_EMPTY)) { ok = false; break; }
+                const int s = it % kSt;
+                if (it >= kSt && !mbar_wait(bars + G_EMPTY + s, ((it / kSt) & 1) ^ 1, abortp, status, GERR_EMPTY)) { ok = false; break; }
                 uint64_t *full = bars + G_FULL + s;
-                mbar_arm(bars, G_FULL + s, kStageBytes, armed);
+                const int nsub = kstage == nk - 1 ? tail : kSub, kbase = kstage * kSub * GK;
+                mbar_arrive_expect_tx(full, (uint32_t)(nsub * kSubBytes));
+                ++armed;
                 const CUtensorMap *ma = &J.A[part], *mb = &J.B[part];
 #pragma unroll
                 for (int sub = 0; sub < kSub; ++sub) {
-                    const int k0 = ((ks - part * nk) * kSub + sub) * GK;
+                    if (sub >= nsub) break;
+                    const int k0 = kbase + sub * GK;
                     uint8_t *sa = sm + s * kStageBytes + sub * kSubBytes, *sb = sa + kABytes;
                     if (!J.a_mn) {
                         tma_load_3d(sa, ma, full, k0, m0, 0);
@@ -586,9 +640,9 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
                         for (int b = 0; b < kN / 64; ++b) tma_load_3d(sb + b * kMnBox, mb, full, n0 + 64 * b, k0, 0);
                     }
                 }
+                if (++kstage == nk) { kstage = 0; ++part; }
             }
         }
-        mbar_drain(bars, armed);      // copies of this CTA still on their way land before it leaves (bounded)
     } else if (warp == 1 && lane == 0) {
         // ------------------------------------------------------------------- UMMA issuer
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kMnBox, 1024);
@@ -601,18 +655,22 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
             const uint64_t ap = J.a_mn ? mn_proto : km_proto, bp = J.b_mn ? mn_proto : km_proto;
             const uint32_t a_hi = (uint32_t)(ap >> 32), b_hi = (uint32_t)(bp >> 32), a_lo0 = (uint32_t)ap, b_lo0 = (uint32_t)bp;
             const uint32_t a_step = (J.a_mn ? 2048 : 32) >> 4, b_step = (J.b_mn ? 2048 : 32) >> 4, idesc = idesc_bf16_f32(GM, kN, J.a_mn, J.b_mn);
-            const int nk_total = stages_of(J) * J.nparts, buf = ti & 1;
+            const int nk = stages_of(J), nk_total = nk * J.nparts, tail = tail_of(J), buf = ti & 1;
             if (!mbar_wait(bars + G_ACCEMPTY + buf, ((ti >> 1) & 1) ^ 1, abortp, status, GERR_ACCEMPTY)) break;
             tc_fence_after();
             const uint32_t acc = tbase + (uint32_t)(buf * kN);
+            int kstage = 0;
             for (int ks = 0; ks < nk_total; ++ks, ++it) {
                 const int s = it % kSt;
+                const bool last = ++kstage == nk;
+                if (last) kstage = 0;
                 if (!mbar_wait(bars + G_FULL + s, (it / kSt) & 1, abortp, status, GERR_FULL)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t a_lo = a_lo0 + ((smem_u32(sm + s * kStageBytes) >> 4) & 0x3FFFu);
                 const uint32_t b_lo = b_lo0 + ((smem_u32(sm + s * kStageBytes + kABytes) >> 4) & 0x3FFFu);
 #pragma unroll
                 for (int sub = 0; sub < kSub; ++sub) {
+                    if (sub > 0 && last && sub >= tail) break;
                     const uint32_t a_s = a_lo + (uint32_t)(sub * (kSubBytes >> 4)), b_s = b_lo + (uint32_t)(sub * (kSubBytes >> 4));
                     if (ks == 0 && sub == 0) umma_ss2<false>(acc, a_s, a_hi, b_s, b_hi, idesc);
                     else                     umma_ss2<true>(acc, a_s, a_hi, b_s, b_hi, idesc);
@@ -675,7 +733,10 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
         if (leader) bulk_wait_read<0>();
     }
     tc_fence_before();
+    __syncwarp();
     __syncthreads();
+    if (*abortp && producer)      // (as in tc_gemm_kernel)
+        for (int s = 0; s < kSt; ++s) mbar_drain_one(bars + G_FULL + s, armed > s ? (armed - s + kSt - 1) / kSt : 0);
     if (warp == 1) tmem_dealloc(tbase, 2 * kN);
 }
 
