@@ -476,8 +476,11 @@ NormPlan norm_plan(int n, int d, bool bwd)
 }
 
 
-// The ring variant serves rows of 256 .. 2048 elements (a warp per row, at most 8 vectors per lane).
-bool norm_uses_ring(int d) { return d >= 256 && d <= 2048; }
+// The ring variant serves rows of 256 .. 2048 elements (a warp per row, at most 8 vectors per lane) from the size on where the bytes in
+// flight decide; below it, a warp's rows of a stage one behind the other are most of the time.  Register and ring variant, in a chain of
+// calls: forward 8192 x 512 4.4 and 4.6 us, 4096 x 2048 7.1 and 7.6, 8192 x 2048 11.8 and 11.4; backward 512 x 256 4.5 and 8.1, 512 x 2048
+// 8.5 and 14.4, 1024 x 1024 7.7 and 9.9, 2048 x 1024 13.6 and 10.9.
+bool norm_uses_ring(int n, int d, bool bwd) { return d >= 256 && d <= 2048 && (long long)n * d > (bwd ? 1LL << 20 : 8LL << 20); }
 struct RingPlan {
     int kV, m, grid;
     size_t smem;
@@ -529,7 +532,7 @@ cudaError_t rmsnorm_fwd(int n, int d, float eps, const void *x, const void *g, v
     const auto *gb = (const __nv_bfloat16 *)g;
     auto *yb = (__nv_bfloat16 *)y;
     LaunchScope scope(MOA_KERNEL_OTHER, st);
-    if (norm_uses_ring(d)) return launch_ring_kv<false>(ring_plan(n, d, false), xb, gb, nullptr, r, nullptr, nullptr, yb, nullptr, n, d, eps, st);
+    if (norm_uses_ring(n, d, false)) return launch_ring_kv<false>(ring_plan(n, d, false), xb, gb, nullptr, r, nullptr, nullptr, yb, nullptr, n, d, eps, st);
     const auto kernel = p.kV == 1 ? rmsnorm_fwd_kernel<1, 2> : p.kV == 2 ? rmsnorm_fwd_kernel<2, 1> : rmsnorm_fwd_kernel<4, 1>;
     return launch_dependent(kernel, dim3(p.grid), dim3(kNormThreads), (size_t)0, st, xb, gb, yb, r, n, d, eps, p.tpr);
 }
@@ -545,7 +548,7 @@ cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, c
     auto *ob = (__nv_bfloat16 *)dx;
     float *part = (float *)ws;
     int parts = p.grid;
-    if (norm_uses_ring(d)) {
+    if (norm_uses_ring(n, d, true)) {
         const RingPlan rp = ring_plan(n, d, true);
         parts = rp.grid;
         LaunchScope scope(MOA_KERNEL_OTHER, st);

@@ -1,0 +1,36 @@
+"""RMSNorm on both sides of the lines between its register and its ring kernels (rows of 256..2048 elements; by n times d, another line
+in the forward than in the backward), with ragged numbers of rows and row lengths that leave vectors over."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+import oracle
+from paper_2609_33916_b200 import inputs as mi
+
+TOL = 1e-2        # bf16 storage, fp32 arithmetic: the bound of the other RMSNorm tests
+
+
+@pytest.mark.parametrize("n,d", [(4096, 256), (4097, 256), (511, 2048), (513, 2048), (1033, 1016), (127, 264), (32767, 256), (32801, 256),
+                                 (8300, 1016)])
+def test_rmsnorm_routes(n, d):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2609_33916_b200 import binding as mb
+    from paper_2609_33916_b200 import build
+    build.build()
+    inp = mi.make_norm_inputs(n, d, seed=7 * n + d)
+    x, g, dy = (torch.from_numpy(np.ascontiguousarray(inp[k])).view(torch.bfloat16).cuda() for k in ("x", "g", "dy"))
+    y, dx, dg = (torch.full_like(t, float("nan")) for t in (x, x, g))
+    r = torch.full((n,), float("nan"), dtype=torch.float32, device="cuda")
+    desc = mb.make_rmsnorm_desc(n, d, 1e-5)
+    ws = torch.full((mb.moa_rmsnorm_workspace_bytes(desc),), 0xFF, dtype=torch.uint8, device="cuda")
+    mb.moa_rmsnorm_fwd(desc, x, g, y, r)
+    mb.moa_rmsnorm_bwd(desc, x, g, r, dy, dx, dg, ws)
+    f = {k: mi.to_f64(v, "bf16") for k, v in inp.items()}
+    ref = oracle.rmsnorm_fwd_bwd(f["x"], f["g"], f["dy"], 1e-5)
+    for k, t in (("y", y), ("dx", dx), ("dg", dg)):
+        got = t.float().cpu().numpy().astype(np.float64)
+        assert np.all(np.isfinite(got)) and mi.rel_err(got, ref[k]) <= TOL, (k, mi.rel_err(got, ref[k]))
+    assert mi.rel_err(r.cpu().numpy().astype(np.float64), ref["r"]) <= 1e-5
