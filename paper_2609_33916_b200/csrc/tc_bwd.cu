@@ -246,8 +246,30 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     const int head0 = kGrouped && kSplit ? it0 / (nqt - i_begin) : 0;       // query heads of the group in front of it
     const TileWalk walk0{(kGrouped ? bh * group : bh) + head0, i_begin + it0 - head0 * (nqt - i_begin), i_begin, nqt};
 
+    // The producer initialises the barriers of its own loads and sends the first ones off at once; the rest of the set-up (the other barriers,
+    // the TMEM allocation) runs under them.  K, V, Q and dO are the caller's tensors; L', D and the cleared dQ accumulator were
+    // written by the kernel in front of this one in the stream (the forward or the preprocess kernel), which may still be running.
+    if (warp == kLoadWarp && lane == 0) {
+        mbar_init(bars + B_KV, 1u);
+        for (int s = 0; s < 2; ++s) { mbar_init(bars + B_QFULL + s, 1u); mbar_init(bars + B_DOFULL + s, 1u); }
+        fence_mbar_init();
+        if ((smem_u32(sm) & 1023u) == 0 && niter_all > 0) {
+            mbar_arrive_expect_tx(bars + B_KV, 2 * SM::kTile);
+            mbar_arrive_expect_tx(bars + B_QFULL, SM::kTile + 1024);       // (with its L' and D, requested later)
+            mbar_arrive_expect_tx(bars + B_DOFULL, SM::kTile);
+            for (int b = 0; b < kBoxes; ++b) {
+                tma_load_4d(sK + b * kBoxBytes, &mapK, bars + B_KV, 64 * b, k0, hk, bb);
+                tma_load_4d(sm + SM::offQ + b * kBoxBytes, &mapQ, bars + B_QFULL, 64 * b, walk0.qi * 128, walk0.qh + hq0, bb);
+            }
+            for (int b = 0; b < kBoxes; ++b) {
+                tma_load_4d(sV + b * kBoxBytes, &mapV, bars + B_KV, 64 * b, k0, hk, bb);
+                tma_load_4d(sm + SM::offdO + b * kBoxBytes, &mapdO, bars + B_DOFULL, 64 * b, walk0.qi * 128, walk0.qh + hq0, bb);
+            }
+        }
+    }
     if (tid == 0) {
         for (int b = 0; b < B_COUNT; ++b) {
+            if (b <= B_QFULL + 1 || b == B_DOFULL || b == B_DOFULL + 1) continue;      // (the producer's own)
             const uint32_t cnt = (b == B_P || b == B_DS || b == B_EPI) ? 256u
                                : (b == B_DQR || b == B_STGFULL || b == B_STGFULL + 1) ? 128u : 1u;
             mbar_init(bars + b, cnt);
@@ -275,27 +297,19 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
       asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
       if (warp == kLoadWarp) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0 && niter > 0) {
-            mbar_arrive_expect_tx(bars + B_KV, 2 * SM::kTile);
-            for (int b = 0; b < kBoxes; ++b) {
-                tma_load_4d(sK + b * kBoxBytes, &mapK, bars + B_KV, 64 * b, k0, hk, bb);
-                tma_load_4d(sV + b * kBoxBytes, &mapV, bars + B_KV, 64 * b, k0, hk, bb);
-            }
-        }
         // Q tiles (with L, D) go through a two-slot ring and are fetched two tiles ahead: S(i+1) is
         // issued in the middle of tile i.  dO has one slot: it is read only by dP(i) and dV(i),
         // early in tile i, and is refilled as soon as dV(i) has completed.
-        // K, V, Q and dO are the caller's tensors; L', D and the cleared dQ accumulator were written by the kernel in front of
-        // this one in the stream (the forward or the preprocess kernel), which may still be running: the first tiles are
-        // requested, then this warp waits for that kernel before it asks for L' and D.
+        // The first tiles were requested in front of the set-up; their L' and D wait for the kernel in front.
         TileWalk wq = walk0, wdo = walk0;     // load_q and load_do are each called for it = 0, 1, 2, ... in order
-        auto load_q = [&](int it, bool wait_first) {
+        auto load_q = [&](int it) {
             const int s = it & 1, q0 = wq.qi * 128, qh = wq.qh;
             wq.next();
-            uint8_t *sQ = sm + SM::offQ + s * SM::kTile;
-            mbar_arrive_expect_tx(bars + B_QFULL + s, SM::kTile + 1024);
-            for (int b = 0; b < kBoxes; ++b) tma_load_4d(sQ + b * kBoxBytes, &mapQ, bars + B_QFULL + s, 64 * b, q0, qh + hq0, bb);
-            if (wait_first) grid_dependency_wait();
+            if (it > 0) {
+                uint8_t *sQ = sm + SM::offQ + s * SM::kTile;
+                mbar_arrive_expect_tx(bars + B_QFULL + s, SM::kTile + 1024);
+                for (int b = 0; b < kBoxes; ++b) tma_load_4d(sQ + b * kBoxBytes, &mapQ, bars + B_QFULL + s, 64 * b, q0, qh + hq0, bb);
+            }
             bulk_load_1d(sL + s * 128, Lp + (size_t)qh * n_pad + q0, 512, bars + B_QFULL + s);
             bulk_load_1d(sD + s * 128, Dp + (size_t)qh * n_pad + q0, 512, bars + B_QFULL + s);
         };
@@ -307,12 +321,14 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             for (int b = 0; b < kBoxes; ++b) tma_load_4d(sdO + b * kBoxBytes, &mapdO, bars + B_DOFULL + s, 64 * b, q0, qh + hq0, bb);
         };
         if (lane == 0 && niter > 0) {
-            load_do(0);
+            wdo.next();
             if (kDoSlots == 2 && niter > 1) load_do(1);
-            load_q(0, true);
-            if (niter > 1) load_q(1, false);
         }
-        grid_dependency_wait();     // (the lanes that issued nothing, and a CTA without tiles)
+        grid_dependency_wait();
+        if (lane == 0 && niter > 0) {
+            load_q(0);
+            if (niter > 1) load_q(1);
+        }
         grid_launch_dependents();   // the dQ conversion that follows may be set up while this grid drains
         for (int it = 0; it < niter; ++it) {
             if (it + kDoSlots < niter) {     // dV(it) done: its dO slot takes tile it + kDoSlots
@@ -321,7 +337,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             }
             if (it + 2 < niter) {     // dK(it) done: its Q slot takes tile it+2
                 if (!mbar_wait(bars + B_QEMPTY + (it & 1), (it >> 1) & 1, abortp, status, ERR_EMPTY)) break;
-                if (lane == 0) load_q(it + 2, false);
+                if (lane == 0) load_q(it + 2);
             }
             __syncwarp();
         }
@@ -545,8 +561,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 }
             }
         }
-        if (kTransposeDQ && dq_bulk && tid == kReduceWarp0 * 32) bulk_wait<0>();   // all reduces done before exit
-        if (!kTransposeDQ && dq_bulk && lane == 0) bulk_wait<0>();                 // (D = 64: every reduce warp sent its own)
+        if (kTransposeDQ && dq_bulk && tid == kReduceWarp0 * 32) bulk_wait_read<0>();   // the stages are read before the CTA may exit
+        if (!kTransposeDQ && dq_bulk && lane == 0) bulk_wait_read<0>();            // (D = 64: every reduce warp sent its own)
     } else {
         // ----------------------------------------------------------- elementwise warps 0-7
         asm volatile("setmaxnreg.inc.sync.aligned.u32 144;");
@@ -677,16 +693,19 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 }
             }
         }
-        if (!kSplit && ok && mbar_wait(bars + B_DQ, (niter - 1) & 1, abortp, status, ERR_DQ) &&
-            (!kDKfromSmem || mbar_wait(bars + B_QEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, ERR_DQ))) {
-            // All UMMAs have completed.  dV and scale*dK go out as bf16 through shared memory (the K and V
-            // tiles are no longer read) and TMA stores: a thread owns a row, so direct stores would be 16
-            // bytes at a 2D-byte stride, one 128-byte line per lane and instruction -- 4096 line requests
-            // per CTA, which kept the load/store unit busy for ~3 us; staged, the tile leaves as
-            // full lines, and rows past n are clipped by the tensor map.
-            tc_fence_after();
+        if (!kSplit && ok) {
+            // dV and scale*dK go out as bf16 through shared memory (the V and K tiles, no longer read) and TMA stores: a thread owns
+            // a row, so direct stores would be 16 bytes at a 2D-byte stride, one 128-byte line per lane and instruction -- 4096
+            // line requests per CTA, which kept the load/store unit busy for ~3 us; staged, the tile leaves as full lines, and
+            // rows past n are clipped by the tensor map.  dV first, under the last dQ and dK: the last dP has read V, and dV is complete
+            // once the last dO slot is free.
 #pragma unroll
             for (int which = 0; which < 2; ++which) {
+                const bool there = which == 0 ? mbar_wait(bars + B_DOEMPTY + (niter - 1) % kDoSlots, ((niter - 1) / kDoSlots) & 1, abortp, status, ERR_DQ)
+                    : mbar_wait(bars + B_DQ, (niter - 1) & 1, abortp, status, ERR_DQ) &&
+                      (!kDKfromSmem || mbar_wait(bars + B_QEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, ERR_DQ));
+                if (!there) break;
+                tc_fence_after();
                 const uint32_t col = (which == 0 ? colDV : colDK) + (D / 2) * wg;
                 const float mul = which == 0 ? 1.f : scale;
                 uint8_t *stage = which == 0 ? sV : sK;
@@ -707,17 +726,14 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                         *reinterpret_cast<uint4 *>(stage + (cabs >> 6) * kBoxBytes + lane_row * 128 + chunk * 16) = v;
                     }
                 }
-            }
-            fence_proxy_async_smem();
-            mbar_arrive(bars + B_EPI);
-            if (tid == 0 && mbar_wait(bars + B_EPI, 0, abortp, status, ERR_DQ)) {
-                for (int b = 0; b < kBoxes; ++b) {
-                    tma_store_4d(&mapdV, sV + b * kBoxBytes, 64 * b, k0, hk, bb);
-                    tma_store_4d(&mapdK, sK + b * kBoxBytes, 64 * b, k0, hk, bb);
+                fence_proxy_async_smem();
+                mbar_arrive(bars + B_EPI);
+                if (tid == 0 && mbar_wait(bars + B_EPI, which, abortp, status, ERR_DQ)) {
+                    for (int b = 0; b < kBoxes; ++b) tma_store_4d(which == 0 ? &mapdV : &mapdK, stage + b * kBoxBytes, 64 * b, k0, hk, bb);
+                    bulk_commit();
                 }
-                bulk_commit();
-                bulk_wait_read<0>();      // shared memory is read before the CTA may exit
             }
+            if (tid == 0) bulk_wait_read<0>();      // shared memory is read before the CTA may exit
         }
     }
     tc_fence_before();
