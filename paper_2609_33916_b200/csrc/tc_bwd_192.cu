@@ -106,9 +106,29 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     const int head0 = kGrouped && kSplit ? it0 / (nqt - i_begin) : 0;       // query heads of the group in front of it
     const TileWalk walk0{(kGrouped ? bh * group : bh) + head0, i_begin + it0 - head0 * (nqt - i_begin), i_begin, nqt};
 
+    // the first loads go out before the rest of the set-up (K, V, Q and dO are the call's inputs; -L, -D and the cleared accumulator
+    // come from the kernel in front)
+    if (warp == kLoadWarp && lane == 0) {
+        mbar_init(bars + X_KV, 1u);
+        for (int s = 0; s < 2; ++s) { mbar_init(bars + X_Q + s, 1u); mbar_init(bars + X_DO + s, 1u); }
+        fence_mbar_init();
+        if ((smem_u32(sm) & 1023u) == 0 && niter_all > 0) {
+            mbar_arrive_expect_tx(bars + X_KV, 2 * NB * SM::kBoxK);
+            mbar_arrive_expect_tx(bars + X_Q, SM::kTile + 512);            // (with its L and D, requested later)
+            mbar_arrive_expect_tx(bars + X_DO, SM::kTile);
+            for (int b = 0; b < NB; ++b) {
+                tma_load_4d(sK + b * SM::kBoxK, &mapK, bars + X_KV, 64 * b, k0, hk, bb);
+                tma_load_4d(sQ + b * SM::kBoxQ, &mapQ, bars + X_Q, 64 * b, walk0.qi * BQ, walk0.qh + hq0, bb);
+            }
+            for (int b = 0; b < NB; ++b) {
+                tma_load_4d(sV + b * SM::kBoxK, &mapV, bars + X_KV, 64 * b, k0, hk, bb);
+                tma_load_4d(sdO + b * SM::kBoxQ, &mapdO, bars + X_DO, 64 * b, walk0.qi * BQ, walk0.qh + hq0, bb);
+            }
+        }
+    }
     if (tid == 0) {
         for (int b = 0; b < X_COUNT; ++b)
-            mbar_init(bars + b, (b == X_P || b == X_DS || b == X_EPI) ? 256u : (b == X_DQR) ? 128u : 1u);
+            if (b > X_Q + 1 && b != X_DO && b != X_DO + 1) mbar_init(bars + b, (b == X_P || b == X_DS || b == X_EPI) ? 256u : (b == X_DQR) ? 128u : 1u);
         *abortp = (smem_u32(sm) & 1023u) ? 1u : 0u;
         if (*abortp && status) atomicCAS(status, 0u, (unsigned)XERR_ALIGN);
         fence_mbar_init();
@@ -136,8 +156,10 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             int qh, q0;
             tile_of(it, qh, q0);
             const int s = it & 1;
-            mbar_arrive_expect_tx(bars + X_Q + s, SM::kTile + 512);
-            for (int b = 0; b < NB; ++b) tma_load_4d(sQ + s * SM::kTile + b * SM::kBoxQ, &mapQ, bars + X_Q + s, 64 * b, q0, qh + hq0, bb);
+            if (it > 0) {
+                mbar_arrive_expect_tx(bars + X_Q + s, SM::kTile + 512);
+                for (int b = 0; b < NB; ++b) tma_load_4d(sQ + s * SM::kTile + b * SM::kBoxQ, &mapQ, bars + X_Q + s, 64 * b, q0, qh + hq0, bb);
+            }
             bulk_load_1d(sL + s * 64, Lp + (size_t)qh * n_pad + q0, 256, bars + X_Q + s);
             bulk_load_1d(sD + s * 64, Dp + (size_t)qh * n_pad + q0, 256, bars + X_Q + s);
         };
@@ -148,16 +170,7 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             mbar_arrive_expect_tx(bars + X_DO + s, SM::kTile);
             for (int b = 0; b < NB; ++b) tma_load_4d(sdO + s * SM::kTile + b * SM::kBoxQ, &mapdO, bars + X_DO + s, 64 * b, q0, qh + hq0, bb);
         };
-        // (K, V, Q and dO are the call's inputs; -L, -D and the cleared accumulator come from the kernel in front)
-        if (lane == 0 && niter > 0) {
-            mbar_arrive_expect_tx(bars + X_KV, 2 * NB * SM::kBoxK);
-            for (int b = 0; b < NB; ++b) {
-                tma_load_4d(sK + b * SM::kBoxK, &mapK, bars + X_KV, 64 * b, k0, hk, bb);
-                tma_load_4d(sV + b * SM::kBoxK, &mapV, bars + X_KV, 64 * b, k0, hk, bb);
-            }
-            load_do(0);
-            if (niter > 1) load_do(1);
-        }
+        if (lane == 0 && niter > 1) load_do(1);
         grid_dependency_wait();
         grid_launch_dependents();
         if (lane == 0 && niter > 0) {
@@ -371,9 +384,10 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             if (it + 1 < niter) ok = p_phase(it + 1);
         }
         // every UMMA has completed once dK of the last tile has (one issuing thread; its phase before is known complete: dP of the last tile is)
-        const bool done = ok && mbar_wait(bars + X_QEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, XERR_DQ);
-        tc_fence_after();
+        auto all_done = [&]() { return mbar_wait(bars + X_QEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, XERR_DQ); };
         if (kSplit) {
+            const bool done = ok && all_done();
+            tc_fence_after();
             // partial dV, dK as floats over K, V, Q and dO, which are no longer read: rows of 192 floats, 16-byte chunks swizzled by the row
 #pragma unroll 1
             for (int which = 0; which < 2; ++which) {
@@ -394,11 +408,14 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                         *reinterpret_cast<uint4 *>(row + ((((c0 + e) / 4) ^ (lane_row & 7)) << 4)) = make_uint4(r[e], r[e + 1], r[e + 2], r[e + 3]);
                 }
             }
-        } else if (done) {
+        } else if (ok) {
             // dV and scale*dK go out as bf16 through the V and K tiles (no longer read) and TMA stores; rows past n and columns past d are
-            // clipped by the tensor map
+            // clipped by the tensor map.  dV first, under the last dQ and dK: it is complete once the last dO slot is free.
 #pragma unroll 1
             for (int which = 0; which < 2; ++which) {
+                const bool there = which == 0 ? mbar_wait(bars + X_DOEMPTY + ((niter - 1) & 1), ((niter - 1) >> 1) & 1, abortp, status, XERR_DQ) : all_done();
+                if (!there) break;
+                tc_fence_after();
                 const float mul = which == 0 ? 1.f : scale;
                 uint8_t *stage = which == 0 ? sV : sK;
 #pragma unroll 1
@@ -419,19 +436,15 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                         *reinterpret_cast<uint4 *>(stage + (cabs >> 6) * SM::kBoxK + lane_row * 128 + chunk * 16) = v;
                     }
                 }
-            }
-            fence_proxy_async_smem();
-            mbar_arrive(bars + X_EPI);
-            if (tid == 0 && mbar_wait(bars + X_EPI, 0, abortp, status, XERR_DQ)) {
-                for (int b = 0; b < NB; ++b) {
-                    if (64 * b < d) {       // (a box wholly past the head dimension has nothing to store)
-                        tma_store_4d(&mapdV, sV + b * SM::kBoxK, 64 * b, k0, hk, bb);
-                        tma_store_4d(&mapdK, sK + b * SM::kBoxK, 64 * b, k0, hk, bb);
-                    }
+                fence_proxy_async_smem();
+                mbar_arrive(bars + X_EPI);
+                if (tid == 0 && mbar_wait(bars + X_EPI, which, abortp, status, XERR_DQ)) {
+                    for (int b = 0; b < NB; ++b)
+                        if (64 * b < d) tma_store_4d(which == 0 ? &mapdV : &mapdK, stage + b * SM::kBoxK, 64 * b, k0, hk, bb);     // (a box wholly past the head dimension has nothing to store)
+                    bulk_commit();
                 }
-                bulk_commit();
-                bulk_wait_read<0>();      // shared memory is read before the CTA may exit
             }
+            if (tid == 0) bulk_wait_read<0>();      // shared memory is read before the CTA may exit
         }
     }
     tc_fence_before();

@@ -322,18 +322,19 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         }
         // ---- epilogue of this stream: O / l as bf16 through the stream's Q tile and a TMA store; the row's logsumexp and, in a fused
         // call, the backward's per-row inputs.  (The barrier's phase before is known complete: the loop has waited for it.)
+        // The dO row is requested in front of the wait, all of it: chunk by chunk inside the loop each request's latency was on the job's end.
+        uint4 dov[D / 8];
+        if (want_d)
+#pragma unroll
+            for (int k = 0; k < D / 8; ++k)      // columns past the head dimension count as zeros
+                dov[k] = 8 * k < prep.d ? *reinterpret_cast<const uint4 *>(prep.dO + doff + 8 * k) : make_uint4(0u, 0u, 0u, 0u);
         if (ok && mbar_wait(bars + F2_OB + h, (nk - 1) & 1, abortp, status, ERR2_O)) {
             tc_fence_after();
             const float inv = 1.f / l;
             float dsum = 0.f;
             uint8_t *stage = sQ + h * kTileBytes;
-#pragma unroll 1
-            for (int c = 0; c < D; c += 32) {
-                uint4 dov[4];
-                if (want_d)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)      // columns past the head dimension count as zeros
-                        dov[k] = c + 8 * k < prep.d ? *reinterpret_cast<const uint4 *>(prep.dO + doff + c + 8 * k) : make_uint4(0u, 0u, 0u, 0u);
+            for (int c = 0; c < D; c += 32) {
                 uint32_t o[32];
                 tmem_ld(lane_addr + ocol + c, o);
                 tc_wait_ld();
@@ -346,7 +347,8 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
 #pragma unroll
                         for (int u = 0; u < 8; ++u) v[u] = 0.f;
                     if (want_d) {
-                        const uint32_t gw[4] = {dov[i / 8].x, dov[i / 8].y, dov[i / 8].z, dov[i / 8].w};
+                        const uint4 g = dov[(c + i) / 8];
+                        const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
                             const float2 gg = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gw[u]));

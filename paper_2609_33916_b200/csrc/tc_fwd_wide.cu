@@ -232,6 +232,12 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         const uint32_t pcol = kColP + 64 * h;
         float m_used = -1e30f, l = 0.f;      // (a warpgroup without tiles contributes nothing)
         bool ok = nkt > 0;
+        const bool want_d = prep.dO != nullptr && row < n;
+        const uint4 *dorow = want_d ? reinterpret_cast<const uint4 *>(prep.dO + prep.so.at(bb, hq, row)) : nullptr;
+        if (want_d) {      // the epilogue reads half of this dO row: ask L2 for it now
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(dorow + 4 * NB * h));
+            if (32 * NB * h + 64 < d) asm volatile("prefetch.global.L2 [%0];" ::"l"(dorow + 4 * NB * h + 8));
+        }
         for (int j = h; ok && j < nkt; j += 2) {
             const int t = j >> 1;
             if (!mbar_wait(bars + FW_S + 2 * h + (t & 1), (t >> 1) & 1, abortp, status, ERRW_S)) { ok = false; break; }
@@ -330,9 +336,10 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         }
         // ---- epilogue: the two row sums on the final reference (the larger of the two last seen), O / l as bf16 through the Q tile and a
         // TMA store, half of the columns per warpgroup
-        const bool want_d = prep.dO != nullptr && row < n;
-        const uint4 *dorow = want_d ? reinterpret_cast<const uint4 *>(prep.dO + prep.so.at(bb, hq, row)) : nullptr;
         float dpart = 0.f;
+        uint4 dov[4 * NB];                   // (the whole half row, in front of the waits)
+#pragma unroll
+        for (int k = 0; k < 4 * NB; ++k) dov[k] = want_d && 32 * NB * h + 8 * k < d ? dorow[4 * NB * h + k] : make_uint4(0u, 0u, 0u, 0u);
         xch[h * 128 + lane_row] = make_float2(m_used, l);
         mbar_arrive(bars + FW_X);
         if (ok && mbar_wait(bars + FW_X, 0, abortp, status, ERRW_P) && mbar_wait(bars + FW_DONE, 0, abortp, status, ERRW_O)) {
@@ -341,13 +348,10 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             const float m_all = fmaxf(m_used, other.x);
             const float l_all = l * ex2(m_used - m_all) + other.y * ex2(other.x - m_all);
             const float inv = 1.f / l_all;
-#pragma unroll 1
+#pragma unroll
             for (int c = 0; c < 32 * NB; c += 32) {
                 const int c0 = 32 * NB * h + c;
                 uint32_t o[32];
-                uint4 g[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) g[k] = want_d && c0 + 8 * k < d ? dorow[c0 / 8 + k] : make_uint4(0u, 0u, 0u, 0u);
                 tmem_ld(lane_addr + kColO + c0, o);
                 tc_wait_ld();
 #pragma unroll
@@ -355,7 +359,8 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     float v[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(o[i + u]) * inv;
-                    const uint32_t gw[4] = {g[i / 8].x, g[i / 8].y, g[i / 8].z, g[i / 8].w};
+                    const uint4 g = dov[(c + i) / 8];
+                    const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const float2 gg = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gw[u]));
