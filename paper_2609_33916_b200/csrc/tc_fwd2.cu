@@ -27,17 +27,17 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.f;
 
-enum : uint32_t { ERR2_Q = 0x121, ERR2_K = 0x122, ERR2_V = 0x123, ERR2_S = 0x124, ERR2_P = 0x125, ERR2_O = 0x126, ERR2_ALIGN = 0x128 };
+enum : uint32_t { ERR2_Q = 0x121, ERR2_K = 0x122, ERR2_V = 0x123, ERR2_S = 0x124, ERR2_P = 0x125, ERR2_O = 0x126, ERR2_DO = 0x127, ERR2_ALIGN = 0x128 };
 
 enum { F2_Q = 0, F2_KFULL = 1 /*2*/, F2_KEMPTY = 3 /*2*/, F2_VFULL = 5 /*2*/, F2_VEMPTY = 7 /*2*/, F2_P = 9 /*2: per stream*/,
        F2_SFREE = 11 /*2: per stream, the tile's scores are in registers*/, F2_OB = 13 /*2: per stream, P V of the stream's tile has completed*/,
-       F2_E = 15 /*2: per stream, O staged*/, F2_S = 17 /*[stream][key tile & 1]: 4, as in tc_fwd.cu*/, F2_COUNT = 21 };
+       F2_E = 15 /*2: per stream, O staged*/, F2_S = 17 /*[stream][key tile & 1]: 4, as in tc_fwd.cu*/,
+       F2_DO = 21 /*2: per stream, its dO tile (fused call)*/, F2_COUNT = 23 };
 
 struct FwdPrep2 {
-    const __nv_bfloat16 *dO;
+    int with_bwd;        // fused call: mapdO, Lp and Dp are there
     float *Lp, *Dp;
     int n_pad;
-    Strides so;
     int d;               // columns of a row in memory (<= D)
 };
 
@@ -45,7 +45,7 @@ struct FwdPrep2 {
 template <int D, int KL>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO, float *__restrict__ L, int n,
+               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapdO, float *__restrict__ L, int n,
                int causal, float scale_log2, int npairs, int hpg, int group, int H, float *__restrict__ zero_acc, FwdPrep2 prep,
                unsigned int *status)
 {
@@ -100,6 +100,11 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             if (want1 > 0)
                 for (int b = 0; b < kBoxes; ++b) tma_load_4d(sQ + kTileBytes + b * kBoxBytes, &mapQ, bars + F2_Q, 64 * b, q01, hq, bb);
             if (early > 1) load_k(1);
+            if (prep.with_bwd)      // (what the end of the job reads: into L2)
+                for (int b = 0; b < kBoxes; ++b) {
+                    if (want1 > 0) tma_prefetch_4d(&mapdO, 64 * b, q01, hq, bb);
+                    tma_prefetch_4d(&mapdO, 64 * b, q00, hq, bb);
+                }
         }
     }
     if (warp == 11 && lane == 0) {
@@ -149,7 +154,25 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             if (lane == 0) { load_k(j); ++nk; }
             __syncwarp();
         }
+        // Fused call: the streams' dO tiles, which the epilogues multiply their rows with, go into the K slots as these come free: stream 1's
+        // into that of the last tile but one (stream 1 ends first), stream 0's into the last tile's.  (Read by the row's owner straight from
+        // global memory, 16 bytes of 32 rows at a time, the two tiles were 2 us of LSU work at the end of a job.)
+        int armed_do = 0;       // bit h
+        if (prep.with_bwd)
+#pragma unroll 1
+            for (int h = 1; h >= 0; --h) {
+                const int s = (n0 - 1 + h) & 1, uses = (n0 - s + 1) / 2;
+                if ((h ? n1 : n0) == 0) continue;
+                if (uses > 0 && !mbar_wait(bars + F2_KEMPTY + s, (uses - 1) & 1, abortp, status, ERR2_K)) break;
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(bars + F2_DO + h, kTileBytes);
+                    armed_do |= 1 << h;
+                    for (int b = 0; b < kBoxes; ++b) tma_load_4d(sK + s * kTileBytes + b * kBoxBytes, &mapdO, bars + F2_DO + h, 64 * b, h ? q01 : q00, hq, bb);
+                }
+                __syncwarp();
+            }
         if (lane == 0 && *abortp) {
+            for (int h = 0; h < 2; ++h) mbar_drain_one(bars + F2_DO + h, (armed_do >> h) & 1);
             mbar_drain_one(bars + F2_Q, early > 0 ? 1 : 0);
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
         }
@@ -232,12 +255,6 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         const uint32_t ocol = kColO + h * D, pcol = kColP + 64 * h;
         float m_used = -1e30f, l = 0.f;
         bool ok = nk > 0;
-        const bool want_d = prep.dO != nullptr && ok && row < n;
-        const size_t doff = want_d ? prep.so.at(bb, hq, row) : 0;
-        if (want_d) {      // the epilogue reads this dO row: ask L2 for it now
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(prep.dO + doff));
-            if (D == 128 && prep.d > 64) asm volatile("prefetch.global.L2 [%0];" ::"l"(prep.dO + doff + 64));
-        }
         for (int t = 0; ok && t < nk; ++t) {
             if (!mbar_wait(bars + F2_S + 2 * h + (t & 1), (t >> 1) & 1, abortp, status, ERR2_S)) { ok = false; break; }
             tc_fence_after();
@@ -322,18 +339,14 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         }
         // ---- epilogue of this stream: O / l as bf16 through the stream's Q tile and a TMA store; the row's logsumexp and, in a fused
         // call, the backward's per-row inputs.  (The barrier's phase before is known complete: the loop has waited for it.)
-        // The dO row is requested in front of the wait, all of it: chunk by chunk inside the loop each request's latency was on the job's end.
-        uint4 dov[D / 8];
-        if (want_d)
-#pragma unroll
-            for (int k = 0; k < D / 8; ++k)      // columns past the head dimension count as zeros
-                dov[k] = 8 * k < prep.d ? *reinterpret_cast<const uint4 *>(prep.dO + doff + 8 * k) : make_uint4(0u, 0u, 0u, 0u);
-        if (ok && mbar_wait(bars + F2_OB + h, (nk - 1) & 1, abortp, status, ERR2_O)) {
+        const bool want_d = prep.with_bwd != 0;
+        const uint8_t *drow = sK + ((n0 - 1 + h) & 1) * kTileBytes + lane_row * 128;       // this row of the dO tile
+        if (ok && mbar_wait(bars + F2_OB + h, (nk - 1) & 1, abortp, status, ERR2_O) && (!want_d || mbar_wait(bars + F2_DO + h, 0, abortp, status, ERR2_DO))) {
             tc_fence_after();
             const float inv = 1.f / l;
             float dsum = 0.f;
             uint8_t *stage = sQ + h * kTileBytes;
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < D; c += 32) {
                 uint32_t o[32];
                 tmem_ld(lane_addr + ocol + c, o);
@@ -346,8 +359,9 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                     if (KL < D / 16 && c + i >= 16 * KL)      // columns no product wrote
 #pragma unroll
                         for (int u = 0; u < 8; ++u) v[u] = 0.f;
-                    if (want_d) {
-                        const uint4 g = dov[(c + i) / 8];
+                    const int cabs = c + i, chunk = ((cabs & 63) >> 3) ^ (lane_row & 7);       // 128-byte swizzle, as the maps expect
+                    if (want_d) {      // (columns past the head dimension and rows past n are zeros)
+                        const uint4 g = *reinterpret_cast<const uint4 *>(drow + (cabs >> 6) * kBoxBytes + chunk * 16);
                         const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
@@ -356,14 +370,13 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                             dsum = fmaf(v[2 * u + 1], gg.y, dsum);
                         }
                     }
-                    const int cabs = c + i, chunk = ((cabs & 63) >> 3) ^ (lane_row & 7);       // 128-byte swizzle, as the map expects
                     *reinterpret_cast<uint4 *>(stage + (cabs >> 6) * kBoxBytes + lane_row * 128 + chunk * 16) =
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
                 }
             }
             fence_proxy_async_smem();
             mbar_arrive(bars + F2_E + h);
-            if (prep.dO != nullptr && row < prep.n_pad) {
+            if (want_d && row < prep.n_pad) {
                 const size_t prow = (size_t)bh * prep.n_pad + row;
                 prep.Dp[prow] = row < n ? -dsum : 0.f;
                 prep.Lp[prow] = row < n ? -(m_used + log2f(l)) : -INFINITY;
@@ -386,7 +399,7 @@ template <int D, int KL>
 cudaError_t launch(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const FwdForBwd &fb, cudaStream_t st)
 {
     constexpr int kSmem = 6 * 128 * D * 2 + 8 * F2_COUNT + 16;
-    CUtensorMap mq, mk, mv, mo;
+    CUtensorMap mq, mk, mv, mo, mdo;
     const auto bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     // p.d <= D columns exist in memory: loads fill the rest of a box with zeros, the store drops it
     if (!make_tensor_map_4d_strided(&mq, Q, bf, 2, p.B, p.H, p.n, p.d, p.sq.row, p.sq.head, p.sq.batch, 128, 64) ||
@@ -394,13 +407,15 @@ cudaError_t launch(const Problem &p, const void *Q, const void *K, const void *V
         !make_tensor_map_4d_strided(&mv, V, bf, 2, p.B, p.kv_heads(), p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64) ||
         !make_tensor_map_4d_strided(&mo, O, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64))
         return cudaErrorInvalidValue;
+    mdo = mo;
+    if (fb.dO && !make_tensor_map_4d_strided(&mdo, fb.dO, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64)) return cudaErrorInvalidValue;
     const cudaError_t e = allow_smem<tc_fwd2_kernel<D, KL>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + BM - 1) / BM, npairs = (nqt + 1) / 2;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_dependent(tc_fwd2_kernel<D, KL>, dim3((unsigned)(npairs * p.BH())), dim3(kThreads), (size_t)kSmem, st, mq, mk, mv, mo, L,
+    return launch_dependent(tc_fwd2_kernel<D, KL>, dim3((unsigned)(npairs * p.BH())), dim3(kThreads), (size_t)kSmem, st, mq, mk, mv, mo, mdo, L,
                             p.n, p.causal, p.scale * kLog2e, npairs, heads_per_group(p, npairs), p.group(), p.H, fb.zero_acc,
-                            FwdPrep2{(const __nv_bfloat16 *)fb.dO, fb.Lp, fb.Dp, nqt * BM, p.so, p.d}, device_status_ptr());
+                            FwdPrep2{fb.dO != nullptr, fb.Lp, fb.Dp, nqt * BM, p.d}, device_status_ptr());
 }
 
 }  // namespace

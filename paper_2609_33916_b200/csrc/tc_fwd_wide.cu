@@ -34,11 +34,13 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.f;
 
-enum : uint32_t { ERRW_Q = 0x141, ERRW_K = 0x142, ERRW_V = 0x143, ERRW_S = 0x144, ERRW_P = 0x145, ERRW_O = 0x146, ERRW_M = 0x147, ERRW_ALIGN = 0x148 };
+enum : uint32_t { ERRW_Q = 0x141, ERRW_K = 0x142, ERRW_V = 0x143, ERRW_S = 0x144, ERRW_P = 0x145, ERRW_O = 0x146, ERRW_M = 0x147, ERRW_ALIGN = 0x148,
+                ERRW_DO = 0x149 };
 
 enum { FW_Q = 0, FW_KFULL = 1 /*3*/, FW_KEMPTY = 4 /*3*/, FW_VFULL = 7 /*3*/, FW_VEMPTY = 10 /*3*/, FW_P = 13 /*2: by tile parity*/,
        FW_SFREE = 15 /*2*/, FW_OB = 17 /*2: P V of the tile has completed*/, FW_M = 19 /*2: the row references of the tile are posted*/,
-       FW_S = 21 /*[parity][tile / 2 & 1]: 4*/, FW_X = 25 /*epilogue exchange*/, FW_E = 26 /*O staged*/, FW_DONE = 27 /*last P V*/, FW_COUNT = 28 };
+       FW_S = 21 /*[parity][tile / 2 & 1]: 4*/, FW_X = 25 /*epilogue exchange*/, FW_E = 26 /*O staged*/, FW_DONE = 27 /*last P V*/,
+       FW_DO = 28 /*the dO tile (fused call)*/, FW_COUNT = 29 };
 
 template <int NB>
 struct WideFwd {
@@ -56,18 +58,16 @@ struct WideFwd {
 };
 static_assert(WideFwd<3>::kTotal <= 232448 && WideFwd<4>::kTotal <= 232448, "shared memory of one CTA");
 
-// Fused call only (dO == nullptr otherwise): the backward's per-row inputs, as in tc_fwd.cu
 struct WidePrep {
-    const __nv_bfloat16 *dO;
+    int with_bwd;        // fused call: mapdO, Lp and Dp are there (what the forward prepares: tc_fwd.cu)
     float *Lp, *Dp, *zero_acc;
     int n_pad;
-    Strides so;
 };
 
 template <int NB>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                   const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO, float *__restrict__ L, int n, int d,
+                   const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapdO, float *__restrict__ L, int n, int d,
                    int causal, float scale_log2, int nqt, int hpg, int group, int H, WidePrep prep,
                    unsigned int *status)
 {
@@ -112,6 +112,8 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             mbar_arrive_expect_tx(bars + FW_Q, S::kQ);
             for (int b = 0; b < NB; ++b) tma_load_4d(sQ + b * S::kBox, &mapQ, bars + FW_Q, 64 * b, q0, hq, bb);
             for (int g = 0; g < early_k; ++g) load_k(g);
+            if (prep.with_bwd)      // (what the end of the job reads: into L2)
+                for (int b = 0; b < NB; ++b) tma_prefetch_4d(&mapdO, 64 * b, q0, hq, bb);
         }
     }
     if (warp == 11 && lane == 0) {
@@ -139,6 +141,7 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     if (gridDim.x <= 512) grid_launch_dependents();      // (short launches only: see tc_fwd.cu)
     const uint32_t tbase = *tmem_base_p;
     const int nkt = (*abortp == 0) ? nkt_want : 0;       // misaligned shared memory: every role is a no-op
+    const int dslot = NB == 3 ? nkt & 1 : 0;             // first K slot of the dO tile: that of the last tile but one, or the first two
 
     if (warp >= 8) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");      // (128 x 88 + 256 x 208 = 384 x 168, the launch's registers)
@@ -154,7 +157,23 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             if (lane == 0) { load_k(g); ++nk; }
             __syncwarp();
         }
+        // fused call: the dO tile, which the epilogue multiplies its rows with, goes over K slots that have come free (see tc_fwd2.cu)
+        int armed_do = 0;
+        if (prep.with_bwd && nkt > 0) {
+            bool free = true;
+            for (int s = dslot; free && s < dslot + (NB == 3 ? 1 : 2); ++s) {
+                const int uses = (nkt * S::kChunks - s + S::kKSlots - 1) / S::kKSlots;
+                free = uses <= 0 || mbar_wait(bars + FW_KEMPTY + s, (uses - 1) & 1, abortp, status, ERRW_K);
+            }
+            if (free && lane == 0) {
+                mbar_arrive_expect_tx(bars + FW_DO, NB * S::kBox);
+                armed_do = 1;
+                for (int b = 0; b < NB; ++b) tma_load_4d(sK + dslot * S::kKSlot + b * S::kBox, &mapdO, bars + FW_DO, 64 * b, q0, hq, bb);
+            }
+            __syncwarp();
+        }
         if (lane == 0 && *abortp) {
+            mbar_drain_one(bars + FW_DO, armed_do);
             mbar_drain_one(bars + FW_Q, early_k > 0 ? 1 : 0);
             for (int s = 0; s < S::kKSlots; ++s) mbar_drain_one(bars + FW_KFULL + s, nk > s ? (nk - s + S::kKSlots - 1) / S::kKSlots : 0);
         }
@@ -232,12 +251,6 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         const uint32_t pcol = kColP + 64 * h;
         float m_used = -1e30f, l = 0.f;      // (a warpgroup without tiles contributes nothing)
         bool ok = nkt > 0;
-        const bool want_d = prep.dO != nullptr && row < n;
-        const uint4 *dorow = want_d ? reinterpret_cast<const uint4 *>(prep.dO + prep.so.at(bb, hq, row)) : nullptr;
-        if (want_d) {      // the epilogue reads half of this dO row: ask L2 for it now
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(dorow + 4 * NB * h));
-            if (32 * NB * h + 64 < d) asm volatile("prefetch.global.L2 [%0];" ::"l"(dorow + 4 * NB * h + 8));
-        }
         for (int j = h; ok && j < nkt; j += 2) {
             const int t = j >> 1;
             if (!mbar_wait(bars + FW_S + 2 * h + (t & 1), (t >> 1) & 1, abortp, status, ERRW_S)) { ok = false; break; }
@@ -337,18 +350,18 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         // ---- epilogue: the two row sums on the final reference (the larger of the two last seen), O / l as bf16 through the Q tile and a
         // TMA store, half of the columns per warpgroup
         float dpart = 0.f;
-        uint4 dov[4 * NB];                   // (the whole half row, in front of the waits)
-#pragma unroll
-        for (int k = 0; k < 4 * NB; ++k) dov[k] = want_d && 32 * NB * h + 8 * k < d ? dorow[4 * NB * h + k] : make_uint4(0u, 0u, 0u, 0u);
+        const bool want_d = prep.with_bwd != 0;
+        const uint8_t *drow = sK + dslot * S::kKSlot + lane_row * 128;       // this row of the dO tile
         xch[h * 128 + lane_row] = make_float2(m_used, l);
         mbar_arrive(bars + FW_X);
-        if (ok && mbar_wait(bars + FW_X, 0, abortp, status, ERRW_P) && mbar_wait(bars + FW_DONE, 0, abortp, status, ERRW_O)) {
+        if (ok && mbar_wait(bars + FW_X, 0, abortp, status, ERRW_P) && mbar_wait(bars + FW_DONE, 0, abortp, status, ERRW_O) &&
+            (!want_d || mbar_wait(bars + FW_DO, 0, abortp, status, ERRW_DO))) {
             tc_fence_after();
             const float2 other = xch[(h ^ 1) * 128 + lane_row];
             const float m_all = fmaxf(m_used, other.x);
             const float l_all = l * ex2(m_used - m_all) + other.y * ex2(other.x - m_all);
             const float inv = 1.f / l_all;
-#pragma unroll
+#pragma unroll 1
             for (int c = 0; c < 32 * NB; c += 32) {
                 const int c0 = 32 * NB * h + c;
                 uint32_t o[32];
@@ -359,15 +372,17 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                     float v[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) v[u] = __uint_as_float(o[i + u]) * inv;
-                    const uint4 g = dov[(c + i) / 8];
-                    const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
+                    const int cabs = c0 + i, chunk = ((cabs & 63) >> 3) ^ (lane_row & 7);       // 128-byte swizzle, as the maps expect
+                    if (want_d) {      // (columns past the head dimension and rows past n are zeros)
+                        const uint4 g = *reinterpret_cast<const uint4 *>(drow + (cabs >> 6) * S::kBox + chunk * 16);
+                        const uint32_t gw[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const float2 gg = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gw[u]));
-                        dpart = fmaf(v[2 * u], gg.x, dpart);
-                        dpart = fmaf(v[2 * u + 1], gg.y, dpart);
+                        for (int u = 0; u < 4; ++u) {
+                            const float2 gg = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gw[u]));
+                            dpart = fmaf(v[2 * u], gg.x, dpart);
+                            dpart = fmaf(v[2 * u + 1], gg.y, dpart);
+                        }
                     }
-                    const int cabs = c0 + i, chunk = ((cabs & 63) >> 3) ^ (lane_row & 7);       // 128-byte swizzle, as the map expects
                     *reinterpret_cast<uint4 *>(sQ + (cabs >> 6) * S::kBox + lane_row * 128 + chunk * 16) =
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
                 }
@@ -375,7 +390,7 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             if (h == 1) mref[lane_row] = dpart;      // (no tile needs the reference any more)
             fence_proxy_async_smem();
             mbar_arrive(bars + FW_E);
-            if (prep.dO != nullptr && h == 0 && mbar_wait(bars + FW_E, 0, abortp, status, ERRW_O)) {
+            if (want_d && h == 0 && mbar_wait(bars + FW_E, 0, abortp, status, ERRW_O)) {
                 // both halves of the row are in: the backward's per-row inputs, in its padded layout
                 const size_t prow = (size_t)bh * prep.n_pad + row;
                 prep.Dp[prow] = row < n ? -(dpart + mref[lane_row]) : 0.f;
@@ -400,7 +415,7 @@ cudaError_t launch(const Problem &p, const void *Q, const void *K, const void *V
                    cudaStream_t st)
 {
     using S = WideFwd<NB>;
-    CUtensorMap mq, mk, mv, mo;
+    CUtensorMap mq, mk, mv, mo, mdo;
     const auto bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     // p.d <= 64 NB columns exist in memory: loads fill the rest of a box with zeros, the store drops it
     if (!make_tensor_map_4d_strided(&mq, Q, bf, 2, p.B, p.H, p.n, p.d, p.sq.row, p.sq.head, p.sq.batch, 128, 64) ||
@@ -408,13 +423,15 @@ cudaError_t launch(const Problem &p, const void *Q, const void *K, const void *V
         !make_tensor_map_4d_strided(&mv, V, bf, 2, p.B, p.kv_heads(), p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 64, 64) ||
         !make_tensor_map_4d_strided(&mo, O, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64))
         return cudaErrorInvalidValue;
+    mdo = mo;
+    if (fb.dO && !make_tensor_map_4d_strided(&mdo, fb.dO, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64)) return cudaErrorInvalidValue;
     const cudaError_t e = allow_smem<tc_fwd_wide_kernel<NB>>(S::kTotal);
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + BM - 1) / BM;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_dependent(tc_fwd_wide_kernel<NB>, dim3((unsigned)(nqt * p.BH())), dim3(kThreads), (size_t)S::kTotal, st, mq, mk, mv, mo, L,
+    return launch_dependent(tc_fwd_wide_kernel<NB>, dim3((unsigned)(nqt * p.BH())), dim3(kThreads), (size_t)S::kTotal, st, mq, mk, mv, mo, mdo, L,
                             p.n, p.d, p.causal, p.scale * kLog2e, nqt, heads_per_group(p, nqt), p.group(), p.H,
-                            WidePrep{(const __nv_bfloat16 *)fb.dO, fb.Lp, fb.Dp, fb.zero_acc, nqt * BM, p.so}, device_status_ptr());
+                            WidePrep{fb.dO != nullptr, fb.Lp, fb.Dp, fb.zero_acc, nqt * BM}, device_status_ptr());
 }
 
 }  // namespace
