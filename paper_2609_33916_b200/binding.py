@@ -1,4 +1,4 @@
-"""ctypes binding of libmoa_attn.so: the same entry points as include/moa_attn.h.
+"""Binding of libmoa_attn.so (ctypes; the launching calls through _pycall): the same entry points as include/moa_attn.h.
 
 Argument marshalling only -- every step of the attention path runs in the
 library's CUDA kernels.  Tensor arguments may be torch CUDA tensors (their
@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libmoa_attn.so")
@@ -170,6 +171,43 @@ def strides_of(t):
     return (t.stride(2), t.stride(1), t.stride(0))
 
 
+# The calls that go through the extension _pycall (csrc/pycall.c): name, descriptor, pointer arguments, whether the last of these is a
+# workspace (whose size follows).  The others are rare and go through ctypes, which takes 2.5 us for the arguments of a decode call where
+# the extension takes 0.8: with a kernel of 3.9 us (B1 H16 n1000 d64) the call went from 5.4 to 4.3.
+_ENTRIES = (("moa_attn_fwd", moa_attn_desc, 6, True), ("moa_attn_bwd", moa_attn_desc, 10, True),
+            ("moa_attn_fused_fwd_bwd", moa_attn_desc, 10, True), ("moa_decode_attn", moa_decode_desc, 6, True),
+            ("moa_rmsnorm_fwd", moa_rmsnorm_desc, 4, False), ("moa_rmsnorm_bwd", moa_rmsnorm_desc, 8, True), ("moa_gemm", moa_gemm_desc, 4, False),
+            ("moa_gated_mlp_fwd", moa_mlp_desc, 9, False), ("moa_gated_mlp_bwd", moa_mlp_desc, 13, True))
+_ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD = range(len(_ENTRIES))
+_invoke = _fill = None
+_load_lock = threading.Lock()
+
+
+def _load():
+    """_pycall.invoke, with the library's functions registered."""
+    global _invoke, _fill
+    with _load_lock:
+        if _invoke is None:
+            L = lib()
+            try:
+                from . import _pycall
+            except ImportError as e:
+                raise RuntimeError("_pycall.so is missing: run `python -m paper_2609_33916_b200.build` (there is no fallback path)") from e
+            for name, desc, pointers, ws in _ENTRIES:
+                _pycall.add_entry(ctypes.cast(getattr(L, name), ctypes.c_void_p).value, desc, pointers, ws)
+            _pycall.set_current_stream(lambda: _current_stream())
+            _fill, _invoke = _pycall.fill, _pycall.invoke
+    return _invoke
+
+
+def fill_pointers(struct, objects):
+    """A tuple of tensors (their addresses), integers or None, in order, into the fields of a struct of pointers and sizes."""
+    if _invoke is None:
+        _load()
+    _fill(struct, objects)
+    return struct
+
+
 def _ptr(x):
     """What a c_void_p argument takes: the address of a torch tensor, an integer address, or None."""
     if x is None or isinstance(x, int):
@@ -193,6 +231,9 @@ def _current_stream() -> int:
     if raw is not None and device is not None:
         global _current_stream
         _current_stream = lambda: raw(device())        # noqa: E731
+        _load()
+        from . import _pycall
+        _pycall.set_current_stream(raw, device)
     return stream
 
 
@@ -221,17 +262,14 @@ def moa_attn_workspace_bytes(desc: moa_attn_desc, op: int) -> int:
 
 
 def moa_attn_fwd(desc, Q, K, V, O, L, ws=None, stream=None, ws_bytes=None, check=True) -> int:
-    s = lib().moa_attn_fwd(ctypes.byref(desc), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(L), _ptr(ws),
-                           _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
+    s = (_invoke or _load())(_ATTN_FWD, desc, Q, K, V, O, L, ws, ws_bytes, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_attn_fwd")
     return s
 
 
 def moa_attn_bwd(desc, Q, K, V, O, L, dO, dQ, dK, dV, ws=None, stream=None, ws_bytes=None, check=True) -> int:
-    s = lib().moa_attn_bwd(ctypes.byref(desc), _ptr(Q), _ptr(K), _ptr(V), _ptr(O), _ptr(L), _ptr(dO),
-                           _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(ws),
-                           _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
+    s = (_invoke or _load())(_ATTN_BWD, desc, Q, K, V, O, L, dO, dQ, dK, dV, ws, ws_bytes, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_attn_bwd")
     return s
@@ -250,9 +288,7 @@ def moa_attn_bwd_static_scratch(desc, Q, K, V, O, L, dO, dQ, dK, dV, stream=None
 
 def moa_attn_fused_fwd_bwd(desc, Q, K, V, dO, O, L, dQ, dK, dV, ws=None, stream=None, ws_bytes=None,
                            check=True) -> int:
-    s = lib().moa_attn_fused_fwd_bwd(ctypes.byref(desc), _ptr(Q), _ptr(K), _ptr(V), _ptr(dO), _ptr(O),
-                                     _ptr(L), _ptr(dQ), _ptr(dK), _ptr(dV), _ptr(ws),
-                                     _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
+    s = (_invoke or _load())(_ATTN_FUSED, desc, Q, K, V, dO, O, L, dQ, dK, dV, ws, ws_bytes, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_attn_fused_fwd_bwd")
     return s
@@ -277,7 +313,7 @@ def moa_rmsnorm_workspace_bytes(desc) -> int:
 
 
 def moa_rmsnorm_fwd(desc, x, g, y, r=None, stream=None, check=True) -> int:
-    s = lib().moa_rmsnorm_fwd(ctypes.byref(desc), _ptr(x), _ptr(g), _ptr(y), _ptr(r), _stream(stream))
+    s = (_invoke or _load())(_NORM_FWD, desc, x, g, y, r, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_rmsnorm_fwd")
     return s
@@ -285,8 +321,7 @@ def moa_rmsnorm_fwd(desc, x, g, y, r=None, stream=None, check=True) -> int:
 
 def moa_rmsnorm_bwd(desc, x, g, r, dy, dx, dg, ws=None, stream=None, ws_bytes=None, check=True, dx_add=None) -> int:
     """dx_add (optional, [n,d]): added to dx (the gradient arriving along a residual connection)."""
-    s = lib().moa_rmsnorm_bwd(ctypes.byref(desc), _ptr(x), _ptr(g), _ptr(r), _ptr(dy), _ptr(dx_add), _ptr(dx), _ptr(dg), _ptr(ws),
-                              _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
+    s = (_invoke or _load())(_NORM_BWD, desc, x, g, r, dy, dx_add, dx, dg, ws, ws_bytes, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_rmsnorm_bwd")
     return s
@@ -310,7 +345,7 @@ def make_gemm_desc(M, N, K, a_layout=0, b_layout=0, dtype=MOA_BF16) -> moa_gemm_
 
 
 def moa_gemm(desc, A, B, C, R=None, stream=None, check=True) -> int:
-    s = lib().moa_gemm(ctypes.byref(desc), _ptr(A), _ptr(B), _ptr(R), _ptr(C), _stream(stream))
+    s = (_invoke or _load())(_GEMM, desc, A, B, R, C, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_gemm")
     return s
@@ -326,8 +361,7 @@ def moa_gated_mlp_workspace_bytes(desc) -> int:
 
 def moa_gated_mlp_fwd(desc, x, W1, W3, W2, a, u, h, y, stream=None, check=True, res=None) -> int:
     """res (optional, [n,d]): added to y (the block's residual connection)."""
-    s = lib().moa_gated_mlp_fwd(ctypes.byref(desc), _ptr(x), _ptr(W1), _ptr(W3), _ptr(W2), _ptr(res), _ptr(a), _ptr(u), _ptr(h),
-                                _ptr(y), _stream(stream))
+    s = (_invoke or _load())(_MLP_FWD, desc, x, W1, W3, W2, res, a, u, h, y, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_gated_mlp_fwd")
     return s
@@ -335,9 +369,7 @@ def moa_gated_mlp_fwd(desc, x, W1, W3, W2, a, u, h, y, stream=None, check=True, 
 
 def moa_gated_mlp_bwd(desc, x, W1, W3, W2, a, u, h, dy, dx, dW1, dW3, dW2, ws=None, stream=None, ws_bytes=None,
                       check=True) -> int:
-    s = lib().moa_gated_mlp_bwd(ctypes.byref(desc), _ptr(x), _ptr(W1), _ptr(W3), _ptr(W2), _ptr(a), _ptr(u), _ptr(h),
-                                _ptr(dy), _ptr(dx), _ptr(dW1), _ptr(dW3), _ptr(dW2), _ptr(ws),
-                                _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
+    s = (_invoke or _load())(_MLP_BWD, desc, x, W1, W3, W2, a, u, h, dy, dx, dW1, dW3, dW2, ws, ws_bytes, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_gated_mlp_bwd")
     return s
@@ -366,8 +398,7 @@ def moa_decode_workspace_bytes(desc: moa_decode_desc) -> int:
 
 
 def moa_decode_attn(desc, q, K, V, out, lse=None, ws=None, stream=None, ws_bytes=None, check=True) -> int:
-    s = lib().moa_decode_attn(ctypes.byref(desc), _ptr(q), _ptr(K), _ptr(V), _ptr(out), _ptr(lse), _ptr(ws),
-                              _nbytes(ws) if ws_bytes is None else ws_bytes, _stream(stream))
+    s = (_invoke or _load())(_DECODE, desc, q, K, V, out, lse, ws, ws_bytes, stream)
     if check and s != MOA_OK:
         raise MoaError(s, "moa_decode_attn")
     return s

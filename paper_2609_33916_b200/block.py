@@ -85,13 +85,11 @@ class TransformerBlock:
     def _arrays(self, x, w, dy):
         """The addresses of this call (taken anew each time: any of the tensors may have been replaced)."""
         g = self.grads
-        return mb.moa_block_arrays(
-            *[t.data_ptr() for t in (x, w["g1"], w["g2"], w["Wqkv"], w["Wo"], w["W1"], w["W3"], w["W2"], self.h1, self.qkv, self.o, self.x2,
-                                     self.h2, self.a, self.u, self.h, self.y, self.r1, self.r2, self.L)],
-            None if dy is None else dy.data_ptr(),
-            *[t.data_ptr() for t in (self.dh2, self.dx2, self.do, self.dqkv, self.dh1, self.dx, g["g1"], g["g2"], self.gqkv, g["Wo"],
-                                     g["W1"], g["W3"], g["W2"], self.nws, self.aws, self.mws)],
-            self.nws.nbytes, self.aws.nbytes, self.mws.nbytes)
+        nws, aws, mws = self.nws, self.aws, self.mws
+        return mb.fill_pointers(mb.moa_block_arrays(), (
+            x, w["g1"], w["g2"], w["Wqkv"], w["Wo"], w["W1"], w["W3"], w["W2"], self.h1, self.qkv, self.o, self.x2, self.h2, self.a, self.u,
+            self.h, self.y, self.r1, self.r2, self.L, dy, self.dh2, self.dx2, self.do, self.dqkv, self.dh1, self.dx, g["g1"], g["g2"],
+            self.gqkv, g["Wo"], g["W1"], g["W3"], g["W2"], nws, aws, mws, nws.nbytes, aws.nbytes, mws.nbytes))
 
     def forward(self, x, w, stream=None):
         if self.packed:

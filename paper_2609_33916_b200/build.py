@@ -5,6 +5,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -12,6 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libmoa_attn.so")
+PYCALL = os.path.join(HERE, "_pycall.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -66,7 +68,19 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if force or jobs or _stale(LIB, objs):
         cmd = [_nvcc(), "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"]
         run(cmd)
+    build_pycall(force)
     return LIB
+
+
+def build_pycall(force: bool = False) -> str:
+    """The marshalling extension of binding.py (plain C, no CUDA)."""
+    src = os.path.join(CSRC, "pycall.c")
+    if force or _stale(PYCALL, [src]):
+        r = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", PYCALL],
+                           capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"the compiler failed for {src}:\n{r.stderr}")
+    return PYCALL
 
 
 if __name__ == "__main__":
