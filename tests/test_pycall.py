@@ -1,0 +1,63 @@
+"""The marshalling extension behind the binding's launching calls: what it takes for an address, a workspace size and a descriptor, seen from
+refusals that need no GPU, and from several threads."""
+import ctypes
+import threading
+
+import pytest
+import torch
+
+from paper_2609_33916_b200 import binding as mb
+from paper_2609_33916_b200 import build
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def _decode(desc, ws, **kw):
+    q = torch.zeros(64)
+    return mb.moa_decode_attn(desc, q, q, q, q, None, ws, check=False, **kw)
+
+
+def test_descriptors_of_another_type_and_things_without_an_address_are_refused():
+    desc = mb.make_decode_desc(1, 1, 8, 64, 0.1)
+    with pytest.raises(TypeError):
+        _decode(mb.make_gemm_desc(8, 8, 8), None)
+    with pytest.raises(AttributeError):
+        mb.moa_decode_attn(desc, "q", None, None, None)
+    with pytest.raises(OverflowError):
+        mb.moa_decode_attn(desc, -1, None, None, None)
+
+
+@pytest.mark.parametrize("ws,ws_bytes,want", [(None, None, "MOA_ERR_WORKSPACE"), (4096, 1, "MOA_ERR_WORKSPACE")])
+def test_workspace_sizes(ws, ws_bytes, want):
+    desc = mb.make_desc(1, 1, 256, 64, False, 0.1)
+    a = 4096
+    got = mb.moa_attn_bwd(desc, a, a, a, a, a, a, a, a, a, ws, stream=0, ws_bytes=ws_bytes, check=False)
+    assert got == getattr(mb, want)
+    with pytest.raises(mb.MoaError):
+        mb.moa_attn_bwd(desc, a, a, a, a, a, a, a, a, a, torch.zeros(8, dtype=torch.uint8), stream=0)
+
+
+@pytest.mark.parametrize("count", [1, 3])
+def test_fill(count):
+    class Words(ctypes.Structure):
+        _fields_ = [("w", ctypes.c_uint64 * 3)]
+
+    t = torch.zeros(4)
+    words = mb.fill_pointers(Words(), (t, None, 7)[:count])
+    assert list(words.w) == [t.data_ptr(), 0, 7 if count == 3 else 0]
+    with pytest.raises(ValueError):
+        mb.fill_pointers(Words(), (1, 2, 3, 4))
+
+
+def test_from_several_threads():
+    desc = mb.make_decode_desc(1, 1, -1, 64, 0.1)
+    got = []
+    threads = [threading.Thread(target=lambda: got.extend(_decode(desc, None, stream=0) for _ in range(500))) for _ in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert got == [mb.MOA_ERR_INVALID_ARG] * 2000
