@@ -120,8 +120,11 @@ template <typename T> __device__ __forceinline__ float4 as_stored(float4 v)
                        to_float(from_float<T>(v.w)));
 }
 
+// kDeep: many steps of the products unrolled, their loads in flight together.  For launches of one tile per CTA and at most a CTA (a warp per
+// scheduler) per SM, where the time is that tile's latency: fused B1 H1 n128 d64 12.3 -> 11.2 us, B1 H1 n128 d128 15.3 -> 14.1, B1 H8 n64 d64
+// 11.6 -> 10.5.  From two tiles per CTA on it was slower (B1 H2 n300 d64 21.7 -> 27.9).
 // out[i][b] = A[a_row0 + i][:] . B[tx + 16 b][:], contraction over D; rows of D + 4 floats
-template <int R, int NB, int D>
+template <int R, int NB, int D, bool kDeep>
 __device__ __forceinline__ void dot_rows(float (&out)[R][NB], const float *A, const float *B, int a_row0, int tx)
 {
     constexpr int LD = D + 4;
@@ -131,7 +134,7 @@ __device__ __forceinline__ void dot_rows(float (&out)[R][NB], const float *A, co
 #pragma unroll
         for (int b = 0; b < NB; ++b) acc[i][b] = 0ull;
     const float *ap = A + a_row0 * LD, *bp = B + tx * LD;
-#pragma unroll 2
+#pragma unroll (kDeep ? 8 : 2)
     for (int k = 0; k < D; k += 4) {
         ulonglong2 av[R], bv[NB];
 #pragma unroll
@@ -158,13 +161,13 @@ __device__ __forceinline__ void dot_rows(float (&out)[R][NB], const float *A, co
 
 // acc[i2][c] (rows 2 i2 and 2 i2 + 1 of the thread's R rows, packed) += sum_{j < K} W[j][R rows] X[j][4 tx + 64 v + 0..3];
 // W: rows of LW floats, the thread's R rows consecutive at w0; X: rows of D + 4 floats
-template <int R, int K, int D>
+template <int R, int K, int D, bool kDeep>
 __device__ __forceinline__ void add_rows(uint64_t (&acc)[R / 2][D / 16], const float *W, int LW, int w0, const float *X, int tx)
 {
     static_assert(R == 2 || R % 4 == 0, "a thread's rows are read 8 or 16 bytes at a time");
     constexpr int LD = D + 4;
     const float *wp = W + w0, *xp = X + 4 * tx;
-#pragma unroll 4
+#pragma unroll (kDeep ? 16 : 4)
     for (int j = 0; j < K; ++j) {
         uint64_t wv[R / 2], xv[D / 16];
         if (R == 2) {
@@ -225,7 +228,7 @@ struct SimtFwd {
     static constexpr size_t kSmem = kFloats * sizeof(float);
 };
 
-template <typename T, int R, int D>
+template <typename T, int R, int D, bool kDeep>
 __global__ void __launch_bounds__(SNT, R == 8 ? 3 : D == 128 ? 2 : 4)
 simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, T *__restrict__ O,
                 float *__restrict__ L, const T *__restrict__ dO, float *__restrict__ Dv, float *__restrict__ dQzero, int n,
@@ -273,7 +276,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         cp_wait<1>();                 // K (and Q) are here; V may still be on its way
         __syncthreads();
         float s[R][4];
-        dot_rows<R, 4, D>(s, Qs, Ks, ty * R, tx);
+        dot_rows<R, 4, D, kDeep>(s, Qs, Ks, ty * R, tx);
         __syncthreads();
         if (more) tile_in<T, BN, D>(Ks, K, k0 + step, n);      // runs under the softmax and the P V product
         cp_commit();
@@ -339,7 +342,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         }
         cp_wait<1>();                 // V is here; the next K may still be on its way
         __syncthreads();              // (also: every lane's part of P^T is written)
-        add_rows<R, BN, D>(o, Pw, LP, (ty % 2) * R, Vs, tx);
+        add_rows<R, BN, D, kDeep>(o, Pw, LP, (ty % 2) * R, Vs, tx);
         __syncthreads();
         if (more) tile_in<T, BN, D>(Vs, V, k0 + step, n);
         cp_commit();
@@ -500,7 +503,7 @@ struct SimtBwd {
     static_assert(BN <= BM, "the partial dK, dV are staged over Q, dO");
 };
 
-template <typename T, int R, int D>
+template <typename T, int R, int D, bool kDeep>
 __global__ void __launch_bounds__(SNT, 2)
 simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
                    const T *__restrict__ dO, const float *__restrict__ L, const float *__restrict__ Dv,
@@ -554,7 +557,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
         __syncthreads();
         const bool mask = k0 + BN > n || q0 + BM > n || (causal && k0 + BN - 1 > q0);
         float p[R][QB];
-        dot_rows<R, QB, D>(p, Ks, Qs, ty * R, tx);
+        dot_rows<R, QB, D, kDeep>(p, Ks, Qs, ty * R, tx);
 #pragma unroll
         for (int b = 0; b < QB; ++b) {
             const int q = tx + 16 * b, row = q0 + q;
@@ -583,10 +586,10 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
             __syncwarp();
         };
         put_rows(p);
-        add_rows<R, BM, D>(dv, Ps, LPS, ty * R, dOs, tx);
+        add_rows<R, BM, D, kDeep>(dv, Ps, LPS, ty * R, dOs, tx);
         if (dK != nullptr || dQacc != nullptr) {
             float ds[R][QB];
-            dot_rows<R, QB, D>(ds, Vs, dOs, ty * R, tx);
+            dot_rows<R, QB, D, kDeep>(ds, Vs, dOs, ty * R, tx);
 #pragma unroll
             for (int b = 0; b < QB; ++b) {
                 const int q = tx + 16 * b;
@@ -599,7 +602,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
             }
             __syncwarp();              // the warp's lanes have read P
             put_rows(ds);
-            add_rows<R, BM, D>(dk, Ps, LPS, ty * R, Qs, tx);
+            add_rows<R, BM, D, kDeep>(dk, Ps, LPS, ty * R, Qs, tx);
         }
         __syncthreads();
         if (q0 + step < n) {           // arrives under the dQ product
@@ -613,7 +616,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
             for (int i = 0; i < RQ / 2; ++i)
 #pragma unroll
                 for (int c = 0; c < NC; ++c) dq[i][c] = 0ull;
-            add_rows<RQ, BN, D>(dq, dSt, LST, ty * RQ, Ks, tx);
+            add_rows<RQ, BN, D, kDeep>(dq, dSt, LST, ty * RQ, Ks, tx);
 #pragma unroll
             for (int i = 0; i < RQ / 2; ++i)
 #pragma unroll
@@ -1045,13 +1048,18 @@ cudaError_t fwd_r(const Problem &p, const void *Q, const void *K, const void *V,
     if (R > 2 && tiles * (nkt < 8 ? nkt : 8) < device_info().sms)
         return fwd_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, O, L, pr, st);
     const int split = simt_split(tiles, nqt, nkt, S::BM, BN, p.causal, R == 8 ? 3 : D == 128 ? 2 : 4);
-    const cudaError_t e = allow_smem<simt_fwd_kernel<T, R, D>>(S::kSmem);
-    if (e != cudaSuccess) return e;
-    LaunchScope scope(MOA_KERNEL_FWD, st);
     // Not a programmatic dependent where an SM gets more than one CTA: those placed while the kernel in front drains pile up on
     // the SMs it leaves first (B2 H1 n2048 d64: 252 us per fused call against 219).
-    return launch_cluster_as(tiles * split <= device_info().sms, simt_fwd_kernel<T, R, D>, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K, (const T *)V,
-                       (T *)O, L, (const T *)pr.dO, pr.Dv, pr.dQzero, p.n, p.causal, p.scale, nqt, split);
+    const bool alone = tiles * split <= device_info().sms;
+    auto go = [&](auto kernel, cudaError_t e) {
+        if (e != cudaSuccess) return e;
+        LaunchScope scope(MOA_KERNEL_FWD, st);
+        return launch_cluster_as(alone, kernel, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K,
+                                 (const T *)V, (T *)O, L, (const T *)pr.dO, pr.Dv, pr.dQzero, p.n, p.causal, p.scale, nqt, split);
+    };
+    if constexpr (R == 2)
+        if (alone && split >= nkt) return go(simt_fwd_kernel<T, R, D, true>, allow_smem<simt_fwd_kernel<T, R, D, true>>(S::kSmem));
+    return go(simt_fwd_kernel<T, R, D, false>, allow_smem<simt_fwd_kernel<T, R, D, false>>(S::kSmem));
 }
 template <typename T, int D>
 cudaError_t fwd_t(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L, const SimtPrep &pr,
@@ -1070,11 +1078,16 @@ cudaError_t bwd_kv_r(const Problem &p, const void *Q, const void *K, const void 
     if (R > 2 && tiles * (nqt < 8 ? nqt : 8) < device_info().sms)
         return bwd_kv_r<T, (R > 2 ? R / 2 : 2), D>(p, Q, K, V, dO, L, Dv, dK, dV, dQacc, st);
     const int split = simt_split(tiles, nkt, nqt, S::BN, S::BM, p.causal, 2);
-    const cudaError_t e = allow_smem<simt_bwd_kv_kernel<T, R, D>>(S::kSmem);
-    if (e != cudaSuccess) return e;
-    LaunchScope scope(MOA_KERNEL_BWD_KV, st);
-    return launch_cluster(simt_bwd_kv_kernel<T, R, D>, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K,
-                       (const T *)V, (const T *)dO, L, Dv, (T *)dK, (T *)dV, dQacc, p.n, p.causal, p.scale, nkt, split);
+    auto go = [&](auto kernel, cudaError_t e) {
+        if (e != cudaSuccess) return e;
+        LaunchScope scope(MOA_KERNEL_BWD_KV, st);
+        return launch_cluster(kernel, (unsigned)split, dim3((unsigned)(tiles * split)), dim3(SNT), S::kSmem, st, (const T *)Q, (const T *)K, (const T *)V,
+                              (const T *)dO, L, Dv, (T *)dK, (T *)dV, dQacc, p.n, p.causal, p.scale, nkt, split);
+    };
+    if constexpr (R == 2)
+        if (tiles * split <= device_info().sms && split >= nqt)
+            return go(simt_bwd_kv_kernel<T, R, D, true>, allow_smem<simt_bwd_kv_kernel<T, R, D, true>>(S::kSmem));
+    return go(simt_bwd_kv_kernel<T, R, D, false>, allow_smem<simt_bwd_kv_kernel<T, R, D, false>>(S::kSmem));
 }
 template <typename T, int D>
 cudaError_t bwd_kv_t(const Problem &p, const void *Q, const void *K, const void *V, const void *dO,
