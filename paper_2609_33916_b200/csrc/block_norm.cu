@@ -150,20 +150,69 @@ rmsnorm_fwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
     }
 }
 
+// dg of 64 columns over all rows: 32 rows of 8 vectors at a time, the row lanes added up in a fixed order.
+constexpr int kDgCols = 64, kDgRows = 768;
+__device__ __forceinline__ void dg_columns(const __nv_bfloat16 *x, const __nv_bfloat16 *dy, const float *r, __nv_bfloat16 *dg, int n, int d, int col0,
+                                           float *acc /*[32][64]*/)
+{
+    constexpr int kLanes = kDgCols / 8, kRows = kNormThreads / kLanes, kBatch = 8;
+    const int v = threadIdx.x % kLanes, rl = threadIdx.x / kLanes, col = col0 + 8 * v;
+    float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (col < d)
+        for (int row0 = rl; row0 < n; row0 += kRows * kBatch) {
+            uint4 xv[kBatch], dv[kBatch];
+            float rv[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int row = row0 + u * kRows;
+                xv[u] = dv[u] = make_uint4(0u, 0u, 0u, 0u);
+                rv[u] = 0.f;
+                if (row < n) {
+                    xv[u] = *reinterpret_cast<const uint4 *>(x + (size_t)row * d + col);
+                    dv[u] = *reinterpret_cast<const uint4 *>(dy + (size_t)row * d + col);
+                    rv[u] = r[row];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                float fx[8], fd[8];
+                unpack8(xv[u], fx);
+                unpack8(dv[u], fd);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) sum[e] = fmaf(fd[e] * fx[e], rv[u], sum[e]);
+            }
+        }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[rl * kDgCols + 8 * v + e] = sum[e];
+    __syncthreads();
+    if (threadIdx.x < kDgCols && col0 + (int)threadIdx.x < d) {
+        float t = 0.f;
+#pragma unroll
+        for (int l = 0; l < kRows; ++l) t += acc[l * kDgCols + threadIdx.x];
+        dg[col0 + threadIdx.x] = __float2bfloat16_rn(t);
+    }
+}
+
 // Backward.  Besides dx, every CTA leaves its partial dg (summed over its rows in a fixed order) in
-// part[blockIdx.x][d]; rmsnorm_dg_kernel adds the partials up.
+// part[blockIdx.x][d]; rmsnorm_dg_kernel adds the partials up.  col_blocks > 0 (few rows): the first col_blocks CTAs compute dg from x, dy and r
+// instead, and there are no partials.
 template <int kV, int R>
 __global__ void __launch_bounds__(kNormThreads)
 rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g,
                    const float *__restrict__ r_in, const __nv_bfloat16 *__restrict__ dy,
-                   const __nv_bfloat16 *__restrict__ dx_add, __nv_bfloat16 *__restrict__ dx, float *__restrict__ part, int n,
-                   int d, float eps, int tpr)
+                   const __nv_bfloat16 *__restrict__ dx_add, __nv_bfloat16 *__restrict__ dx, float *__restrict__ part,
+                   __nv_bfloat16 *__restrict__ dg, int col_blocks, int n, int d, float eps, int tpr)
 {
     __shared__ float red[8 * R];
     __shared__ float acc[kNormThreads * 8];              // [row lane][tpr*8] for one j at a time
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     x = ptx::after_wait(x); g = ptx::after_wait(g); r_in = ptx::after_wait(r_in); dy = ptx::after_wait(dy); dx_add = ptx::after_wait(dx_add);
+    if ((int)blockIdx.x < col_blocks) {
+        dg_columns(x, dy, r_in, dg, n, d, (int)blockIdx.x * kDgCols, acc);
+        return;
+    }
+    const int block = (int)blockIdx.x - col_blocks, blocks = (int)gridDim.x - col_blocks;
     const int c = threadIdx.x % tpr, rl = threadIdx.x / tpr, lanes = kNormThreads / tpr;
     const int nvec = d / 8;
     float gf[kV][8], dgacc[kV][8];
@@ -176,9 +225,9 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
 #pragma unroll
         for (int e = 0; e < 8; ++e) dgacc[j][e] = 0.f;
     }
-    const long long rows_per_iter = (long long)gridDim.x * lanes * R;
+    const long long rows_per_iter = (long long)blocks * lanes * R;
     const int iters = (int)((n + rows_per_iter - 1) / rows_per_iter);
-    const long long first = ((long long)blockIdx.x * lanes + rl) * R;
+    const long long first = ((long long)block * lanes + rl) * R;
     const float inv_d = 1.f / (float)d;
     RowRegs<kV, R> xc, dc, xn, dn;
     load_rows<kV, R>(xc, x, first, n, d, c, tpr);
@@ -236,8 +285,9 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
         xc = xn;
         dc = dn;
     }
+    if (col_blocks > 0) return;
     // CTA partial of dg: the row lanes' sums added in lane order
-    float *mine = part + (size_t)blockIdx.x * d;
+    float *mine = part + (size_t)block * d;
 #pragma unroll
     for (int j = 0; j < kV; ++j) {
         __syncthreads();
@@ -548,6 +598,11 @@ cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, c
     auto *ob = (__nv_bfloat16 *)dx;
     float *part = (float *)ws;
     int parts = p.grid;
+    // Few rows: dg from CTAs of their own in the same launch, 64 columns each; they read x and dy once more, from L2, while the others work on dx,
+    // and need as long for a thousand rows as a second launch (in a chain of calls 128 x 64 4.1 -> 2.3 us, 512 x 64 3.9 -> 2.8, 512 x 1024 5.0
+    // -> 3.0, 512 x 2048 8.6 -> 4.0; 1024 x 64 4.4 either way, 1024 x 512 4.4 and 4.6).
+    // (Not where dx is written over x or dy: the other CTAs may be a row ahead.)
+    const int col_blocks = r != nullptr && n <= kDgRows && !norm_uses_ring(n, d, true) && dx != x && dx != dy ? (d + kDgCols - 1) / kDgCols : 0;
     if (norm_uses_ring(n, d, true)) {
         const RingPlan rp = ring_plan(n, d, true);
         parts = rp.grid;
@@ -557,8 +612,9 @@ cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, c
     } else {
         LaunchScope scope(MOA_KERNEL_OTHER, st);
         const auto kernel = p.kV == 1 ? rmsnorm_bwd_kernel<1, 2> : p.kV == 2 ? rmsnorm_bwd_kernel<2, 1> : rmsnorm_bwd_kernel<4, 2>;
-        const cudaError_t e = launch_dependent(kernel, dim3(p.grid), dim3(kNormThreads), (size_t)0, st, xb, gb, r, db, ab, ob, part, n, d, eps, p.tpr);
-        if (e != cudaSuccess) return e;
+        const cudaError_t e = launch_dependent(kernel, dim3(p.grid + col_blocks), dim3(kNormThreads), (size_t)0, st, xb, gb, r, db, ab, ob, part,
+                                               (__nv_bfloat16 *)dg, col_blocks, n, d, eps, p.tpr);
+        if (e != cudaSuccess || col_blocks > 0) return e;
     }
     LaunchScope scope(MOA_KERNEL_OTHER, st);
     return launch_dependent(rmsnorm_dg_kernel, dim3((d + 31) / 32), dim3(32 * kDgWarps), (size_t)0, st, (const float *)part, (__nv_bfloat16 *)dg,

@@ -1,5 +1,6 @@
 """RMSNorm on both sides of the lines between its register and its ring kernels (rows of 256..2048 elements; by n times d, another line
-in the forward than in the backward), with ragged numbers of rows and row lengths that leave vectors over."""
+in the forward than in the backward) and of the line up to which the backward is one launch, with ragged numbers of rows and row lengths that
+leave vectors over."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,7 @@ TOL = 1e-2        # bf16 storage, fp32 arithmetic: the bound of the other RMSNor
 
 
 @pytest.mark.parametrize("n,d", [(4096, 256), (4097, 256), (511, 2048), (513, 2048), (1033, 1016), (127, 264), (32767, 256), (32801, 256),
-                                 (8300, 1016)])
+                                 (8300, 1016), (768, 64), (769, 64), (1, 8), (33, 72), (700, 4104)])
 def test_rmsnorm_routes(n, d):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
