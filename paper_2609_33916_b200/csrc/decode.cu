@@ -577,7 +577,7 @@ template <typename T, int D>
 cudaError_t launch_decode(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse,
                           float *ws, cudaStream_t st)
 {
-    const int splits = decode_splits(p);
+    const int splits = decode_splits(p, sizeof(T) == 4 ? MOA_F32 : MOA_BF16);
     const int keys_per_split = (p.n + splits - 1) / splits;
     const size_t BH = (size_t)p.B * p.H;
     float *part_o = ws, *part_ml = ws + (size_t)splits * BH * D;
@@ -624,17 +624,39 @@ static void decode_tc_splits(const DecodeProblem &p, int *splits, int *tiles_per
     *splits = (nkt + tps - 1) / tps;          // every segment has at least one tile
 }
 
-// Segments of the cache per K/V head: enough CTAs to fill the GPU a few times over, each with at least 128 keys (one round of
-// loads of the bf16 d = 64 kernel; with 256 a short cache left half of the SMs idle: B1 H16 n1000 8.2 -> 5.3 us) or, in the
-// ring kernel, of which an SM holds one CTA, 256 (with 128: fp32 groups of 8 over 4359 keys 54 -> 66 us).  Up to eight
-// segments, a power of two, are one cluster.
-int decode_splits(const DecodeProblem &p)
+// Segments of the cache per K/V head, each with at least 128 keys (one round of loads of the bf16 d = 64 kernel; with 256 a short
+// cache left half of the SMs idle: B1 H16 n1000 8.2 -> 5.3 us) or, in the ring kernel, of which an SM holds one CTA, 256 (with 128: fp32
+// groups of 8 over 4359 keys 54 -> 66 us).
+// Up to eight segments, a power of two, are one cluster.  The streaming kernel's CTAs all run at once, four or (pairs of heads) three to an SM:
+// a few more than that begin when the others end (B1 H32 n16000 d128 with 19 segments, 608 CTAs, 61.9 us, with 16 46.2; B8 H16 n600 d64 with
+// 8 9.3, with 4 6.4).  More segments than a cluster has cost the clearing of the counters and a merge through memory, about 4 us: they
+// pay only where a segment of eight would stream for longer than that by itself, at 25 (bf16) or 41 (fp32) bytes per ns, and there is room for twice as
+// many (B6 H8 n4390 d64 8: 14.1 us, 13: 18.1; B4 H16 n8000 d128 8: 43.5, 10: 59.4; but B1 H8 n30000 d64 8: 45.1, 74: 17.9).
+// Single heads with segments of 500 KB or more take more of them, in several waves, where those fill the slots a fifth better
+// (B20 H32 n8000 d64, 640 heads, 1: 254.5, 4: 206.4; B20 H16 n4000 d128 1: 125.5, 4: 115.6; B25 H8 n16000 d64 2: 135.7, 8: 129.4; the same fill,
+// B16 H16 n8192 d128, 2: 157.9, 4: 161.3; shorter segments, B20 H8 n3000 d128 fp32, 2: 73.1, 8: 79.3; pairs, B16 H32/16 n6000 d128, 1: 132.0, 8: 159.9).
+// The one shape found where the former rule, more than slots, is better: B13 H8 n8000 d128 fp32, 4: 132.9, 8: 128.4.
+int decode_splits(const DecodeProblem &p, int dtype)
 {
     const int group = p.H / p.Hkv;
     const int gc = group_chunk(group);
-    const long long ctas_per_split = (long long)p.B * p.Hkv * ((group + gc - 1) / gc);
-    long long s = (4LL * device_info().sms + ctas_per_split - 1) / ctas_per_split;
+    const long long sms = device_info().sms, heads = (long long)p.B * p.Hkv * ((group + gc - 1) / gc);
     const long long least = gc >= 4 ? 256 : 128, cap = (p.n + least - 1) / least;
+    if (gc < 4) {
+        const long long slots = sms * (gc == 1 ? 4 : 3), fit = slots / heads;
+        const double head_bytes = 2.0 * p.n * p.d * (dtype == MOA_F32 ? 4 : 2);
+        if (fit >= 16 && cap > kMaxCluster && head_bytes / kMaxCluster > 7000.0 * (dtype == MOA_F32 ? 41 : 25)) {
+            const long long s = fit < cap ? fit : cap;
+            return (int)(s > 1024 ? 1024 : s);
+        }
+        int c = kMaxCluster;
+        while (c > 1 && (heads * c > slots || c / 2 >= cap)) c /= 2;
+        const auto fill = [&](int k) { return (double)(heads * k) / (double)((heads * k + slots - 1) / slots * slots); };
+        for (int k = c * 2; gc == 1 && k <= kMaxCluster && head_bytes / k >= 5e5; k *= 2)
+            if (fill(k) >= 1.2 * fill(c)) c = k;
+        return c;
+    }
+    long long s = (4LL * sms + heads - 1) / heads;
     if (s > cap) s = cap;
     if (s < 1) s = 1;
     if (s > 1024) s = 1024;
@@ -654,7 +676,7 @@ size_t decode_workspace_bytes(const DecodeProblem &p, int dtype)
         return ((heads * p.d * 2 + 255) / 256) * 256 + heads * sizeof(float);
     }
     // partial results of the segments, then one counter per (K/V head, chunk of query heads)
-    return (size_t)decode_splits(p) * p.B * p.H * (p.d + 2) * sizeof(float) + (size_t)p.B * p.H * sizeof(unsigned int);
+    return (size_t)decode_splits(p, dtype) * p.B * p.H * (p.d + 2) * sizeof(float) + (size_t)p.B * p.H * sizeof(unsigned int);
 }
 
 cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const void *K, const void *V, void *out,
