@@ -328,7 +328,6 @@ __device__ __forceinline__ void finish_segment(DecodeState<T, D, GC> &st, const 
         out[head * D + c] = from_float<T>(o / ls);
         if (lse && c == 0) lse[head] = (mt + log2f(ls)) * kLn2;
     }
-    __syncwarp();
     if (splits > 1) ptx::cluster_sync_all();       // nobody leaves while another CTA may still read its shared memory
 }
 

@@ -237,12 +237,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
             float lt = l[h];
             lt += __shfl_xor_sync(0xffffffffu, lt, 1);
             lt += __shfl_xor_sync(0xffffffffu, lt, 2);
-            asm volatile("bar.sync 1, 256;" ::: "memory");          // (the merge before has been read)
+            named_barrier(1, 256);          // (the merge before has been read)
             float *row = merge + (warp * 8 + r0) * kLd;
 #pragma unroll
             for (int i2 = 0; i2 < kNT; ++i2) *reinterpret_cast<float2 *>(row + 8 * i2 + c0) = make_float2(o[i2][2 * h], o[i2][2 * h + 1]);
             if (lane % 4 == 0) { row[D] = m[h]; row[D + 1] = lt; }
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+            named_barrier(1, 256);
             for (int idx = tid; idx < min(8, G - 8 * h) * D; idx += 256) {
                 const int r = idx / D, c = idx - r * D, g = 8 * h + r;
                 float mt = -INFINITY, ot = 0.f, ls = 0.f;
@@ -269,7 +269,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
             }
         }
         if (cl > 1) {       // (the only segment)
-            __syncwarp();
             cluster_sync_all();
             auto peer = [&](const float *mine, int k) {
                 float v;
@@ -289,7 +288,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constan
                 out[((size_t)head * G + g) * D + c] = __float2bfloat16_rn(ot / ls);
                 if (lse && c == 0) lse[(size_t)head * G + g] = (mt + log2f(ls)) * kLn2;
             }
-            __syncwarp();
             cluster_sync_all();       // nobody leaves while another CTA may still read its shared memory
         }
     }

@@ -306,10 +306,18 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t cta_addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(cta_addr), "r"(rank));
     return r;
 }
-// every thread of every CTA of the cluster (hardware barrier; all threads reach it, also after an expired wait)
+// every thread of every CTA of the cluster (hardware barrier; all threads reach it, also after an expired wait).  The aligned form
+// is undefined for a warp whose lanes arrive apart, as they may behind a loop that half of them leave early: they meet first.
 __device__ __forceinline__ void cluster_sync_all()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// `threads` threads of the CTA, whole warps (an aligned barrier as well)
+__device__ __forceinline__ void named_barrier(int id, int threads)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {

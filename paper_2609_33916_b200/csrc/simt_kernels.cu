@@ -205,17 +205,6 @@ __device__ __forceinline__ void unpack_rows(const uint64_t (&acc)[C], int v, flo
     ptx::unpack_f32x2(acc[4 * v + 3], even.w, odd.w);
 }
 
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_barrier()
-{
-    asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
-}
-
 // ------------------------------------------------------------------------- forward
 // CTA: BM = 8 R query rows; a warp has 2 R rows to itself, a thread R rows x 4 keys of the score tile and R rows x D / 16
 // columns of O.  The `split` ranks of a cluster take the key tiles of their rows in turn (rank r: tiles r, r + split, ...), each
@@ -244,7 +233,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
     ptx::grid_launch_dependents();
     Q = ptx::after_wait(Q); K = ptx::after_wait(K); V = ptx::after_wait(V); dO = ptx::after_wait(dO);
 
-    const int rank = split > 1 ? (int)cluster_rank() : 0;
+    const int rank = split > 1 ? (int)ptx::cluster_ctarank() : 0;
     const int job = (int)blockIdx.x / split;
     int qt = job % nqt;
     const int bh = job / nqt;
@@ -365,7 +354,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         const float li = group16_sum(l[i]);
         if (tx == 0) { Mm[ty * R + i] = m[i]; Lm[ty * R + i] = li; }
     }
-    if (split > 1) cluster_barrier();
+    if (split > 1) ptx::cluster_sync_all();
     else __syncthreads();
     constexpr int LPR = D / 4;         // lanes per row, 16 bytes each
     const int per = (BM + split - 1) / split;        // rows this rank finishes (the last rank: what is left)
@@ -414,7 +403,7 @@ simt_fwd_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
             if (live && c == 0) Dv[(size_t)bh * n + row] = dot;
         }
     }
-    if (split > 1) cluster_barrier();      // nobody leaves while another rank may still read its shared memory
+    if (split > 1) ptx::cluster_sync_all();      // nobody leaves while another rank may still read its shared memory
 }
 
 // ---------------------------------------- rowsum(dO o O), and dQ (or its accumulator) cleared: one warp per row
@@ -517,7 +506,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
     float *Ps = dOs + BM * LD, *dSt = Ps + BM * LPS, *Ls = dSt + BN * LST, *Ds = Ls + BM;
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
 
-    const int rank = split > 1 ? (int)cluster_rank() : 0;
+    const int rank = split > 1 ? (int)ptx::cluster_ctarank() : 0;
     const int job = (int)blockIdx.x / split;
     const int kt = job % nkt;   // causal: key tile 0 has the most work and comes first
     const int bh = job / nkt;
@@ -668,7 +657,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
                 *reinterpret_cast<float4 *>(dOs + at) = g[e];
             }
         }
-    cluster_barrier();
+    ptx::cluster_sync_all();
     constexpr int LPR = D / 4;
     const int per = (BN + split - 1) / split;
     for (int r = tid / LPR; r < per && rank * per + r < BN; r += SNT / LPR) {
@@ -690,7 +679,7 @@ simt_bwd_kv_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
         if (dK) store4(dK + (size_t)row * D + c, a);
         store4(dV + (size_t)row * D + c, g);
     }
-    cluster_barrier();
+    ptx::cluster_sync_all();
 }
 
 // ----------------------------------------- backward, one CTA per query tile: dQ, no atomics

@@ -741,7 +741,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
     if (kSplit) {
         // the ranks add up the partial results, 128 / split rows each, and write them out
-        __syncwarp();
         cluster_sync_all();
         if (warp < kLoadWarp) {
             const int per = 128 / split;
@@ -755,7 +754,6 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
             }
         }
-        __syncwarp();
         cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
     }
     if (*abortp && tid == kLoadWarp * 32) {

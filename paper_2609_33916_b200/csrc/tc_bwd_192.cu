@@ -452,7 +452,6 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
     if (warp == kMmaWarp) tmem_dealloc(tbase, kTmemCols);
     if (kSplit) {
         // the ranks add up the partial results, 128 / split rows each, and write them out
-        __syncwarp();
         cluster_sync_all();
         if (warp < kLoadWarp) {
             const int per = 128 / split;
@@ -466,7 +465,6 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
                         make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
             }
         }
-        __syncwarp();
         cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
     }
     if (*abortp && tid == kLoadWarp * 32) {

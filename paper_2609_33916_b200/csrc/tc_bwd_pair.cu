@@ -639,7 +639,6 @@ tc_bwd_pair_kernel(const __grid_constant__ CUtensorMap mapQr, const __grid_const
     }
     // neither CTA leaves, or frees its TMEM, while the other may still read its shared memory, write into it,
     // write its accumulators or arrive on its barriers
-    __syncwarp();
     cluster_sync_all();
     if (warp == kMmaWarp) tmem_dealloc_pair(tbase, kTmemCols);
 }

@@ -518,7 +518,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     if (kPair) {
         // neither CTA leaves, or frees its TMEM, while the other may still read its shared memory, write its
         // accumulator or arrive on its barriers
-        __syncwarp();
         cluster_sync_all();
         if (warp == 1) tmem_dealloc_pair(tbase, 512);
     } else if (warp == 1) {
