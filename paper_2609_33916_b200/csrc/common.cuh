@@ -216,6 +216,14 @@ cudaError_t allow_smem(size_t bytes)
     return e;
 }
 
+// Whether two arrays share memory.  A caller may lay an output over an input that only earlier kernels of a call read (dx over dy, say); a
+// rule that lets kernels of a call run side by side has to look.
+inline bool arrays_meet(const void *a, size_t a_bytes, const void *b, size_t b_bytes)
+{
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x < y + b_bytes && y < x + a_bytes;
+}
+
 // Device address of the status word kernels write when a bounded wait expires.
 unsigned int *device_status_ptr();
 

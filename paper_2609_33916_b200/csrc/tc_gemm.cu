@@ -898,6 +898,13 @@ struct Product {
     void *C;                     // [M, N]
     int M, N, K, a_mn, b_mn;
     long long tiles(int n) const { return (long long)((M + GM - 1) / GM) * ((N + n - 1) / n); }
+    bool writes_into(const void *p, long long rows, long long cols) const { return arrays_meet(C, (size_t)M * N * 2, p, (size_t)(rows * cols) * 2); }
+    bool disturbs(const Product &o) const       // writes what `o` reads or writes
+    {
+        for (const Operand *r : {&o.A0, &o.B0, o.A1, o.B1})
+            if (r && writes_into(r->p, r->rows, r->cols)) return true;
+        return writes_into(o.C, o.M, o.N);
+    }
 };
 
 template <int kN>
@@ -937,11 +944,16 @@ cudaError_t launch_group_n(const Product *p, int count, cudaStream_t st)
 }
 
 // Whether `count` products go out as one launch: while their 128-column tiles fit on the SMs at once (then no wider tile and no pair
-// would have been faster for any of them), and MOA_GEMM_PAIR does not ask for pairs.
+// would have been faster for any of them), none writes what another one reads (one after the other they may: dx over dy or x), and
+// MOA_GEMM_PAIR does not ask for pairs.
 bool group_fits(const Product *p, int count)
 {
     long long t = 0;
-    for (int i = 0; i < count; ++i) t += p[i].tiles(128);
+    for (int i = 0; i < count; ++i) {
+        t += p[i].tiles(128);
+        for (int j = 0; j < count; ++j)
+            if (i != j && p[i].disturbs(p[j])) return false;
+    }
     return gemm_pair_mode() != 2 && t <= device_info().sms;
 }
 cudaError_t launch_group(const Product *p, int count, cudaStream_t st)
