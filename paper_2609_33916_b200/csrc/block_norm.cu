@@ -601,8 +601,12 @@ cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, c
     // Few rows: dg from CTAs of their own in the same launch, 64 columns each; they read x and dy once more, from L2, while the others work on dx,
     // and need as long for a thousand rows as a second launch (in a chain of calls 128 x 64 4.1 -> 2.3 us, 512 x 64 3.9 -> 2.8, 512 x 1024 5.0
     // -> 3.0, 512 x 2048 8.6 -> 4.0; 1024 x 64 4.4 either way, 1024 x 512 4.4 and 4.6).
-    // (Not where dx is written over x or dy: the other CTAs may be a row ahead.)
-    const int col_blocks = r != nullptr && n <= kDgRows && !norm_uses_ring(n, d, true) && dx != x && dx != dy ? (d + kDgCols - 1) / kDgCols : 0;
+    // (Not where dx lies over what the CTAs of dg read, or dg over what those of dx read: either may be rows ahead.)
+    const size_t all = (size_t)n * d * 2, cols = (size_t)d * 2, rows = (size_t)n * 4;
+    const bool apart = !arrays_meet(dx, all, x, all) && !arrays_meet(dx, all, dy, all) && !arrays_meet(dx, all, r, rows) &&
+                       !arrays_meet(dg, cols, g, cols) && !arrays_meet(dg, cols, x, all) && !arrays_meet(dg, cols, dy, all) &&
+                       !arrays_meet(dg, cols, r, rows) && !(dx_add && arrays_meet(dg, cols, dx_add, all));
+    const int col_blocks = r != nullptr && n <= kDgRows && !norm_uses_ring(n, d, true) && apart ? (d + kDgCols - 1) / kDgCols : 0;
     if (norm_uses_ring(n, d, true)) {
         const RingPlan rp = ring_plan(n, d, true);
         parts = rp.grid;

@@ -80,3 +80,34 @@ def test_block_weight_gradient_over_the_weight(rt):
     assert res[1][2] == res[0][2] + 1
     for a, b in zip(res[0][:2], res[1][:2]):      # (dQ's atomic sums in another order, and their bf16 roundings down the chain)
         assert (a - b).abs().max().item() <= 1.6e-2 * a.abs().max().item()
+
+
+# register kernel with one and with several CTAs; dx over x or dy row for row; dg over what the other rows' CTAs still read
+@pytest.mark.parametrize("over,under", [("dx", "x"), ("dx", "dy"), ("dx", "dx_add"), ("dg", "g"), ("dg", "x"), ("dg", "dy"), ("dg", "dx_add"), ("dg", "r")])
+@pytest.mark.parametrize("n,d", [(700, 64), (512, 1024), (64, 72), (1, 256)])
+def test_rmsnorm_backward(rt, n, d, over, under):
+    torch, mb = rt
+    gen = torch.Generator(device="cuda").manual_seed(n + d)
+    R = lambda *s: torch.randn(s, generator=gen, device="cuda").bfloat16()      # noqa: E731
+    t = {"x": R(n, d), "g": 1 + 0.25 * R(d), "dy": R(n, d), "dx_add": R(n, d), "r": torch.empty(n, dtype=torch.float32, device="cuda")}
+    desc = mb.make_rmsnorm_desc(n, d, 1e-5)
+    mb.moa_rmsnorm_fwd(desc, t["x"], t["g"], torch.empty_like(t["x"]), t["r"])
+    if t[under].nbytes < 2 * d:
+        pytest.skip("the output does not fit into this input")
+
+    def run(reused):
+        a = {k: v.clone() for k, v in t.items()}
+        out = {"dx": torch.empty_like(a["x"]), "dg": torch.empty_like(a["g"])}
+        if reused:
+            like = out[over]
+            out[over] = a[under].view(torch.bfloat16).flatten()[:like.numel()].view(like.shape)
+        ws = torch.empty(mb.moa_rmsnorm_workspace_bytes(desc), dtype=torch.uint8, device="cuda")
+        before = mb.moa_launch_count()
+        mb.moa_rmsnorm_bwd(desc, a["x"], a["g"], a["r"], a["dy"], out["dx"], out["dg"], ws, dx_add=a["dx_add"])
+        return out["dx"].double(), out["dg"].double(), mb.moa_launch_count() - before
+
+    ref, got = run(False), run(True)
+    assert ref[2] == 1 and got[2] == (1 if under == "dx_add" and over == "dx" else 2)
+    # dx does not depend on the route; dg's sums are taken in another order: fp32 sums of n terms, then one rounding to bf16 (2^-8 of an element)
+    assert torch.equal(ref[0], got[0])
+    assert (ref[1] - got[1]).abs().max().item() <= 2 ** -7 * ref[1].abs().max().item()
