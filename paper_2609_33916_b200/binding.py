@@ -178,14 +178,15 @@ _ENTRIES = (("moa_attn_fwd", moa_attn_desc, 6, True), ("moa_attn_bwd", moa_attn_
             ("moa_attn_fused_fwd_bwd", moa_attn_desc, 10, True), ("moa_decode_attn", moa_decode_desc, 6, True),
             ("moa_rmsnorm_fwd", moa_rmsnorm_desc, 4, False), ("moa_rmsnorm_bwd", moa_rmsnorm_desc, 8, True), ("moa_gemm", moa_gemm_desc, 4, False),
             ("moa_gated_mlp_fwd", moa_mlp_desc, 9, False), ("moa_gated_mlp_bwd", moa_mlp_desc, 13, True))
-_ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD = range(len(_ENTRIES))
+# their indexes in the extension's table, which outlives a reload of this module: set by _load, which runs before they are read
+_ATTN_FWD = _ATTN_BWD = _ATTN_FUSED = _DECODE = _NORM_FWD = _NORM_BWD = _GEMM = _MLP_FWD = _MLP_BWD = None
 _invoke = _fill = None
 _load_lock = threading.Lock()
 
 
 def _load():
     """_pycall.invoke, with the library's functions registered."""
-    global _invoke, _fill
+    global _invoke, _fill, _ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD
     with _load_lock:
         if _invoke is None:
             L = lib()
@@ -193,8 +194,8 @@ def _load():
                 from . import _pycall
             except ImportError as e:
                 raise RuntimeError("_pycall.so is missing: run `python -m paper_2609_33916_b200.build` (there is no fallback path)") from e
-            for name, desc, pointers, ws in _ENTRIES:
-                _pycall.add_entry(ctypes.cast(getattr(L, name), ctypes.c_void_p).value, desc, pointers, ws)
+            _ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD = (
+                _pycall.add_entry(ctypes.cast(getattr(L, name), ctypes.c_void_p).value, desc, pointers, ws) for name, desc, pointers, ws in _ENTRIES)
             _pycall.set_current_stream(lambda: _current_stream())
             _fill, _invoke = _pycall.fill, _pycall.invoke
     return _invoke

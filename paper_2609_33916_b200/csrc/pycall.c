@@ -8,15 +8,14 @@
 #include <Python.h>
 #include <stdint.h>
 
-#define MAX_ENTRIES 32
 #define MAX_ARGS 16 /* pointers, workspace bytes and stream */
 
-static struct {
+static struct entry {
     uintptr_t fn;
     PyTypeObject *desc_type;
     Py_ssize_t npointers; /* pointer arguments, the workspace included */
     int has_ws;
-} entries[MAX_ENTRIES];
+} *entries; /* (grows: a reloaded binding registers its own descriptor types) */
 static int nentries;
 static PyObject *s_data_ptr, *s_nbytes, *s_cuda_stream;
 static PyObject *stream_getter, *device_getter; /* stream_getter(device_getter()), or stream_getter() without the second */
@@ -27,12 +26,16 @@ static PyObject *add_entry(PyObject *self, PyObject *args)
     PyObject *type;
     Py_ssize_t npointers;
     int has_ws;
+    struct entry *more;
     (void)self;
     if (!PyArg_ParseTuple(args, "KO!np", &fn, &PyType_Type, &type, &npointers, &has_ws)) return NULL;
-    if (nentries == MAX_ENTRIES || npointers < 1 || npointers + 2 > MAX_ARGS) {
-        PyErr_SetString(PyExc_ValueError, "too many entries or arguments");
+    if (npointers < 1 || npointers + 2 > MAX_ARGS) {
+        PyErr_SetString(PyExc_ValueError, "too many arguments");
         return NULL;
     }
+    more = PyMem_Realloc(entries, (size_t)(nentries + 1) * sizeof *entries);
+    if (!more) return PyErr_NoMemory();
+    entries = more;
     Py_INCREF(type);
     entries[nentries].fn = (uintptr_t)fn;
     entries[nentries].desc_type = (PyTypeObject *)type;
@@ -102,6 +105,7 @@ static PyObject *invoke(PyObject *self, PyObject *const *args, Py_ssize_t nargs)
     uint64_t a[MAX_ARGS] = {0};
     Py_ssize_t np, i;
     Py_buffer desc;
+    struct entry entry; /* (a copy: the table may move while other code runs) */
     int status;
     const long e = nargs > 0 ? PyLong_AsLong(args[0]) : -1;
     (void)self;
@@ -109,18 +113,19 @@ static PyObject *invoke(PyObject *self, PyObject *const *args, Py_ssize_t nargs)
         if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "unknown entry");
         return NULL;
     }
-    np = entries[e].npointers;
-    if (nargs != 3 + np + (entries[e].has_ws ? 1 : 0)) {
+    entry = entries[e];
+    np = entry.npointers;
+    if (nargs != 3 + np + (entry.has_ws ? 1 : 0)) {
         PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
         return NULL;
     }
-    if (!PyObject_TypeCheck(args[1], entries[e].desc_type)) {
-        PyErr_Format(PyExc_TypeError, "expected a %s", entries[e].desc_type->tp_name);
+    if (!PyObject_TypeCheck(args[1], entry.desc_type)) {
+        PyErr_Format(PyExc_TypeError, "expected a %s", entry.desc_type->tp_name);
         return NULL;
     }
     for (i = 0; i < np; ++i)
         if (address(args[2 + i], s_data_ptr, 1, &a[i])) return NULL;
-    if (entries[e].has_ws) {
+    if (entry.has_ws) {
         PyObject *ws = args[1 + np], *bytes = args[2 + np];
         if (bytes != Py_None) {
             Py_INCREF(bytes);
@@ -136,7 +141,7 @@ static PyObject *invoke(PyObject *self, PyObject *const *args, Py_ssize_t nargs)
     /* (every argument is a pointer, a size_t or a stream, an integer register or a stack slot each: one call with all the slots serves every
      * count, the callee reads as many as it has) */
     status = ((int (*)(void *, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t, uint64_t,
-                       uint64_t, uint64_t, uint64_t, uint64_t, uint64_t))entries[e].fn)(
+                       uint64_t, uint64_t, uint64_t, uint64_t, uint64_t))entry.fn)(
         desc.buf, a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7], a[8], a[9], a[10], a[11], a[12], a[13], a[14], a[15]);
     Py_END_ALLOW_THREADS
     PyBuffer_Release(&desc);

@@ -1,6 +1,8 @@
 """The marshalling extension behind the binding's launching calls: what it takes for an address, a workspace size and a descriptor, seen from
 refusals that need no GPU, and from several threads."""
 import ctypes
+import subprocess
+import sys
 import threading
 
 import pytest
@@ -61,3 +63,18 @@ def test_from_several_threads():
     for t in threads:
         t.join()
     assert got == [mb.MOA_ERR_INVALID_ARG] * 2000
+
+
+def test_after_reloads_of_the_binding():
+    """(In a process of its own: the reload makes new descriptor classes.)  More reloads than any fixed table would hold."""
+    code = """
+import importlib
+from paper_2609_33916_b200 import binding as mb
+for k in range(12):
+    for make, call, args in ((mb.make_decode_desc, mb.moa_decode_attn, 6), (mb.make_mlp_desc, mb.moa_gated_mlp_bwd, 13)):
+        desc = make(1, 1, -1, 64, 0.1) if args == 6 else make(-1, 8, 8)
+        assert call(desc, *[4096] * args, ws_bytes=0, stream=0, check=False) == mb.MOA_ERR_INVALID_ARG
+    importlib.reload(mb)
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=build.ROOT)
+    assert r.returncode == 0, r.stderr[-2000:]
