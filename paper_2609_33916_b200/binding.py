@@ -184,16 +184,44 @@ _invoke = _fill = None
 _load_lock = threading.Lock()
 
 
+def _address(x) -> int:
+    """An address as the extension takes it: None, an integer, or an object with data_ptr()."""
+    a = 0 if x is None else x if isinstance(x, int) else x.data_ptr()
+    if not 0 <= a < 1 << 64:
+        raise OverflowError("an address has 64 bits")
+    return a
+
+
+def _invoke_ctypes(e, desc, *args):
+    """_pycall.invoke without the extension."""
+    name, desc_type, pointers, has_ws = _ENTRIES[e]
+    if not isinstance(desc, desc_type):
+        raise TypeError(f"expected a {desc_type.__name__}")
+    values = [_address(x) for x in args[:pointers]]
+    if has_ws:
+        values.append(_nbytes(args[pointers - 1]) if args[pointers] is None else _address(args[pointers]))
+    return getattr(lib(), name)(ctypes.byref(desc), *values, _stream(args[-1]))
+
+
+def _fill_ctypes(struct, objects):
+    """_pycall.fill without the extension."""
+    if 8 * len(objects) > ctypes.sizeof(struct):
+        raise ValueError("more objects than words")
+    (ctypes.c_uint64 * len(objects)).from_buffer(struct)[:] = [_address(x) for x in objects]
+
+
 def _load():
-    """_pycall.invoke, with the library's functions registered."""
+    """_pycall.invoke, with the library's functions registered, or its form in ctypes where the extension is not there."""
     global _invoke, _fill, _ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD
     with _load_lock:
         if _invoke is None:
             L = lib()
             try:
                 from . import _pycall
-            except ImportError as e:
-                raise RuntimeError("_pycall.so is missing: run `python -m paper_2609_33916_b200.build` (there is no fallback path)") from e
+            except ImportError:          # not built for this interpreter: the same through ctypes
+                _ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD = range(len(_ENTRIES))
+                _fill, _invoke = _fill_ctypes, _invoke_ctypes
+                return _invoke
             _ATTN_FWD, _ATTN_BWD, _ATTN_FUSED, _DECODE, _NORM_FWD, _NORM_BWD, _GEMM, _MLP_FWD, _MLP_BWD = (
                 _pycall.add_entry(ctypes.cast(getattr(L, name), ctypes.c_void_p).value, desc, pointers, ws) for name, desc, pointers, ws in _ENTRIES)
             _pycall.set_current_stream(lambda: _current_stream())
@@ -232,9 +260,9 @@ def _current_stream() -> int:
     if raw is not None and device is not None:
         global _current_stream
         _current_stream = lambda: raw(device())        # noqa: E731
-        _load()
-        from . import _pycall
-        _pycall.set_current_stream(raw, device)
+        if _load() is not _invoke_ctypes:
+            from . import _pycall
+            _pycall.set_current_stream(raw, device)
     return stream
 
 

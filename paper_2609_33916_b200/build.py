@@ -6,6 +6,7 @@ import os
 import subprocess
 import sys
 import sysconfig
+import warnings
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -13,7 +14,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libmoa_attn.so")
-PYCALL = os.path.join(HERE, "_pycall.so")
+# (the suffix names the interpreter and its ABI: a tree built by one and used by another does not load the wrong module)
+PYCALL = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -72,14 +74,28 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
-def build_pycall(force: bool = False) -> str:
-    """The marshalling extension of binding.py (plain C, no CUDA)."""
+def build_pycall(force: bool = False) -> str | None:
+    """The marshalling extension of binding.py (plain C, no CUDA).  None where it cannot be compiled (no compiler or no Python headers):
+    the binding then marshals through ctypes."""
+    untagged = os.path.join(HERE, "_pycall.so")
+    if untagged != PYCALL and os.path.exists(untagged):      # (any interpreter would load it)
+        os.remove(untagged)
     src = os.path.join(CSRC, "pycall.c")
     if force or _stale(PYCALL, [src]):
-        r = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], src, "-o", PYCALL],
-                           capture_output=True, text=True)
+        include = sysconfig.get_paths()["include"]
+        partial = f"{PYCALL}.{os.getpid()}"
+        try:
+            r = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", include, src, "-o", partial],
+                               capture_output=True, text=True)
+        except OSError as e:
+            warnings.warn(f"no C compiler for {src} ({e}): short calls take about 2 us longer")
+            return None
         if r.returncode != 0:
-            raise RuntimeError(f"the compiler failed for {src}:\n{r.stderr}")
+            if os.path.exists(os.path.join(include, "Python.h")):
+                raise RuntimeError(f"the compiler failed for {src}:\n{r.stderr}")
+            warnings.warn(f"no Python headers for {src}: short calls take about 2 us longer")
+            return None
+        os.replace(partial, PYCALL)
     return PYCALL
 
 

@@ -1,8 +1,11 @@
 """The marshalling extension behind the binding's launching calls: what it takes for an address, a workspace size and a descriptor, seen from
 refusals that need no GPU, and from several threads."""
 import ctypes
+import importlib.machinery
+import os
 import subprocess
 import sys
+import sysconfig
 import threading
 
 import pytest
@@ -75,6 +78,45 @@ for k in range(12):
         desc = make(1, 1, -1, 64, 0.1) if args == 6 else make(-1, 8, 8)
         assert call(desc, *[4096] * args, ws_bytes=0, stream=0, check=False) == mb.MOA_ERR_INVALID_ARG
     importlib.reload(mb)
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=build.ROOT)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_the_module_belongs_to_one_interpreter(monkeypatch, tmp_path):
+    assert build.PYCALL.endswith(sysconfig.get_config_var("EXT_SUFFIX")) and os.path.exists(build.PYCALL)
+    assert importlib.machinery.EXTENSION_SUFFIXES[0] == sysconfig.get_config_var("EXT_SUFFIX")
+    # an untagged one, which every interpreter would load, goes; without a compiler or headers there is none, and that is no error
+    monkeypatch.setattr(build, "HERE", str(tmp_path))
+    monkeypatch.setattr(build, "PYCALL", str(tmp_path / "_pycall.tag.so"))
+    (tmp_path / "_pycall.so").write_bytes(b"")
+    monkeypatch.setenv("CC", str(tmp_path / "none"))
+    with pytest.warns(UserWarning):
+        assert build.build_pycall() is None
+    assert os.listdir(tmp_path) == []
+    monkeypatch.delenv("CC")
+    monkeypatch.setattr(sysconfig, "get_paths", lambda: {"include": str(tmp_path)})
+    with pytest.warns(UserWarning):
+        assert build.build_pycall() is None
+    assert os.listdir(tmp_path) == []
+
+
+def test_without_the_extension():
+    """The same answers through ctypes (a process of its own, in which the module cannot be imported)."""
+    code = """
+import ctypes, sys
+sys.modules["paper_2609_33916_b200._pycall"] = None
+import pytest, torch
+sys.path.insert(0, "tests")
+import test_pycall as t
+from paper_2609_33916_b200 import binding as mb
+t.test_descriptors_of_another_type_and_things_without_an_address_are_refused()
+t.test_workspace_sizes(None, None, "MOA_ERR_WORKSPACE")
+t.test_workspace_sizes(4096, 1, "MOA_ERR_WORKSPACE")
+t.test_fill(1)
+t.test_fill(3)
+t.test_from_several_threads()
+assert mb._load() is mb._invoke_ctypes
 """
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=build.ROOT)
     assert r.returncode == 0, r.stderr[-2000:]
