@@ -10,7 +10,8 @@ With `packed_qkv` (the default) the three projections are one GEMM against the s
 ([3 H d, H d]): its [T, 3 H d] output is a packed [B, n, 3, H, d] array whose thirds go to the attention as Q, K, V through
 explicit strides (MOA_LAYOUT_STRIDED, no copy), dQ, dK, dV come back into one such array, and the backward of the
 projection is one GEMM for dh1 and one for dWqkv.  That form's 6 + 8 calls are made by the library (moa_block_fwd,
-moa_block_bwd: one call per direction from here); without it: 8 and 12 calls, made here."""
+moa_block_bwd: one call per direction from here) as long as the block's descriptors (nd, ad, md) are the ones it was built with; with
+changed ones (another dq_mode, say), and without `packed_qkv`, the calls (8 and 12) are made here."""
 from __future__ import annotations
 
 import math
@@ -43,6 +44,10 @@ class TransformerBlock:
         self.proj = mb.make_gemm_desc(T, dm, dm)              # y = x W^T
         self.back = mb.make_gemm_desc(T, dm, dm, 0, 1)        # dx = dy W
         self.wgrad = mb.make_gemm_desc(dm, dm, T, 1, 1)       # dW = dy^T x
+        self.proj3 = mb.make_gemm_desc(T, 3 * dm, dm)         # qkv = h1 Wqkv^T
+        self.back3 = mb.make_gemm_desc(T, dm, 3 * dm, 0, 1)   # dh1 = dqkv Wqkv
+        self.wgrad3 = mb.make_gemm_desc(3 * dm, dm, T, 1, 1)  # dWqkv = dqkv^T h1
+        self._built_with = self._descriptors()
         self.nws = u8(mb.moa_rmsnorm_workspace_bytes(self.nd))
         self.aws = u8(mb.moa_attn_workspace_bytes(self.ad, mb.MOA_OP_BWD))
         self.mws = u8(mb.moa_gated_mlp_workspace_bytes(self.md))
@@ -82,6 +87,9 @@ class TransformerBlock:
         att = 14.0 * self.B * self.H * float(self.n) ** 2 * self.d * (0.5 if self.causal else 1.0)
         return 4 * 6.0 * T * dm * dm + att + 18.0 * T * dm * self.d_ff
 
+    def _descriptors(self):
+        return bytes(self.ad), bytes(self.nd), bytes(self.md)
+
     def _arrays(self, x, w, dy):
         """The addresses of this call (taken anew each time: any of the tensors may have been replaced)."""
         g = self.grads
@@ -92,14 +100,17 @@ class TransformerBlock:
             self.gqkv, g["Wo"], g["W1"], g["W3"], g["W2"], nws, aws, mws, nws.nbytes, aws.nbytes, mws.nbytes))
 
     def forward(self, x, w, stream=None):
-        if self.packed:
+        if self.packed and self._descriptors() == self._built_with:
             mb.moa_block_fwd(self.bd, self._arrays(x, w, None), stream)
             return self.y
         s = stream
         mb.moa_rmsnorm_fwd(self.nd, x, w["g1"], self.h1, self.r1, s)
-        mb.moa_gemm(self.proj, self.h1, w["Wq"], self.q, stream=s)
-        mb.moa_gemm(self.proj, self.h1, w["Wk"], self.k, stream=s)
-        mb.moa_gemm(self.proj, self.h1, w["Wv"], self.v, stream=s)
+        if self.packed:
+            mb.moa_gemm(self.proj3, self.h1, w["Wqkv"], self.qkv, stream=s)
+        else:
+            mb.moa_gemm(self.proj, self.h1, w["Wq"], self.q, stream=s)
+            mb.moa_gemm(self.proj, self.h1, w["Wk"], self.k, stream=s)
+            mb.moa_gemm(self.proj, self.h1, w["Wv"], self.v, stream=s)
         mb.moa_attn_fwd(self.ad, self.q, self.k, self.v, self.o, self.L, self.aws, s)
         mb.moa_gemm(self.proj, self.o, w["Wo"], self.x2, R=x, stream=s)
         mb.moa_rmsnorm_fwd(self.nd, self.x2, w["g2"], self.h2, self.r2, s)
@@ -108,7 +119,7 @@ class TransformerBlock:
 
     def backward(self, x, w, dy, stream=None):
         s, g = stream, self.grads
-        if self.packed:
+        if self.packed and self._descriptors() == self._built_with:
             mb.moa_block_bwd(self.bd, self._arrays(x, w, dy), s)
             return self.dx, g
         mb.moa_gated_mlp_bwd(self.md, self.h2, w["W1"], w["W3"], w["W2"], self.a, self.u, self.h, dy, self.dh2,
@@ -117,11 +128,15 @@ class TransformerBlock:
         mb.moa_gemm(self.wgrad, self.dx2, self.o, g["Wo"], stream=s)
         mb.moa_gemm(self.back, self.dx2, w["Wo"], self.do, stream=s)
         mb.moa_attn_bwd(self.ad, self.q, self.k, self.v, self.o, self.L, self.do, self.dq, self.dk, self.dv, self.aws, s)
-        mb.moa_gemm(self.back, self.dq, w["Wq"], self.dh1, stream=s)
-        mb.moa_gemm(self.back, self.dk, w["Wk"], self.dh1, R=self.dh1, stream=s)
-        mb.moa_gemm(self.back, self.dv, w["Wv"], self.dh1, R=self.dh1, stream=s)
-        mb.moa_gemm(self.wgrad, self.dq, self.h1, g["Wq"], stream=s)
-        mb.moa_gemm(self.wgrad, self.dk, self.h1, g["Wk"], stream=s)
-        mb.moa_gemm(self.wgrad, self.dv, self.h1, g["Wv"], stream=s)
+        if self.packed:
+            mb.moa_gemm(self.back3, self.dqkv, w["Wqkv"], self.dh1, stream=s)
+            mb.moa_gemm(self.wgrad3, self.dqkv, self.h1, self.gqkv, stream=s)
+        else:
+            mb.moa_gemm(self.back, self.dq, w["Wq"], self.dh1, stream=s)
+            mb.moa_gemm(self.back, self.dk, w["Wk"], self.dh1, R=self.dh1, stream=s)
+            mb.moa_gemm(self.back, self.dv, w["Wv"], self.dh1, R=self.dh1, stream=s)
+            mb.moa_gemm(self.wgrad, self.dq, self.h1, g["Wq"], stream=s)
+            mb.moa_gemm(self.wgrad, self.dk, self.h1, g["Wk"], stream=s)
+            mb.moa_gemm(self.wgrad, self.dv, self.h1, g["Wv"], stream=s)
         mb.moa_rmsnorm_bwd(self.nd, x, w["g1"], self.r1, self.dh1, self.dx, g["g1"], self.nws, s, dx_add=self.dx2)
         return self.dx, g
