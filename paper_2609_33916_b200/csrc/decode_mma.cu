@@ -378,7 +378,7 @@ cudaError_t launch(const DecodeProblem &p, const void *q, const void *K, const v
     // kernel costs about what an SM streams in that time.
     int cl = 0;
     for (int c = 1; c <= 8 && c <= nt && heads * c * 100 <= sms * (c == 8 ? 85 : c == 4 ? 90 : 100); c *= 2) cl = c;
-    if (cl && ((nt + cl - 1) / cl - (units + sms - 1) / sms) * 2 * S::kTile > 192 * 1024) cl = 0;
+    if (cl && (long long)((nt + cl - 1) / cl - (units + sms - 1) / sms) * 2 * S::kTile > 192 * 1024) cl = 0;
     const int ctas = cl ? heads * cl : units < sms ? units : sms;
     float *part_o = (float *)ws, *part_ml = part_o + (size_t)2 * sms * G * D;
     {
