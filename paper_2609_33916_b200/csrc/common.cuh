@@ -131,7 +131,6 @@ struct DecodeProblem {
     int B, H, Hkv, n, d;     // Hkv resolved (never 0)
     float scale;
 };
-int decode_splits(const DecodeProblem &p, int dtype);                      // cache segments per K/V head (CUDA-core route)
 size_t decode_workspace_bytes(const DecodeProblem &p, int dtype);    // partial results of all segments
 // q [B,H,d], K, V [B,Hkv,n,d] -> out [B,H,d] (dtype of the inputs), lse [B,H] fp32 (may be null)
 cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const void *K, const void *V, void *out,

@@ -538,54 +538,144 @@ namespace {
 
 int group_chunk(int group) { return group >= 8 ? 8 : group >= 4 ? 4 : group >= 2 ? 2 : 1; }
 
+// Clusters of `size` CTAs of Kernel that run at once on this device: fewer than its SMs hold CTAs, since a cluster does not reach over GPCs (of
+// four CTAs per SM 592, 296, 187, 142, 112, 93, 78, 71 clusters of 1 ... 8).  Asked once per kernel, size and device.
+template <auto Kernel>
+int clusters_at_once(int size, int threads, size_t smem)
+{
+    constexpr int kMaxDev = 64;
+    static std::atomic<int> known[kMaxDev][kMaxCluster + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return 1;
+    int n = known[dev][size].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(size * 4 * device_info().sms));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, Kernel, &cfg) != cudaSuccess || n <= 0) {
+        (void)cudaGetLastError();
+        n = device_info().sms / size > 0 ? device_info().sms / size : 1;
+    }
+    known[dev][size].store(n, std::memory_order_relaxed);
+    return n;
+}
+
+// How the cache of a K/V head is cut into segments, in bytes of cache that a CTA streams one behind the other.
+//   * Up to eight segments are one cluster.  Its time is the rounds that the heads' clusters take times (segment + 200 KB): what a round costs beside
+//     its bytes was 3.5 us where an SM holds one CTA (49 bytes/ns) and 5 where it holds four.
+//   * More of them leave partial results that the last CTA merges, behind a kernel that clears its counters: about 4 us, another 200 KB.
+//     Worth it with few heads and long caches only: where there is room for sixteen segments per head at once and one of eight would
+//     stream for 7 us by itself (at 25 (bf16) or 41 (fp32) bytes/ns); in the ring kernel, whose SMs hold one CTA, where the sum says so.
+// A cluster whose size is no power of two costs about 1 us more (B1 H8 n1500 d64 fp32: 4 segments 7.5 us, 5 7.0, 7 6.5, 8 5.4). Single heads
+// take powers of two, and 3 where that is one round: of the other sizes some gain up to 15 % and others, at the memory's rate already, lose 7 %
+// (fp32 d64, 88 heads of 12000 keys: 4 segments 79.7 us, 6 84.1).
+// us, with powers of two that fill the slots (which placed the last cluster of eight in a round of its own) and now: single heads B9 H8 n12000 d64
+// fp32 81.4 and 67.5, B9 H8 n3000 d128 bf16 30.2 and 25.8; pairs B9 H16/8 n6000 d128 bf16 64.2 and 47.6; ring B17 H32/8 n4700 d128 fp32 188 and
+// 114, B27 H32/8 n4700 d128 fp32 224 and 178.  Segments of less than 128 keys (one round of loads; 256 in the ring kernel) are not worth a CTA.
+constexpr double kRoundBytes = 200e3;
+double odd_size_bytes(int k, int gc) { return (k & (k - 1)) == 0 ? 0.0 : gc == 1 ? 150e3 : 50e3; }
+int single_ctas(int gc, size_t elem) { return gc == 1 ? 4 : gc == 2 ? (elem == 4 ? 3 : 2) : 1; }      // per SM (registers; the ring's shared memory)
+long long work_items(const DecodeProblem &p) { const int g = p.H / p.Hkv, gc = group_chunk(g); return (long long)p.B * p.Hkv * ((g + gc - 1) / gc); }
+long long segment_cap(const DecodeProblem &p) { const long long least = group_chunk(p.H / p.Hkv) >= 4 ? 256 : 128; return (p.n + least - 1) / least; }
+
+// Segments that merge through memory: j rounds of them where the ring kernel's launch may choose (0: none); 1024 at most
+int segments_through_memory(const DecodeProblem &p, size_t elem, int j)
+{
+    const int gc = group_chunk(p.H / p.Hkv);
+    const long long slots = (long long)device_info().sms * single_ctas(gc, elem), items = work_items(p), cap = segment_cap(p);
+    if (gc < 4 && (slots / items < 16 || 2.0 * p.n * p.d * elem / kMaxCluster <= 7000.0 * (elem == 4 ? 41 : 25))) return 0;
+    long long s = j * slots / items;
+    if (s > cap) s = cap;
+    if (s > 1024) s = 1024;
+    return s > kMaxCluster ? (int)s : 0;
+}
+
+// AtOnce: size -> clusters of that size that run at once
+template <typename AtOnce>
+int choose_segments(const DecodeProblem &p, size_t elem, AtOnce at_once)
+{
+    const int gc = group_chunk(p.H / p.Hkv);
+    const long long items = work_items(p), cap = segment_cap(p);
+    const double bytes = 2.0 * p.n * p.d * elem;
+    if (gc < 4)
+        if (const int s = segments_through_memory(p, elem, 1)) return s;
+    int best = 1;
+    double least = 0;
+    for (int k = 1; k <= kMaxCluster && (k == 1 || k < 2 * cap); k = gc == 1 && k >= 3 ? (k == 3 ? 4 : k * 2) : k + 1) {
+        const long long slots = at_once(k);
+        if (gc == 1 && k == 3 && items > slots) continue;
+        const double cost = (double)((items + slots - 1) / slots) * (bytes / k + kRoundBytes + odd_size_bytes(k, gc));
+        if (k == 1 || cost < least) { least = cost; best = k; }
+    }
+    if (gc >= 4)
+        for (int j = 1; j <= 4; ++j) {
+            const int s = segments_through_memory(p, elem, j);
+            if (s == 0) continue;
+            const long long slots = device_info().sms;
+            const double cost = (double)((items * s + slots - 1) / slots) * (bytes / s + kRoundBytes) + kRoundBytes;
+            if (cost < least) { least = cost; best = s; }
+        }
+    return best;
+}
+
 template <typename T, int D, int GC>
-cudaError_t launch_split(const DecodeProblem &p, const void *q, const void *K, const void *V, float *part_o,
-                         float *part_ml, void *out, float *lse, unsigned int *counters, int splits, int keys_per_split,
-                         cudaStream_t st)
+cudaError_t launch_split(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse, float *ws, cudaStream_t st)
 {
     const int group = p.H / p.Hkv;
-    dim3 grid((unsigned)(p.B * p.Hkv * splits), (unsigned)((group + GC - 1) / GC));
     // warps' states and this segment's result; or what the threads of merge_heads pass on
     size_t merge_smem = (size_t)(kWarps + 1) * GC * (D + 2) * sizeof(float);
     if (merge_smem < kMergeFloats * sizeof(float)) merge_smem = kMergeFloats * sizeof(float);
-    const int clustered = splits <= kMaxCluster ? 1 : 0;
-    if (!clustered) {       // one counter per (K/V head, chunk of query heads): the last of its CTAs to finish merges
-        const cudaError_t ce = decode_clear(counters, (int)(p.B * p.Hkv * grid.y), st);
-        if (ce != cudaSuccess) return ce;
-    }
-    const unsigned cluster = clustered ? (unsigned)splits : 1u;
-    LaunchScope scope(MOA_KERNEL_OTHER, st);
-    if (GC >= 4) {
+    auto go = [&](auto launch, auto at_once) {
+        const int splits = choose_segments(p, sizeof(T), at_once), keys_per_split = (p.n + splits - 1) / splits;
+        const size_t BH = (size_t)p.B * p.H;
+        float *part_o = ws, *part_ml = ws + (size_t)splits * BH * D;
+        unsigned int *counters = reinterpret_cast<unsigned int *>(part_ml + (size_t)splits * BH * 2);
+        const dim3 grid((unsigned)(p.B * p.Hkv * splits), (unsigned)((group + GC - 1) / GC));
+        const int clustered = splits <= kMaxCluster ? 1 : 0;
+        if (!clustered) {       // one counter per (K/V head, chunk of query heads): the last of its CTAs to finish merges
+            const cudaError_t ce = decode_clear(counters, (int)(p.B * p.Hkv * grid.y), st);
+            if (ce != cudaSuccess) return ce;
+        }
+        LaunchScope scope(MOA_KERNEL_OTHER, st);
+        return launch(grid, clustered ? (unsigned)splits : 1u, part_o, part_ml, counters, clustered, splits, keys_per_split, BH);
+    };
+    if constexpr (GC >= 4) {
         constexpr int kStages = Ring<T, D>::kStages;
         const size_t ring_smem = (size_t)kStages * 2 * kTileRows * D * sizeof(T) + 2 * kStages * sizeof(uint64_t) + 16;
         const size_t smem = ring_smem > merge_smem ? ring_smem : merge_smem;
-        cudaError_t e = allow_smem<decode_ring_kernel<T, D, GC>>(smem);
+        const cudaError_t e = allow_smem<decode_ring_kernel<T, D, GC>>(smem);
         if (e != cudaSuccess) return e;
-        return launch_cluster(decode_ring_kernel<T, D, GC>, cluster, grid, dim3(kRingThreads), smem, st, (const T *)q, (const T *)K,
-                              (const T *)V, part_o, part_ml, (T *)out, lse, counters, clustered, p.n, p.H, p.Hkv, group, splits,
-                              keys_per_split, (size_t)p.B * p.H, p.scale * kLog2e, device_status_ptr());
+        return go([&](dim3 grid, unsigned cluster, float *part_o, float *part_ml, unsigned int *counters, int clustered, int splits, int keys, size_t BH) {
+            return launch_cluster(decode_ring_kernel<T, D, GC>, cluster, grid, dim3(kRingThreads), smem, st, (const T *)q, (const T *)K, (const T *)V,
+                                  part_o, part_ml, (T *)out, lse, counters, clustered, p.n, p.H, p.Hkv, group, splits, keys, BH, p.scale * kLog2e,
+                                  device_status_ptr());
+        }, [&](int size) { return clusters_at_once<decode_ring_kernel<T, D, GC>>(size, kRingThreads, smem); });
+    } else {
+        const cudaError_t e = allow_smem<decode_split_kernel<T, D, GC>>(merge_smem);
+        if (e != cudaSuccess) return e;
+        return go([&](dim3 grid, unsigned cluster, float *part_o, float *part_ml, unsigned int *counters, int clustered, int splits, int keys, size_t BH) {
+            return launch_cluster(decode_split_kernel<T, D, GC>, cluster, grid, dim3(kThreads), merge_smem, st, (const T *)q, (const T *)K, (const T *)V,
+                                  part_o, part_ml, (T *)out, lse, counters, clustered, p.n, p.H, p.Hkv, group, splits, keys, BH, p.scale * kLog2e);
+        }, [&](int size) { return clusters_at_once<decode_split_kernel<T, D, GC>>(size, kThreads, merge_smem); });
     }
-    cudaError_t e = allow_smem<decode_split_kernel<T, D, GC>>(merge_smem);
-    if (e != cudaSuccess) return e;
-    return launch_cluster(decode_split_kernel<T, D, GC>, cluster, grid, dim3(kThreads), merge_smem, st, (const T *)q, (const T *)K,
-                          (const T *)V, part_o, part_ml, (T *)out, lse, counters, clustered, p.n, p.H, p.Hkv, group, splits, keys_per_split,
-                          (size_t)p.B * p.H, p.scale * kLog2e);
 }
 
 template <typename T, int D>
 cudaError_t launch_decode(const DecodeProblem &p, const void *q, const void *K, const void *V, void *out, float *lse,
                           float *ws, cudaStream_t st)
 {
-    const int splits = decode_splits(p, sizeof(T) == 4 ? MOA_F32 : MOA_BF16);
-    const int keys_per_split = (p.n + splits - 1) / splits;
-    const size_t BH = (size_t)p.B * p.H;
-    float *part_o = ws, *part_ml = ws + (size_t)splits * BH * D;
-    unsigned int *counters = reinterpret_cast<unsigned int *>(part_ml + (size_t)splits * BH * 2);
     const int gc = group_chunk(p.H / p.Hkv);
-    return gc == 8 ? launch_split<T, D, 8>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st)
-         : gc == 4 ? launch_split<T, D, 4>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st)
-         : gc == 2 ? launch_split<T, D, 2>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st)
-                   : launch_split<T, D, 1>(p, q, K, V, part_o, part_ml, out, lse, counters, splits, keys_per_split, st);
+    return gc == 8 ? launch_split<T, D, 8>(p, q, K, V, out, lse, ws, st)
+         : gc == 4 ? launch_split<T, D, 4>(p, q, K, V, out, lse, ws, st)
+         : gc == 2 ? launch_split<T, D, 2>(p, q, K, V, out, lse, ws, st)
+                   : launch_split<T, D, 1>(p, q, K, V, out, lse, ws, st);
 }
 
 }  // namespace
@@ -623,48 +713,6 @@ static void decode_tc_splits(const DecodeProblem &p, int *splits, int *tiles_per
     *splits = (nkt + tps - 1) / tps;          // every segment has at least one tile
 }
 
-// Segments of the cache per K/V head, each with at least 128 keys (one round of loads of the bf16 d = 64 kernel; with 256 a short
-// cache left half of the SMs idle: B1 H16 n1000 8.2 -> 5.3 us) or, in the ring kernel, of which an SM holds one CTA, 256 (with 128: fp32
-// groups of 8 over 4359 keys 54 -> 66 us).
-// Up to eight segments, a power of two, are one cluster.  The streaming kernel's CTAs all run at once, four or (pairs of heads) three to an SM:
-// a few more than that begin when the others end (B1 H32 n16000 d128 with 19 segments, 608 CTAs, 61.9 us, with 16 46.2; B8 H16 n600 d64 with
-// 8 9.3, with 4 6.4).  More segments than a cluster has cost the clearing of the counters and a merge through memory, about 4 us: they
-// pay only where a segment of eight would stream for longer than that by itself, at 25 (bf16) or 41 (fp32) bytes per ns, and there is room for twice as
-// many (B6 H8 n4390 d64 8: 14.1 us, 13: 18.1; B4 H16 n8000 d128 8: 43.5, 10: 59.4; but B1 H8 n30000 d64 8: 45.1, 74: 17.9).
-// Single heads with segments of 500 KB or more take more of them, in several waves, where those fill the slots a fifth better
-// (B20 H32 n8000 d64, 640 heads, 1: 254.5, 4: 206.4; B20 H16 n4000 d128 1: 125.5, 4: 115.6; B25 H8 n16000 d64 2: 135.7, 8: 129.4; the same fill,
-// B16 H16 n8192 d128, 2: 157.9, 4: 161.3; shorter segments, B20 H8 n3000 d128 fp32, 2: 73.1, 8: 79.3; pairs, B16 H32/16 n6000 d128, 1: 132.0, 8: 159.9).
-// The one shape found where the former rule, more than slots, is better: B13 H8 n8000 d128 fp32, 4: 132.9, 8: 128.4.
-int decode_splits(const DecodeProblem &p, int dtype)
-{
-    const int group = p.H / p.Hkv;
-    const int gc = group_chunk(group);
-    const long long sms = device_info().sms, heads = (long long)p.B * p.Hkv * ((group + gc - 1) / gc);
-    const long long least = gc >= 4 ? 256 : 128, cap = (p.n + least - 1) / least;
-    if (gc < 4) {
-        const long long slots = sms * (gc == 1 ? 4 : 3), fit = slots / heads;
-        const double head_bytes = 2.0 * p.n * p.d * (dtype == MOA_F32 ? 4 : 2);
-        if (fit >= 16 && cap > kMaxCluster && head_bytes / kMaxCluster > 7000.0 * (dtype == MOA_F32 ? 41 : 25)) {
-            const long long s = fit < cap ? fit : cap;
-            return (int)(s > 1024 ? 1024 : s);
-        }
-        int c = kMaxCluster;
-        while (c > 1 && (heads * c > slots || c / 2 >= cap)) c /= 2;
-        const auto fill = [&](int k) { return (double)(heads * k) / (double)((heads * k + slots - 1) / slots * slots); };
-        for (int k = c * 2; gc == 1 && k <= kMaxCluster && head_bytes / k >= 5e5; k *= 2)
-            if (fill(k) >= 1.2 * fill(c)) c = k;
-        return c;
-    }
-    long long s = (4LL * sms + heads - 1) / heads;
-    if (s > cap) s = cap;
-    if (s < 1) s = 1;
-    if (s > 1024) s = 1024;
-    if (s <= kMaxCluster)
-        for (int c = 1; c <= kMaxCluster; c *= 2)
-            if (c >= s) { s = c; break; }
-    return (int)s;
-}
-
 size_t decode_workspace_bytes(const DecodeProblem &p, int dtype)
 {
     if (decode_uses_mma(p, dtype)) return decode_mma_workspace_bytes(p);
@@ -674,8 +722,10 @@ size_t decode_workspace_bytes(const DecodeProblem &p, int dtype)
         const size_t heads = (size_t)splits * p.B * p.H;
         return ((heads * p.d * 2 + 255) / 256) * 256 + heads * sizeof(float);
     }
-    // partial results of the segments, then one counter per (K/V head, chunk of query heads)
-    return (size_t)decode_splits(p, dtype) * p.B * p.H * (p.d + 2) * sizeof(float) + (size_t)p.B * p.H * sizeof(unsigned int);
+    // partial results of the segments (of the most that a launch merges through memory; clusters leave none), then one counter per (K/V head,
+    // chunk of query heads)
+    const int most = segments_through_memory(p, dtype == MOA_F32 ? 4 : 2, group_chunk(p.H / p.Hkv) >= 4 ? 4 : 1);
+    return (size_t)most * p.B * p.H * (p.d + 2) * sizeof(float) + (size_t)p.B * p.H * sizeof(unsigned int);
 }
 
 cudaError_t decode_attn(const DecodeProblem &p, int dtype, const void *q, const void *K, const void *V, void *out,
