@@ -71,9 +71,10 @@ struct RowRegs {
     uint4 v[R][kV];
 };
 
-template <int kV, int R>
+// kToken: `token` keeps the loads behind the wait; otherwise `src` has gone through after_wait().
+template <int kV, int R, bool kToken = false>
 __device__ __forceinline__ void load_rows(RowRegs<kV, R> &dst, const __nv_bfloat16 *__restrict__ src, long long row0,
-                                          int n, int d, int c, int tpr)
+                                          int n, int d, int c, int tpr, uint32_t token = 0)
 {
     const int nvec = d / 8;
 #pragma unroll
@@ -82,7 +83,10 @@ __device__ __forceinline__ void load_rows(RowRegs<kV, R> &dst, const __nv_bfloat
         for (int j = 0; j < kV; ++j) {
             const int v = c + j * tpr;
             dst.v[i][j] = make_uint4(0u, 0u, 0u, 0u);
-            if (row0 + i < n && v < nvec) dst.v[i][j] = __ldcs(reinterpret_cast<const uint4 *>(src + (size_t)(row0 + i) * d) + v);
+            if (row0 + i < n && v < nvec) {
+                const uint4 *at = reinterpret_cast<const uint4 *>(src + (size_t)(row0 + i) * d) + v;
+                dst.v[i][j] = kToken ? ptx::ld_cs_v4(at, token) : __ldcs(at);
+            }
         }
 }
 
@@ -194,9 +198,10 @@ __device__ __forceinline__ void dg_columns(const __nv_bfloat16 *x, const __nv_bf
 }
 
 // Backward.  Besides dx, every CTA leaves its partial dg (summed over its rows in a fixed order) in
-// part[blockIdx.x][d]; rmsnorm_dg_kernel adds the partials up.  col_blocks > 0 (few rows): the first col_blocks CTAs compute dg from x, dy and r
-// instead, and there are no partials.
-template <int kV, int R>
+// part[blockIdx.x][d]; rmsnorm_dg_kernel adds the partials up.  kCols (few rows): the first col_blocks CTAs compute dg from x, dy and r
+// instead, and there are no partials.  (A kernel of its own, and r requested an iteration ahead: with the branch, and r's load held behind the
+// stores before it, 25579 x 2632 took 132 us, 124 before there was a wait for the kernel in front, 121 so.)
+template <int kV, int R, bool kCols>
 __global__ void __launch_bounds__(kNormThreads)
 rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g,
                    const float *__restrict__ r_in, const __nv_bfloat16 *__restrict__ dy,
@@ -205,14 +210,16 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
 {
     __shared__ float red[8 * R];
     __shared__ float acc[kNormThreads * 8];              // [row lane][tpr*8] for one j at a time
-    ptx::grid_dependency_wait();
+    constexpr bool kToken = !kCols && kV <= 2;
+    const uint32_t token = ptx::grid_dependency_wait_token();
     ptx::grid_launch_dependents();
-    x = ptx::after_wait(x); g = ptx::after_wait(g); r_in = ptx::after_wait(r_in); dy = ptx::after_wait(dy); dx_add = ptx::after_wait(dx_add);
-    if ((int)blockIdx.x < col_blocks) {
+    g = ptx::after_wait(g);
+    if (!kToken) { x = ptx::after_wait(x); r_in = ptx::after_wait(r_in); dy = ptx::after_wait(dy); dx_add = ptx::after_wait(dx_add); }
+    if (kCols && (int)blockIdx.x < col_blocks) {
         dg_columns(x, dy, r_in, dg, n, d, (int)blockIdx.x * kDgCols, acc);
         return;
     }
-    const int block = (int)blockIdx.x - col_blocks, blocks = (int)gridDim.x - col_blocks;
+    const int block = kCols ? (int)blockIdx.x - col_blocks : (int)blockIdx.x, blocks = kCols ? (int)gridDim.x - col_blocks : (int)gridDim.x;
     const int c = threadIdx.x % tpr, rl = threadIdx.x / tpr, lanes = kNormThreads / tpr;
     const int nvec = d / 8;
     float gf[kV][8], dgacc[kV][8];
@@ -230,18 +237,23 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
     const long long first = ((long long)block * lanes + rl) * R;
     const float inv_d = 1.f / (float)d;
     RowRegs<kV, R> xc, dc, xn, dn;
-    load_rows<kV, R>(xc, x, first, n, d, c, tpr);
-    load_rows<kV, R>(dc, dy, first, n, d, c, tpr);
+    // the stored r of an iteration's rows: requested with its x and dy an iteration ahead, or (kToken = false) ahead of its reductions
+    float rc[R], rn[R];
+    auto load_r = [&](float (&to)[R], long long row0) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) to[i] = (r_in != nullptr && row0 + i < n) ? (kToken ? ptx::ld_f32(r_in + row0 + i, token) : r_in[row0 + i]) : 0.f;
+    };
+    load_rows<kV, R, kToken>(xc, x, first, n, d, c, tpr, token);
+    load_rows<kV, R, kToken>(dc, dy, first, n, d, c, tpr, token);
+    if (kToken) load_r(rc, first);
     for (int it = 0; it < iters; ++it) {
         const long long row0 = it * rows_per_iter + first;
         if (it + 1 < iters) {
-            load_rows<kV, R>(xn, x, row0 + rows_per_iter, n, d, c, tpr);
-            load_rows<kV, R>(dn, dy, row0 + rows_per_iter, n, d, c, tpr);
+            load_rows<kV, R, kToken>(xn, x, row0 + rows_per_iter, n, d, c, tpr, token);
+            load_rows<kV, R, kToken>(dn, dy, row0 + rows_per_iter, n, d, c, tpr, token);
         }
-        // the stored r of this iteration's rows: requested here, ahead of the reductions and their barriers
-        float rr[R];
-#pragma unroll
-        for (int i = 0; i < R; ++i) rr[i] = (r_in != nullptr && row0 + i < n) ? r_in[row0 + i] : 0.f;
+        if (!kToken) load_r(rc, row0);
+        else if (it + 1 < iters) load_r(rn, row0 + rows_per_iter);
         // per row: t = sum_k x_k g_k dy_k, and sum_k x_k^2 when r is not given
         float t[R], ss[R];
 #pragma unroll
@@ -264,7 +276,7 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
 #pragma unroll
         for (int i = 0; i < R; ++i) {
             if (row0 + i >= n) continue;
-            const float r = r_in != nullptr ? rr[i] : rsqrtf(ss[i] * inv_d + eps);
+            const float r = r_in != nullptr ? rc[i] : rsqrtf(ss[i] * inv_d + eps);
             const float coef = r * r * r * t[i] * inv_d;
 #pragma unroll
             for (int j = 0; j < kV; ++j) {
@@ -273,7 +285,10 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
                 float fx[8], fd[8], o[8], fa[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 unpack8(xc.v[i][j], fx);
                 unpack8(dc.v[i][j], fd);
-                if (dx_add != nullptr) unpack8(__ldcs(reinterpret_cast<const uint4 *>(dx_add + (size_t)(row0 + i) * d) + v), fa);
+                if (dx_add != nullptr) {
+                    const uint4 *at = reinterpret_cast<const uint4 *>(dx_add + (size_t)(row0 + i) * d) + v;
+                    unpack8(kToken ? ptx::ld_cs_v4(at, token) : __ldcs(at), fa);
+                }
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     o[e] = r * gf[j][e] * fd[e] - fx[e] * coef + fa[e];
@@ -284,8 +299,10 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
         }
         xc = xn;
         dc = dn;
+#pragma unroll
+        for (int i = 0; kToken && i < R; ++i) rc[i] = rn[i];
     }
-    if (col_blocks > 0) return;
+    if (kCols) return;
     // CTA partial of dg: the row lanes' sums added in lane order
     float *mine = part + (size_t)block * d;
 #pragma unroll
@@ -314,12 +331,15 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
 // straight to global memory in whole 512-byte runs.  A row is read from shared memory twice (sums,
 // then results) rather than held in registers, and the gain sits in shared memory as floats, which
 // keeps the kernel near 100 registers.  Every wait is bounded.
+// kAdd: with dx_add.  Registers decide the backward at 2048 columns: with the addresses of r and dx_add made opaque behind the wait, and the null
+// test of dx_add in the loop, 65536 x 2048 took 176 us (163 before there was a wait), with their loads pinned where they are and kAdd 149; with
+// dx_add 259 and 256.
 constexpr int kRingWarps = 8;                 // consumer warps per group = rows per stage / m
 constexpr int kRingGroups = 2;                // consumer groups; group q takes the CTA's stages q, q + 2, ...
 constexpr int kRingThreads = 32 * (kRingGroups * kRingWarps + 1), kRingStages = 3;
 enum { NERR_EMPTY = 0x401, NERR_FULL = 0x402 };
 
-template <int kV, bool kBwd>
+template <int kV, bool kBwd, bool kAdd>
 __global__ void __launch_bounds__(kRingThreads, 1)
 rmsnorm_ring_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__restrict__ g, const float *__restrict__ r_in,
                     float *__restrict__ r_out, const __nv_bfloat16 *__restrict__ dy, const __nv_bfloat16 *__restrict__ dx_add,
@@ -346,7 +366,7 @@ rmsnorm_ring_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__
     }
     grid_dependency_wait();
     grid_launch_dependents();
-    g = after_wait(g); r_in = after_wait(r_in); dx_add = after_wait(dx_add);
+    g = after_wait(g);
     for (int i = threadIdx.x; i < d; i += kRingThreads) gs[i] = __bfloat162float(g[i]);
     __syncthreads();
     float dgacc[kV][8];          // backward only (dead otherwise)
@@ -390,7 +410,7 @@ rmsnorm_ring_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__
                 const long long row = row0 + lr;
                 if (row >= n) break;                          // warp-uniform
                 float rr = 0.f;
-                if (kBwd && r_in != nullptr) rr = r_in[row];
+                if (kBwd && r_in != nullptr) rr = ld_f32_here(r_in + row);
                 float ss = 0.f, t = 0.f;
 #pragma unroll
                 for (int j = 0; j < kV; ++j) {
@@ -423,7 +443,7 @@ rmsnorm_ring_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__
                     float fx[8], fd[8], o8[8], fa[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                     unpack8(*reinterpret_cast<const uint4 *>(sx + lr * row_bytes + 16 * v), fx);
                     if (kBwd) unpack8(*reinterpret_cast<const uint4 *>(sd + lr * row_bytes + 16 * v), fd);
-                    if (kBwd && dx_add != nullptr) unpack8(__ldcs(reinterpret_cast<const uint4 *>(dx_add + (size_t)row * d) + v), fa);
+                    if (kAdd) unpack8(ld_cs_v4_here(dx_add + (size_t)row * d + 8 * v), fa);
                     const float4 g0 = *reinterpret_cast<const float4 *>(gs + 8 * v), g1 = *reinterpret_cast<const float4 *>(gs + 8 * v + 4);
                     const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
 #pragma unroll
@@ -554,10 +574,14 @@ cudaError_t launch_ring(const RingPlan &p, const __nv_bfloat16 *x, const __nv_bf
                         const __nv_bfloat16 *dy, const __nv_bfloat16 *dx_add, __nv_bfloat16 *out, float *part, int n, int d,
                         float eps, cudaStream_t st)
 {
-    cudaError_t e = allow_smem<rmsnorm_ring_kernel<kV, kBwd>>(p.smem);
-    if (e != cudaSuccess) return e;
-    return launch_dependent(rmsnorm_ring_kernel<kV, kBwd>, dim3(p.grid), dim3(kRingThreads), p.smem, st, x, g, r_in, r_out, dy, dx_add, out,
-                            part, n, d, eps, p.m, device_status_ptr());
+    auto go = [&](auto kernel, cudaError_t e) {
+        if (e != cudaSuccess) return e;
+        return launch_dependent(kernel, dim3(p.grid), dim3(kRingThreads), p.smem, st, x, g, r_in, r_out, dy, dx_add, out, part, n, d, eps, p.m,
+                                device_status_ptr());
+    };
+    if constexpr (kBwd)
+        if (dx_add != nullptr) return go(rmsnorm_ring_kernel<kV, kBwd, true>, allow_smem<rmsnorm_ring_kernel<kV, kBwd, true>>(p.smem));
+    return go(rmsnorm_ring_kernel<kV, kBwd, false>, allow_smem<rmsnorm_ring_kernel<kV, kBwd, false>>(p.smem));
 }
 template <bool kBwd>
 cudaError_t launch_ring_kv(const RingPlan &p, const __nv_bfloat16 *x, const __nv_bfloat16 *g, const float *r_in, float *r_out,
@@ -615,7 +639,8 @@ cudaError_t rmsnorm_bwd(int n, int d, float eps, const void *x, const void *g, c
         if (e != cudaSuccess) return e;
     } else {
         LaunchScope scope(MOA_KERNEL_OTHER, st);
-        const auto kernel = p.kV == 1 ? rmsnorm_bwd_kernel<1, 2> : p.kV == 2 ? rmsnorm_bwd_kernel<2, 1> : rmsnorm_bwd_kernel<4, 2>;
+        const auto kernel = col_blocks > 0 ? (p.kV == 1 ? rmsnorm_bwd_kernel<1, 2, true> : p.kV == 2 ? rmsnorm_bwd_kernel<2, 1, true> : rmsnorm_bwd_kernel<4, 2, true>)
+                                           : (p.kV == 1 ? rmsnorm_bwd_kernel<1, 2, false> : p.kV == 2 ? rmsnorm_bwd_kernel<2, 1, false> : rmsnorm_bwd_kernel<4, 2, false>);
         const cudaError_t e = launch_dependent(kernel, dim3(p.grid + col_blocks), dim3(kNormThreads), (size_t)0, st, xb, gb, r, db, ab, ob, part,
                                                (__nv_bfloat16 *)dg, col_blocks, n, d, eps, p.tpr);
         if (e != cudaSuccess || col_blocks > 0) return e;

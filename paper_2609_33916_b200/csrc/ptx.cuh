@@ -47,6 +47,40 @@ template <typename T> __device__ __forceinline__ T *after_wait(T *p)
     asm volatile("" : "+l"(p) :: "memory");
     return p;
 }
+// The wait with a token, and loads of what no CTA of this kernel writes, which take it: they cannot be moved in front of the wait and are
+// otherwise free, through the kernel's own parameters.  Where registers are short, a pointer that after_wait() has made opaque costs two of
+// them, its null test an instruction each time, and its loads stay in order with the stores.
+__device__ __forceinline__ uint32_t grid_dependency_wait_token()
+{
+    uint32_t t;
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(t) :: "memory");
+    return t;
+}
+__device__ __forceinline__ uint4 ld_cs_v4(const void *p, uint32_t token)
+{
+    uint4 v;
+    asm("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "r"(token));
+    return v;
+}
+__device__ __forceinline__ float ld_f32(const float *p, uint32_t token)
+{
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p), "r"(token));
+    return v;
+}
+// The same, kept where they are written (volatile, like the wait: behind it in program order)
+__device__ __forceinline__ uint4 ld_cs_v4_here(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_f32_here(const float *p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)

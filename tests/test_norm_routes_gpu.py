@@ -35,3 +35,31 @@ def test_rmsnorm_routes(n, d):
         got = t.float().cpu().numpy().astype(np.float64)
         assert np.all(np.isfinite(got)) and mi.rel_err(got, ref[k]) <= TOL, (k, mi.rel_err(got, ref[k]))
     assert mi.rel_err(r.cpu().numpy().astype(np.float64), ref["r"]) <= 1e-5
+
+
+@pytest.mark.parametrize("with_r", [True, False])
+@pytest.mark.parametrize("with_add", [True, False])
+@pytest.mark.parametrize("n,d", [(513, 2048), (4099, 264), (1033, 1016), (8193, 136), (1537, 2056), (800, 4104), (900, 8192), (300, 72)])
+def test_rmsnorm_backward_forms(n, d, with_add, with_r):
+    """With and without the added gradient and the stored r, in the ring kernel (first three), the register kernels and the one-launch form."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2609_33916_b200 import binding as mb
+    from paper_2609_33916_b200 import build
+    build.build()
+    inp = mi.make_norm_inputs(n, d, seed=5 * n + d)
+    x, g, dy = (torch.from_numpy(np.ascontiguousarray(inp[k])).view(torch.bfloat16).cuda() for k in ("x", "g", "dy"))
+    add = torch.randn(x.shape, generator=torch.Generator(device="cuda").manual_seed(n), device="cuda").bfloat16() if with_add else None
+    y, dx, dg = (torch.full_like(t, float("nan")) for t in (x, x, g))
+    r = torch.full((n,), float("nan"), dtype=torch.float32, device="cuda")
+    desc = mb.make_rmsnorm_desc(n, d, 1e-5)
+    ws = torch.full((mb.moa_rmsnorm_workspace_bytes(desc),), 0xFF, dtype=torch.uint8, device="cuda")
+    mb.moa_rmsnorm_fwd(desc, x, g, y, r)
+    mb.moa_rmsnorm_bwd(desc, x, g, r if with_r else None, dy, dx, dg, ws, dx_add=add)
+    f = {k: mi.to_f64(v, "bf16") for k, v in inp.items()}
+    ref = oracle.rmsnorm_fwd_bwd(f["x"], f["g"], f["dy"], 1e-5)
+    want = ref["dx"] + (add.double().cpu().numpy() if with_add else 0.0)
+    for got, r_ in ((dx, want), (dg, ref["dg"])):
+        got = got.float().cpu().numpy().astype(np.float64)
+        assert np.all(np.isfinite(got)) and mi.rel_err(got, r_) <= TOL
