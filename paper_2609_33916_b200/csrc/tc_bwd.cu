@@ -793,7 +793,13 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     Problem pkv = p;
     pkv.H = p.kv_heads();
     pkv.Hkv = 0;
-    return launch_cluster(tc_bwd_kernel<D, kBulk, kGrouped, kSplit, KL>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)),
+    // A long walk is launched plainly: CTAs that wait for the kernel in front are let go at one instant, walk the query tiles of their head in step, and
+    // their reduces meet on the same dQ tile.  Plain / dependent, d = 128: B1 H32/4 n4096 698 / 785 us, B2 H32/8 n4096 1410 / 1538, causal B4 H16/4
+    // n4096 806 / 867; but short walks want the early start (B1 H32/8 n1000 71.0 / 68.9), and so do causal jobs that all run at once (B1 H32/4
+    // n4096 440 / 416) and 64 columns, whose reduces are smaller (within 2 % either way).
+    const long long walk = (long long)nkt * p.group();
+    const bool apart = D == 128 && kBulk && !kSplit && (p.causal ? walk >= 100 && (long long)nkt * p.BHkv() > device_info().sms : walk >= 48);
+    return launch_cluster_as(!apart, tc_bwd_kernel<D, kBulk, kGrouped, kSplit, KL>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)),
                           dim3(kThreads), (size_t)kSmem, st,
                             mq, mk, mv, mdo, mdq, mdk, mdv, Lp, Dp, dQacc, p.n, nkt * 128, p.causal, p.scale, p.scale * kLog2e, nkt,
                             heads_per_group(pkv, nkt), p.group(), p.kv_heads(), dQacc == nullptr ? 1 : 0, device_status_ptr(),
