@@ -33,8 +33,12 @@
 // with two of them, and the tile takes about 1550.
 // The O tile leaves through the Q tile's shared memory and a TMA store.
 //
-// KL: 16-column steps of the head dimension that hold anything (6 for 72..96 in the 128-column kernel).  Head dimensions 136..256:
-// tc_fwd_wide.cu.
+// KC = 2, head dimensions 200..256 where there are few query tiles (more of them: tc_fwd_wide.cu): the scores need the whole head dimension, the
+// output does not.  S = Q K^T is accumulated over two chunks of 128 columns -- Q holds both, the K ring carries one chunk per slot, so a key
+// tile passes through it twice -- and the grid has two CTAs per (head, query tile), each with the V columns and the O columns of one
+// 128-column half (the scores and the softmax are computed twice).  The backward's per-row inputs are not prepared here (a CTA holds half of an
+// O row).
+// KL: 16-column steps of the head dimension that hold anything (6 for 72..96 in the 128-column kernel).
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tensormap.cuh"
@@ -82,7 +86,7 @@ struct FwdPrep {
     int d;               // columns of a dO row in memory (<= D)
 };
 
-template <int D, int KL>
+template <int D, int KC, int KL>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapO,
@@ -94,16 +98,18 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     constexpr int kBoxes = D / 64;         // 64-column (128-byte) swizzled boxes per tile
     constexpr int kBoxBytes = 128 * 128;   // 128 rows x 128 bytes
     extern __shared__ __align__(1024) uint8_t sm[];
-    uint8_t *sQ = sm, *sK = sm + kTileBytes /*2 slots*/, *sV = sm + 3 * kTileBytes /*2 slots*/;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + 5 * kTileBytes);
+    uint8_t *sQ = sm /*KC chunks*/, *sK = sm + KC * kTileBytes /*2 slots of one chunk*/, *sV = sm + (KC + 2) * kTileBytes /*2 slots*/;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + (KC + 4) * kTileBytes);
     uint32_t *tmem_base_p = reinterpret_cast<uint32_t *>(bars + F_COUNT);
     volatile uint32_t *abortp = reinterpret_cast<uint32_t *>(bars + F_COUNT + 1);
 
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     int bh, t;
-    const int blk = (int)blockIdx.x;
+    // KC > 1: KC consecutive CTAs share a job, CTA `pass` computes output columns [D pass, D pass + D)
+    const int pass = KC > 1 ? (int)blockIdx.x % KC : 0;
+    const int blk = KC > 1 ? (int)blockIdx.x / KC : (int)blockIdx.x;
     const int split = sp.splits > 1 ? blk % sp.splits : 0;
-    const int heads_all = (int)gridDim.x / sp.splits / nqt;
+    const int heads_all = (int)gridDim.x / KC / sp.splits / nqt;
     job_from_block(sp.splits > 1 ? blk / sp.splits : blk, nqt, heads_all, hpg, bh, t);
     const int bb = bh / H, hq = bh - bb * H;    // batch and query head: coordinates of the 4-D tensor maps
     const int hk = hq / group;                  // the K/V head this query head reads (group > 1: shared heads)
@@ -117,7 +123,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     // Q, the first two K chunks and the first two V tiles are on their way while the rest of the set-up (the other
     // barriers, the TMEM allocation, the CTA-wide barrier) still runs, instead of starting behind it.
     const bool aligned = (smem_u32(sm) & 1023u) == 0;      // (swizzled tiles need the 1024-byte alignment)
-    const int early_k = aligned ? min(nkt_want, 2) : 0, early_v = aligned ? min(nkt_want, 2) : 0;
+    const int early_k = aligned ? min(nkt_want * KC, 2) : 0, early_v = aligned ? min(nkt_want, 2) : 0;
     if (warp == 8 && lane == 0) {
         mbar_init(bars + F_Q, 1u);
         mbar_init(bars + F_KFULL, 1u);
@@ -125,12 +131,13 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         fence_mbar_init();
         grid_dependency_wait();
         if (early_k > 0) {
-            mbar_arrive_expect_tx(bars + F_Q, kTileBytes);
-            for (int b = 0; b < kBoxes; ++b) tma_load_4d(sQ + b * kBoxBytes, &mapQ, bars + F_Q, 64 * b, q0, hq, bb);
-            for (int j = 0; j < early_k; ++j) {
-                mbar_arrive_expect_tx(bars + F_KFULL + j, kTileBytes);
+            mbar_arrive_expect_tx(bars + F_Q, KC * kTileBytes);
+            for (int b = 0; b < KC * kBoxes; ++b) tma_load_4d(sQ + b * kBoxBytes, &mapQ, bars + F_Q, 64 * b, q0, hq, bb);
+            for (int g = 0; g < early_k; ++g) {       // chunk g: columns [D c, D c + D) of key tile j, g = j KC + c
+                const int j = g / KC, c = g % KC;
+                mbar_arrive_expect_tx(bars + F_KFULL + g, kTileBytes);
                 for (int b = 0; b < kBoxes; ++b)
-                    tma_load_4d(sK + j * kTileBytes + b * kBoxBytes, &mapK, bars + F_KFULL + j, 64 * b, (kt0 + j) * BN, hk, bb);
+                    tma_load_4d(sK + g * kTileBytes + b * kBoxBytes, &mapK, bars + F_KFULL + g, D * c + 64 * b, (kt0 + j) * BN, hk, bb);
             }
         }
     }
@@ -142,7 +149,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         for (int j = 0; j < early_v; ++j) {
             mbar_arrive_expect_tx(bars + F_VFULL + j, kTileBytes);
             for (int b = 0; b < kBoxes; ++b)
-                tma_load_4d(sV + j * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + j, 64 * b, (kt0 + j) * BN, hk, bb);
+                tma_load_4d(sV + j * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + j, D * pass + 64 * b, (kt0 + j) * BN, hk, bb);
         }
     }
     if (tid == 0) {
@@ -174,24 +181,31 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
       asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
       if (warp == 8) {
         // ------------------------------------------------------------------ TMA producer
-        int nk = early_k;       // K tiles requested so far (slot = count & 1): Q and the first two went out before the set-up
+        int nk = early_k;       // K chunks requested so far (slot = count & 1): Q and the first two went out before the set-up
+        // chunk g of the K stream: 128 columns [D c, D c + D) of key tile j, g = j KC + c, ring slot g & 1
+        auto load_k = [&](int g) {
+            const int s = g & 1, j = g / KC, c = g % KC;
+            mbar_arrive_expect_tx(bars + F_KFULL + s, kTileBytes);
+            ++nk;
+            for (int b = 0; b < kBoxes; ++b)
+                tma_load_4d(sK + s * kTileBytes + b * kBoxBytes, &mapK, bars + F_KFULL + s, D * c + 64 * b, (kt0 + j) * BN, hk, bb);
+        };
         if (zero_acc != nullptr) {
-            // Fused forward+backward: this CTA's 128 rows of the fp32 dQ accumulator ([B*H, n, D]) are
+            // Fused forward+backward (KC = 1): this CTA's 128 rows of the fp32 dQ accumulator ([B*H, n, D]) are
             // cleared here, by the producer warp while its first loads are in flight (the next slot
             // frees two tiles from now), so that the step needs no separate clearing pass.
             const int rows = min(BM, n - q0);
             float4 *dst = reinterpret_cast<float4 *>(zero_acc + ((size_t)bh * n + q0) * D);
             for (int i = lane; i < rows * (D / 4); i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        for (int j = early_k; j < nkt; ++j) {
-            if (j >= 2 && !mbar_wait(bars + F_KEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR_K)) break;
-            if (lane == 0) {
-                const int s = j & 1;
-                mbar_arrive_expect_tx(bars + F_KFULL + s, kTileBytes);
-                ++nk;
-                for (int b = 0; b < kBoxes; ++b)
-                    tma_load_4d(sK + s * kTileBytes + b * kBoxBytes, &mapK, bars + F_KFULL + s, 64 * b, (kt0 + j) * BN, hk, bb);
+        bool live = true;
+        for (int j = early_k / KC; live && j < nkt; ++j) {
+            for (int c = (j == early_k / KC ? early_k % KC : 0); c < KC; ++c) {
+                const int g = j * KC + c;
+                if (g >= 2 && !mbar_wait(bars + F_KEMPTY + (g & 1), ((g >> 1) - 1) & 1, abortp, status, ERR_K)) { live = false; break; }
+                if (lane == 0) load_k(g);
             }
+            if (!live) break;
             __syncwarp();
         }
         if (lane == 0 && *abortp) {
@@ -211,7 +225,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 mbar_arrive_expect_tx(bars + F_VFULL + s, kTileBytes);
                 ++nv;
                 for (int b = 0; b < kBoxes; ++b)
-                    tma_load_4d(sV + s * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + s, 64 * b, (kt0 + j) * BN, hk, bb);
+                    tma_load_4d(sV + s * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + s, D * pass + 64 * b, (kt0 + j) * BN, hk, bb);
             }
             __syncwarp();
         }
@@ -231,22 +245,27 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         auto field = [](const void *ptr) { return (smem_u32(ptr) >> 4) & 0x3FFFu; };
         const uint32_t q_lo = (uint32_t)km_proto + field(sQ), k_lo0 = (uint32_t)km_proto + field(sK);
         constexpr uint32_t kSlot = (uint32_t)(kTileBytes >> 4);
-        const bool ok = nkt > 0 && mbar_wait(bars + F_Q, 0, abortp, status, ERR_Q);
+        bool ok = nkt > 0 && mbar_wait(bars + F_Q, 0, abortp, status, ERR_Q);
         for (int j = 0; ok && j < nkt; ++j) {
             const uint32_t dcol = tbase + kColS;
-            const int sl = j & 1;
-            const uint32_t k_lo = k_lo0 + sl * kSlot;
-            if (!mbar_wait(bars + F_KFULL + sl, (j >> 1) & 1, abortp, status, ERR_K)) break;
-            // the one score buffer is free once the warpgroup of tile j-1 holds that tile's scores in registers
-            if (j >= 1 && !mbar_wait(bars + F_SFREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, abortp, status, ERR_O)) break;
-            tc_fence_after();
-            umma_ss2<false>(dcol, q_lo, km_hi, k_lo, km_hi, idesc_s);
 #pragma unroll
-            for (int ks = 1; ks < KL; ++ks) {
-                const uint32_t off = (uint32_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4);
-                umma_ss2<true>(dcol, q_lo + off, km_hi, k_lo + off, km_hi, idesc_s);
+            for (int c = 0; c < KC; ++c) {          // the contraction over the head dimension, 128 columns per K chunk
+                const int g = j * KC + c, sl = g & 1;
+                const uint32_t k_lo = k_lo0 + sl * kSlot, q_c = q_lo + c * kSlot;
+                if (!mbar_wait(bars + F_KFULL + sl, (g >> 1) & 1, abortp, status, ERR_K)) { ok = false; break; }
+                // the one score buffer is free once the warpgroup of tile j-1 holds that tile's scores in registers
+                if (c == 0 && j >= 1 && !mbar_wait(bars + F_SFREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, abortp, status, ERR_O)) { ok = false; break; }
+                tc_fence_after();
+                if (c == 0) umma_ss2<false>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
+                else        umma_ss2<true>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
+#pragma unroll
+                for (int ks = 1; ks < KL; ++ks) {
+                    const uint32_t off = (uint32_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4);
+                    umma_ss2<true>(dcol, q_c + off, km_hi, k_lo + off, km_hi, idesc_s);
+                }
+                umma_commit(bars + F_KEMPTY + sl);
             }
-            umma_commit(bars + F_KEMPTY + sl);
+            if (!ok) break;
             umma_commit(bars + F_S + 2 * (j & 1) + ((j >> 1) & 1));
         }
       } else if (warp == 10 && lane == 0) {
@@ -465,12 +484,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             }
             if (tid == 0 && mbar_wait(bars + F_E, 0, abortp, status, ERR_O)) {
                 for (int b = 0; b < kBoxes; ++b)
-                    if (64 * b < prep.d)       // (a box wholly past the head dimension has nothing to store)
-                        tma_store_4d(&mapO, sQ + b * kBoxBytes, 64 * b, q0, hq, split * (heads_all / H) + bb);
+                    if (D * pass + 64 * b < prep.d)       // (a box wholly past the head dimension has nothing to store)
+                        tma_store_4d(&mapO, sQ + b * kBoxBytes, D * pass + 64 * b, q0, hq, split * (heads_all / H) + bb);
                 bulk_commit();
                 bulk_wait_read<0>();      // shared memory is read before the CTA may exit
             }
-            if (row < sp.n_q && h == 0) L[((size_t)split * heads_all + bh) * sp.n_q + row] = m_all * kLn2 + logf(l_all);
+            if (row < sp.n_q && h == 0 && pass == 0) L[((size_t)split * heads_all + bh) * sp.n_q + row] = m_all * kLn2 + logf(l_all);
         }
     }
     tc_fence_before();
@@ -478,11 +497,12 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     if (warp == 9) tmem_dealloc(tbase, kTmemCols);
 }
 
-template <int D, int KL>
+template <int D, int KC, int KL>
 cudaError_t launch_fwd(const Problem &p, const void *Q, const void *K, const void *V, void *O, float *L,
                        const FwdForBwd &fb, cudaStream_t st)
 {
-    constexpr int kSmem = 5 * 128 * D * 2 + 8 * (F_COUNT + 2) + 2 * 128 * 8 + 2 * 128 * 4;
+    constexpr int kSmem = (KC + 4) * 128 * D * 2 + 8 * (F_COUNT + 2) + 2 * 128 * 8 + 2 * 128 * 4;
+    if (KC > 1 && (fb.dO != nullptr || fb.zero_acc != nullptr)) return cudaErrorInvalidValue;   // no fused preparation with KC > 1
     CUtensorMap mq, mk, mv, mo;
     const auto bf = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     // p.d <= D columns exist in memory: loads fill the rest of a box with zeros, the store drops it
@@ -491,11 +511,11 @@ cudaError_t launch_fwd(const Problem &p, const void *Q, const void *K, const voi
         !make_tensor_map_4d_strided(&mv, V, bf, 2, p.B, p.kv_heads(), p.n, p.d, p.skv.row, p.skv.head, p.skv.batch, 128, 64) ||
         !make_tensor_map_4d_strided(&mo, O, bf, 2, p.B, p.H, p.n, p.d, p.so.row, p.so.head, p.so.batch, 128, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem<tc_fwd_kernel<D, KL>>(kSmem);
+    cudaError_t e = allow_smem<tc_fwd_kernel<D, KC, KL>>(kSmem);
     if (e != cudaSuccess) return e;
     const int nqt = (p.n + BM - 1) / BM;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_dependent(tc_fwd_kernel<D, KL>, dim3((unsigned)(nqt * p.BH())), dim3(kThreads), (size_t)kSmem, st,
+    return launch_dependent(tc_fwd_kernel<D, KC, KL>, dim3((unsigned)(nqt * p.BH() * KC)), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mo, L, p.n, p.causal, p.scale * kLog2e, nqt, heads_per_group(p, nqt), p.group(), p.H,
         FwdSplit{p.n, 1, (p.n + BN - 1) / BN}, fb.zero_acc,
         FwdPrep{(const __nv_bfloat16 *)fb.dO, fb.Lp, fb.Dp, nqt * BM, p.so, p.d}, device_status_ptr());
@@ -517,10 +537,10 @@ cudaError_t launch_fwd_decode(int B, int Hkv, int G, int n, float scale, const v
         !make_tensor_map_4d(&mv, V, bf, 2, B, Hkv, n, D, false, 128, 64) ||
         !make_tensor_map_4d(&mo, O_part, bf, 2, (uint64_t)splits * B, Hkv, G, D, false, 128, 64))
         return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem<tc_fwd_kernel<D, D / 16>>(kSmem);
+    cudaError_t e = allow_smem<tc_fwd_kernel<D, 1, D / 16>>(kSmem);
     if (e != cudaSuccess) return e;
     LaunchScope scope(MOA_KERNEL_FWD, st);
-    return launch_dependent(tc_fwd_kernel<D, D / 16>, dim3((unsigned)(B * Hkv * splits)), dim3(kThreads), (size_t)kSmem, st,
+    return launch_dependent(tc_fwd_kernel<D, 1, D / 16>, dim3((unsigned)(B * Hkv * splits)), dim3(kThreads), (size_t)kSmem, st,
         mq, mk, mv, mo, L_part, n, 0, scale * kLog2e, 1, 1, 1, Hkv, FwdSplit{G, splits, tiles_per_split},
         nullptr, FwdPrep{nullptr, nullptr, nullptr, 0, Strides{0, 0, 0}, D}, device_status_ptr());
 }
@@ -540,9 +560,17 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
 {
     if (p.d < 8 || p.d > 256 || p.d % 8) return cudaErrorInvalidValue;
     if (p.d <= 128 && fwd_pairs_pay(p)) return tc_fwd_pairs(p, Q, K, V, O, L, fb, st);
-    if (p.d > 128) return tc_fwd_wide(p, Q, K, V, O, L, fb, st);
-    if (p.d <= 64) return launch_fwd<64, 4>(p, Q, K, V, O, L, fb, st);
-    return p.d <= 96 ? launch_fwd<128, 6>(p, Q, K, V, O, L, fb, st) : launch_fwd<128, 8>(p, Q, K, V, O, L, fb, st);
+    if (p.d > 128) {
+        // Two CTAs per query tile take 0.7 to 0.85 of the time per key tile of one with all columns, which is worth it while all of them run at once
+        // (with the causal mask: while the longest outlasts the others' share), and from three key tiles on.  Two / one, B1 H4 n1500 d200 22.6 / 29.3
+        // us, causal H2 n3000 d256 31.6 / 40.9, H2 n282 d256 9.7 / 10.4; but 96 tiles of n1500 d256 0.67 the other way, and equal at n130.
+        const long long nqt = (p.n + BM - 1) / BM, jobs = nqt * p.BH(), sms = device_info().sms;
+        const bool few = p.causal ? 4 * (jobs * (nqt + 1) / 2) * 2 <= 3 * nqt * sms : 2 * jobs <= sms;
+        if (p.d > 192 && fb.dO == nullptr && fb.zero_acc == nullptr && nqt >= 3 && few) return launch_fwd<128, 2, 8>(p, Q, K, V, O, L, fb, st);
+        return tc_fwd_wide(p, Q, K, V, O, L, fb, st);
+    }
+    if (p.d <= 64) return launch_fwd<64, 1, 4>(p, Q, K, V, O, L, fb, st);
+    return p.d <= 96 ? launch_fwd<128, 1, 6>(p, Q, K, V, O, L, fb, st) : launch_fwd<128, 1, 8>(p, Q, K, V, O, L, fb, st);
 }
 
 }  // namespace moa

@@ -38,3 +38,12 @@ def test_row_maximum_grows_from_tile_to_tile(H, B, Hq, Hkv, n, d, causal, op, la
     ref = oracle.attn_fwd_bwd_gqa(f["Q"], f["K"], f["V"], f["dO"], causal, scale)
     H.assert_close(got, ref, H.TOL_BF16, keys=("O",) if op == "fwd" else ("O", "dQ", "dK", "dV"), tag=f"H{Hq}/{Hkv} n{n} d{d} {op}")
     assert mi.rel_err(got["L"], ref["L"]) <= 1e-3
+
+
+# two CTAs per query tile: the fewest key tiles, ragged ones, all that run at once and one head more; columns that fill half, most and all of the
+# second half
+@pytest.mark.parametrize("B,Hq,Hkv,n,d,causal", [(1, 2, 2, 265, 200, False), (1, 3, 1, 257, 256, True), (1, 4, 2, 700, 224, True), (2, 1, 1, 1000, 256, True), (1, 1, 1, 1409, 208, False),
+                                                 (1, 18, 18, 500, 256, False), (1, 19, 19, 500, 256, False), (1, 8, 1, 1500, 240, True)])
+@pytest.mark.parametrize("op,layout", [("fwd", 1), ("split", 0)])
+def test_few_query_tiles(H, B, Hq, Hkv, n, d, causal, op, layout):
+    test_row_maximum_grows_from_tile_to_tile(H, B, Hq, Hkv, n, d, causal, op, layout)
