@@ -868,7 +868,9 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
     const bool fits = pair_tiles >= 8 && (pair_tiles + pairs - 1) / pairs <= (tiles(256) + sms - 1) / sms;   // (a few tiles: launch-bound)
     const bool pair_ok = mode && fits && (kEpi == EPI_STORE || K >= 1024);
     // Where the 256-column tiles leave SMs idle, the narrower ones compete: cycles of a K block (UMMAs at 256 columns, its
-    // operands' way from L2 below that), of a chunk of the epilogue, and the rounds the grid takes.
+    // operands' way from L2 below that, which is longer for operands that come in by blocks of columns: a long K loop of 128-column tiles then takes up
+    // to a fifth more than of K-major ones, 1208 x 5048 x 1664 (1,1) 35.5 us, 30.4 in pairs), of a chunk of the epilogue, and the rounds the
+    // grid takes.
     constexpr double kChunk = kEpi == EPI_STORE ? 1100 : kEpi == EPI_SWIGLU_FWD ? 2500 : 3500;
     const double blocks = (double)K64 * ((A1 && !kDualN && nbatch == 1) ? 2 : 1);
     auto cost = [&](long long t, long long slots, double block, int n) {
@@ -879,7 +881,7 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
     bool pair = mode == 2 || pair_ok;
     if (mode != 2 && tiles(256) < 2 * sms) {
         double best = pair ? cost(pair_tiles, pairs, 530, 256) : cost(tiles(256), sms, 520, 256);
-        const double c128 = cost(tiles(128), sms, 360, 128);
+        const double c128 = cost(tiles(128), sms, K64 < 12 ? 360 : kAMn ? 430 : kBMn ? 390 : 360, 128);
         if (c128 < 0.95 * best) { best = c128; n = 128; pair = false; }
         const double c64 = kDualN ? 1e30 : cost(tiles(64), sms, 290, 64);
         if (c64 < 0.95 * best) { n = 64; pair = false; }
