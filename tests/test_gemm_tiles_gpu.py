@@ -65,8 +65,9 @@ def test_gated_mlp_widths(rt, n, d, dff):
 
 @pytest.mark.parametrize("B,n,H,d,dff", [(1, 40, 1, 64, 72), (2, 186, 4, 128, 1360), (1, 700, 8, 64, 1024), (1, 1613, 16, 64, 1000)])
 def test_block_products_side_by_side(rt, B, n, H, d, dff):
-    """The products a block's backward may launch together, against the block's three-projection form, which makes every call by itself:
-    same sums in the same order, so the same weight gradients up to the atomics in dQ."""
+    """The products a block's backward may launch together.  dWo against the block's three-projection form, where it is a launch of its own, bit
+    for bit; dx and what comes from dqkv up to the atomics in dQ.  (The MLP's four products are launched together, or not, in both forms alike:
+    test_mlp_products_side_by_side.)"""
     torch, mb = rt
     from paper_2609_33916_b200.block import TransformerBlock
     gen = torch.Generator(device="cuda").manual_seed(n)
@@ -87,3 +88,39 @@ def test_block_products_side_by_side(rt, B, n, H, d, dff):
         assert torch.equal(out[0][k], out[1][k]), k
     for k in ("dx", "Wq", "Wk", "Wv", "g1"):      # bf16 results of dQ sums in another order (and dh1 as one sum of three)
         assert (out[0][k] - out[1][k]).abs().max().item() <= 1.6e-2 * out[1][k].abs().max().item(), k
+
+
+# 64-column tiles of all four products within a wave, 128-column tiles within one, and neither; tails of rows, columns and of the K loop
+@pytest.mark.parametrize("n,d,dff,launches", [(40, 64, 72, 2), (700, 128, 264, 2), (520, 512, 1000, 2), (700, 1024, 1032, 4)])
+def test_mlp_products_side_by_side(rt, n, d, dff, launches):
+    """dW2, dW1, dW3 and dx of a gated MLP's backward against the same products one by one, from the da, du that the call left in its workspace:
+    one fp32 accumulation over K in the same order whichever tile or launch, so the same bits (dx: two sums instead of one of both)."""
+    torch, mb = rt
+    gen = torch.Generator(device="cuda").manual_seed(n + dff)
+    R = lambda *s: torch.randn(s, generator=gen, device="cuda").bfloat16()      # noqa: E731
+    x, W1, W3, W2, dy = R(n, d), R(dff, d) * d ** -0.5, R(dff, d) * d ** -0.5, R(d, dff) * dff ** -0.5, R(n, d)
+    a, u, h = R(n, dff), R(n, dff), R(n, dff)
+    E = lambda *s: torch.full(s, float("nan"), device="cuda", dtype=torch.bfloat16)      # noqa: E731
+    dx, dW1, dW3, dW2 = E(n, d), E(dff, d), E(dff, d), E(d, dff)
+    desc = mb.make_mlp_desc(n, d, dff)
+    ws = torch.empty(mb.moa_gated_mlp_workspace_bytes(desc), dtype=torch.uint8, device="cuda")
+    before = mb.moa_launch_count()
+    mb.moa_gated_mlp_bwd(desc, x, W1, W3, W2, a, u, h, dy, dx, dW1, dW3, dW2, ws)
+    assert mb.moa_launch_count() - before == launches
+    half = ws.numel() // 2
+    da, du = (ws[i * half:i * half + 2 * n * dff].view(torch.bfloat16).view(n, dff) for i in range(2))
+    f = lambda t: t.double()                                                     # noqa: E731
+    s = torch.sigmoid(f(a))
+    dh = f(dy) @ f(W2)
+    for got, ref in ((da, dh * f(u) * s * (1 + f(a) * (1 - s))), (du, dh * f(a) * s)):
+        assert (f(got) - ref).abs().max().item() <= 2 ** -7 * ref.abs().max().item()      # one rounding to bf16, a fast sigmoid below it
+
+    def product(M, N, K, A, B, a_layout, b_layout, add=None):
+        C = E(M, N)
+        mb.moa_gemm(mb.make_gemm_desc(M, N, K, a_layout, b_layout), A, B, C, R=add)
+        return C
+    for name, got, A, B, M, N in (("dW2", dW2, dy, h, d, dff), ("dW1", dW1, da, x, dff, d), ("dW3", dW3, du, x, dff, d)):
+        assert torch.equal(got, product(M, N, n, A, B, 1, 1)), name
+    ref = f(da) @ f(W1) + f(du) @ f(W3)
+    assert (f(dx) - ref).abs().max().item() <= 2 ** -8 * ref.abs().max().item()
+    assert mb.moa_last_device_status() == mb.MOA_OK
