@@ -33,8 +33,9 @@
  *  - Outputs are overwritten, never accumulated into.
  *  - A call is one to four kernels in stream order.  Most are launched as programmatic dependents of the kernel in
  *    front of them, the caller's included: they set themselves up while that kernel drains and wait for its completion before
- *    they touch memory (the backward kernels, which follow another kernel of their own call, may read the call's
- *    inputs before; everything the caller enqueued earlier has completed by then).  MOA_PDL=0 in the environment
+ *    they touch memory.  Kernels that follow another kernel of their own call may read the call's inputs before that (the
+ *    backward kernels; decode's streaming kernels behind the one that clears their counters): the kernel in front lets them start only
+ *    after its own wait, so everything the caller enqueued earlier has completed by then.  MOA_PDL=0 in the environment
  *    (read once per process) launches everything in plain stream order.
  *  - Errors are reported only through the returned moa_status; the library does
  *    not abort or throw.  Argument, workspace, scratch-limit and architecture errors

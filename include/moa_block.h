@@ -10,8 +10,11 @@
  * Conventions (the same as moa_attn.h): every tensor argument is a DEVICE pointer to a
  * contiguous row-major array, 16-byte aligned; the caller owns every buffer, workspace
  * included; calls enqueue kernels on `stream` (a cudaStream_t passed as void*) and return
- * without synchronising; outputs are overwritten; errors come back only as moa_status and
- * nothing has been enqueued when one is returned.  bf16 storage, fp32 arithmetic.
+ * without synchronising; outputs are overwritten; errors come back only as moa_status.  When an argument, workspace or
+ * architecture error is returned nothing has been enqueued -- except by moa_block_fwd and moa_block_bwd, which are sequences
+ * of calls and return the first error of any of them, with the calls in front of it enqueued.  Where an output lies over an
+ * input (dx over dy, say), a call gives what its steps, in the order of the formulas below, give one after the other.  bf16
+ * storage, fp32 arithmetic.
  */
 #ifndef MOA_BLOCK_H
 #define MOA_BLOCK_H
@@ -91,8 +94,10 @@ moa_status moa_gated_mlp_bwd(const moa_mlp_desc *desc, const void *x, const void
  * the running sum of a chain of products.  M, N, K >= 1; the row length of every array a multiple of
  * 8 (rows stay 16-byte aligned); dtype MOA_BF16; fp32 accumulation.
  * Tiling: 256 x 256 tiles on pairs of CTAs (one cluster of two, UMMAs of M = 256 reading half of B from each CTA's
- * shared memory), or 128 x 256 output tiles on single CTAs where M is so small that pairs would need more waves.  The environment variable MOA_GEMM_PAIR, read once per process, overrides the choice for
- * tests and measurements: 0 = never pairs, 2 = always pairs; the results do not depend on it beyond rounding order
+ * shared memory), 128 x 256 output tiles on single CTAs where M is so small that pairs would need more waves, or 128 x 128 and
+ * 128 x 64 where the wider ones would leave SMs idle; a small block's or gated MLP's backward sends out several products as one launch.
+ * The environment variable MOA_GEMM_PAIR, read once per process, overrides the choice for
+ * tests and measurements: 0 = never pairs, 2 = always pairs (no narrow tiles and no joint launches); the results do not depend on it beyond rounding order
  * (they are the same bits: every output element is one fp32 accumulation over K in the same order). */
 typedef struct {
     int32_t M, N, K;
@@ -108,7 +113,7 @@ moa_status moa_gemm(const moa_gemm_desc *desc, const void *A, const void *B, con
  *     o = attention(Q, K, V)    x2 = x + o Wo^T    h2 = RMSNorm(x2; g2)    y = x2 + gated_mlp(h2)
  * Every array is [T, H d] unless said otherwise; weights are stored [out,in].  The forward reads x and the weights and writes
  * the activations; the backward reads those, the weights and dy and writes the gradients.  Workspaces as for the single calls
- * (attention: MOA_OP_BWD).  The first error of a call of the sequence is returned. */
+ * (attention: MOA_OP_BWD).  The first error of a call of the sequence is returned; the calls in front of it have been enqueued. */
 typedef struct {
     int32_t B, n, H, d, d_ff;
     int32_t causal;

@@ -160,7 +160,9 @@ struct LaunchScope {
 // dependent launch), in clusters of `cluster` CTAs.  Every kernel launched like this keeps to two rules, which together
 // make the early start invisible:
 //   * it calls ptx::grid_dependency_wait() before it reads or writes global memory -- except that a kernel that is never the
-//     first of a call (the attention backward kernels) may read the call's own inputs before that;
+//     first of a call may read the call's own inputs before that: the attention backward kernels, and decode's streaming kernels where they
+//     merge through memory.  (The latter rest on decode_clear_kernel in front of them, which triggers only after its own wait: without it they
+//     would read the cache while the caller's update of it still runs.)
 //   * it calls ptx::grid_launch_dependents() only after that wait.  So once a kernel's successor runs at all, everything in
 //     front of the kernel itself, the caller's work included, has completed.
 // What overlaps is the set-up (barriers, TMEM allocation, tensor-map fetches) and the launch latency.

@@ -260,8 +260,8 @@ __device__ __noinline__ void merge_heads(const float *__restrict__ part_o, const
 
 // The CTA that finishes last among the `splits` CTAs of a group of query heads merges their partial results, so
 // the merge needs no launch of its own and runs while other heads are still streaming.  No CTA waits for another:
-// each one publishes its partials (fence), then adds one to the group's counter (zeroed by the host before the
-// launch); whoever reads splits - 1 is the last.
+// each one publishes its partials (fence), then adds one to the group's counter (zeroed by the kernel in front); whoever reads splits - 1
+// is the last.
 template <typename T, int D>
 __device__ __forceinline__ void merge_if_last(unsigned int *counters, const DecodeJob &job, int splits, size_t BH,
                                               const float *part_o, const float *part_ml, T *out, float *lse, float *sh)
