@@ -213,8 +213,9 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
     constexpr bool kToken = !kCols && kV <= 2;
     const uint32_t token = ptx::grid_dependency_wait_token();
     ptx::grid_launch_dependents();
+    if (!kToken) x = ptx::after_wait(x);
     g = ptx::after_wait(g);
-    if (!kToken) { x = ptx::after_wait(x); r_in = ptx::after_wait(r_in); dy = ptx::after_wait(dy); dx_add = ptx::after_wait(dx_add); }
+    if (!kToken) { r_in = ptx::after_wait(r_in); dy = ptx::after_wait(dy); dx_add = ptx::after_wait(dx_add); }
     if (kCols && (int)blockIdx.x < col_blocks) {
         dg_columns(x, dy, r_in, dg, n, d, (int)blockIdx.x * kDgCols, acc);
         return;
@@ -302,7 +303,7 @@ rmsnorm_bwd_kernel(const __nv_bfloat16 *__restrict__ x, const __nv_bfloat16 *__r
 #pragma unroll
         for (int i = 0; kToken && i < R; ++i) rc[i] = rn[i];
     }
-    if (kCols) return;
+    if (kCols && col_blocks > 0) return;
     // CTA partial of dg: the row lanes' sums added in lane order
     float *mine = part + (size_t)block * d;
 #pragma unroll
