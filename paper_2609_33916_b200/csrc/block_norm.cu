@@ -551,7 +551,14 @@ NormPlan norm_plan(int n, int d, bool bwd)
 // flight decide; below it, a warp's rows of a stage one behind the other are most of the time.  Register and ring variant, in a chain of
 // calls: forward 8192 x 512 4.4 and 4.6 us, 4096 x 2048 7.1 and 7.6, 8192 x 2048 11.8 and 11.4; backward 512 x 256 4.5 and 8.1, 512 x 2048
 // 8.5 and 14.4, 1024 x 1024 7.7 and 9.9, 2048 x 1024 13.6 and 10.9.
-bool norm_uses_ring(int n, int d, bool bwd) { return d >= 256 && d <= 2048 && (long long)n * d > (bwd ? 1LL << 20 : 8LL << 20); }
+// In the forward rows just above 1024 elements are two warps' in the register kernel, with a barrier of the block and half of a thread's four vectors empty:
+// there the ring pays from 2M elements on (register / ring: 4845 x 1032 7.8 and 6.8, 5719 x 1224 8.0 and 7.4, 1938 x 1032 4.3 and 4.2; but 1497 x 1336 4.1
+// and 4.6).
+bool norm_uses_ring(int n, int d, bool bwd)
+{
+    const long long line = bwd ? 1LL << 20 : d > 1024 && d <= 1280 ? 2LL << 20 : 8LL << 20;
+    return d >= 256 && d <= 2048 && (long long)n * d > line;
+}
 struct RingPlan {
     int kV, m, grid;
     size_t smem;

@@ -63,3 +63,9 @@ def test_rmsnorm_backward_forms(n, d, with_add, with_r):
     for got, r_ in ((dx, want), (dg, ref["dg"])):
         got = got.float().cpu().numpy().astype(np.float64)
         assert np.all(np.isfinite(got)) and mi.rel_err(got, r_) <= TOL
+
+
+@pytest.mark.parametrize("n,d", [(2032, 1032), (2033, 1032), (1638, 1280), (1639, 1280), (2100, 1288)])
+def test_rmsnorm_rows_above_1024(n, d):
+    """Both sides of the forward's other line, for rows of 1032..1280 elements, and the first rows past them."""
+    test_rmsnorm_routes(n, d)
