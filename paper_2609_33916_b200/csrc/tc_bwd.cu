@@ -341,7 +341,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             }
             __syncwarp();
         }
-      } else if (warp == kMmaWarp && lane == 0) {
+      } else if (warp == kMmaWarp && elect_one()) {
         // the whole role runs in one thread: no warp re-convergence between waits and issues
         // ------------------------------------------------------------------- UMMA issuer
         // Issue order per query tile i:  dP(i), dV(i), S(i+1), dQ(i), dK(i)  (D = 64: dK(i), dQ(i)).
@@ -377,7 +377,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         ok = ok && mbar_wait(bars + B_QFULL + 0, 0, abortp, status, ERR_FULL);
         if (ok) {
             tc_fence_after();
-            if (lane == 0) issue_S(q_km0);
+            issue_S(q_km0);
         }
         for (int it = 0; ok && it < niter; ++it) {
             const int s = it & 1;
@@ -386,7 +386,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (!mbar_wait(bars + B_DOFULL + sdo, (it / kDoSlots) & 1, abortp, status, ERR_FULL)) break;
             if (kAliasDQ && !skip_dq && it > 0 && !mbar_wait(bars + B_DQR, (it - 1) & 1, abortp, status, ERR_DQR)) break;
             tc_fence_after();
-            if (lane == 0) {
+            {
                 umma_ss2<false>(tbase + colDP, v_km, km_hi, do_km, km_hi, idesc_st);
 #pragma unroll
                 for (int ks = 1; ks < KL; ++ks)
@@ -399,7 +399,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             // arrives -- 150-185 cycles per such point in a replay of this loop's issue pattern)
             if (it + 1 < niter && !mbar_wait(bars + B_QFULL + ((it + 1) & 1), ((it + 1) >> 1) & 1, abortp, status, ERR_FULL)) break;
             tc_fence_after();
-            if (lane == 0) {
+            {
                 // 16 queries per step; the very first UMMA of the CTA overwrites the accumulator
                 if (it > 0) umma_ts2<true>(tbase + colDV, tbase + colS, do_mn, mn_hi, idesc_acc);
                 else        umma_ts2<false>(tbase + colDV, tbase + colS, do_mn, mn_hi, idesc_acc);
@@ -414,7 +414,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (!mbar_wait(bars + B_DS, it & 1, abortp, status, ERR_PDS)) break;
             if (!kAliasDQ && !skip_dq && it > 0 && !mbar_wait(bars + B_DQR, (it - 1) & 1, abortp, status, ERR_DQR)) break;
             tc_fence_after();
-            if (lane == 0 && kDKfromSmem) {
+            if (kDKfromSmem) {
                 // dQ^T first (16 keys per step), then dK += dS^T Q_i with dS^T from shared memory (16 queries per step)
                 if (!skip_dq) {
                     umma_ss2<false>(tbase + colDQ, k_mn, mn_hi, ds_mn, mn_hi, idesc_dqt);
@@ -430,7 +430,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                     umma_ss2<true>(tbase + colDK, ds_km + koff(ks), km_hi, q_mn + moff(ks), mn_hi, idesc_acc);
                 umma_commit(bars + B_QEMPTY + s);   // Q slot (and, on the last tile, everything issued) is done
             }
-            if (lane == 0 && !kDKfromSmem) {
+            if (!kDKfromSmem) {
                 if (it > 0) umma_ts2<true>(tbase + colDK, tbase + colDP, q_mn, mn_hi, idesc_acc);
                 else        umma_ts2<false>(tbase + colDK, tbase + colDP, q_mn, mn_hi, idesc_acc);
 #pragma unroll

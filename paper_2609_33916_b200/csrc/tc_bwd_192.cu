@@ -184,7 +184,7 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
             if (lane == 0) load_q(it + 2);
             __syncwarp();
         }
-      } else if (warp == kMmaWarp && lane == 0) {
+      } else if (warp == kMmaWarp && elect_one()) {
         // ------------------------------------------------------------------- UMMA issuer (one thread)
         constexpr uint32_t idesc_st = idesc_bf16_f32(128, 64, 0, 0);          // S^T, dP^T: 128 keys x 64 queries
         constexpr uint32_t idesc_acc = idesc_bf16_f32(128, 64 * NB, 0, 1);    // dV, dK: B MN-major, all columns of d

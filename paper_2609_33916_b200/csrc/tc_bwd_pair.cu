@@ -282,7 +282,7 @@ tc_bwd_pair_kernel(const __grid_constant__ CUtensorMap mapQr, const __grid_const
             }
             __syncwarp();
         }
-      } else if (warp == kMmaWarp && lane == 0 && rank == 0) {
+      } else if (warp == kMmaWarp && rank == 0 && elect_one()) {
         // ------------------------------------------------------------------- UMMA issuer (rank 0 only)
         // Issue order per query tile i:  dP(i), dV(i), S(i+1), dK(i), dQ(i).
         constexpr uint32_t idesc_st = idesc_bf16_f32(256, 128, 0, 0);    // S^T, dP^T

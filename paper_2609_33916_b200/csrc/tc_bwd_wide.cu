@@ -190,7 +190,7 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             }
             __syncwarp();
         }
-      } else if (warp == kMmaWarp && lane == 0) {
+      } else if (warp == kMmaWarp && elect_one()) {
         // ------------------------------------------------------------------- UMMA issuer (one thread)
         constexpr uint32_t idesc_st = idesc_bf16_f32(128, 64, 0, 0);     // S^T, dP^T: 128 keys x 64 queries
         constexpr uint32_t idesc_acc = idesc_bf16_f32(128, 128, 0, 1);   // dV, dK: A in TMEM, B MN-major, 128 columns of d

@@ -102,7 +102,7 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ C
             __syncwarp();
         }
         if (lane == 0) mbar_drain(bars, armed);     // copies of this CTA still on their way land before it leaves (bounded)
-    } else if (warp == 9 && lane == 0) {
+    } else if (warp == 9 && elect_one()) {
         // ------------------------------------------------------- UMMA issuer (one thread)
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
         constexpr uint32_t idesc_dq = idesc_bf16_f32(128, D, 0, 1);

@@ -231,7 +231,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         }
         if (lane == 0 && *abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
-      } else if (warp == 9 && lane == 0) {
+      } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer for the score GEMMs (one thread)
         // Two issuing threads (this one for S = Q K^T, warp 10 for O += P V): a successful barrier
         // probe or a commit costs an issuing thread ~100 cycles during which it feeds nothing, and
@@ -268,7 +268,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (!ok) break;
             umma_commit(bars + F_S + 2 * (j & 1) + ((j >> 1) & 1));
         }
-      } else if (warp == 10 && lane == 0) {
+      } else if (warp == 10 && elect_one()) {
         // ------------------------------------------------ UMMA issuer for O += P V (one thread)
         const uint32_t idesc_pv = KL < D / 16 ? idesc_bf16_f32(128, 16 * KL, 0, 1) : idesc_bf16_f32(128, D, 0, 1);
         const uint64_t mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);

@@ -186,7 +186,7 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         }
         if (lane == 0 && *abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
-      } else if (warp == 9 && lane == 0) {
+      } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer for the score products (one thread)
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024);
@@ -216,7 +216,7 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 before = h;
             }
         }
-      } else if (warp == 10 && lane == 0) {
+      } else if (warp == 10 && elect_one()) {
         // ------------------------------------------------ UMMA issuer for O += P V (one thread)
         constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 16 * KL, 0, 1);
         const uint64_t mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);

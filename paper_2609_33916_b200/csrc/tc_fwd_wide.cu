@@ -188,7 +188,7 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         }
         if (lane == 0 && *abortp)
             for (int s = 0; s < S::kVSlots; ++s) mbar_drain_one(bars + FW_VFULL + s, nv > s ? (nv - s + S::kVSlots - 1) / S::kVSlots : 0);
-      } else if (warp == 9 && lane == 0) {
+      } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer for the score products (one thread)
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024);
@@ -216,7 +216,7 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             if (!ok) break;
             umma_commit(bars + FW_S + 2 * (j & 1) + ((j >> 1) & 1));
         }
-      } else if (warp == 10 && lane == 0) {
+      } else if (warp == 10 && elect_one()) {
         // ------------------------------------------------ UMMA issuer for O += P V (one thread)
         constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 64 * NB, 0, 1);
         const uint64_t mn_proto = smem_desc_sw128(0, S::kVBox, 1024);

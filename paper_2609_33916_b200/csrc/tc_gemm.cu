@@ -262,7 +262,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 if (++kstage == nk) { kstage = 0; ++part; }
             }
         }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
+    } else if (warp == 1 && rank == 0 && elect_one()) {
         // ------------------------------------------------------------------- UMMA issuer
         constexpr uint32_t idesc = idesc_bf16_f32(kTileM, kN, kAMn ? 1 : 0, kBMn ? 1 : 0);
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kMnBox, 1024);
@@ -642,7 +642,7 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
                 if (++kstage == nk) { kstage = 0; ++part; }
             }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1 && elect_one()) {
         // ------------------------------------------------------------------- UMMA issuer
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kMnBox, 1024);
         int it = 0, ti = 0, jx = 0;

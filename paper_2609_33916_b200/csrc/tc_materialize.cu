@@ -113,7 +113,7 @@ mat_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             __syncwarp();
         }
         if (lane == 0) mbar_drain(bars, armed);     // copies still on their way land before the CTA leaves (bounded)
-    } else if (warp == 5 && lane == 0) {
+    } else if (warp == 5 && elect_one()) {
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
         constexpr uint32_t idesc_pv = idesc_bf16_f32(128, D, 0, 1);
         const DescParts dp = desc_parts();
@@ -307,7 +307,7 @@ mat_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             __syncwarp();
         }
         if (lane == 0) mbar_drain(bars, armed);     // copies still on their way land before the CTA leaves (bounded)
-    } else if (warp == 9 && lane == 0) {
+    } else if (warp == 9 && elect_one()) {
         constexpr uint32_t idesc_st = idesc_bf16_f32(128, 128, 0, 0);
         constexpr uint32_t idesc_acc = idesc_bf16_f32(128, D, 0, 1);
         const DescParts dp = desc_parts();
@@ -484,7 +484,7 @@ mat_dq_kernel(const __grid_constant__ CUtensorMap mapGST, const __grid_constant_
             __syncwarp();
         }
         if (lane == 0) mbar_drain(bars, armed);     // copies still on their way land before the CTA leaves (bounded)
-    } else if (warp == 5 && lane == 0) {
+    } else if (warp == 5 && elect_one()) {
         constexpr uint32_t idesc = idesc_bf16_f32(128, D, 1, 1);   // A = dS^T tile (MN-major), B = K (MN-major)
         const DescParts dp = desc_parts();
         const uint32_t g_mn0 = dp.mn_lo + addr_field(sG), k_mn0 = dp.mn_lo + addr_field(sK);
