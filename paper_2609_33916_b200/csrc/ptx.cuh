@@ -622,5 +622,29 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
+// Backward: r[e] = r[e] * sl2 + Ls[e] (a row of S^T in place; Ls = -L log2 e in shared memory, 16-byte aligned), the argument of exp2, and where
+// `masked` -inf for the queries e < first, which do not see this key.  The mask stands in a branch of its own: written beside each
+// exponential it was two instructions per score in every tile, masked or not.  (Behind the addition of L, so that a masked P is 0 whatever L is.)
+template <int N>
+__device__ __forceinline__ void score_exponents(uint32_t (&r)[N], const float *Ls, uint64_t sl2, bool masked, int first)
+{
+#pragma unroll
+    for (int e = 0; e < N; e += 4) {
+        const ulonglong2 l4 = *reinterpret_cast<const ulonglong2 *>(Ls + e);   // two pairs
+        float a0, a1, a2, a3;
+        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sl2, l4.x), a0, a1);
+        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sl2, l4.y), a2, a3);
+        r[e] = __float_as_uint(a0);
+        r[e + 1] = __float_as_uint(a1);
+        r[e + 2] = __float_as_uint(a2);
+        r[e + 3] = __float_as_uint(a3);
+    }
+    if (masked) {
+#pragma unroll
+        for (int e = 0; e < N; ++e)
+            if (e < first) r[e] = 0xff800000u;   // -inf
+    }
+}
+
 }  // namespace ptx
 }  // namespace moa

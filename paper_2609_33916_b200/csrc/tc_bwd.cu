@@ -249,7 +249,7 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     // The producer initialises the barriers of its own loads and sends the first ones off at once; the rest of the set-up (the other barriers,
     // the TMEM allocation) runs under them.  K, V, Q and dO are the caller's tensors; L', D and the cleared dQ accumulator were
     // written by the kernel in front of this one in the stream (the forward or the preprocess kernel), which may still be running.
-    if (warp == kLoadWarp && lane == 0) {
+    if (warp == kLoadWarp && elect_one()) {
         mbar_init(bars + B_KV, 1u);
         for (int s = 0; s < 2; ++s) { mbar_init(bars + B_QFULL + s, 1u); mbar_init(bars + B_DOFULL + s, 1u); }
         fence_mbar_init();
@@ -295,8 +295,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     if (warp >= kLoadWarp) {
       // one instruction for the whole last warpgroup (TMA warp, UMMA warp, two idle warps)
       asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-      if (warp == kLoadWarp) {
-        // ------------------------------------------------------------------ TMA producer
+      if (warp == kLoadWarp && elect_one()) {
+        // ------------------------------------------------------------------ TMA producer (one thread)
         // Q tiles (with L, D) go through a two-slot ring and are fetched two tiles ahead: S(i+1) is
         // issued in the middle of tile i.  dO has one slot: it is read only by dP(i) and dV(i),
         // early in tile i, and is refilled as soon as dV(i) has completed.
@@ -320,12 +320,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             mbar_arrive_expect_tx(bars + B_DOFULL + s, SM::kTile);
             for (int b = 0; b < kBoxes; ++b) tma_load_4d(sdO + b * kBoxBytes, &mapdO, bars + B_DOFULL + s, 64 * b, q0, qh + hq0, bb);
         };
-        if (lane == 0 && niter > 0) {
+        if (niter > 0) {
             wdo.next();
             if (kDoSlots == 2 && niter > 1) load_do(1);
         }
         grid_dependency_wait();
-        if (lane == 0 && niter > 0) {
+        if (niter > 0) {
             load_q(0);
             if (niter > 1) load_q(1);
         }
@@ -333,13 +333,12 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         for (int it = 0; it < niter; ++it) {
             if (it + kDoSlots < niter) {     // dV(it) done: its dO slot takes tile it + kDoSlots
                 if (!mbar_wait(bars + B_DOEMPTY + it % kDoSlots, (it / kDoSlots) & 1, abortp, status, ERR_EMPTY)) break;
-                if (lane == 0) load_do(it + kDoSlots);
+                load_do(it + kDoSlots);
             }
             if (it + 2 < niter) {     // dK(it) done: its Q slot takes tile it+2
                 if (!mbar_wait(bars + B_QEMPTY + (it & 1), (it >> 1) & 1, abortp, status, ERR_EMPTY)) break;
-                if (lane == 0) load_q(it + 2);
+                load_q(it + 2);
             }
-            __syncwarp();
         }
       } else if (warp == kMmaWarp && elect_one()) {
         // the whole role runs in one thread: no warp re-convergence between waits and issues
@@ -591,26 +590,13 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 uint32_t rs[32];
                 tmem_ld(lane_addr + colS + qc0, rs);
                 tc_wait_ld();
+                score_exponents<32>(rs, Ls + qc0, sl2, diag, lane_row - qc0);
                 uint32_t pk[16];
 #pragma unroll
-                for (int e = 0; e < 32; e += 4) {
-                    const ulonglong2 l4 = *reinterpret_cast<const ulonglong2 *>(Ls + qc0 + e);   // two pairs
-                    const uint64_t t0 = fma_f32x2(pack_f32x2(__uint_as_float(rs[e]), __uint_as_float(rs[e + 1])), sl2, l4.x);
-                    const uint64_t t1 = fma_f32x2(pack_f32x2(__uint_as_float(rs[e + 2]), __uint_as_float(rs[e + 3])), sl2, l4.y);
-                    float a0, a1, a2, a3;
-                    unpack_f32x2(t0, a0, a1);
-                    unpack_f32x2(t1, a2, a3);
-                    a0 = ex2(a0); a1 = ex2(a1); a2 = ex2(a2); a3 = ex2(a3);
-                    if (diag) {   // query index < key index: masked
-                        if (qc0 + e < lane_row) a0 = 0.f;
-                        if (qc0 + e + 1 < lane_row) a1 = 0.f;
-                        if (qc0 + e + 2 < lane_row) a2 = 0.f;
-                        if (qc0 + e + 3 < lane_row) a3 = 0.f;
-                    }
+                for (int e = 0; e < 32; e += 2) {
+                    const float a0 = ex2(__uint_as_float(rs[e])), a1 = ex2(__uint_as_float(rs[e + 1]));
                     p2[16 * c + e / 2] = pack_f32x2(a0, a1);
-                    p2[16 * c + e / 2 + 1] = pack_f32x2(a2, a3);
                     pk[e / 2] = pack_bf16(a0, a1);
-                    pk[e / 2 + 1] = pack_bf16(a2, a3);
                 }
                 tmem_st(lane_addr + colS + 64 * wg + 16 * c, pk);
             }

@@ -126,9 +126,9 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
 
     if (warp >= kLoadWarp) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-      if (warp == kLoadWarp) {
-        // ------------------------------------------------------------------ TMA producer
-        if (lane == 0 && niter > 0) {
+      if (warp == kLoadWarp && elect_one()) {
+        // ------------------------------------------------------------------ TMA producer (one thread)
+        if (niter > 0) {
             mbar_arrive_expect_tx(bars + W_KV, 8 * SM::kBoxK);
             for (int b = 0; b < 4; ++b) {
                 tma_load_4d(sK + b * SM::kBoxK, &mapK, bars + W_KV, 64 * b, k0, hk, bb);
@@ -164,13 +164,13 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             for (int b = 0; b < 4; ++b) tma_load_4d(sdO + b * SM::kBoxQ, &mapdO, bars + W_DOFULL, 64 * b, q0, qh + hq0, bb);
         };
         // (K, V, Q and dO are the call's inputs; -L, -D and the cleared accumulator come from the kernel in front)
-        if (lane == 0 && niter > 0) {
+        if (niter > 0) {
             load_qoth(0);
             load_do(0);
         }
         grid_dependency_wait();
         grid_launch_dependents();
-        if (lane == 0 && niter > 0) {
+        if (niter > 0) {
             load_qown(0);
             if (niter > 1) load_qown(1);
         }
@@ -180,15 +180,14 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         for (int it = 0; it < niter; ++it) {
             if (it + 1 < niter) {
                 if (!mbar_wait(bars + W_S, it & 1, abortp, status, WERR_EMPTY)) break;
-                if (lane == 0) load_qoth(it + 1);
+                load_qoth(it + 1);
                 if (!mbar_wait(bars + W_DOEMPTY, it & 1, abortp, status, WERR_EMPTY)) break;
-                if (lane == 0) load_do(it + 1);
+                load_do(it + 1);
             }
             if (it + 2 < niter) {
                 if (!mbar_wait(bars + W_QEMPTY + (it & 1), (it >> 1) & 1, abortp, status, WERR_EMPTY)) break;
-                if (lane == 0) load_qown(it + 2);
+                load_qown(it + 2);
             }
-            __syncwarp();
         }
       } else if (warp == kMmaWarp && elect_one()) {
         // ------------------------------------------------------------------- UMMA issuer (one thread)
@@ -328,27 +327,13 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             uint32_t rs[32];
             tmem_ld(lane_addr + colS + qc0, rs);
             tc_wait_ld();
+            score_exponents<32>(rs, Ls + qc0, sl2, masked, lane_row - qc0 - rel);
             uint32_t pk[16];
 #pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-                const ulonglong2 l4 = *reinterpret_cast<const ulonglong2 *>(Ls + qc0 + e);   // two pairs
-                const uint64_t t0 = fma_f32x2(pack_f32x2(__uint_as_float(rs[e]), __uint_as_float(rs[e + 1])), sl2, l4.x);
-                const uint64_t t1 = fma_f32x2(pack_f32x2(__uint_as_float(rs[e + 2]), __uint_as_float(rs[e + 3])), sl2, l4.y);
-                float a0, a1, a2, a3;
-                unpack_f32x2(t0, a0, a1);
-                unpack_f32x2(t1, a2, a3);
-                a0 = ex2(a0); a1 = ex2(a1); a2 = ex2(a2); a3 = ex2(a3);
-                if (masked) {
-                    const int q = qc0 + e + rel;
-                    if (q < lane_row) a0 = 0.f;
-                    if (q + 1 < lane_row) a1 = 0.f;
-                    if (q + 2 < lane_row) a2 = 0.f;
-                    if (q + 3 < lane_row) a3 = 0.f;
-                }
+            for (int e = 0; e < 32; e += 2) {
+                const float a0 = ex2(__uint_as_float(rs[e])), a1 = ex2(__uint_as_float(rs[e + 1]));
                 p2[e / 2] = pack_f32x2(a0, a1);
-                p2[e / 2 + 1] = pack_f32x2(a2, a3);
                 pk[e / 2] = pack_bf16(a0, a1);
-                pk[e / 2 + 1] = pack_bf16(a2, a3);
             }
             tmem_st(lane_addr + colS + qc0, pk);          // over the first 16 of the 32 columns just read
             tc_wait_st();

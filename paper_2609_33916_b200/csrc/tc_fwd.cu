@@ -124,7 +124,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     // barriers, the TMEM allocation, the CTA-wide barrier) still runs, instead of starting behind it.
     const bool aligned = (smem_u32(sm) & 1023u) == 0;      // (swizzled tiles need the 1024-byte alignment)
     const int early_k = aligned ? min(nkt_want * KC, 2) : 0, early_v = aligned ? min(nkt_want, 2) : 0;
-    if (warp == 8 && lane == 0) {
+    if (warp == 8 && elect_one()) {
         mbar_init(bars + F_Q, 1u);
         mbar_init(bars + F_KFULL, 1u);
         mbar_init(bars + F_KFULL + 1, 1u);
@@ -141,7 +141,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             }
         }
     }
-    if (warp == 11 && lane == 0) {
+    if (warp == 11 && elect_one()) {
         mbar_init(bars + F_VFULL, 1u);
         mbar_init(bars + F_VFULL + 1, 1u);
         fence_mbar_init();
@@ -198,38 +198,37 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             float4 *dst = reinterpret_cast<float4 *>(zero_acc + ((size_t)bh * n + q0) * D);
             for (int i = lane; i < rows * (D / 4); i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        if (elect_one()) {      // (one thread from here on)
         bool live = true;
         for (int j = early_k / KC; live && j < nkt; ++j) {
             for (int c = (j == early_k / KC ? early_k % KC : 0); c < KC; ++c) {
                 const int g = j * KC + c;
                 if (g >= 2 && !mbar_wait(bars + F_KEMPTY + (g & 1), ((g >> 1) - 1) & 1, abortp, status, ERR_K)) { live = false; break; }
-                if (lane == 0) load_k(g);
+                load_k(g);
             }
-            if (!live) break;
-            __syncwarp();
         }
-        if (lane == 0 && *abortp) {
+        if (*abortp) {
             // a wait expired somewhere in the CTA: copies still on their way land before it leaves (bounded)
             mbar_drain_one(bars + F_Q, nkt > 0 ? 1 : 0);
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
         }
-      } else if (warp == 11) {
+        }
+      } else if (warp == 11 && elect_one()) {
         // ------------------------------------------------------------------ TMA producer of the V stream
         // (a thread of its own: the V ring follows the P V products, the K ring the score products, and neither waits
         // for the other's slots)
         int nv = early_v;       // (the first two tiles went out before the set-up)
         for (int j = early_v; j < nkt; ++j) {
             if (j >= 2 && !mbar_wait(bars + F_VEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR_V)) break;
-            if (lane == 0) {
+            {
                 const int s = j & 1;
                 mbar_arrive_expect_tx(bars + F_VFULL + s, kTileBytes);
                 ++nv;
                 for (int b = 0; b < kBoxes; ++b)
                     tma_load_4d(sV + s * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + s, D * pass + 64 * b, (kt0 + j) * BN, hk, bb);
             }
-            __syncwarp();
         }
-        if (lane == 0 && *abortp)
+        if (*abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
       } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer for the score GEMMs (one thread)

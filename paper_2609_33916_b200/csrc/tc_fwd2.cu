@@ -87,7 +87,7 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         for (int b = 0; b < kBoxes; ++b) tma_load_4d(sV + s * kTileBytes + b * kBoxBytes, &mapV, bars + F2_VFULL + s, 64 * b, j * BN, hk, bb);
     };
     // the first loads go out before the rest of the set-up
-    if (warp == 8 && lane == 0) {
+    if (warp == 8 && elect_one()) {
         mbar_init(bars + F2_Q, 1u);
         mbar_init(bars + F2_KFULL, 1u);
         mbar_init(bars + F2_KFULL + 1, 1u);
@@ -107,7 +107,7 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 }
         }
     }
-    if (warp == 11 && lane == 0) {
+    if (warp == 11 && elect_one()) {
         mbar_init(bars + F2_VFULL, 1u);
         mbar_init(bars + F2_VFULL + 1, 1u);
         fence_mbar_init();
@@ -148,11 +148,12 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 for (int i = lane; i < rows * (D / 4); i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
+        if (elect_one()) {      // (one thread from here on)
         int nk = early;
         for (int j = early; j < n0; ++j) {
             if (!mbar_wait(bars + F2_KEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR2_K)) break;
-            if (lane == 0) { load_k(j); ++nk; }
-            __syncwarp();
+            load_k(j);
+            ++nk;
         }
         // Fused call: the streams' dO tiles, which the epilogues multiply their rows with, go into the K slots as these come free: stream 1's
         // into that of the last tile but one (stream 1 ends first), stream 0's into the last tile's.  (Read by the row's owner straight from
@@ -164,27 +165,27 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 const int s = (n0 - 1 + h) & 1, uses = (n0 - s + 1) / 2;
                 if ((h ? n1 : n0) == 0) continue;
                 if (uses > 0 && !mbar_wait(bars + F2_KEMPTY + s, (uses - 1) & 1, abortp, status, ERR2_K)) break;
-                if (lane == 0) {
+                {
                     mbar_arrive_expect_tx(bars + F2_DO + h, kTileBytes);
                     armed_do |= 1 << h;
                     for (int b = 0; b < kBoxes; ++b) tma_load_4d(sK + s * kTileBytes + b * kBoxBytes, &mapdO, bars + F2_DO + h, 64 * b, h ? q01 : q00, hq, bb);
                 }
-                __syncwarp();
             }
-        if (lane == 0 && *abortp) {
+        if (*abortp) {
             for (int h = 0; h < 2; ++h) mbar_drain_one(bars + F2_DO + h, (armed_do >> h) & 1);
             mbar_drain_one(bars + F2_Q, early > 0 ? 1 : 0);
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
         }
-      } else if (warp == 11) {
+        }
+      } else if (warp == 11 && elect_one()) {
         // ------------------------------------------------------------------ TMA producer of V
         int nv = early;
         for (int j = early; j < n0; ++j) {
             if (!mbar_wait(bars + F2_VEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR2_V)) break;
-            if (lane == 0) { load_v(j); ++nv; }
-            __syncwarp();
+            load_v(j);
+            ++nv;
         }
-        if (lane == 0 && *abortp)
+        if (*abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
       } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer for the score products (one thread)

@@ -104,7 +104,7 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
     const int nk_all = aligned ? nkt_want * S::kChunks : 0, nv_all = aligned ? nkt_want * 2 : 0;
     const int early_k = min(nk_all, S::kKSlots), early_v = min(nv_all, S::kVSlots);
     // the first loads go out before the rest of the set-up
-    if (warp == 8 && lane == 0) {
+    if (warp == 8 && elect_one()) {
         mbar_init(bars + FW_Q, 1u);
         for (int s = 0; s < 3; ++s) mbar_init(bars + FW_KFULL + s, 1u);
         fence_mbar_init();
@@ -117,7 +117,7 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 for (int b = 0; b < NB; ++b) tma_prefetch_4d(&mapdO, 64 * b, q0, hq, bb);
         }
     }
-    if (warp == 11 && lane == 0) {
+    if (warp == 11 && elect_one()) {
         for (int s = 0; s < 3; ++s) mbar_init(bars + FW_VFULL + s, 1u);
         fence_mbar_init();
         grid_dependency_wait();
@@ -153,10 +153,11 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             float4 *dst = reinterpret_cast<float4 *>(prep.zero_acc + ((size_t)bh * n + q0) * 256);
             for (int i = lane; i < min(BM, n - q0) * 64; i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        if (elect_one()) {      // (one thread from here on)
         for (int g = early_k; g < nkt * S::kChunks; ++g) {
             if (!mbar_wait(bars + FW_KEMPTY + g % S::kKSlots, (g / S::kKSlots - 1) & 1, abortp, status, ERRW_K)) break;
-            if (lane == 0) { load_k(g); ++nk; }
-            __syncwarp();
+            load_k(g);
+            ++nk;
         }
         // fused call: the dO tile, which the epilogue multiplies its rows with, goes over K slots that have come free (see tc_fwd2.cu)
         int armed_do = 0;
@@ -166,27 +167,27 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
                 const int uses = (nkt * S::kChunks - s + S::kKSlots - 1) / S::kKSlots;
                 free = uses <= 0 || mbar_wait(bars + FW_KEMPTY + s, (uses - 1) & 1, abortp, status, ERRW_K);
             }
-            if (free && lane == 0) {
+            if (free) {
                 mbar_arrive_expect_tx(bars + FW_DO, NB * S::kBox);
                 armed_do = 1;
                 for (int b = 0; b < NB; ++b) tma_load_4d(sK + dslot * S::kKSlot + b * S::kBox, &mapdO, bars + FW_DO, 64 * b, q0, hq, bb);
             }
-            __syncwarp();
         }
-        if (lane == 0 && *abortp) {
+        if (*abortp) {
             mbar_drain_one(bars + FW_DO, armed_do);
             mbar_drain_one(bars + FW_Q, early_k > 0 ? 1 : 0);
             for (int s = 0; s < S::kKSlots; ++s) mbar_drain_one(bars + FW_KFULL + s, nk > s ? (nk - s + S::kKSlots - 1) / S::kKSlots : 0);
         }
-      } else if (warp == 11) {
+        }
+      } else if (warp == 11 && elect_one()) {
         // ------------------------------------------------------------------ TMA producer of V
         int nv = early_v;
         for (int g = early_v; g < nkt * 2; ++g) {
             if (!mbar_wait(bars + FW_VEMPTY + g % S::kVSlots, (g / S::kVSlots - 1) & 1, abortp, status, ERRW_V)) break;
-            if (lane == 0) { load_v(g); ++nv; }
-            __syncwarp();
+            load_v(g);
+            ++nv;
         }
-        if (lane == 0 && *abortp)
+        if (*abortp)
             for (int s = 0; s < S::kVSlots; ++s) mbar_drain_one(bars + FW_VFULL + s, nv > s ? (nv - s + S::kVSlots - 1) / S::kVSlots : 0);
       } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer for the score products (one thread)

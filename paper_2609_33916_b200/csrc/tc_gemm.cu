@@ -186,13 +186,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     if (kPair) cluster_sync_all();       // the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after();
     const uint32_t tbase = *tmem_slot;
-    const bool producer = warp == 0 && lane == 0;
-    if (!producer) {
+    if (warp != 0) {
         grid_dependency_wait();
         grid_launch_dependents();
     }
 
-    if (producer) {
+    bool producer = false;
+    if (warp == 0 && elect_one()) {
+        producer = true;
         // ------------------------------------------------------------------ TMA producer
         int it = 0, tm = 0, tn = 0, second = 0;
         bool ok = true;
@@ -585,14 +586,15 @@ tc_gemm_group_kernel(const __grid_constant__ GroupJobs jobs, unsigned int *statu
     auto stages_of = [&](const GroupJob &J) { return (J.K + GK * kSub - 1) / (GK * kSub); };      // per operand pair
 
     auto tail_of = [&](const GroupJob &J) { return (J.K + GK - 1) / GK - (stages_of(J) - 1) * kSub; };   // K blocks of a pair's last stage
-    const bool producer = warp == 0 && lane == 0;
     int armed = 0;       // stages the producer armed
-    if (!producer) {
+    if (warp != 0) {
         grid_dependency_wait();
         grid_launch_dependents();
     }
 
-    if (producer) {
+    bool producer = false;
+    if (warp == 0 && elect_one()) {
+        producer = true;
         // ------------------------------------------------------------------ TMA producer
         int it = 0, jx = 0, m0 = 0, n0 = 0;
         bool ok = true;
