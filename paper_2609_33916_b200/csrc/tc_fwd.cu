@@ -14,16 +14,12 @@
 //              ring follows the score products, the V ring the P V products, and a single producer made
 //              the next K tile wait for a V slot, i.e. for a P V product).
 //   warp 9     UMMA issuer (one thread) for S = Q K^T (SS, both operands K-major) into the ONE score
-//              buffer: S(j+1) is issued as soon as the warpgroup of tile j holds that tile's scores in
-//              registers, and runs under tile j's exponentials.
-//   warp 10    UMMA issuer (one thread) for O_h += P V (TS: P from TMEM, V MN-major in smem).  It lets
-//              S(j+2) through the pipe before it issues P V(j): the warpgroup that waits for those scores
-//              has nothing else to do, and UMMAs of two threads issued together interleave, so that both
-//              products take twice as long.
+//              buffer, S(j+1) as soon as the warpgroup of tile j holds that tile's scores in registers, so
+//              that it runs under tile j's exponentials, and for O_h += P V (TS: P from TMEM, V MN-major in
+//              smem), P V(j) behind S(j+2).  (64 columns: warp 10 issues the P V, see the role.)
 // The two warpgroups take turns on the score buffer, so one is in its exp2 loop while the other waits,
 // loads and takes its maxima; with both working on halves of the same tile (the earlier form of this
 // kernel) the two exp2 loops ran together, the MUFU unit was saturated during them and idle otherwise.
-// UMMAs of different threads are unordered; every hazard between them goes through an mbarrier.
 // TMEM (512 columns): scores [0,128), P of stream 0 / 1 [128,192) / [192,256), O_0 [256,256+D),
 // O_1 [256+D,256+2D).  S, P and the O accumulators never leave the SM: nothing of size n x n reaches HBM.
 //
@@ -50,7 +46,7 @@ using namespace ptx;
 
 constexpr int BM = 128;            // query rows per CTA
 constexpr int BN = 128;            // keys per tile
-constexpr int kThreads = 384;      // warps 0-7 softmax, 8 TMA, 9 UMMA issuer for S, 10 UMMA issuer for PV, 11 idle
+constexpr int kThreads = 384;      // warps 0-7 softmax, 8 TMA of Q and K, 9 UMMA issuer (D = 64: for S, and 10 for P V), 11 TMA of V
 constexpr int kTmemCols = 512;     // scores [0,128); bf16 P of the two streams [128,192), [192,256); two O accumulators from 256
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 256;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -97,6 +93,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     constexpr int kTileBytes = 128 * D * 2;
     constexpr int kBoxes = D / 64;         // 64-column (128-byte) swizzled boxes per tile
     constexpr int kBoxBytes = 128 * 128;   // 128 rows x 128 bytes
+    constexpr bool kOneIssuer = D == 128;
     extern __shared__ __align__(1024) uint8_t sm[];
     uint8_t *sQ = sm /*KC chunks*/, *sK = sm + KC * kTileBytes /*2 slots of one chunk*/, *sV = sm + (KC + 2) * kTileBytes /*2 slots*/;
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + (KC + 4) * kTileBytes);
@@ -173,7 +170,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
     const uint32_t tbase = *tmem_base_p;
     const int nkt = (*abortp == 0) ? nkt_want : 0;   // misaligned shared memory: every role is a no-op
 
-    // 384 threads start with 168 registers each; the last warpgroup (TMA, the two issuers, an idle warp) gives most of its
+    // 384 threads start with 168 registers each; the last warpgroup (TMA, UMMA) gives most of its
     // share to the softmax warpgroups, whose threads hold the 128 scores of a row.  The two counts must add up to what the
     // CTA was launched with (128 x 88 + 256 x 208 = 384 x 168): an increase that asks for more than the decrease frees
     // waits for registers forever.
@@ -230,68 +227,63 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         }
         if (*abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
-      } else if (warp == 9 && elect_one()) {
-        // ------------------------------------------- UMMA issuer for the score GEMMs (one thread)
-        // Two issuing threads (this one for S = Q K^T, warp 10 for O += P V): a successful barrier
-        // probe or a commit costs an issuing thread ~100 cycles during which it feeds nothing, and
-        // the tensor pipe only queues a few UMMAs, so with a single issuer the pipe idled for a
-        // third of every tile.  UMMAs of different threads are not ordered, so every hazard between
-        // the two streams goes through an mbarrier: S(j) may overwrite score buffer j&1 only after
-        // PV(j-2), which read P(j-2) there, has completed (F_OB).
+      } else if ((warp == 9 || (!kOneIssuer && warp == 10)) && elect_one()) {
+        // ------------------------------------------- UMMA issuer: scores and O += P V
+        // 128 columns: one thread, and the products go through the pipe in the order S(j + 2), P V(j), S(j + 3), ...: what S(j + 2) waits for (the scores of tile
+        // j + 1 in registers) comes before P(j), which its warpgroup writes before it loads tile j + 2, which is what S(j + 3) waits for.  64 columns:
+        // warp 10 issues the P V (both measured: tc_fwd2.cu).  UMMAs of different threads are not ordered, so every hazard between the two goes
+        // through an mbarrier.
+        const bool scores = kOneIssuer || warp == 9, values = kOneIssuer || warp == 10;
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
-        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024);
-        const uint32_t km_hi = (uint32_t)(km_proto >> 32);
-        auto field = [](const void *ptr) { return (smem_u32(ptr) >> 4) & 0x3FFFu; };
-        const uint32_t q_lo = (uint32_t)km_proto + field(sQ), k_lo0 = (uint32_t)km_proto + field(sK);
-        constexpr uint32_t kSlot = (uint32_t)(kTileBytes >> 4);
-        bool ok = nkt > 0 && mbar_wait(bars + F_Q, 0, abortp, status, ERR_Q);
-        for (int j = 0; ok && j < nkt; ++j) {
-            const uint32_t dcol = tbase + kColS;
-#pragma unroll
-            for (int c = 0; c < KC; ++c) {          // the contraction over the head dimension, 128 columns per K chunk
-                const int g = j * KC + c, sl = g & 1;
-                const uint32_t k_lo = k_lo0 + sl * kSlot, q_c = q_lo + c * kSlot;
-                if (!mbar_wait(bars + F_KFULL + sl, (g >> 1) & 1, abortp, status, ERR_K)) { ok = false; break; }
-                // the one score buffer is free once the warpgroup of tile j-1 holds that tile's scores in registers
-                if (c == 0 && j >= 1 && !mbar_wait(bars + F_SFREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, abortp, status, ERR_O)) { ok = false; break; }
-                tc_fence_after();
-                if (c == 0) umma_ss2<false>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
-                else        umma_ss2<true>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
-#pragma unroll
-                for (int ks = 1; ks < KL; ++ks) {
-                    const uint32_t off = (uint32_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4);
-                    umma_ss2<true>(dcol, q_c + off, km_hi, k_lo + off, km_hi, idesc_s);
-                }
-                umma_commit(bars + F_KEMPTY + sl);
-            }
-            if (!ok) break;
-            umma_commit(bars + F_S + 2 * (j & 1) + ((j >> 1) & 1));
-        }
-      } else if (warp == 10 && elect_one()) {
-        // ------------------------------------------------ UMMA issuer for O += P V (one thread)
         const uint32_t idesc_pv = KL < D / 16 ? idesc_bf16_f32(128, 16 * KL, 0, 1) : idesc_bf16_f32(128, D, 0, 1);
-        const uint64_t mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);
-        const uint32_t mn_hi = (uint32_t)(mn_proto >> 32);
-        const uint32_t v_lo0 = (uint32_t)mn_proto + ((smem_u32(sV) >> 4) & 0x3FFFu);
+        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);
+        const uint32_t km_hi = (uint32_t)(km_proto >> 32), mn_hi = (uint32_t)(mn_proto >> 32);
+        auto field = [](const void *ptr) { return (smem_u32(ptr) >> 4) & 0x3FFFu; };
+        const uint32_t q_lo = (uint32_t)km_proto + field(sQ), k_lo0 = (uint32_t)km_proto + field(sK), v_lo0 = (uint32_t)mn_proto + field(sV);
         constexpr uint32_t kSlot = (uint32_t)(kTileBytes >> 4);
-        for (int j = 0; j < nkt; ++j) {
-            const int b = j & 1;        // V ring slot and stream of tile j
-            const uint32_t v_lo = v_lo0 + b * kSlot, acol = tbase + kColP + 64 * b, ocol = tbase + kColO + b * D;
-            if (!mbar_wait(bars + F_VFULL + b, (j >> 1) & 1, abortp, status, ERR_V)) break;
-            if (!mbar_wait(bars + F_P + b, (j >> 1) & 1, abortp, status, ERR_P)) break;
-            // The scores come first: this product waits until S(j+2), which is issued the moment tile j+1's scores are in
-            // registers, is through the pipe (two issuing threads' UMMAs interleave and both products take twice as long).
-            if (j + 2 < nkt && !mbar_wait(bars + F_S + 2 * (j & 1) + (((j + 2) >> 1) & 1), ((j + 2) >> 2) & 1, abortp, status, ERR_S)) break;
-            tc_fence_after();
-            // O_b (+)= P(j) V(j): 128 keys = eight k-steps; P (bf16) is 64 TMEM columns, V rows 16 ks .. 16 ks + 15
-            if (j > 1) umma_ts2<true>(ocol, acol, v_lo, mn_hi, idesc_pv);
-            else       umma_ts2<false>(ocol, acol, v_lo, mn_hi, idesc_pv);      // the stream's first tile
+        bool ok = nkt > 0 && (!scores || mbar_wait(bars + F_Q, 0, abortp, status, ERR_Q));
+        for (int j = 0; ok && j < nkt + 2; ++j) {
+            if (scores && j < nkt) {
+                const uint32_t dcol = tbase + kColS;
 #pragma unroll
-            for (int ks = 1; ks < 8; ++ks)
-                umma_ts2<true>(ocol, acol + ks * 8, v_lo + (uint32_t)((ks * 2048) >> 4), mn_hi, idesc_pv);
-            umma_commit(bars + F_OB + b);
-            umma_commit(bars + F_VEMPTY + b);
-            if (j == nkt - 1) umma_commit(bars + F_DONE);
+                for (int c = 0; c < KC; ++c) {          // the contraction over the head dimension, 128 columns per K chunk
+                    const int g = j * KC + c, sl = g & 1;
+                    const uint32_t k_lo = k_lo0 + sl * kSlot, q_c = q_lo + c * kSlot;
+                    if (!mbar_wait(bars + F_KFULL + sl, (g >> 1) & 1, abortp, status, ERR_K)) { ok = false; break; }
+                    // the one score buffer is free once the warpgroup of tile j-1 holds that tile's scores in registers
+                    if (c == 0 && j >= 1 && !mbar_wait(bars + F_SFREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, abortp, status, ERR_O)) { ok = false; break; }
+                    tc_fence_after();
+                    if (c == 0) umma_ss2<false>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
+                    else        umma_ss2<true>(dcol, q_c, km_hi, k_lo, km_hi, idesc_s);
+#pragma unroll
+                    for (int ks = 1; ks < KL; ++ks) {
+                        const uint32_t off = (uint32_t)(((ks / 4) * kBoxBytes + (ks % 4) * 32) >> 4);
+                        umma_ss2<true>(dcol, q_c + off, km_hi, k_lo + off, km_hi, idesc_s);
+                    }
+                    umma_commit(bars + F_KEMPTY + sl);
+                }
+                if (!ok) break;
+                umma_commit(bars + F_S + 2 * (j & 1) + ((j >> 1) & 1));
+            }
+            if (values && j >= 2) {
+                const int i = j - 2, b = i & 1;        // V ring slot and stream of tile i
+                const uint32_t v_lo = v_lo0 + b * kSlot, acol = tbase + kColP + 64 * b, ocol = tbase + kColO + b * D;
+                if (!mbar_wait(bars + F_VFULL + b, (i >> 1) & 1, abortp, status, ERR_V)) break;
+                if (!mbar_wait(bars + F_P + b, (i >> 1) & 1, abortp, status, ERR_P)) break;
+                // Two threads: the scores come first.  This product waits until S(i+2), which is issued the moment tile i+1's scores are in
+                // registers, is through the pipe (two issuing threads' UMMAs interleave and both products take twice as long).
+                if (!kOneIssuer && i + 2 < nkt && !mbar_wait(bars + F_S + 2 * b + (((i + 2) >> 1) & 1), ((i + 2) >> 2) & 1, abortp, status, ERR_S)) break;
+                tc_fence_after();
+                // O_b (+)= P(i) V(i): 128 keys = eight k-steps; P (bf16) is 64 TMEM columns, V rows 16 ks .. 16 ks + 15
+                if (i > 1) umma_ts2<true>(ocol, acol, v_lo, mn_hi, idesc_pv);
+                else       umma_ts2<false>(ocol, acol, v_lo, mn_hi, idesc_pv);      // the stream's first tile
+#pragma unroll
+                for (int ks = 1; ks < 8; ++ks)
+                    umma_ts2<true>(ocol, acol + ks * 8, v_lo + (uint32_t)((ks * 2048) >> 4), mn_hi, idesc_pv);
+                umma_commit(bars + F_OB + b);
+                umma_commit(bars + F_VEMPTY + b);
+                if (i == nkt - 1) umma_commit(bars + F_DONE);
+            }
         }
       }
     } else {

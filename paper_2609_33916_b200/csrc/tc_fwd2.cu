@@ -6,7 +6,7 @@
 //   * what a job costs beside its tiles (set-up, first loads, epilogue: 7.5 us of tc_fwd.cu) is paid once per 256 rows;
 //   * the streams share nothing, so the epilogue merges nothing: a stream that has finished writes its rows while the other still works.
 // The order of the products is that of tc_fwd.cu with its tile number j read as (key tile j / 2, query tile j % 2), and so are the roles, the
-// barriers, the one score buffer used in turn, the P V issuer's yield to the score products and the TMEM plan.  With the causal mask the
+// barriers, the one score buffer used in turn, the order of the products and the TMEM plan.  With the causal mask the
 // longer query tile of a pair (one key tile more) is stream 0; a query tile without a partner (odd count: the last one, causal the
 // first, which is the shortest) runs alone in stream 0.
 // Shared memory: two Q tiles, two K and two V slots (192 KB at D = 128).  A stream's O leaves through its own Q tile.
@@ -20,7 +20,7 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BN = 128;
-constexpr int kThreads = 384;      // warps 0-7 softmax, 8 TMA of Q and K, 9 UMMA issuer for S, 10 UMMA issuer for P V, 11 TMA of V
+constexpr int kThreads = 384;      // warps 0-7 softmax, 8 TMA of Q and K, 9 UMMA issuer (D = 64: for S, and 10 for P V), 11 TMA of V
 constexpr int kTmemCols = 512;     // scores [0,128); bf16 P of the two streams [128,192), [192,256); two O accumulators from 256
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 256;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -50,6 +50,7 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                unsigned int *status)
 {
     constexpr int kTileBytes = 128 * D * 2, kBoxes = D / 64, kBoxBytes = 128 * 128;
+    constexpr bool kOneIssuer = D == 128;
     extern __shared__ __align__(1024) uint8_t sm[];
     uint8_t *sQ = sm /*2 tiles: stream 0, 1*/, *sK = sm + 2 * kTileBytes, *sV = sm + 4 * kTileBytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + 6 * kTileBytes);
@@ -187,25 +188,32 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         }
         if (*abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
-      } else if (warp == 9 && elect_one()) {
-        // ------------------------------------------- UMMA issuer for the score products (one thread)
-        constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
-        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024);
-        const uint32_t km_hi = (uint32_t)(km_proto >> 32);
+      } else if ((warp == 9 || (!kOneIssuer && warp == 10)) && elect_one()) {
+        // ------------------------------------------- UMMA issuer: scores and O += P V
+        // 128 columns: one thread, and the products go through the pipe in the order S(q + 2), P V(q), S(q + 3), ... with q counting the tiles of both streams:
+        // what S(q + 2) waits for (the scores of tile q + 1 in registers) comes before P(q), which its warpgroup writes before it loads tile q + 2, which is
+        // what S(q + 3) waits for.  A P V is queued behind its S instead of being issued once that has been seen to complete.  (Two threads were the faster
+        // form while a probe between two batches drained the pipe.)  Two / one, forward alone: B1 H16 n16384 1765 / 1556 us, B1 H8 n8192 216.3 / 214.5,
+        // B2 H16 n4096 causal 139 / 131.  64 columns: two threads, warp 10 for P V, whose products are short and should not wait for a late K tile
+        // (B1 H8 n8192 causal 100.2 / 102.5 us).
+        const bool scores = kOneIssuer || warp == 9, values = kOneIssuer || warp == 10;
+        constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0), idesc_pv = idesc_bf16_f32(128, 16 * KL, 0, 1);
+        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);
+        const uint32_t km_hi = (uint32_t)(km_proto >> 32), mn_hi = (uint32_t)(mn_proto >> 32);
         auto field = [](const void *ptr) { return (smem_u32(ptr) >> 4) & 0x3FFFu; };
-        const uint32_t q_lo0 = (uint32_t)km_proto + field(sQ), k_lo0 = (uint32_t)km_proto + field(sK);
+        const uint32_t q_lo0 = (uint32_t)km_proto + field(sQ), k_lo0 = (uint32_t)km_proto + field(sK), v_lo0 = (uint32_t)mn_proto + field(sV);
         constexpr uint32_t kSlot = (uint32_t)(kTileBytes >> 4);
-        bool ok = n0 > 0 && mbar_wait(bars + F2_Q, 0, abortp, status, ERR2_Q);
-        int before = -1;            // stream of the tile issued last; its scores have to be in registers
-        for (int kt = 0; ok && kt < n0; ++kt) {
-            const uint32_t k_lo = k_lo0 + (kt & 1) * kSlot;
-            if (!mbar_wait(bars + F2_KFULL + (kt & 1), (kt >> 1) & 1, abortp, status, ERR2_K)) break;
-#pragma unroll 1
-            for (int h = 0; h < (kt < n1 ? 2 : 1); ++h) {
-                // (stream 1's last tile was kt - 1 or, when h = 1, stream 0's is kt)
-                if (before >= 0 && !mbar_wait(bars + F2_SFREE + before, (before < h ? kt : kt - 1) & 1, abortp, status, ERR2_O)) { ok = false; break; }
+        bool ok = n0 > 0 && (!scores || mbar_wait(bars + F2_Q, 0, abortp, status, ERR2_Q));
+        int kt = 0, h = 0, pk = 0, ph = 0;      // the tile (key tile, stream) whose scores come next, and whose P V
+        int bk = -1, bh0 = 0;                   // the tile of the scores issued last
+        const int total = n0 + n1;
+        for (int step = 0; ok && step < total + 2; ++step) {
+            if (scores && step < total) {
+                if (h == 0 && !mbar_wait(bars + F2_KFULL + (kt & 1), (kt >> 1) & 1, abortp, status, ERR2_K)) break;
+                // the one score buffer: the tile before is in registers
+                if (bk >= 0 && !mbar_wait(bars + F2_SFREE + bh0, bk & 1, abortp, status, ERR2_O)) break;
                 tc_fence_after();
-                const uint32_t q_lo = q_lo0 + h * kSlot;
+                const uint32_t k_lo = k_lo0 + (kt & 1) * kSlot, q_lo = q_lo0 + h * kSlot;
                 umma_ss2<false>(tbase + kColS, q_lo, km_hi, k_lo, km_hi, idesc_s);
 #pragma unroll
                 for (int ks = 1; ks < KL; ++ks) {
@@ -214,34 +222,27 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 }
                 if (h == 1 || kt >= n1) umma_commit(bars + F2_KEMPTY + (kt & 1));       // the K tile's last product
                 umma_commit(bars + F2_S + 2 * h + (kt & 1));
-                before = h;
+                bk = kt;
+                bh0 = h;
+                if (h == 0 && kt < n1) h = 1;
+                else { h = 0; ++kt; }
             }
-        }
-      } else if (warp == 10 && elect_one()) {
-        // ------------------------------------------------ UMMA issuer for O += P V (one thread)
-        constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 16 * KL, 0, 1);
-        const uint64_t mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);
-        const uint32_t mn_hi = (uint32_t)(mn_proto >> 32);
-        const uint32_t v_lo0 = (uint32_t)mn_proto + ((smem_u32(sV) >> 4) & 0x3FFFu);
-        constexpr uint32_t kSlot = (uint32_t)(kTileBytes >> 4);
-        bool ok = true;
-        for (int kt = 0; ok && kt < n0; ++kt) {
-            const uint32_t v_lo = v_lo0 + (kt & 1) * kSlot;
-            if (!mbar_wait(bars + F2_VFULL + (kt & 1), (kt >> 1) & 1, abortp, status, ERR2_V)) break;
-#pragma unroll 1
-            for (int h = 0; h < (kt < n1 ? 2 : 1); ++h) {
-                if (!mbar_wait(bars + F2_P + h, kt & 1, abortp, status, ERR2_P)) { ok = false; break; }
-                // the scores come first: let the stream's next score product through the pipe (see tc_fwd.cu)
-                if (kt + 1 < (h ? n1 : n0) && !mbar_wait(bars + F2_S + 2 * h + ((kt + 1) & 1), ((kt + 1) >> 1) & 1, abortp, status, ERR2_S)) { ok = false; break; }
+            if (values && step >= 2) {
+                if (ph == 0 && !mbar_wait(bars + F2_VFULL + (pk & 1), (pk >> 1) & 1, abortp, status, ERR2_V)) break;
+                if (!mbar_wait(bars + F2_P + ph, pk & 1, abortp, status, ERR2_P)) break;
+                // (two threads: the scores come first, their UMMAs and these would interleave and both take twice as long)
+                if (!kOneIssuer && pk + 1 < (ph ? n1 : n0) && !mbar_wait(bars + F2_S + 2 * ph + ((pk + 1) & 1), ((pk + 1) >> 1) & 1, abortp, status, ERR2_S)) break;
                 tc_fence_after();
-                const uint32_t ocol = tbase + kColO + h * D, acol = tbase + kColP + 64 * h;
-                if (kt > 0) umma_ts2<true>(ocol, acol, v_lo, mn_hi, idesc_pv);
+                const uint32_t v_lo = v_lo0 + (pk & 1) * kSlot, ocol = tbase + kColO + ph * D, acol = tbase + kColP + 64 * ph;
+                if (pk > 0) umma_ts2<true>(ocol, acol, v_lo, mn_hi, idesc_pv);
                 else        umma_ts2<false>(ocol, acol, v_lo, mn_hi, idesc_pv);
 #pragma unroll
                 for (int ks = 1; ks < 8; ++ks)
                     umma_ts2<true>(ocol, acol + ks * 8, v_lo + (uint32_t)((ks * 2048) >> 4), mn_hi, idesc_pv);
-                umma_commit(bars + F2_OB + h);
-                if (h == 1 || kt >= n1) umma_commit(bars + F2_VEMPTY + (kt & 1));       // the V tile's last product
+                umma_commit(bars + F2_OB + ph);
+                if (ph == 1 || pk >= n1) umma_commit(bars + F2_VEMPTY + (pk & 1));       // the V tile's last product
+                if (ph == 0 && pk < n1) ph = 1;
+                else { ph = 0; ++pk; }
             }
         }
       }
