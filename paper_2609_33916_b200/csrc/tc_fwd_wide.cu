@@ -4,8 +4,8 @@
 // still the faster one where there are few query tiles: the rule is in tc_fwd.cu.)
 //
 // CTA = 128 query rows of one (batch, head); roles, barriers and the order of the products as in tc_fwd.cu: two softmax warpgroups take
-// the key tiles in turn, one score buffer, K and V rings with a producer thread each, an issuing thread for S = Q K^T and one for
-// O += P V, which yields to the next scores.  What differs: TMEM has room for ONE accumulator of 192 or 256 columns beside the scores
+// the key tiles in turn, one score buffer, K and V rings with a producer thread each, one issuing thread, which queues
+// S(j + 2), P V(j), S(j + 3), ...  What differs: TMEM has room for ONE accumulator of 192 or 256 columns beside the scores
 // and the two P buffers, so both warpgroups' products go into it, and their weights have to be relative to one maximum per row:
 //   * the reference m of a row lives in shared memory and passes from the warpgroup of tile j - 1 to that of tile j through a barrier: the
 //     warpgroup takes its own tile's maximum, waits for the reference, raises it if the maximum is more than 8 (log2 domain) above,
@@ -28,7 +28,7 @@ namespace {
 using namespace ptx;
 
 constexpr int BM = 128, BN = 128;
-constexpr int kThreads = 384;      // warps 0-7 softmax, 8 TMA of Q and K, 9 UMMA issuer for S, 10 UMMA issuer for P V, 11 TMA of V
+constexpr int kThreads = 384;      // warps 0-7 softmax, 8 TMA of Q and K, 9 UMMA issuer, 11 TMA of V
 constexpr int kTmemCols = 512;
 constexpr uint32_t kColS = 0, kColP = 128, kColO = 256;
 constexpr float kLog2e = 1.4426950408889634f;
@@ -190,57 +190,54 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         if (*abortp)
             for (int s = 0; s < S::kVSlots; ++s) mbar_drain_one(bars + FW_VFULL + s, nv > s ? (nv - s + S::kVSlots - 1) / S::kVSlots : 0);
       } else if (warp == 9 && elect_one()) {
-        // ------------------------------------------- UMMA issuer for the score products (one thread)
-        constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0);
-        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024);
-        const uint32_t km_hi = (uint32_t)(km_proto >> 32);
+        // ------------------------------------------- UMMA issuer (one thread): S(j + 2), P V(j), S(j + 3), ... (why: tc_fwd2.cu)
+        // Two threads / one, forward alone: B1 H16/4 n3001 d192 causal 58.5 / 54.6 us, B1 H8 n8192 d192 316.5 / 304, B2 H16 n4096 d256 causal 234 / 227.5.
+        constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0), idesc_pv = idesc_bf16_f32(128, 64 * NB, 0, 1);
+        const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, S::kVBox, 1024);
+        const uint32_t km_hi = (uint32_t)(km_proto >> 32), mn_hi = (uint32_t)(mn_proto >> 32);
         auto field = [](const void *ptr) { return (smem_u32(ptr) >> 4) & 0x3FFFu; };
         const uint32_t q_lo = (uint32_t)km_proto + field(sQ);
         bool ok = nkt > 0 && mbar_wait(bars + FW_Q, 0, abortp, status, ERRW_Q);
-        for (int j = 0; ok && j < nkt; ++j) {
+        for (int step = 0; ok && step < nkt + 2; ++step) {
+            if (step < nkt) {
+                const int j = step;
 #pragma unroll
-            for (int c = 0; c < S::kChunks; ++c) {
-                const int g = j * S::kChunks + c, sl = g % S::kKSlots;
-                const uint32_t k_lo = (uint32_t)km_proto + field(sK + sl * S::kKSlot);
-                if (!mbar_wait(bars + FW_KFULL + sl, (g / S::kKSlots) & 1, abortp, status, ERRW_K)) { ok = false; break; }
-                // the one score buffer is free once the warpgroup of tile j-1 holds that tile's scores in registers
-                if (c == 0 && j >= 1 && !mbar_wait(bars + FW_SFREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, abortp, status, ERRW_O)) { ok = false; break; }
-                tc_fence_after();
+                for (int c = 0; c < S::kChunks; ++c) {
+                    const int g = j * S::kChunks + c, sl = g % S::kKSlots;
+                    const uint32_t k_lo = (uint32_t)km_proto + field(sK + sl * S::kKSlot);
+                    if (!mbar_wait(bars + FW_KFULL + sl, (g / S::kKSlots) & 1, abortp, status, ERRW_K)) { ok = false; break; }
+                    // the one score buffer is free once the warpgroup of tile j-1 holds that tile's scores in registers
+                    if (c == 0 && j >= 1 && !mbar_wait(bars + FW_SFREE + ((j - 1) & 1), ((j - 1) >> 1) & 1, abortp, status, ERRW_O)) { ok = false; break; }
+                    tc_fence_after();
 #pragma unroll
-                for (int ks = 0; ks < 4 * S::kChunkBoxes; ++ks) {
-                    const uint32_t koff = (uint32_t)(((ks / 4) * S::kBox + (ks % 4) * 32) >> 4), qoff = koff + (uint32_t)((c * S::kKSlot) >> 4);
-                    if (c == 0 && ks == 0) umma_ss2<false>(tbase + kColS, q_lo, km_hi, k_lo, km_hi, idesc_s);
-                    else                   umma_ss2<true>(tbase + kColS, q_lo + qoff, km_hi, k_lo + koff, km_hi, idesc_s);
+                    for (int ks = 0; ks < 4 * S::kChunkBoxes; ++ks) {
+                        const uint32_t koff = (uint32_t)(((ks / 4) * S::kBox + (ks % 4) * 32) >> 4), qoff = koff + (uint32_t)((c * S::kKSlot) >> 4);
+                        if (c == 0 && ks == 0) umma_ss2<false>(tbase + kColS, q_lo, km_hi, k_lo, km_hi, idesc_s);
+                        else                   umma_ss2<true>(tbase + kColS, q_lo + qoff, km_hi, k_lo + koff, km_hi, idesc_s);
+                    }
+                    umma_commit(bars + FW_KEMPTY + sl);
                 }
-                umma_commit(bars + FW_KEMPTY + sl);
+                if (!ok) break;
+                umma_commit(bars + FW_S + 2 * (j & 1) + ((j >> 1) & 1));
             }
-            if (!ok) break;
-            umma_commit(bars + FW_S + 2 * (j & 1) + ((j >> 1) & 1));
-        }
-      } else if (warp == 10 && elect_one()) {
-        // ------------------------------------------------ UMMA issuer for O += P V (one thread)
-        constexpr uint32_t idesc_pv = idesc_bf16_f32(128, 64 * NB, 0, 1);
-        const uint64_t mn_proto = smem_desc_sw128(0, S::kVBox, 1024);
-        const uint32_t mn_hi = (uint32_t)(mn_proto >> 32);
-        for (int j = 0; j < nkt; ++j) {
-            const int b = j & 1, g = 2 * j, s0 = g % S::kVSlots, s1 = (g + 1) % S::kVSlots;
-            if (!mbar_wait(bars + FW_VFULL + s0, (g / S::kVSlots) & 1, abortp, status, ERRW_V)) break;
-            if (!mbar_wait(bars + FW_P + b, (j >> 1) & 1, abortp, status, ERRW_P)) break;
-            // the scores come first (see tc_fwd.cu)
-            if (j + 2 < nkt && !mbar_wait(bars + FW_S + 2 * (j & 1) + (((j + 2) >> 1) & 1), ((j + 2) >> 2) & 1, abortp, status, ERRW_S)) break;
-            if (!mbar_wait(bars + FW_VFULL + s1, ((g + 1) / S::kVSlots) & 1, abortp, status, ERRW_V)) break;
-            tc_fence_after();
-            const uint32_t acol = tbase + kColP + 64 * b, ocol = tbase + kColO;
+            if (step >= 2) {
+                const int j = step - 2, b = j & 1, g = 2 * j, s0 = g % S::kVSlots, s1 = (g + 1) % S::kVSlots;
+                if (!mbar_wait(bars + FW_VFULL + s0, (g / S::kVSlots) & 1, abortp, status, ERRW_V)) break;
+                if (!mbar_wait(bars + FW_VFULL + s1, ((g + 1) / S::kVSlots) & 1, abortp, status, ERRW_V)) break;
+                if (!mbar_wait(bars + FW_P + b, (j >> 1) & 1, abortp, status, ERRW_P)) break;
+                tc_fence_after();
+                const uint32_t acol = tbase + kColP + 64 * b, ocol = tbase + kColO;
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {          // 16 keys each; P (bf16) is 64 TMEM columns
-                const uint32_t v_lo = (uint32_t)mn_proto + ((smem_u32(sV + (ks < 4 ? s0 : s1) * S::kVSlot) >> 4) & 0x3FFFu) + (uint32_t)(((ks & 3) * 2048) >> 4);
-                if (ks == 0 && j == 0) umma_ts2<false>(ocol, acol, v_lo, mn_hi, idesc_pv);
-                else                   umma_ts2<true>(ocol, acol + ks * 8, v_lo, mn_hi, idesc_pv);
-                if (ks == 3) umma_commit(bars + FW_VEMPTY + s0);
+                for (int ks = 0; ks < 8; ++ks) {          // 16 keys each; P (bf16) is 64 TMEM columns
+                    const uint32_t v_lo = (uint32_t)mn_proto + field(sV + (ks < 4 ? s0 : s1) * S::kVSlot) + (uint32_t)(((ks & 3) * 2048) >> 4);
+                    if (ks == 0 && j == 0) umma_ts2<false>(ocol, acol, v_lo, mn_hi, idesc_pv);
+                    else                   umma_ts2<true>(ocol, acol + ks * 8, v_lo, mn_hi, idesc_pv);
+                    if (ks == 3) umma_commit(bars + FW_VEMPTY + s0);
+                }
+                umma_commit(bars + FW_VEMPTY + s1);
+                umma_commit(bars + FW_OB + b);
+                if (j == nkt - 1) umma_commit(bars + FW_DONE);
             }
-            umma_commit(bars + FW_VEMPTY + s1);
-            umma_commit(bars + FW_OB + b);
-            if (j == nkt - 1) umma_commit(bars + FW_DONE);
         }
       }
     } else {
