@@ -56,11 +56,11 @@ constexpr int kABytes = GM * GK * 2;
 // A CTA on its own stages 16 KB of A and 32 KB of B per 64 K-elements, four stages (three measured 7-16 % slower: the
 // ring has to cover the L2 latency).  A CTA of a pair stages 16 KB of A and its half of B, 16 KB: six stages.
 // In a pair a stage holds two such blocks (128 K-elements, 64 KB) and the ring has three: one wait and one commit of
-// the issuing thread per eight UMMAs instead of per four (that thread's time per stage is on the critical path: a
-// second commit per stage cost 3-4 %).
+// the issuing thread per eight UMMAs instead of per four (six stages of one block: 4096^3 94.9 / 97.5 us, 8192 x 2048 x 8192
+// 187 / 191).
 // Narrower tiles are for launches whose 256-column tiles would leave SMs idle: less work per SM and a shorter epilogue, at more operand
-// traffic per unit of work.  Their stages hold two K blocks as well: a wait, four short UMMAs and a commit take the issuing thread 640
-// cycles a block whatever the width, so that with one block per stage they gained nothing.
+// traffic per unit of work.  Their stages hold two K blocks as well: with one (six stages at 128 columns, eight at 64) operands stored by
+// columns, whose copies are many, fall behind (512 x 512 x 2048 (1,1) 7.8 / 9.7 us, 1024 x 1024 x 1613 (1,1) 7.7 / 9.1; others level).
 constexpr int kMaxStages = 6;
 __host__ __device__ constexpr int gemm_sub(bool pair, int n) { return pair || n < 256 ? 2 : 1; }       // 64-element K blocks per stage
 __host__ __device__ constexpr int gemm_stages(bool pair, int n) { return pair ? 3 : n == 256 ? 4 : n == 128 ? 3 : 4; }
@@ -868,13 +868,19 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
     const long long pair_tiles = (long long)((M + 2 * GM - 1) / (2 * GM)) * (tiles(256) / rows);
     const int mode = gemm_pair_mode();
     const bool fits = pair_tiles >= 8 && (pair_tiles + pairs - 1) / pairs <= (tiles(256) + sms - 1) / sms;   // (a few tiles: launch-bound)
-    const bool pair_ok = mode && fits && (kEpi == EPI_STORE || K >= 1024);
+    // A plain product whose single tiles all run at once, and whose K loop is not long, is over before the pairs' cluster start is paid: pairs / single
+    // 4096 x 1024 x 1024 11.3 / 10.4 us, 1300 x 3072 x 1024 11.4 / 10.3, 4096 x 1024 x 3072 (0,1) 21.2 / 20.6, 3072 x 1024 x 1300 (1,1) 12.7 / 12.2; but
+    // not where an operand stored by columns comes in by many copies (1024 x 2728 x 1300 (1,1) 13.0 / 14.8).
+    const long long parts = (A1 && !kDualN && nbatch == 1) ? 2 : 1;
+    const bool few_copies = (!kAMn || A0.cols % 64 == 0) && (!kBMn || B0.cols % 64 == 0);
+    const bool one_wave = kEpi == EPI_STORE && tiles(256) <= sms && K64 * parts <= 48 && few_copies;
+    const bool pair_ok = mode && fits && !one_wave && (kEpi == EPI_STORE || K >= 1024);
     // Where the 256-column tiles leave SMs idle, the narrower ones compete: cycles of a K block (UMMAs at 256 columns, its
     // operands' way from L2 below that, which is longer for operands that come in by blocks of columns: a long K loop of 128-column tiles then takes up
     // to a fifth more than of K-major ones, 1208 x 5048 x 1664 (1,1) 35.5 us, 30.4 in pairs), of a chunk of the epilogue, and the rounds the
     // grid takes.
     constexpr double kChunk = kEpi == EPI_STORE ? 1100 : kEpi == EPI_SWIGLU_FWD ? 2500 : 3500;
-    const double blocks = (double)K64 * ((A1 && !kDualN && nbatch == 1) ? 2 : 1);
+    const double blocks = (double)(K64 * parts);
     auto cost = [&](long long t, long long slots, double block, int n) {
         const double epi = kChunk * (kDualN ? n / 128 : n / 64), main = blocks * block;
         return (double)((t + slots - 1) / slots) * (main > epi ? main : epi) + epi;
