@@ -1,7 +1,8 @@
 // Backward attention for head dimensions 136..192 on the sm_100a tensor cores, bf16 in, fp32 accumulate: the whole head dimension in
 // ONE pass.  (tc_bwd_wide.cu, which runs 200..256, computes the scores and dP in each of two passes over the halves of d; run on 192
 // columns, 40 UMMAs per pass and 64-query tile against 56 here for both, and its loop is bound by the chain of hand-offs, which
-// is paid once here: B1 H16 H_kv4 n3001 causal backward 385 -> 279 us, B1 H8 n8192 2108 -> 1420 us.)
+// is paid once here: B1 H16 H_kv4 n3001 causal backward 385 -> 279 us, B1 H8 n8192 2108 -> 1420 us; since the UMMAs are issued by an elected thread
+// 256 and 1115.)
 //
 // Same mathematics, the same key-tile-parallel structure and the same one-writer rule for dK and dV as tc_bwd.cu.  CTA = 128 keys of one
 // K/V head (or, kSplit, its part of their query tiles); query tiles of 64 rows.

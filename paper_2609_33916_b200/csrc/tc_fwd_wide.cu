@@ -1,6 +1,6 @@
 // Forward attention for head dimensions 136..256 on the sm_100a tensor cores, bf16 in, fp32 accumulate: the whole head dimension in one
 // CTA.  (Two CTAs per query tile, each with half of the output columns, compute every score and every exponential twice: B1 H16
-// H_kv4 n3001 d192 causal 99 us, here 58; B1 H8 n8192 d192 552, here 325; B1 H8 n8192 d256 600, here 434.  From 200 columns on that form is
+// H_kv4 n3001 d192 causal 99 us, here 55; B1 H8 n8192 d192 552, here 304; B1 H8 n8192 d256 600, here 434 (two issuing threads).  From 200 columns on that form is
 // still the faster one where there are few query tiles: the rule is in tc_fwd.cu.)
 //
 // CTA = 128 query rows of one (batch, head); roles, barriers and the order of the products as in tc_fwd.cu: two softmax warpgroups take
