@@ -41,6 +41,7 @@
 //   EPI_SWIGLU_BWD  C = dh; reads the stored a, u; writes da = dh u s (1 + a (1 - s)) and
 //                   du = dh a s, s = sigmoid(a).  dh itself never reaches memory.
 #include "common.cuh"
+#include "gemm_rule.cuh"
 #include "ptx.cuh"
 #include "tensormap.cuh"
 #include "moa_block.h"
@@ -50,7 +51,7 @@ namespace {
 
 using namespace ptx;
 
-constexpr int GM = 128, GK = 64;
+constexpr int GM = 128, GK = 64;                       // (gemm_rule.cuh counts in these)
 constexpr int kGemmThreads = 320;                      // producer, issuer, eight epilogue warps
 constexpr int kABytes = GM * GK * 2;
 // A CTA on its own stages 16 KB of A and 32 KB of B per 64 K-elements, four stages (three measured 7-16 % slower: the
@@ -860,44 +861,12 @@ cudaError_t launch_gemm(const Operand &A0, const Operand &B0, const Operand *A1,
                         const void *C2, const void *C3, int c_rows, int ldc, int M, int N, int K, cudaStream_t st,
                         int nbatch = 1, bool has_res = false)
 {
-    // Pairs unless they would need more waves than single CTAs (tiny M); the two gate GEMMs only when the main loop outlasts
-    // their epilogue.
     constexpr bool kDualN = kEpi == EPI_SWIGLU_FWD;
-    const long long sms = device_info().sms, pairs = sms / 2, rows = (M + GM - 1) / GM, K64 = (K + GK - 1) / GK;
-    auto tiles = [&](int n) { return rows * ((N + (kDualN ? n / 2 : n) - 1) / (kDualN ? n / 2 : n)) * nbatch; };
-    const long long pair_tiles = (long long)((M + 2 * GM - 1) / (2 * GM)) * (tiles(256) / rows);
-    const int mode = gemm_pair_mode();
-    const bool fits = pair_tiles >= 8 && (pair_tiles + pairs - 1) / pairs <= (tiles(256) + sms - 1) / sms;   // (a few tiles: launch-bound)
-    // A plain product whose single tiles all run at once, and whose K loop is not long, is over before the pairs' cluster start is paid: pairs / single
-    // 4096 x 1024 x 1024 11.3 / 10.4 us, 1300 x 3072 x 1024 11.4 / 10.3, 4096 x 1024 x 3072 (0,1) 21.2 / 20.6, 3072 x 1024 x 1300 (1,1) 12.7 / 12.2; but
-    // not where an operand stored by columns comes in by many copies (1024 x 2728 x 1300 (1,1) 13.0 / 14.8).
-    const long long parts = (A1 && !kDualN && nbatch == 1) ? 2 : 1;
-    const bool few_copies = (!kAMn || A0.cols % 64 == 0) && (!kBMn || B0.cols % 64 == 0);
-    const bool one_wave = kEpi == EPI_STORE && tiles(256) <= sms && K64 * parts <= 48 && few_copies;
-    const bool pair_ok = mode && fits && !one_wave && (kEpi == EPI_STORE || K >= 1024);
-    // Where the 256-column tiles leave SMs idle, the narrower ones compete: cycles of a K block (UMMAs at 256 columns, its
-    // operands' way from L2 below that, which is longer for operands that come in by blocks of columns: a long K loop of 128-column tiles then takes up
-    // to a fifth more than of K-major ones, 1208 x 5048 x 1664 (1,1) 35.5 us, 30.4 in pairs), of a chunk of the epilogue, and the rounds the
-    // grid takes.
-    constexpr double kChunk = kEpi == EPI_STORE ? 1100 : kEpi == EPI_SWIGLU_FWD ? 2500 : 3500;
-    const double blocks = (double)(K64 * parts);
-    auto cost = [&](long long t, long long slots, double block, int n) {
-        const double epi = kChunk * (kDualN ? n / 128 : n / 64), main = blocks * block;
-        return (double)((t + slots - 1) / slots) * (main > epi ? main : epi) + epi;
-    };
-    int n = 256;
-    bool pair = mode == 2 || pair_ok;
-    if (mode != 2 && tiles(256) < 2 * sms) {
-        double best = pair ? cost(pair_tiles, pairs, 530, 256) : cost(tiles(256), sms, 520, 256);
-        const double c128 = cost(tiles(128), sms, K64 < 12 ? 360 : kAMn ? 430 : kBMn ? 390 : 360, 128);
-        if (c128 < 0.95 * best) { best = c128; n = 128; pair = false; }
-        const double c64 = kDualN ? 1e30 : cost(tiles(64), sms, 290, 64);
-        if (c64 < 0.95 * best) { n = 64; pair = false; }
-    }
-    if (pair) return launch_gemm_as<kAMn, kBMn, kEpi, true, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+    const GemmTile tile = gemm_tile(M, N, K, kAMn, kBMn, kEpi == EPI_STORE, kDualN, A1 && !kDualN && nbatch == 1, nbatch, device_info().sms, gemm_pair_mode());
+    if (tile.pair) return launch_gemm_as<kAMn, kBMn, kEpi, true, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
     if constexpr (!kDualN)
-        if (n == 64) return launch_gemm_as<kAMn, kBMn, kEpi, false, 64>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
-    if (n == 128) return launch_gemm_as<kAMn, kBMn, kEpi, false, 128>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+        if (tile.columns == 64) return launch_gemm_as<kAMn, kBMn, kEpi, false, 64>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
+    if (tile.columns == 128) return launch_gemm_as<kAMn, kBMn, kEpi, false, 128>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
     return launch_gemm_as<kAMn, kBMn, kEpi, false, 256>(A0, B0, A1, B1, C0, C1, C2, C3, c_rows, ldc, M, N, K, st, nbatch, has_res);
 }
 
