@@ -458,9 +458,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         const int lane_row = 32 * (warp % 4) + lane;
         const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp % 4)) << 16);
         TileWalk wr = walk0;
-        for (int it = 0; it < (skip_dq ? 0 : niter); ++it) {
+        for (int it = 0; it < (skip_dq ? 0 : niter); ++it, wr.next()) {
             const int qtile = wr.qi, qh = wr.qh, qrow = qtile * 128 + lane_row;
-            wr.next();
             if (!mbar_wait(bars + B_DQ, it & 1, abortp, status, ERR_DQ)) break;
             tc_fence_after();
             uint32_t r[D / 32][32];
@@ -497,12 +496,11 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                         }
                         mbar_arrive(bars + B_STGFULL + st);
                         if (leader && stage_ok && mbar_wait(bars + B_STGFULL + st, (g >> 1) & 1, abortp, status, ERR_STAGE)) {
-                            // (query head, tile) of this iteration: recomputed here, by the one thread that
-                            // needs them, rather than kept live beside the 128 registers of the tile
-                            const int nq_per = nqt - i_begin, at = it0 + it;
-                            const int hh = kGrouped ? at / nq_per : 0;
-                            tma_reduce_add_3d(&mapdQ, stage, 0, (i_begin + at - hh * nq_per) * 128 + 32 * c,
-                                              (kGrouped ? bh * group : bh) + hh);
+                            // (query head, tile) of this iteration.  One head: counted from the iteration, rather than kept live beside the 128
+                            // registers of the tile.  Shared K/V heads: from the walker, since a division here, in front of every quarter of a
+                            // tile, stands in the chain of hand-offs that paces these warps (division / walker: B1 H8/1 n2300 causal 71.1 / 66.1 us,
+                            // H32/1 n1000 109.4 / 101.4, H32/4 n4096 753 / 702).
+                            tma_reduce_add_3d(&mapdQ, stage, 0, (kGrouped ? wr.qi : i_begin + it0 + it) * 128 + 32 * c, kGrouped ? wr.qh : bh);
                             bulk_commit();
                         }
                     }
