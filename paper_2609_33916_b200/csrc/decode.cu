@@ -689,9 +689,9 @@ static bool decode_uses_tc(const DecodeProblem &p, int dtype)
 }
 
 // Tensor-core route: key tiles of 128 per CTA segment, one CTA per SM at a time.  All CTAs are equal,
-// so the run takes ceil(CTAs / SMs) rounds of (fixed cost + tiles per segment); the fixed cost of a CTA
-// (pipeline fill, epilogue) was measured at about 3.5 tile times.  Take the segment count that
-// minimises rounds x (3.5 + tiles).
+// so the run takes ceil(CTAs / SMs) rounds of (fixed cost + tiles per segment).  Take the segment count that
+// minimises rounds x (3.5 + tiles).  (3.5 tile times were the fixed cost, pipeline fill and epilogue, of an earlier form of the kernel; calls of one and
+// of two rounds over the same cache now differ by 8.7 tile times at 128 columns and 6.7 at 64, the merge of twice the segments included.)
 static void decode_tc_splits(const DecodeProblem &p, int *splits, int *tiles_per_split)
 {
     const int nkt = (p.n + 127) / 128;

@@ -31,9 +31,11 @@ inline GemmTile gemm_tile(long long M, long long N, long long K, bool a_mn, bool
     const bool one_wave = plain && tiles(256) <= sms && K64 * parts <= 48 && few_copies && whole_rows;
     const bool pair_ok = mode && fits && !one_wave && (plain || K >= 1024);
     // Where the 256-column tiles leave SMs idle, the narrower ones compete: cycles of a K block (UMMAs at 256 columns, its
-    // operands' way from L2 below that, which is longer for operands that come in by blocks of columns: a long K loop of 128-column tiles then takes up
-    // to a fifth more than of K-major ones, 1208 x 5048 x 1664 (1,1) 35.5 us, 30.4 in pairs), of a chunk of the epilogue, and the rounds the
-    // grid takes.
+    // operands' way from L2 below that), of a chunk of the epilogue, and the rounds the grid takes.  The cycles are of issuers that were not elected; as
+    // slopes over K (1024 to 3072, 128 tiles at once, 1965 MHz) a block now takes 287 at 64 columns, 387 to 395 at 128 in every storage order, 690 at 256
+    // columns and 655 in pairs (615 and 590 at 64 tiles at once).  The choice holds up: over 70 products of random sizes and storage each width forced is
+    // at most 4.5 % faster from K 512 on (368 x 3600 x 2104 (0,1) 14.6 us, 14.0 at 128 columns), up to 14 % below (408 x 3840 x 136 5.7, 5.0 at 128), and
+    // for operands that come in by blocks of columns a long K loop at 128 columns loses to pairs (1208 x 5048 x 1664 (1,1) 35.0 us, 27.5 in pairs).
     const double chunk = plain ? 1100 : dual ? 2500 : 3500;
     const double blocks = (double)(K64 * parts);
     auto cost = [&](long long t, long long slots, double block, int n) {

@@ -284,11 +284,12 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// One thread of the warp (every lane calls it together).  The roles that issue UMMAs or TMA copies run behind it, not behind `lane == 0`:
-// these instructions take their operands from registers that the whole warp shares, and only behind elect.sync does the compiler know that a single
-// thread is there; behind a test of the lane each instruction was wrapped so that it would hold for any number of threads.  Measured (148 SMs,
-// batches of eight UMMAs, a commit and a barrier probe, cycles per batch, lane == 0 / elect): 128 x 128 x 16 from shared memory 608 / 512, with
-// two probes 679 / 512; A from TMEM 593 / 512; N = 64 608 / 428, A from TMEM 593 / 268; N = 256 1024 either way.
+// One thread of the warp, the same one each time (every lane calls it together).  All roles that issue UMMAs, and the TMA producers of the attention and GEMM kernels, run
+// behind it, not behind `lane == 0`: the instruction promises a single thread, a test of the lane does not, and the issue of UMMAs is slower behind
+// the test.  Measured (148 SMs, batches of eight UMMAs, a commit and a barrier probe, cycles per batch, lane == 0 / elect): 128 x 128 x 16 from shared
+// memory 608 / 512, with two probes 679 / 512; A from TMEM 593 / 512; N = 64 608 / 428, A from TMEM 593 / 268; N = 256 1024 either way.
+// (Still behind a test of the lane or thread: the threads that send dQ, stores and residual loads, the decode and RMSNorm producers, the producers
+// of tc_materialize.cu, and in tc_bwd_pair.cu all but the UMMA issuer.)
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t one;

@@ -385,28 +385,24 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             if (!mbar_wait(bars + B_DOFULL + sdo, (it / kDoSlots) & 1, abortp, status, ERR_FULL)) break;
             if (kAliasDQ && !skip_dq && it > 0 && !mbar_wait(bars + B_DQR, (it - 1) & 1, abortp, status, ERR_DQR)) break;
             tc_fence_after();
-            {
-                umma_ss2<false>(tbase + colDP, v_km, km_hi, do_km, km_hi, idesc_st);
+            umma_ss2<false>(tbase + colDP, v_km, km_hi, do_km, km_hi, idesc_st);
 #pragma unroll
-                for (int ks = 1; ks < KL; ++ks)
-                    umma_ss2<true>(tbase + colDP, v_km + koff(ks), km_hi, do_km + koff(ks), km_hi, idesc_st);
-                umma_commit(bars + B_DP);
-            }
+            for (int ks = 1; ks < KL; ++ks)
+                umma_ss2<true>(tbase + colDP, v_km + koff(ks), km_hi, do_km + koff(ks), km_hi, idesc_st);
+            umma_commit(bars + B_DP);
             if (!mbar_wait(bars + B_P, it & 1, abortp, status, ERR_PDS)) break;
             // (the probe for S(i+1)'s operand sits here, so that dV and S are issued back to back)
             if (it + 1 < niter && !mbar_wait(bars + B_QFULL + ((it + 1) & 1), ((it + 1) >> 1) & 1, abortp, status, ERR_FULL)) break;
             tc_fence_after();
-            {
-                // 16 queries per step; the very first UMMA of the CTA overwrites the accumulator
-                if (it > 0) umma_ts2<true>(tbase + colDV, tbase + colS, do_mn, mn_hi, idesc_acc);
-                else        umma_ts2<false>(tbase + colDV, tbase + colS, do_mn, mn_hi, idesc_acc);
+            // 16 queries per step; the very first UMMA of the CTA overwrites the accumulator
+            if (it > 0) umma_ts2<true>(tbase + colDV, tbase + colS, do_mn, mn_hi, idesc_acc);
+            else        umma_ts2<false>(tbase + colDV, tbase + colS, do_mn, mn_hi, idesc_acc);
 #pragma unroll
-                for (int ks = 1; ks < 8; ++ks) {
-                    const uint32_t a_col = 64 * (ks / 4) + 8 * (ks % 4);
-                    umma_ts2<true>(tbase + colDV, tbase + colS + a_col, do_mn + moff(ks), mn_hi, idesc_acc);
-                }
-                umma_commit(bars + B_DOEMPTY + sdo);
+            for (int ks = 1; ks < 8; ++ks) {
+                const uint32_t a_col = 64 * (ks / 4) + 8 * (ks % 4);
+                umma_ts2<true>(tbase + colDV, tbase + colS + a_col, do_mn + moff(ks), mn_hi, idesc_acc);
             }
+            umma_commit(bars + B_DOEMPTY + sdo);
             if (it + 1 < niter) issue_S(q_km0 + ((it + 1) & 1) * kSlot);
             if (!mbar_wait(bars + B_DS, it & 1, abortp, status, ERR_PDS)) break;
             if (!kAliasDQ && !skip_dq && it > 0 && !mbar_wait(bars + B_DQR, (it - 1) & 1, abortp, status, ERR_DQR)) break;
@@ -739,8 +735,8 @@ tc_bwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
     }
     if (*abortp && tid == kLoadWarp * 32) {
-        // A wait expired: copies this thread asked for may still be on their way into the CTA's shared memory.  It
-        // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) before the CTA can leave.  (The other
+        // A wait expired: copies the producer asked for may still be on their way into the CTA's shared memory.  It
+        // stays for a fixed 400,000 cycles (hundreds of times a copy's latency; any one thread keeps it) before the CTA can leave.  (The other
         // kernels wait on the barriers they armed; here that bookkeeping cost 1.5-3 % under the role's register cap.)
         const long long t0 = clock64();
         while (clock64() - t0 < 400000LL) { }
@@ -776,9 +772,10 @@ cudaError_t launch_bwd_g(const Problem &p, const void *Q, const void *K, const v
     pkv.H = p.kv_heads();
     pkv.Hkv = 0;
     // A long walk is launched plainly: CTAs that wait for the kernel in front are let go at one instant, walk the query tiles of their head in step, and
-    // their reduces meet on the same dQ tile.  Plain / dependent, d = 128: B1 H32/4 n4096 698 / 785 us, B2 H32/8 n4096 1410 / 1538, causal B4 H16/4
-    // n4096 806 / 867; but short walks want the early start (B1 H32/8 n1000 71.0 / 68.9), and so do causal jobs that all run at once (B1 H32/4
-    // n4096 440 / 416) and 64 columns, whose reduces are smaller (within 2 % either way).
+    // their reduces meet on the same dQ tile.  Plain / dependent, d = 128: B1 H32/4 n4096 734 / 804 us, B2 H32/8 n4096 1468 / 1538, causal B4 H16/4
+    // n4096 826 / 854; short walks are level (B1 H32/8 n1000 63.7 / 63.4) and keep the early start, and so do 64 columns, whose reduces are smaller (within
+    // 3 %).  Causal jobs that all run at once keep it too: they were ahead with it when the line was drawn (B1 H32/4 n4096 440 / 416), but no longer are
+    // (414 / 439, H16/4 211 / 219).
     const long long walk = (long long)nkt * p.group();
     const bool apart = D == 128 && kBulk && !kSplit && (p.causal ? walk >= 100 && (long long)nkt * p.BHkv() > device_info().sms : walk >= 48);
     return launch_cluster_as(!apart, tc_bwd_kernel<D, kBulk, kGrouped, kSplit, KL>, (unsigned)split, dim3((unsigned)(nkt * p.BHkv() * split)),
@@ -795,7 +792,8 @@ cudaError_t launch_bwd(const Problem &p, const void *Q, const void *K, const voi
     if constexpr (kBulk) {        // (AUTO is the bulk reduce at these head dimensions)
         const long long nkt = (p.n + 127) / 128, jobs = nkt * p.BHkv(), longest = nkt * p.group();
         const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) / 2 : jobs * longest, p.causal, 2.0, 2.5);
-        // (both sides, d = 128: 8 tiles per job 30.8 us alone, 28.1 in pairs; 4 tiles 21.3 alone, 22.7 in pairs; 3 tiles 17.3, 20.3)
+        // (both sides, d = 128, alone / pairs: 64 jobs of 8 tiles 30.2 / 28.5 us, of 4 tiles 20.9 / 23.4, 48 of 3 tiles 17.9 / 21.6.  The two constants are of
+        // kernels whose UMMAs took longer to issue, and for 32 jobs of 4 tiles they are too low: the estimate takes fours, 22.7, alone 19.8)
         if (split > 1)
             return p.group() > 1 ? launch_bwd_g<D, kBulk, true, true, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
                                  : launch_bwd_g<D, kBulk, false, true, KL>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);

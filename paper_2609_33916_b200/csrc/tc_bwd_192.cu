@@ -1,8 +1,8 @@
 // Backward attention for head dimensions 136..192 on the sm_100a tensor cores, bf16 in, fp32 accumulate: the whole head dimension in
 // ONE pass.  (tc_bwd_wide.cu, which runs 200..256, computes the scores and dP in each of two passes over the halves of d; run on 192
 // columns, 40 UMMAs per pass and 64-query tile against 56 here for both, and its loop is bound by the chain of hand-offs, which
-// is paid once here: B1 H16 H_kv4 n3001 causal backward 385 -> 279 us, B1 H8 n8192 2108 -> 1420 us; since the UMMAs are issued by an elected thread
-// 256 and 1115.)
+// is paid once here: B1 H16 H_kv4 n3001 causal backward 385 -> 279 us, B1 H8 n8192 2108 -> 1420 us; with elected producers and
+// issuers 253, and 1285 in runs of 40 ms under the power cap, 1452 before, or 1162 in short ones.)
 //
 // Same mathematics, the same key-tile-parallel structure and the same one-writer rule for dK and dV as tc_bwd.cu.  CTA = 128 keys of one
 // K/V head (or, kSplit, its part of their query tiles); query tiles of 64 rows.
@@ -454,8 +454,8 @@ tc_bwd192_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant
         cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
     }
     if (*abortp && tid == kLoadWarp * 32) {
-        // A wait expired: copies this thread asked for may still be on their way into the CTA's shared memory.  It
-        // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) before the CTA can leave.
+        // A wait expired: copies the producer asked for may still be on their way into the CTA's shared memory.  It
+        // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) (any one thread keeps it) before the CTA can leave.
         const long long t0 = clock64();
         while (clock64() - t0 < 400000LL) { }
     }
@@ -499,7 +499,8 @@ cudaError_t tc_bwd_kv_192(const Problem &p, const void *Q, const void *K, const 
     const long long nkt = (p.n + 127) / 128, nqt = (p.n + BQ - 1) / BQ, jobs = nkt * p.BHkv(), longest = nqt * p.group();     // query tiles of 64
     const long long total = p.causal ? (nkt * nqt - nkt * (nkt - 1)) * p.BHkv() * p.group() : jobs * longest;
     const int split = !share ? 1 : bwd_split(jobs, longest, total, p.causal, 2.5, 3.0);
-    // (both sides: 16 tiles per job 54.7 us alone, 43.1 in pairs; 8 tiles 34.2 and 31.4; 5 tiles 26.2 and 28.2)
+    // (both sides, alone / pairs: 64 jobs of 16 tiles 50.1 / 40.6 us, of 8 tiles 32.4 / 31.5.  24 jobs of 6 tiles 24.5 / 25.3, of 5 tiles 21.8 / 25.0, where
+    // the estimate, whose constants are older than the elected issuers, takes fours: 28.5 and 28.3)
     if (split > 1)
         return p.group() > 1 ? launch_192<true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
                              : launch_192<false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);

@@ -472,8 +472,8 @@ tc_bwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
         cluster_sync_all();       // nobody leaves while another rank may still read its shared memory
     }
     if (*abortp && tid == kLoadWarp * 32) {
-        // A wait expired: copies this thread asked for may still be on their way into the CTA's shared memory.  It
-        // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) before the CTA can leave.
+        // A wait expired: copies the producer asked for may still be on their way into the CTA's shared memory.  It
+        // stays for a fixed 400,000 cycles (hundreds of times a copy's latency) (any one thread keeps it) before the CTA can leave.
         const long long t0 = clock64();
         while (clock64() - t0 < 400000LL) { }
     }
@@ -517,7 +517,8 @@ cudaError_t tc_bwd_kv_wide(const Problem &p, const void *Q, const void *K, const
     if (p.d <= 128 || p.d > 256 || p.d % 8 || dQacc == nullptr) return cudaErrorInvalidValue;
     const long long nkt = (p.n + 127) / 128, jobs = 2 * nkt * p.BHkv(), longest = 2 * nkt * p.group();     // query tiles of 64
     const int split = !share ? 1 : bwd_split(jobs, longest, p.causal ? jobs * p.group() * (nkt + 1) : jobs * longest, p.causal, 2.5, 3.0);
-    // (both sides, d = 256: 64 tiles per job 176 us alone, 100 in pairs, 64 in fours; 7 tiles 27.1 alone, 25.5 in pairs)
+    // (both sides, d = 256: 16 jobs of 64 tiles 132 us alone, 78 in pairs, 49 in fours; 16 of 8 tiles 23.6, 22.0 and 20.8; 32 of 8 tiles 23.8, 22.4 and 23.6,
+    // where the estimate takes fours)
     if (split > 1)
         return p.group() > 1 ? launch_wide<true, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st)
                              : launch_wide<false, true>(p, Q, K, V, dO, Lp, Dp, dK, dV, dQacc, split, st);

@@ -92,12 +92,10 @@ tc_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ C
         for (int j = 0; j < nkt; ++j) {
             const int s = j & 1;
             if (j >= 2 && !mbar_wait(bars + B_KVEMPTY + s, ((j >> 1) - 1) & 1, abortp, status, ERR_EMPTY)) break;
-            {
-                mbar_arm(bars, bars + B_KVFULL + s, 2 * SM::kTile, armed);
-                for (int b = 0; b < kBoxes; ++b) {
-                    tma_load_4d(sm + SM::offK + s * SM::kTile + b * kBoxBytes, &mapK, bars + B_KVFULL + s, 64 * b, j * 128, hk, bb);
-                    tma_load_4d(sm + SM::offV + s * SM::kTile + b * kBoxBytes, &mapV, bars + B_KVFULL + s, 64 * b, j * 128, hk, bb);
-                }
+            mbar_arm(bars, bars + B_KVFULL + s, 2 * SM::kTile, armed);
+            for (int b = 0; b < kBoxes; ++b) {
+                tma_load_4d(sm + SM::offK + s * SM::kTile + b * kBoxBytes, &mapK, bars + B_KVFULL + s, 64 * b, j * 128, hk, bb);
+                tma_load_4d(sm + SM::offV + s * SM::kTile + b * kBoxBytes, &mapV, bars + B_KVFULL + s, 64 * b, j * 128, hk, bb);
             }
         }
         mbar_drain(bars, armed);     // copies of this CTA still on their way land before it leaves (bounded)

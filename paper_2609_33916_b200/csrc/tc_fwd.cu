@@ -59,8 +59,8 @@ enum { F_Q = 0, F_KFULL = 1 /*2*/, F_KEMPTY = 3 /*2*/, F_VFULL = 5 /*2*/, F_VEMP
        F_P = 11 /*2: per stream*/, F_SFREE = 13 /*2: per stream, the tile's scores are in registers*/, F_O = 15 /*unused*/,
        F_X = 16 /*epilogue exchange*/, F_OB = 17 /*2: per stream, P V of the stream's tile has completed*/,
        F_E = 19 /*O tile staged in shared memory*/, F_DONE = 20 /*last P V of the job has completed*/, 
-       F_S = 21 /*[stream][tile count of the stream & 1]: 4.  Two barriers per stream, taken in turn: the P V issuer, which
-                  lets S(j+2) pass before it issues P V(j), may be stalled on the V ring while the scores run two tiles of
+       F_S = 21 /*[stream][tile count of the stream & 1]: 4.  Two barriers per stream, taken in turn.  With two issuers (64 columns) the one
+                  of P V, which lets S(j+2) pass before it issues P V(j), may be stalled on the V ring while the scores run two tiles of
                   the stream ahead of it, and a parity wait must never fall two phases of one barrier behind*/,
        F_COUNT = 25 };
 
@@ -196,19 +196,19 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
             for (int i = lane; i < rows * (D / 4); i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (elect_one()) {      // (one thread from here on)
-        bool live = true;
-        for (int j = early_k / KC; live && j < nkt; ++j) {
-            for (int c = (j == early_k / KC ? early_k % KC : 0); c < KC; ++c) {
-                const int g = j * KC + c;
-                if (g >= 2 && !mbar_wait(bars + F_KEMPTY + (g & 1), ((g >> 1) - 1) & 1, abortp, status, ERR_K)) { live = false; break; }
-                load_k(g);
+            bool live = true;
+            for (int j = early_k / KC; live && j < nkt; ++j) {
+                for (int c = (j == early_k / KC ? early_k % KC : 0); c < KC; ++c) {
+                    const int g = j * KC + c;
+                    if (g >= 2 && !mbar_wait(bars + F_KEMPTY + (g & 1), ((g >> 1) - 1) & 1, abortp, status, ERR_K)) { live = false; break; }
+                    load_k(g);
+                }
             }
-        }
-        if (*abortp) {
-            // a wait expired somewhere in the CTA: copies still on their way land before it leaves (bounded)
-            mbar_drain_one(bars + F_Q, nkt > 0 ? 1 : 0);
-            for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
-        }
+            if (*abortp) {
+                // a wait expired somewhere in the CTA: copies still on their way land before it leaves (bounded)
+                mbar_drain_one(bars + F_Q, nkt > 0 ? 1 : 0);
+                for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
+            }
         }
       } else if (warp == 11 && elect_one()) {
         // ------------------------------------------------------------------ TMA producer of the V stream
@@ -217,13 +217,11 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         int nv = early_v;       // (the first two tiles went out before the set-up)
         for (int j = early_v; j < nkt; ++j) {
             if (j >= 2 && !mbar_wait(bars + F_VEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR_V)) break;
-            {
-                const int s = j & 1;
-                mbar_arrive_expect_tx(bars + F_VFULL + s, kTileBytes);
-                ++nv;
-                for (int b = 0; b < kBoxes; ++b)
-                    tma_load_4d(sV + s * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + s, D * pass + 64 * b, (kt0 + j) * BN, hk, bb);
-            }
+            const int s = j & 1;
+            mbar_arrive_expect_tx(bars + F_VFULL + s, kTileBytes);
+            ++nv;
+            for (int b = 0; b < kBoxes; ++b)
+                tma_load_4d(sV + s * kTileBytes + b * kBoxBytes, &mapV, bars + F_VFULL + s, D * pass + 64 * b, (kt0 + j) * BN, hk, bb);
         }
         if (*abortp)
             for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F_VFULL + s, nv > s ? (nv - s + 1) / 2 : 0);
@@ -383,7 +381,7 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                     ls2[(i >> 1) & 1] = add_f32x2(ls2[(i >> 1) & 1], pack_f32x2(p0, p1));
                     pk[i / 2] = pack_bf16(p0, p1);
                 }
-                // P(j) goes where P(j-2) was: P V(j-2), which gave way to S(j) in the pipe, has read it by now (the first
+                // P(j) goes where P(j-2) was: P V(j-2), behind S(j) in the pipe, has read it by now (the first
                 // 32 exponentials of the tile ran under the rest of that product)
                 if (c == 0 && t > 0 && !mbar_wait(bars + F_OB + h, (t - 1) & 1, abortp, status, ERR_O)) { ok = false; break; }
                 tmem_st(lane_addr + pcol + 16 * c, pk);
@@ -416,11 +414,10 @@ tc_fwd_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
         mbar_arrive(bars + F_X);
         if (ok && mbar_wait(bars + F_X, 0, abortp, status, ERR_P) &&
             mbar_wait(bars + F_DONE, 0, abortp, status, ERR_O)) {
-            // (F_DONE, not the per-tile F_O with the last tile's parity: the softmax threads can finish the last
-            // tile while the P V products of the last TWO tiles are still pending -- the S and P V issuers are
-            // different threads -- and a wait on F_O's parity would then be satisfied by the tile before those,
-            // which has the same parity.  Seen in decode through this kernel, where tiles arrive at HBM pace:
-            // about one CTA in a hundred wrote an O that missed its last tiles.)
+            // (F_DONE, not a per-tile barrier with the last tile's parity: the softmax threads can finish the last tile while the P V
+            // products of the last TWO tiles are still pending, and such a wait would then be satisfied by the tile before those, which
+            // has the same parity.  Seen with two issuing threads in decode through this kernel, where tiles arrive at HBM
+            // pace: about one CTA in a hundred wrote an O that missed its last tiles.)
             tc_fence_after();
             const float2 other = xch[(h ^ 1) * 128 + lane_row];
             const float m_all = fmaxf(m_used, other.x);
@@ -552,9 +549,9 @@ cudaError_t tc_fwd(const Problem &p, const void *Q, const void *K, const void *V
     if (p.d < 8 || p.d > 256 || p.d % 8) return cudaErrorInvalidValue;
     if (p.d <= 128 && fwd_pairs_pay(p)) return tc_fwd_pairs(p, Q, K, V, O, L, fb, st);
     if (p.d > 128) {
-        // Two CTAs per query tile take 0.7 to 0.85 of the time per key tile of one with all columns, which is worth it while all of them run at once
-        // (with the causal mask: while the longest outlasts the others' share), and from three key tiles on.  Two / one, B1 H4 n1500 d200 22.6 / 29.3
-        // us, causal H2 n3000 d256 31.6 / 40.9, H2 n282 d256 9.7 / 10.4; but 96 tiles of n1500 d256 0.67 the other way, and equal at n130.
+        // Two CTAs per query tile take 0.82 to 0.9 of the time per key tile of one with all columns, which is worth it while all of them run at once
+        // (with the causal mask: while the longest outlasts the others' share), and from three key tiles on.  Two / one, B1 H4 n1500 d200 23.5 / 26.1
+        // us, causal H2 n3000 d256 27.9 / 33.4, H8 n1500 d256 18.4 / 20.4, H2 n282 d256 8.3 / 10.0; but 96 tiles of n1500 d256 34.8 / 22.3.
         const long long nqt = (p.n + BM - 1) / BM, jobs = nqt * p.BH(), sms = device_info().sms;
         const bool few = p.causal ? 4 * (jobs * (nqt + 1) / 2) * 2 <= 3 * nqt * sms : 2 * jobs <= sms;
         if (p.d > 192 && fb.dO == nullptr && fb.zero_acc == nullptr && nqt >= 3 && few) return launch_fwd<128, 2, 8>(p, Q, K, V, O, L, fb, st);

@@ -150,33 +150,31 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             }
         }
         if (elect_one()) {      // (one thread from here on)
-        int nk = early;
-        for (int j = early; j < n0; ++j) {
-            if (!mbar_wait(bars + F2_KEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR2_K)) break;
-            load_k(j);
-            ++nk;
-        }
-        // Fused call: the streams' dO tiles, which the epilogues multiply their rows with, go into the K slots as these come free: stream 1's
-        // into that of the last tile but one (stream 1 ends first), stream 0's into the last tile's.  (Read by the row's owner straight from
-        // global memory, 16 bytes of 32 rows at a time, the two tiles were 2 us of LSU work at the end of a job.)
-        int armed_do = 0;       // bit h
-        if (prep.with_bwd)
+            int nk = early;
+            for (int j = early; j < n0; ++j) {
+                if (!mbar_wait(bars + F2_KEMPTY + (j & 1), ((j >> 1) - 1) & 1, abortp, status, ERR2_K)) break;
+                load_k(j);
+                ++nk;
+            }
+            // Fused call: the streams' dO tiles, which the epilogues multiply their rows with, go into the K slots as these come free: stream 1's
+            // into that of the last tile but one (stream 1 ends first), stream 0's into the last tile's.  (Read by the row's owner straight from
+            // global memory, 16 bytes of 32 rows at a time, the two tiles were 2 us of LSU work at the end of a job.)
+            int armed_do = 0;       // bit h
+            if (prep.with_bwd)
 #pragma unroll 1
-            for (int h = 1; h >= 0; --h) {
-                const int s = (n0 - 1 + h) & 1, uses = (n0 - s + 1) / 2;
-                if ((h ? n1 : n0) == 0) continue;
-                if (uses > 0 && !mbar_wait(bars + F2_KEMPTY + s, (uses - 1) & 1, abortp, status, ERR2_K)) break;
-                {
+                for (int h = 1; h >= 0; --h) {
+                    const int s = (n0 - 1 + h) & 1, uses = (n0 - s + 1) / 2;
+                    if ((h ? n1 : n0) == 0) continue;
+                    if (uses > 0 && !mbar_wait(bars + F2_KEMPTY + s, (uses - 1) & 1, abortp, status, ERR2_K)) break;
                     mbar_arrive_expect_tx(bars + F2_DO + h, kTileBytes);
                     armed_do |= 1 << h;
                     for (int b = 0; b < kBoxes; ++b) tma_load_4d(sK + s * kTileBytes + b * kBoxBytes, &mapdO, bars + F2_DO + h, 64 * b, h ? q01 : q00, hq, bb);
                 }
+            if (*abortp) {
+                for (int h = 0; h < 2; ++h) mbar_drain_one(bars + F2_DO + h, (armed_do >> h) & 1);
+                mbar_drain_one(bars + F2_Q, early > 0 ? 1 : 0);
+                for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
             }
-        if (*abortp) {
-            for (int h = 0; h < 2; ++h) mbar_drain_one(bars + F2_DO + h, (armed_do >> h) & 1);
-            mbar_drain_one(bars + F2_Q, early > 0 ? 1 : 0);
-            for (int s = 0; s < 2; ++s) mbar_drain_one(bars + F2_KFULL + s, nk > s ? (nk - s + 1) / 2 : 0);
-        }
         }
       } else if (warp == 11 && elect_one()) {
         // ------------------------------------------------------------------ TMA producer of V
@@ -192,10 +190,12 @@ tc_fwd2_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         // ------------------------------------------- UMMA issuer: scores and O += P V
         // 128 columns: one thread, and the products go through the pipe in the order S(q + 2), P V(q), S(q + 3), ... with q counting the tiles of both streams:
         // what S(q + 2) waits for (the scores of tile q + 1 in registers) comes before P(q), which its warpgroup writes before it loads tile q + 2, which is
-        // what S(q + 3) waits for.  A P V is queued behind its S instead of being issued once that has been seen to complete.  (Two threads were the faster
-        // form while a probe between two batches drained the pipe.)  Two / one, forward alone: B1 H16 n16384 1765 / 1556 us, B1 H8 n8192 216.3 / 214.5,
-        // B2 H16 n4096 causal 139 / 131.  64 columns: two threads, warp 10 for P V, whose products are short and should not wait for a late K tile
-        // (B1 H8 n8192 causal 100.2 / 102.5 us).
+        // what S(q + 3) waits for.  A P V is queued behind its S instead of being issued once that has been seen to complete.  Two / one, forward alone, in
+        // turn: under the power cap (runs of 40 ms) B1 H16 n16384 1806 / 1784 us at 1567 MHz, B1 H8 n8192 245 / 242, B2 H16 n4096 causal 139.3 / 138.1; at
+        // 1965 MHz the last one 125.6 / 122.9.  A query tile that is alone (n1 == 0: the last one of an odd count) is the exception to the order's reason: tile
+        // q + 1 is the same warpgroup's, which writes P(q) first, so that P V(q) could go before S(q + 2).  It costs nothing there but in one of the shapes timed
+        // (B1 H30 n640 13.28 / 13.02, H74 n384 10.53 / 10.39, H32 n1152 25.4 / 25.4; H64 n640 23.85 / 24.24).  64 columns: two threads, warp 10 for P V, whose
+        // products are short and should not wait for a late K tile (B1 H8 n8192 causal 96.9 / 98.9 us, not causal 194.4 / 198.7).
         const bool scores = kOneIssuer || warp == 9, values = kOneIssuer || warp == 10;
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0), idesc_pv = idesc_bf16_f32(128, 16 * KL, 0, 1);
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, kBoxBytes, 1024);
@@ -424,8 +424,8 @@ cudaError_t launch(const Problem &p, const void *Q, const void *K, const void *V
 
 // Whether pairs of query tiles finish before single ones (tc_fwd.cu), in units of one key tile of one query tile: a job costs about 8
 // (9 for a pair) beside its tiles; equal jobs go in rounds over the SMs, causal ones longest first.  Forward alone, single / pairs:
-// B2 H16 n4096 d128 causal 141 / 124 us, B1 H16 n16384 1913 / 1845, B4 H8 n1024 d64 24.3 / 19.0, B4 H32 n200 causal 18.0 / 11.3, but
-// B1 H8 n2048 23.5 / 37.7 (64 pairs on 148 SMs) and B1 H32 n512 causal 11.0 / 13.2.
+// B2 H16 n4096 d128 causal 145 / 128 us, B1 H16 n16384 1795 / 1780, B4 H8 n1024 d64 20.6 / 16.1, B4 H32 n200 causal 13.4 / 8.2, but
+// B1 H8 n2048 18.4 / 30.1 (64 pairs on 148 SMs) and B1 H32 n512 causal 9.1 / 10.8; close to the line B1 H32 n1024 causal 17.6 / 17.9, H8 n4096 62.5 / 61.5.
 bool fwd_pairs_pay(const Problem &p)
 {
     const long long sms = device_info().sms, nqt = (p.n + BM - 1) / BM, np = (nqt + 1) / 2, bh = p.BH();

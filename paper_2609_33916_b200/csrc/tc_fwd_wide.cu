@@ -1,7 +1,7 @@
 // Forward attention for head dimensions 136..256 on the sm_100a tensor cores, bf16 in, fp32 accumulate: the whole head dimension in one
 // CTA.  (Two CTAs per query tile, each with half of the output columns, compute every score and every exponential twice: B1 H16
-// H_kv4 n3001 d192 causal 99 us, here 55; B1 H8 n8192 d192 552, here 304; B1 H8 n8192 d256 600, here 434 (two issuing threads).  From 200 columns on that form is
-// still the faster one where there are few query tiles: the rule is in tc_fwd.cu.)
+// H_kv4 n3001 d192 causal 110 us, here 57; B1 H8 n8192 d192 637, here 350; B1 H8 n8192 d256 638, here 460 (in turn, runs of 20 ms under the power cap).  From 200
+// columns on that form is still the faster one where there are few query tiles: the rule is in tc_fwd.cu.)
 //
 // CTA = 128 query rows of one (batch, head); roles, barriers and the order of the products as in tc_fwd.cu: two softmax warpgroups take
 // the key tiles in turn, one score buffer, K and V rings with a producer thread each, one issuing thread, which queues
@@ -154,30 +154,30 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             for (int i = lane; i < min(BM, n - q0) * 64; i += 32) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (elect_one()) {      // (one thread from here on)
-        for (int g = early_k; g < nkt * S::kChunks; ++g) {
-            if (!mbar_wait(bars + FW_KEMPTY + g % S::kKSlots, (g / S::kKSlots - 1) & 1, abortp, status, ERRW_K)) break;
-            load_k(g);
-            ++nk;
-        }
-        // fused call: the dO tile, which the epilogue multiplies its rows with, goes over K slots that have come free (see tc_fwd2.cu)
-        int armed_do = 0;
-        if (prep.with_bwd && nkt > 0) {
-            bool free = true;
-            for (int s = dslot; free && s < dslot + (NB == 3 ? 1 : 2); ++s) {
-                const int uses = (nkt * S::kChunks - s + S::kKSlots - 1) / S::kKSlots;
-                free = uses <= 0 || mbar_wait(bars + FW_KEMPTY + s, (uses - 1) & 1, abortp, status, ERRW_K);
+            for (int g = early_k; g < nkt * S::kChunks; ++g) {
+                if (!mbar_wait(bars + FW_KEMPTY + g % S::kKSlots, (g / S::kKSlots - 1) & 1, abortp, status, ERRW_K)) break;
+                load_k(g);
+                ++nk;
             }
-            if (free) {
-                mbar_arrive_expect_tx(bars + FW_DO, NB * S::kBox);
-                armed_do = 1;
-                for (int b = 0; b < NB; ++b) tma_load_4d(sK + dslot * S::kKSlot + b * S::kBox, &mapdO, bars + FW_DO, 64 * b, q0, hq, bb);
+            // fused call: the dO tile, which the epilogue multiplies its rows with, goes over K slots that have come free (see tc_fwd2.cu)
+            int armed_do = 0;
+            if (prep.with_bwd && nkt > 0) {
+                bool free = true;
+                for (int s = dslot; free && s < dslot + (NB == 3 ? 1 : 2); ++s) {
+                    const int uses = (nkt * S::kChunks - s + S::kKSlots - 1) / S::kKSlots;
+                    free = uses <= 0 || mbar_wait(bars + FW_KEMPTY + s, (uses - 1) & 1, abortp, status, ERRW_K);
+                }
+                if (free) {
+                    mbar_arrive_expect_tx(bars + FW_DO, NB * S::kBox);
+                    armed_do = 1;
+                    for (int b = 0; b < NB; ++b) tma_load_4d(sK + dslot * S::kKSlot + b * S::kBox, &mapdO, bars + FW_DO, 64 * b, q0, hq, bb);
+                }
             }
-        }
-        if (*abortp) {
-            mbar_drain_one(bars + FW_DO, armed_do);
-            mbar_drain_one(bars + FW_Q, early_k > 0 ? 1 : 0);
-            for (int s = 0; s < S::kKSlots; ++s) mbar_drain_one(bars + FW_KFULL + s, nk > s ? (nk - s + S::kKSlots - 1) / S::kKSlots : 0);
-        }
+            if (*abortp) {
+                mbar_drain_one(bars + FW_DO, armed_do);
+                mbar_drain_one(bars + FW_Q, early_k > 0 ? 1 : 0);
+                for (int s = 0; s < S::kKSlots; ++s) mbar_drain_one(bars + FW_KFULL + s, nk > s ? (nk - s + S::kKSlots - 1) / S::kKSlots : 0);
+            }
         }
       } else if (warp == 11 && elect_one()) {
         // ------------------------------------------------------------------ TMA producer of V
@@ -191,7 +191,8 @@ tc_fwd_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_consta
             for (int s = 0; s < S::kVSlots; ++s) mbar_drain_one(bars + FW_VFULL + s, nv > s ? (nv - s + S::kVSlots - 1) / S::kVSlots : 0);
       } else if (warp == 9 && elect_one()) {
         // ------------------------------------------- UMMA issuer (one thread): S(j + 2), P V(j), S(j + 3), ... (why: tc_fwd2.cu)
-        // Two threads / one, forward alone: B1 H16/4 n3001 d192 causal 58.5 / 54.6 us, B1 H8 n8192 d192 316.5 / 304, B2 H16 n4096 d256 causal 234 / 227.5.
+        // Two threads / one, forward alone, in turn: runs of 40 ms under the power cap B1 H16/4 n3001 d192 causal 60.1 / 57.0 us, B1 H8 n8192 d192 360 / 346,
+        // B2 H16 n4096 d256 causal 268 / 261; at 1965 MHz B1 H8 n1500 d256 24.6 / 22.3.
         constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 0, 0), idesc_pv = idesc_bf16_f32(128, 64 * NB, 0, 1);
         const uint64_t km_proto = smem_desc_sw128(0, 16, 1024), mn_proto = smem_desc_sw128(0, S::kVBox, 1024);
         const uint32_t km_hi = (uint32_t)(km_proto >> 32), mn_hi = (uint32_t)(mn_proto >> 32);
